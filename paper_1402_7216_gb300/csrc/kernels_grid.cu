@@ -2731,6 +2731,7 @@ cudaError_t configure_kernels() {
   set((const void*)k_interp_bwd<double, 5, double>);
   set((const void*)k_interp_bwd<double, 5, float>);
   if (e == cudaSuccess) e = configure_fft_kernels();
+  if (e == cudaSuccess) e = configure_pair64_kernels();
   return e;
 }
 

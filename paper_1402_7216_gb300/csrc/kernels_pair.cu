@@ -1,5 +1,5 @@
-// kernels_pair.cu -- short-range part of MSM (Sec. "Multilevel Summation
-// Method"): u_i^short = sum_{j != i, r_ij < a} q_j g*(r_ij) with
+// kernels_pair.cu -- short-range part of MSM on mixed plans (FP64 plans:
+// kernels_pair64.cu) (Sec. "Multilevel Summation Method"): u_i^short = sum_{j != i, r_ij < a} q_j g*(r_ij) with
 // g*(r) = 1/r - gamma(r/a)/a (Eq. msmgrid), and the force
 // F_i = -q_i grad_i u_i^short.
 //
@@ -13,15 +13,25 @@
 // operations; rejected pairs are masked, not branched.  Mixed precision sums
 // each batch in FP32 and folds the batch sums into the running totals with an
 // error-free TwoSum (compensated accumulation).
-#include <climits>
-#include <cmath>
 #include <new>
 
-#include "msm_internal.h"
+#include "pair_common.h"
 
 namespace msm {
 
 namespace {
+
+PairArgs pair_args(const Plan& P) {
+  PairArgs A;
+  for (int d = 0; d < 3; ++d) A.nc[d] = P.nc[d];
+  A.periodic = P.P.periodic;
+  const double a = P.P.cutoff;
+  A.a2f = (float)(a * a);
+  A.inv_af = (float)(1.0 / a);
+  A.inv_a2f = (float)(1.0 / (a * a));
+  A.two_inv_a3f = (float)(2.0 / (a * a * a));
+  return A;
+}
 
 template <typename T, int M>
 struct Smooth;  // gamma(rho) and d gamma / d s as polynomials in s = rho^2 < 1
@@ -53,64 +63,6 @@ __device__ __forceinline__ void two_sum_add(T& s, T& c, T x) {
   s = t;
 }
 
-// Cutoff constants are precomputed on the host in both precisions: a divide
-// in FP64 on every thread would cost dozens of FP64-pipe operations.
-struct PairArgs {
-  int nc[3];
-  int periodic;
-  int noff;
-  double a2, inv_a, inv_a2, two_inv_a3;
-  float a2f, inv_af, inv_a2f, two_inv_a3f;
-};
-
-// Constants of the Wolf pair function (damped, shifted force) with damping
-// alpha and cutoff R = a: v(r) = erfc(alpha r)/r - vR + c1 (r - R),
-// vR = erfc(alpha R)/R, c1 = erfc(alpha R)/R^2 + c2 exp(-alpha^2 R^2)/R,
-// c2 = 2 alpha/sqrt(pi).
-template <typename T>
-struct WolfC {
-  T alpha, alpha2, c2, vR, c1, R;
-};
-
-template <typename T>
-WolfC<T> wolf_consts(double alpha, double R) {
-  const double c2 = 2.0 * alpha / std::sqrt(M_PI);
-  const double vR = std::erfc(alpha * R) / R;
-  const double c1 = std::erfc(alpha * R) / (R * R) + c2 * std::exp(-alpha * alpha * R * R) / R;
-  return WolfC<T>{(T)alpha, (T)(alpha * alpha), (T)c2, (T)vR, (T)c1, (T)R};
-}
-
-__device__ __forceinline__ float d_erfc(float x) { return erfcf(x); }
-__device__ __forceinline__ double d_erfc(double x) { return erfc(x); }
-__device__ __forceinline__ float d_exp(float x) { return expf(x); }
-__device__ __forceinline__ double d_exp(double x) { return exp(x); }
-
-template <typename T>
-struct CutoffConsts;
-template <>
-struct CutoffConsts<double> {
-  __device__ static void get(const PairArgs& A, double& a2, double& ia, double& ia2, double& t3) {
-    a2 = A.a2; ia = A.inv_a; ia2 = A.inv_a2; t3 = A.two_inv_a3;
-  }
-};
-
-PairArgs pair_args(const Plan& P) {
-  PairArgs A;
-  for (int d = 0; d < 3; ++d) A.nc[d] = P.nc[d];
-  A.periodic = P.P.periodic;
-  A.noff = P.noff;
-  const double a = P.P.cutoff;
-  A.a2 = a * a;
-  A.inv_a = 1.0 / a;
-  A.inv_a2 = 1.0 / (a * a);
-  A.two_inv_a3 = 2.0 / (a * a * a);
-  A.a2f = (float)A.a2;
-  A.inv_af = (float)A.inv_a;
-  A.inv_a2f = (float)A.inv_a2;
-  A.two_inv_a3f = (float)A.two_inv_a3;
-  return A;
-}
-
 constexpr int kWarps = 4;
 #ifndef MSM_PAIR_BATCH
 #define MSM_PAIR_BATCH 64
@@ -119,25 +71,12 @@ constexpr int kWarps = 4;
 #define MSM_PAIR_MINB 6
 #endif
 constexpr int kBatch = MSM_PAIR_BATCH;  // sources per queue drain (pairs per lane per drain)
-constexpr unsigned kFull = 0xffffffffu;
 
 __device__ __forceinline__ float fast_rsqrt(float x) {  // one MUFU.RSQ; inputs are >= a^2/... never denormal
   float y;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-__device__ __forceinline__ double fast_rsqrt(double x) { return rsqrt(x); }
-
-template <typename T>
-__device__ __forceinline__ T far_away() { return T(1e18); }
-
-// Pair functions: K = 0 is MSM's short-range kernel g*(r) = 1/r - gamma(r/a)/a
-// (zero with its derivative at r = a); K = 1 is the plain Coulomb law 1/r of
-// the cutoff method (the parareal section's coarse propagator G), which is
-// not zero at a, so sources beyond the cutoff are masked; K = 2 is Wolf
-// summation's damped, shifted-force pair potential (another coarse function
-// of that section), masked beyond a as well.
-constexpr int kPairMSM = 0, kPairCutoff = 1, kPairWolf = 2;
 
 // One pair, scalar: target ai against source b (skipped at r = 0, the atom
 // itself, and beyond the cutoff); adds q_j times the pair potential to pphi
@@ -170,119 +109,6 @@ __device__ __forceinline__ void pair1(const R4<T>& ai, const R4<T>& b, T a2, T i
   pz += f * dz;
 }
 
-// One batch: the lane's target atom against the kBatch queued sources.
-template <typename T, int M, bool COMP, int K = kPairMSM, int NB = kBatch>
-__device__ __forceinline__ void pair_batch(const R4<T>* __restrict__ Q, const R4<T>& ai, T a2, T inv_a,
-                                           T inv_a2, T two_inv_a3, const WolfC<T>& W, T& phi, T& fx, T& fy,
-                                           T& fz, T& cphi, T& cfx, T& cfy, T& cfz) {
-  T pphi = 0, px = 0, py = 0, pz = 0;
-#pragma unroll 8
-  for (int jj = 0; jj < NB; ++jj) pair1<T, M, K>(ai, Q[jj], a2, inv_a, inv_a2, two_inv_a3, W, pphi, px, py, pz);
-  if (COMP) {
-    two_sum_add(phi, cphi, pphi);
-    two_sum_add(fx, cfx, px);
-    two_sum_add(fy, cfy, py);
-    two_sum_add(fz, cfz, pz);
-  } else {
-    phi += pphi;
-    fx += px;
-    fy += py;
-    fz += pz;
-  }
-}
-
-// One warp per cell.  For every neighbour cell in reach, the warp stages 32
-// source atoms at a time (shifted into the target cell's frame), drops those
-// farther than a from the bounding box of its target atoms, and appends the
-// rest to a per-warp queue in shared memory; each full queue of kBatch
-// sources is one fully unrolled batch of pair evaluations.
-template <typename T, int M, bool COMP, int K>
-__global__ void __launch_bounds__(32 * kWarps) k_short_range(
-    const R4<T>* __restrict__ atoms, const int* __restrict__ cell_start,
-    const int4* __restrict__ offs, const R4<T>* __restrict__ shifts, PairArgs A, WolfC<T> W, int ncell,
-    T* __restrict__ phis, R4<T>* __restrict__ fs) {
-  __shared__ R4<T> queue[kWarps][2 * kBatch];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  R4<T>* Q = queue[warp];
-  const int cell = blockIdx.x * kWarps + warp;
-  if (cell >= ncell) return;  // warp-uniform
-  const int cx = cell % A.nc[0], cy = (cell / A.nc[0]) % A.nc[1], cz = cell / (A.nc[0] * A.nc[1]);
-  T a2, inv_a, inv_a2, two_inv_a3;
-  CutoffConsts<T>::get(A, a2, inv_a, inv_a2, two_inv_a3);
-  const R4<T> dummy = {far_away<T>(), far_away<T>(), far_away<T>(), T(0)};
-  const int i0 = cell_start[cell], i1 = cell_start[cell + 1];
-  for (int ib = i0; ib < i1; ib += 32) {
-    const int i = ib + lane;
-    const bool iv = i < i1;
-    R4<T> ai = iv ? atoms[i] : R4<T>{T(0), T(0), T(0), T(0)};
-    // bounding box of this chunk's target atoms
-    T lx = iv ? ai.x : far_away<T>(), ly = iv ? ai.y : far_away<T>(), lz = iv ? ai.z : far_away<T>();
-    T hx = iv ? ai.x : -far_away<T>(), hy = iv ? ai.y : -far_away<T>(), hz = iv ? ai.z : -far_away<T>();
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      lx = min(lx, __shfl_xor_sync(kFull, lx, o));
-      ly = min(ly, __shfl_xor_sync(kFull, ly, o));
-      lz = min(lz, __shfl_xor_sync(kFull, lz, o));
-      hx = max(hx, __shfl_xor_sync(kFull, hx, o));
-      hy = max(hy, __shfl_xor_sync(kFull, hy, o));
-      hz = max(hz, __shfl_xor_sync(kFull, hz, o));
-    }
-    T phi = 0, fx = 0, fy = 0, fz = 0, cphi = 0, cfx = 0, cfy = 0, cfz = 0;
-    int qn = 0;  // queued sources (warp-uniform)
-    for (int o = 0; o < A.noff; ++o) {
-      const int4 off = offs[o];
-      int nx = cx + off.x, ny = cy + off.y, nz = cz + off.z;
-      if (A.periodic) {
-        nx = (nx + A.nc[0]) % A.nc[0];
-        ny = (ny + A.nc[1]) % A.nc[1];
-        nz = (nz + A.nc[2]) % A.nc[2];
-      } else if (nx < 0 || ny < 0 || nz < 0 || nx >= A.nc[0] || ny >= A.nc[1] || nz >= A.nc[2]) {
-        continue;
-      }
-      const int nb = (nz * A.nc[1] + ny) * A.nc[0] + nx;
-      const R4<T> sh = shifts[o];
-      const int j0 = cell_start[nb], j1 = cell_start[nb + 1];
-      for (int jb = j0; jb < j1; jb += 32) {
-        const int j = jb + lane;
-        R4<T> aj = dummy;
-        if (j < j1) {
-          aj = atoms[j];
-          aj.x += sh.x;
-          aj.y += sh.y;
-          aj.z += sh.z;
-        }
-        const T ex = max(max(lx - aj.x, aj.x - hx), T(0));
-        const T ey = max(max(ly - aj.y, aj.y - hy), T(0));
-        const T ez = max(max(lz - aj.z, aj.z - hz), T(0));
-        const bool keep = (j < j1) && (ex * ex + ey * ey + ez * ez < a2);
-        const unsigned bal = __ballot_sync(kFull, keep);
-        if (keep) Q[qn + __popc(bal & ((1u << lane) - 1u))] = aj;
-        qn += __popc(bal);
-        __syncwarp();
-        if (qn >= kBatch) {
-          pair_batch<T, M, COMP, K>(Q, ai, a2, inv_a, inv_a2, two_inv_a3, W, phi, fx, fy, fz, cphi, cfx, cfy, cfz);
-          __syncwarp();
-          if (lane < qn - kBatch) Q[lane] = Q[kBatch + lane];
-          qn -= kBatch;
-          __syncwarp();
-        }
-      }
-    }
-    if (qn > 0) {  // last partial batch, padded with far-away zero charges
-      for (int t = lane; t < kBatch; t += 32)
-        if (t >= qn) Q[t] = dummy;
-      __syncwarp();
-      pair_batch<T, M, COMP, K>(Q, ai, a2, inv_a, inv_a2, two_inv_a3, W, phi, fx, fy, fz, cphi, cfx, cfy, cfz);
-      __syncwarp();
-    }
-    if (iv) {
-      phis[i] = phi + cphi;
-      const T qi = ai.w;
-      fs[i] = R4<T>{-qi * (fx + cfx), -qi * (fy + cfy), -qi * (fz + cfz), T(0)};
-    }
-  }
-}
-
 // ---- mixed precision: packed FP32x2 arithmetic (two sources per instruction) ----
 // The queue is stored as four FP32 arrays (x, y, z, q), so sources j..j+3
 // load as one float4 per array and feed FFMA2/FMUL2/FADD2 as two pairs.  With
@@ -293,17 +119,6 @@ __global__ void __launch_bounds__(32 * kWarps) k_short_range(
 // sits at 1e6 so that the unmasked polynomial stays finite.
 struct alignas(16) QueueF {
   float x[2 * kBatch], y[2 * kBatch], z[2 * kBatch], q[2 * kBatch];
-};
-
-// gamma(r/a)/a and (2/a^3) dgamma/ds written straight as polynomials in r^2
-// (host-scaled coefficients, duplicated into float2 pairs):
-//   pot = 1/r - sum_k G[k] r2^k,   f' = 1/r^3 + sum_k D[k] r2^k.
-// Beyond the cutoff r2 is clamped to a^2: pot and f' are zero there up to
-// FP32 rounding (a few 1e-8 / a per source, measured to leave the energy and
-// forces of the 1.07M-atom water box unchanged at the 1e-8 / 1e-7 level).
-struct PairCoef {
-  float2 G[4];
-  float2 D[3];
 };
 
 template <int M>
@@ -422,32 +237,10 @@ __device__ __forceinline__ void pair_batch_f2(const QueueF& Q, float2 nax, float
 // chunks of 32 sources, loading the next chunk's atoms before it works on the
 // current one.  The x offset of a source's cell follows from comparing its
 // index with the cell starts inside its segment.
-constexpr int kMaxRows = 32;  // rows per cell: cells at least a/2 wide give at most 26
-
 struct SegTable {
   int4 rec[2 * kMaxRows + 1];   // (first atom, flat start, x offset of the first cell, -); sentinel at the end
   int4 bnd[2 * kMaxRows];       // first atom of the segment's 2nd..5th cell (INT_MAX where absent)
   float2 shift[2 * kMaxRows];   // (y, z) shift of the row
-};
-
-// Arguments of the packed pair kernel (one system).
-struct PairKArgs {
-  const R4<float>* atoms;
-  const int* cell_start;
-  const int4* rows;
-  int nrows;
-  PairArgs A;
-  PairCoef C;
-  WolfC<float> W;
-  float cwx, cwy, cwz;
-  int ncell;
-  float* phis;
-  R4<float>* fs;
-  // target runs (short_range_run_body): cell of every input atom, the sorted
-  // order's input indices and the atom count
-  const int* key;
-  const int* perm;
-  int natoms;
 };
 
 // The segment table of cell (cx, cy, cz), built by the warp (lane r: row r);
@@ -929,117 +722,6 @@ __device__ __forceinline__ void short_range_c8_body(const PairKArgs& K, int blk)
 // own cells), walked as one flat index space, culled against the piece's
 // bounding box and queued.  A periodic row then spans up to seven cells, so
 // the runs need at least seven cells in x.
-constexpr int kRunBnd = 6;  // boundaries inside a row segment of up to 7 cells
-struct SegTableR {
-  int4 rec[2 * kMaxRows + 1];         // (first atom, flat start, x offset of the first cell, -); sentinel at the end
-  int4 bnd[2 * kMaxRows];             // first atom of the segment's 2nd..5th cell (INT_MAX where absent)
-  int2 bnd2[2 * kMaxRows];            // ... of its 6th and 7th cell
-  float2 shift[2 * kMaxRows];         // (y, z) shift of the row
-};
-
-// The segment table of the rows about cells (cx .. cx + span, cy, cz): as
-// build_seg_table, each row widened by span cells in +x (the home row's
-// right part moved past the piece's cells), then narrowed to the cells a
-// source within a of the targets' bounding box (lx..hx, ly..hy, lz..hz, in
-// the frame of cell cx) can lie in: a row at y gap gy and z gap gz from the
-// box reaches sqrt(a^2 - gy^2 - gz^2) beyond it in x (with a margin for
-// rounding; the culling tests each source exactly).
-__device__ __forceinline__ int build_seg_table_run(SegTableR& T, const PairKArgs& K, int cx, int cy, int cz, int span,
-                                                   float lx, float ly, float lz, float hx, float hy, float hz,
-                                                   int lane) {
-  const int* __restrict__ cell_start = K.cell_start;
-  const PairArgs& A = K.A;
-  const int ncx = A.nc[0], ncy = A.nc[1], ncz = A.nc[2];
-  const int nrows = K.nrows;
-  const float cwy = K.cwy, cwz = K.cwz;
-  int len[2] = {0, 0}, j0s[2] = {0, 0}, ox0s[2] = {0, 0};
-  int bb[2][kRunBnd];
-#pragma unroll
-  for (int g = 0; g < 2; ++g)
-#pragma unroll
-    for (int t = 0; t < kRunBnd; ++t) bb[g][t] = INT_MAX;
-  float2 sh = make_float2(0.f, 0.f);
-  if (lane < nrows) {
-    int4 row = K.rows[lane];  // (dy, dz, xlo, xhi)
-    if (row.x == 0 && row.y == 0) {
-      if (row.z > 0) { row.z += span; row.w += span; }  // the home row's right part
-    } else {
-      row.w += span;
-    }
-    const float gy = fmaxf(fmaxf(row.x * cwy - hy, ly - (row.x + 1) * cwy), 0.f);
-    const float gz = fmaxf(fmaxf(row.y * cwz - hz, lz - (row.y + 1) * cwz), 0.f);
-    const float r2 = A.a2f - gy * gy - gz * gz;
-    bool inside = r2 > 0.f;
-    if (inside) {
-      const float reach = sqrtf(r2) * 1.0001f + 1e-3f;
-      row.z = max(row.z, (int)floorf((lx - reach) / K.cwx));
-      row.w = min(row.w, (int)floorf((hx + reach) / K.cwx));
-      inside = row.z <= row.w;
-    }
-    int ny = cy + row.x, nz = cz + row.y;
-    if (A.periodic) {
-      ny += (ny < 0) ? ncy : ((ny >= ncy) ? -ncy : 0);
-      nz += (nz < 0) ? ncz : ((nz >= ncz) ? -ncz : 0);
-    } else if (ny < 0 || nz < 0 || ny >= ncy || nz >= ncz) {
-      inside = false;
-    }
-    const int rbase = (nz * ncy + ny) * ncx;
-    sh = make_float2(row.x * cwy, row.y * cwz);
-#pragma unroll
-    for (int seg = 0; seg < 2; ++seg) {
-      int ox0 = 0, ox1 = -1;
-      if (!inside) {
-      } else if (A.periodic) {  // at most 7 <= ncx cells: the row wraps at one end at most
-        const int xa = cx + row.z, xb = cx + row.w;
-        if (xa < 0) {
-          if (seg == 0) { ox0 = row.z; ox1 = -cx - 1; } else { ox0 = -cx; ox1 = row.w; }
-        } else if (xb >= ncx) {
-          if (seg == 0) { ox0 = row.z; ox1 = ncx - 1 - cx; } else { ox0 = ncx - cx; ox1 = row.w; }
-        } else if (seg == 0) {
-          ox0 = row.z; ox1 = row.w;
-        }
-      } else if (seg == 0) {
-        ox0 = max(row.z, -cx);
-        ox1 = min(row.w, ncx - 1 - cx);
-      }
-      if (ox0 <= ox1) {
-        int x0 = cx + ox0, x1 = cx + ox1;
-        if (A.periodic) {
-          x0 += (x0 < 0) ? ncx : ((x0 >= ncx) ? -ncx : 0);
-          x1 += (x1 < 0) ? ncx : ((x1 >= ncx) ? -ncx : 0);
-        }
-        const int j0 = cell_start[rbase + x0], j1 = cell_start[rbase + x1 + 1];
-#pragma unroll
-        for (int t = 0; t < kRunBnd; ++t) bb[seg][t] = (x0 + 1 + t <= x1) ? cell_start[rbase + x0 + 1 + t] : INT_MAX;
-        len[seg] = j1 - j0;
-        j0s[seg] = j0;
-        ox0s[seg] = ox0;
-      }
-    }
-  }
-  const int mine = len[0] + len[1];
-  int incl = mine;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(kFull, incl, o);
-    if (lane >= o) incl += y;
-  }
-  const int total = __shfl_sync(kFull, incl, 31);
-  const int start = incl - mine;
-  if (lane < nrows) {
-#pragma unroll
-    for (int seg = 0; seg < 2; ++seg) {
-      T.rec[2 * lane + seg] = make_int4(j0s[seg], seg ? start + len[0] : start, ox0s[seg], 0);
-      T.bnd[2 * lane + seg] = make_int4(bb[seg][0], bb[seg][1], bb[seg][2], bb[seg][3]);
-      T.bnd2[2 * lane + seg] = make_int2(bb[seg][4], bb[seg][5]);
-      T.shift[2 * lane + seg] = sh;
-    }
-  }
-  if (lane == 0) T.rec[2 * nrows] = make_int4(0, INT_MAX, 0, 0);
-  __syncwarp();
-  return total;
-}
-
 template <int M, int KIND>
 __device__ __forceinline__ void short_range_run_body(const PairKArgs& K, int blk) {
   const R4<float>* __restrict__ atoms = K.atoms;
@@ -1226,31 +908,6 @@ __global__ void __launch_bounds__(32 * kWarps, MSM_PAIR_MINB) kb_short_range_f2(
   short_range_f2_body<M, kPairMSM>(tab[r], blockIdx.x - first[r]);
 }
 
-template <typename T, bool COMP, int K>
-void launch_t(Plan& P, cudaStream_t st, double alpha = 0.0) {
-  PairArgs A = pair_args(P);
-  const WolfC<T> W = wolf_consts<T>(alpha, P.P.cutoff);
-  int blocks = (P.ncell + kWarps - 1) / kWarps;
-  auto* at = (const R4<T>*)P.d.atoms;
-  auto* sh = (const R4<T>*)P.d.cell_shift;
-  auto* ph = (T*)P.d.phis;
-  auto* fs = (R4<T>*)P.d.fs;
-  switch (P.P.splitting) {
-    case 1:
-      k_short_range<T, 1, COMP, K><<<blocks, 32 * kWarps, 0, st>>>(at, P.d.cell_start, P.d.cell_off, sh, A, W,
-                                                               P.ncell, ph, fs);
-      break;
-    case 2:
-      k_short_range<T, 2, COMP, K><<<blocks, 32 * kWarps, 0, st>>>(at, P.d.cell_start, P.d.cell_off, sh, A, W,
-                                                               P.ncell, ph, fs);
-      break;
-    default:
-      k_short_range<T, 3, COMP, K><<<blocks, 32 * kWarps, 0, st>>>(at, P.d.cell_start, P.d.cell_off, sh, A, W,
-                                                               P.ncell, ph, fs);
-      break;
-  }
-}
-
 }  // namespace
 
 PairKArgs pair_kargs(const Plan& P) {
@@ -1324,25 +981,25 @@ void launch_f2(Plan& P, int64_t n, cudaStream_t st, double alpha = 0.0) {
 
 cudaError_t launch_short_range(Plan& P, int64_t n, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  if (P.fp64) launch_t<double, false, kPairMSM>(P, st);
-  else launch_f2<kPairMSM>(P, n, st);
   P.launches += 1;
+  if (P.fp64) return launch_pair64(P, kPairMSM, n, 0.0, st);
+  launch_f2<kPairMSM>(P, n, st);
   return cudaGetLastError();
 }
 
 cudaError_t launch_cutoff_pairs(Plan& P, int64_t n, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  if (P.fp64) launch_t<double, false, kPairCutoff>(P, st);
-  else launch_f2<kPairCutoff>(P, n, st);
   P.launches += 1;
+  if (P.fp64) return launch_pair64(P, kPairCutoff, n, 0.0, st);
+  launch_f2<kPairCutoff>(P, n, st);
   return cudaGetLastError();
 }
 
 cudaError_t launch_wolf_pairs(Plan& P, int64_t n, double alpha, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  if (P.fp64) launch_t<double, false, kPairWolf>(P, st, alpha);
-  else launch_f2<kPairWolf>(P, n, st, alpha);
   P.launches += 1;
+  if (P.fp64) return launch_pair64(P, kPairWolf, n, alpha, st);
+  launch_f2<kPairWolf>(P, n, st, alpha);
   return cudaGetLastError();
 }
 

@@ -1,0 +1,376 @@
+// kernels_pair64.cu -- the short-range pair sums of FP64 plans (the same sums
+// as kernels_pair.cu, every pair function in FP64).
+//
+// This GPU issues FP64 at 1/64 of the FP32 rate (2 lanes per SM and clock), so
+// the kernel is bound by the number of FP64 instructions and nothing else:
+// 22 per MSM pair, and only pairs inside the cutoff are worth them.  The
+// candidates of a target's neighbourhood are ~2,000 sources (culled against
+// the bounding box of a warp's targets), ~750 of them inside a 12 A cutoff at
+// water density.  So the kernel separates finding from evaluating:
+//   - sources are staged 32 at a time in a ring of shared memory (FP64
+//     coordinates in the targets' frame, and their FP32 truncation), and every
+//     lane tests every staged source against its own target in FP32, with a
+//     margin for the truncation; a hit goes onto the lane's own list (one byte,
+//     the ring slot).  This costs ~10 FP32-rate instructions per source, under
+//     5 % of the FP64 time.
+//   - the lanes then pop their lists in step and evaluate one pair each, all
+//     lanes on real pairs.  The cutoff and r > 0 are decided again in FP64 (on
+//     the bit patterns, which order like the values and cost no FP64
+//     instruction).  Lists of different lanes fill unevenly as the walk passes
+//     through the neighbourhood; the ring keeps up to 256 sources alive so that
+//     a lane ahead of the others still has entries.
+// The reciprocal square root is seeded by the FP32 one and refined once by
+// Halley's third-order iteration (5 FP64 instructions, error below 1 ulp more
+// than half a rounding).
+//
+// A group of T = 8, 16 or 32 consecutive sorted atoms is a warp's targets,
+// 32 / T lanes sharing one (each tests every (32 / T)-th source); small systems
+// also split a group's sources over 2 to 8 warps of a block, combined in a
+// fixed order.  Groups are cut into pieces of one cell row as the target runs
+// of kernels_pair.cu are.
+#include <algorithm>
+
+#include "pair_common.h"
+
+namespace msm {
+
+namespace {
+
+constexpr int kRing = 256;   // staged sources (a list entry is one byte)
+constexpr int kChunk = 32;   // sources staged together
+constexpr int kMaxSplit = 8; // warps sharing a group
+constexpr int kShift0 = 3;   // index of offset 0 in the shift tables
+
+struct Pair64Args {
+  PairKArgs g;  // geometry: cell widths and cutoff in FP32, scaled by 2^esc (a in [1, 2))
+  const R4<double>* atoms;
+  double* phis;
+  R4<double>* fs;
+  double a2;
+  double G[4], D[3];  // pot = 1/r + sum_k G[k] r2^k, f' = 1/r^3 + sum_k D[k] r2^k
+  WolfC<double> W;
+  double shx[8], shy[8], shz[8];  // offset (index - kShift0) times the cell width
+  float a2test;                   // scaled cutoff^2 with the margin of the FP32 test
+  int esc;                        // exponent added to coordinates before the FP32 test
+  int lt;                         // log2 of the targets per group
+  int nsplit;                     // warps sharing a group (1: a block's warps take groups of their own)
+  int maxspan;                    // cells a piece may add to its first one
+};
+
+struct alignas(16) Warp64 {
+  double src[kRing][4];  // x, y, z, q in the piece's frame
+  float fx[kRing], fy[kRing], fz[kRing];
+  unsigned char list[kRing][32];
+  SegTableR tab;
+};
+
+// x 2^esc truncated to FP32 (integer operations only: conversions from FP64
+// run at the FP64 rate).
+__device__ __forceinline__ float trunc_scaled(double x, int esc) {
+  const int hi = __double2hiint(x);
+  const int e = ((hi >> 20) & 0x7ff) - 896 + esc;
+  if (e <= 0) return 0.f;
+  return __int_as_float((hi & 0x80000000) | (e << 23) | ((hi & 0xfffff) << 3) |
+                        (int)((unsigned)__double2loint(x) >> 29));
+}
+
+// 1 / sqrt(x), x > 0 and normal: the FP32 approximation of the mantissa, its
+// exponent halved with integers, then y (1 + r/2 + 3 r^2/8), r = 1 - x y^2
+// (Halley's iteration; the next term, 5 r^3/16 with |r| < 2^-21, is below
+// 2^-64).
+__device__ __forceinline__ double rsqrt_halley(double x) {
+  const int hi = __double2hiint(x);
+  const int e = (hi >> 20) - 1023, odd = e & 1;
+  const float m = __int_as_float(((127 + odd) << 23) | ((hi & 0xfffff) << 3) |
+                                 (int)((unsigned)__double2loint(x) >> 29));
+  float s;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"(m));
+  const int sb = __float_as_int(s);
+  const double y = __hiloint2double((sb >> 3) + ((896 - ((e - odd) >> 1)) << 20), sb << 29);
+  const double r = fma(-(x * y), y, 1.0);
+  return fma(y * r, fma(0.375, r, 0.5), y);
+}
+
+// One pair: q_j times the pair potential onto phi, f' (r_i - r_j) onto
+// (px, py, pz), with the force on i being q_i times that sum.
+template <int M, int K>
+__device__ __forceinline__ void pair64(const Pair64Args& A, double tx, double ty, double tz, const double* src,
+                                       double& phi, double& px, double& py, double& pz) {
+  const double2 xy = *reinterpret_cast<const double2*>(src), zq = *reinterpret_cast<const double2*>(src + 2);
+  const double dx = tx - xy.x, dy = ty - xy.y, dz = tz - zq.x;
+  const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
+  const long long rb = __double_as_longlong(r2);
+  const bool ok = rb < __double_as_longlong(A.a2) && rb > 0;  // inside the cutoff, not the atom itself
+  const double r2s = ok ? r2 : A.a2, q = ok ? zq.y : 0.0;
+  const double ri = rsqrt_halley(r2s);
+  double f;
+  if (K == kPairMSM) {
+    double g = A.G[M];
+#pragma unroll
+    for (int k = M - 1; k >= 0; --k) g = fma(g, r2s, A.G[k]);
+    double d = A.D[M - 1];
+#pragma unroll
+    for (int k = M - 2; k >= 0; --k) d = fma(d, r2s, A.D[k]);
+    phi = fma(q, ri + g, phi);
+    f = q * fma(ri * ri, ri, d);
+  } else if (K == kPairWolf) {
+    const double r = r2s * ri;
+    const double e = d_erfc(A.W.alpha * r) * ri, x = A.W.c2 * d_exp(-A.W.alpha2 * r2s);
+    phi = fma(q, e - A.W.vR + A.W.c1 * (r - A.W.R), phi);
+    f = q * ((e + x) * ri * ri - A.W.c1 * ri);
+  } else {
+    phi = fma(q, ri, phi);
+    f = q * (ri * ri * ri);
+  }
+  px = fma(f, dx, px);
+  py = fma(f, dy, py);
+  pz = fma(f, dz, pz);
+}
+
+template <int M, int K>
+__global__ void __launch_bounds__(32 * kMaxSplit) k_pair64(const __grid_constant__ Pair64Args A) {
+  extern __shared__ __align__(16) unsigned char smem64[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  Warp64& S = reinterpret_cast<Warp64*>(smem64)[warp];
+  const PairKArgs& g = A.g;
+  const int T = 1 << A.lt, t = lane & (T - 1), h = lane >> A.lt, lpt = 32 >> A.lt;
+  const bool split = A.nsplit > 1;
+  const int group = split ? blockIdx.x : blockIdx.x * (blockDim.x >> 5) + warp, part = split ? warp : 0;
+  const int s0 = group << A.lt;
+  if (s0 >= g.natoms) return;  // warp-uniform; block-uniform where the block shares the group
+  const int nval = min(T, g.natoms - s0);
+  const int ncx = g.A.nc[0], ncy = g.A.nc[1];
+  const float FAR = 1e6f;
+  const bool sv = t < nval;
+  const int mycell = sv ? g.key[g.perm[s0 + t]] : INT_MAX;
+  const R4<double> me = sv ? A.atoms[s0 + t] : R4<double>{0.0, 0.0, 0.0, 0.0};
+  for (int l0 = 0; l0 < nval;) {  // one piece per step (the same for every warp of the group)
+    const int c0 = __shfl_sync(kFull, mycell, l0);
+    const int cx = c0 % ncx, cy = (c0 / ncx) % ncy, cz = c0 / (ncx * ncy);
+    const int climit = c0 + min(A.maxspan, ncx - 1 - cx);
+    const bool inp = t >= l0 && mycell <= climit;
+    const unsigned pb = __ballot_sync(kFull, inp) & (kFull >> (32 - T));
+    const int l1 = 32 - __clz(pb);
+    const int span = __shfl_sync(kFull, mycell, l1 - 1) - c0;
+    // the home block: the atoms of the piece's cells
+    const int h0 = g.cell_start[c0];
+    const int b1 = span >= 1 ? g.cell_start[c0 + 1] : INT_MAX;
+    const int b2 = span >= 2 ? g.cell_start[c0 + 2] : INT_MAX;
+    const int hlen = g.cell_start[c0 + span + 1] - h0;
+    const double tx = me.x + A.shx[(inp ? mycell - c0 : 0) + kShift0], ty = me.y, tz = me.z;
+    const float ux = trunc_scaled(tx, A.esc), uy = trunc_scaled(ty, A.esc), uz = trunc_scaled(tz, A.esc);
+    float lx = inp ? ux : FAR, ly = inp ? uy : FAR, lz = inp ? uz : FAR;
+    float hx = inp ? ux : -FAR, hy = inp ? uy : -FAR, hz = inp ? uz : -FAR;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      lx = fminf(lx, __shfl_xor_sync(kFull, lx, o));
+      ly = fminf(ly, __shfl_xor_sync(kFull, ly, o));
+      lz = fminf(lz, __shfl_xor_sync(kFull, lz, o));
+      hx = fmaxf(hx, __shfl_xor_sync(kFull, hx, o));
+      hy = fmaxf(hy, __shfl_xor_sync(kFull, hy, o));
+      hz = fmaxf(hz, __shfl_xor_sync(kFull, hz, o));
+    }
+    const int flat = hlen + build_seg_table_run(S.tab, g, cx, cy, cz, span, lx, ly, lz, hx, hy, hz, lane);
+    const int nchunk = (flat + kChunk - 1) / kChunk;
+    double phi = 0.0, px = 0.0, py = 0.0, pz = 0.0;
+    unsigned staged = 0, oldest = 0;  // sources staged so far; the oldest one a list still names
+    unsigned head = 0, tail = 0;      // the lane's list: entries popped, entries pushed
+    int seg = 0, c = part;
+    for (;;) {
+      // find: stage chunks while the ring has room, test the new sources
+      while (c < nchunk && staged - oldest <= kRing - kChunk) {
+        const int f = c * kChunk + lane;
+        c += A.nsplit;
+        R4<double> a = {0.0, 0.0, 0.0, 0.0};
+        bool keep = f < flat;
+        if (keep) {
+          int j, ox, oyz = kShift0 | (kShift0 << 4);
+          if (f < hlen) {
+            j = h0 + f;
+            ox = (j >= b1) + (j >= b2);
+          } else {
+            const int v = f - hlen;
+            while (S.tab.rec[seg + 1].y <= v) ++seg;
+            const int4 r = S.tab.rec[seg], b = S.tab.bnd[seg];
+            const int2 e = S.tab.bnd2[seg];
+            j = r.x + (v - r.y);
+            ox = r.z + (j >= b.x) + (j >= b.y) + (j >= b.z) + (j >= b.w) + (j >= e.x) + (j >= e.y);
+            oyz = r.w;
+          }
+          a = A.atoms[j];
+          a.x += A.shx[ox + kShift0];
+          a.y += A.shy[oyz & 15];
+          a.z += A.shz[oyz >> 4];
+        }
+        const float ax = trunc_scaled(a.x, A.esc), ay = trunc_scaled(a.y, A.esc), az = trunc_scaled(a.z, A.esc);
+        const float ex = fmaxf(fmaxf(lx - ax, ax - hx), 0.f);
+        const float ey = fmaxf(fmaxf(ly - ay, ay - hy), 0.f);
+        const float ez = fmaxf(fmaxf(lz - az, az - hz), 0.f);
+        keep = keep && ex * ex + ey * ey + ez * ez < A.a2test;
+        const unsigned bal = __ballot_sync(kFull, keep);
+        if (keep) {
+          const int p = (staged + __popc(bal & ((1u << lane) - 1u))) & (kRing - 1);
+          S.fx[p] = ax;
+          S.fy[p] = ay;
+          S.fz[p] = az;
+          *reinterpret_cast<double2*>(&S.src[p][0]) = make_double2(a.x, a.y);
+          *reinterpret_cast<double2*>(&S.src[p][2]) = make_double2(a.z, a.w);
+        }
+        __syncwarp();
+        const unsigned end = staged + __popc(bal);
+#pragma unroll 4
+        for (unsigned s = staged + ((h - staged) & (lpt - 1)); s < end; s += lpt) {
+          const int p = s & (kRing - 1);
+          const float dx = ux - S.fx[p], dy = uy - S.fy[p], dz = uz - S.fz[p];
+          if (inp && dx * dx + dy * dy + dz * dz < A.a2test) S.list[tail++ & (kRing - 1)][lane] = (unsigned char)p;
+        }
+        staged = end;
+      }
+      // evaluate: every lane pops its own list; while more sources follow, as
+      // many steps as all lanes have entries for (at least 8, so that the
+      // ring's oldest source is let go)
+      const unsigned have = tail - head;
+      const bool more = c < nchunk;
+      const unsigned steps = more ? max(8u, __reduce_min_sync(kFull, inp ? have : 0xffffffffu))
+                                  : __reduce_max_sync(kFull, have);
+      double sphi = 0.0, sx = 0.0, sy = 0.0, sz = 0.0;
+      for (unsigned k = 0; k < steps; ++k)
+        if (head < tail) {
+          const int p = S.list[head++ & (kRing - 1)][lane];
+          pair64<M, K>(A, tx, ty, tz, S.src[p], sphi, sx, sy, sz);
+        }
+      phi += sphi;
+      px += sx;
+      py += sy;
+      pz += sz;
+      if (!more) break;
+      // the ring index of the lane's next entry lies 1 .. kRing sources back
+      const unsigned back = head < tail ? ((staged - 1u - S.list[head & (kRing - 1)][lane]) & (kRing - 1)) + 1u : 0u;
+      oldest = staged - __reduce_max_sync(kFull, back);
+      __syncwarp();
+    }
+    // the lanes of a target, then the parts of a group, in a fixed order
+    for (int o = T; o < 32; o <<= 1) {
+      phi += __shfl_xor_sync(kFull, phi, o);
+      px += __shfl_xor_sync(kFull, px, o);
+      py += __shfl_xor_sync(kFull, py, o);
+      pz += __shfl_xor_sync(kFull, pz, o);
+    }
+    if (split) {
+      __syncwarp();
+      if (lane < T) {
+        S.src[lane][0] = phi;
+        S.src[lane][1] = px;
+        S.src[lane][2] = py;
+        S.src[lane][3] = pz;
+      }
+      __syncthreads();
+      if (part == 0 && lane < T)
+        for (int p = 1; p < A.nsplit; ++p) {
+          const double* o = reinterpret_cast<Warp64*>(smem64)[p].src[lane];
+          phi += o[0];
+          px += o[1];
+          py += o[2];
+          pz += o[3];
+        }
+      __syncthreads();
+    }
+    if (part == 0 && h == 0 && inp) {
+      const int i = s0 + t;
+      A.phis[i] = phi;
+      A.fs[i] = R4<double>{me.w * px, me.w * py, me.w * pz, 0.0};
+    }
+    __syncwarp();
+    l0 = l1;
+  }
+}
+
+// Targets per group and warps per group: full warps of targets once their
+// number fills the GPU (152 SMs x 8 warps), else smaller groups, then several
+// warps per group.
+void group_shape(int64_t n, int& lt, int& nsplit) {
+  constexpr int64_t kFill = 152 * 8;
+  lt = 5;
+  nsplit = 1;
+  while (lt > 3 && ((n + (1 << lt) - 1) >> lt) < kFill) --lt;
+  while (nsplit < kMaxSplit && ((n + (1 << lt) - 1) >> lt) * nsplit < kFill * 3 / 4) nsplit *= 2;
+}
+
+Pair64Args pair64_args(const Plan& P, int64_t n, double alpha) {
+  Pair64Args A;
+  const double a = P.P.cutoff;
+  A.g = pair_kargs(P);
+  A.g.natoms = (int)n;
+  A.esc = -std::ilogb(a);
+  const double sc = std::ldexp(1.0, A.esc);
+  A.g.cwx = (float)(P.cw[0] * sc);
+  A.g.cwy = (float)(P.cw[1] * sc);
+  A.g.cwz = (float)(P.cw[2] * sc);
+  // a coordinate lies within X = 8 cell widths of the origin and its
+  // truncation is off by at most 2^-23 X, a difference by three times that
+  // (with its own rounding): r^2 near a^2 by 2 sqrt(3) a 3 2^-23 X (1 + small)
+  double X = 0.0;
+  for (int d = 0; d < 3; ++d) X = std::max(X, 8.0 * P.cw[d] * sc);
+  const double as = a * sc;
+  const double a2t = as * as + 16.0 * as * X * std::ldexp(1.0, -23) + 16.0 * X * X * std::ldexp(1.0, -46);
+  A.a2test = (float)(a2t * (1.0 + 1e-6));
+  A.g.A.a2f = A.a2test;
+  A.atoms = (const R4<double>*)P.d.atoms;
+  A.phis = (double*)P.d.phis;
+  A.fs = (R4<double>*)P.d.fs;
+  A.a2 = a * a;
+  static const double cf[4][4] = {{0, 0, 0, 0}, {1.5, -0.5, 0, 0}, {1.875, -1.25, 0.375, 0},
+                                  {2.1875, -2.1875, 1.3125, -0.3125}};
+  const int m = P.P.splitting;
+  for (int k = 0; k < 4; ++k) A.G[k] = k <= m ? -cf[m][k] / std::pow(a, 2 * k + 1) : 0.0;
+  for (int k = 0; k < 3; ++k) A.D[k] = k + 1 <= m ? 2.0 * (k + 1) * cf[m][k + 1] / std::pow(a, 2 * k + 3) : 0.0;
+  A.W = wolf_consts<double>(alpha, a);
+  for (int o = 0; o < 8; ++o) {
+    A.shx[o] = (o - kShift0) * P.cw[0];
+    A.shy[o] = (o - kShift0) * P.cw[1];
+    A.shz[o] = (o - kShift0) * P.cw[2];
+  }
+  group_shape(n, A.lt, A.nsplit);
+  // a piece widens the rows of neighbour cells by its span: a periodic row
+  // must not meet itself
+  A.maxspan = 2;
+  if (P.P.periodic) A.maxspan = std::max(0, std::min(2, P.nc[0] - P.row_cells));
+  return A;
+}
+
+template <int M, int K>
+cudaError_t launch_k(const Pair64Args& A, cudaStream_t st) {
+  const int64_t groups = ((int64_t)A.g.natoms + (1 << A.lt) - 1) >> A.lt;
+  const int warps = A.nsplit > 1 ? A.nsplit : 2;
+  const unsigned blocks = (unsigned)(A.nsplit > 1 ? groups : (groups + warps - 1) / warps);
+  k_pair64<M, K><<<blocks, 32 * warps, warps * sizeof(Warp64), st>>>(A);
+  return cudaGetLastError();
+}
+
+template <int M, int K>
+cudaError_t set_smem() {
+  return cudaFuncSetAttribute((const void*)k_pair64<M, K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)(kMaxSplit * sizeof(Warp64)));
+}
+
+}  // namespace
+
+cudaError_t configure_pair64_kernels() {
+  cudaError_t e = set_smem<1, kPairMSM>();
+  if (e == cudaSuccess) e = set_smem<2, kPairMSM>();
+  if (e == cudaSuccess) e = set_smem<3, kPairMSM>();
+  if (e == cudaSuccess) e = set_smem<2, kPairCutoff>();
+  if (e == cudaSuccess) e = set_smem<2, kPairWolf>();
+  return e;
+}
+
+cudaError_t launch_pair64(Plan& P, int kind, int64_t n, double alpha, cudaStream_t st) {
+  const Pair64Args A = pair64_args(P, n, alpha);
+  if (kind == kPairCutoff) return launch_k<2, kPairCutoff>(A, st);  // M unused
+  if (kind == kPairWolf) return launch_k<2, kPairWolf>(A, st);
+  if (P.P.splitting == 1) return launch_k<1, kPairMSM>(A, st);
+  if (P.P.splitting == 2) return launch_k<2, kPairMSM>(A, st);
+  return launch_k<3, kPairMSM>(A, st);
+}
+
+}  // namespace msm

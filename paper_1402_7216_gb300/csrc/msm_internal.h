@@ -78,9 +78,6 @@ struct DeviceBuffers {
   void* seg = nullptr;         // Segment<T>[nseg]
   void* seg2 = nullptr;        // Segment2[nseg] (mixed precision only, instead of seg)
   int* seg_start = nullptr;    // [2*Ez+2]: segments of plane dz live in [start[dz+Ez], start[dz+Ez+1])
-  // neighbour cell offsets (x, y, z) of the pair kernel
-  int4* cell_off = nullptr;    // [noff]
-  void* cell_shift = nullptr;  // R4<T>[noff]: offset times cell width, in the plan's precision
   int4* cell_rows = nullptr;   // [nrows]: (dy, dz, xlo, xhi) rows of neighbour cell offsets
   // reductions and status
   double* partial = nullptr;   // per-block energy partials
@@ -121,8 +118,8 @@ struct Plan {
   int nc[3];
   double cw[3];
   int ncell = 1;
-  int noff = 0;
   int nrows = 0;
+  int row_cells = 5;           // cells of the widest row of neighbour cells (the home cell's)
   // anterpolation patches: blocks of ablk^3 cells, patches of apd^3 points
   int ablk = 1, apd = 1;
   int ablk_batch = 1, apd_batch = 1;  // the same for the batched launches (at least as large)
@@ -335,6 +332,7 @@ bool fft_size_ok(int n);
 cudaError_t fft_build_level(Plan& P, int k, const std::vector<double>& K, void* work);
 void fft_free_level(FftLevel& F);
 cudaError_t configure_fft_kernels();
+cudaError_t configure_pair64_kernels();
 // One launch per pass over every listed level (of one plan, or of every
 // replica of a batch).  Each item is one level: its tables, its FP64
 // charges, its potential (FP32, or FP64 with fp64) and a complex workspace

@@ -358,24 +358,34 @@ int build_plan(const msm_params* pp, const msm_tuning* tune, Plan* P) {
         if (g2 >= p.cutoff * p.cutoff) continue;  // no pair of points closer than a
         offs.push_back(make_int4(ox, oy, oz, 0));
       }
-  P->noff = (int)offs.size();
-  // the same offsets grouped by (dy, dz) into contiguous x runs (cells are numbered x fastest)
+  // the same offsets grouped by (dy, dz) into contiguous x runs (cells are
+  // numbered x fastest), every row followed by its mirror image: a walk then
+  // meets sources on both sides of the targets in turn, which keeps the
+  // targets' lists of the FP64 pair kernel equally long
   std::vector<int4> rowv;
-  for (int oz = -2; oz <= 2; ++oz)
-    for (int oy = -2; oy <= 2; ++oy) {
-      int xlo = 99, xhi = -99;
-      for (auto& o : offs)
-        if (o.y == oy && o.z == oz) {
-          xlo = std::min(xlo, o.x);
-          xhi = std::max(xhi, o.x);
-        }
-      if (xlo > xhi) continue;
-      if (oy == 0 && oz == 0) {  // the home cell (offset 0) is evaluated separately, with the self test
-        if (xlo <= -1) rowv.push_back(make_int4(oy, oz, xlo, -1));
-        if (xhi >= 1) rowv.push_back(make_int4(oy, oz, 1, xhi));
-      } else {
-        rowv.push_back(make_int4(oy, oz, xlo, xhi));
+  int reach = 0;
+  for (auto& o : offs) reach = std::max(reach, std::max(o.x, -o.x));
+  P->row_cells = 2 * reach + 1;
+  auto add_row = [&](int oy, int oz) {
+    int xlo = 99, xhi = -99;
+    for (auto& o : offs)
+      if (o.y == oy && o.z == oz) {
+        xlo = std::min(xlo, o.x);
+        xhi = std::max(xhi, o.x);
       }
+    if (xlo > xhi) return;
+    if (oy == 0 && oz == 0) {  // the home cell (offset 0) is evaluated separately, with the self test
+      if (xlo <= -1) rowv.push_back(make_int4(oy, oz, xlo, -1));
+      if (xhi >= 1) rowv.push_back(make_int4(oy, oz, 1, xhi));
+    } else {
+      rowv.push_back(make_int4(oy, oz, xlo, xhi));
+    }
+  };
+  for (int oz = 0; oz <= 2; ++oz)
+    for (int oy = -2; oy <= 2; ++oy) {
+      if (oz == 0 && oy < 0) continue;
+      add_row(oy, oz);
+      if (oz != 0 || oy != 0) add_row(-oy, -oz);
     }
   P->nrows = (int)rowv.size();
   // the packed pair kernel builds its row table one row per lane; with cells
@@ -588,18 +598,7 @@ int build_plan(const msm_params* pp, const msm_tuning* tune, Plan* P) {
     P->lattice_fft = true;
   }
   if (upload((void**)&D.topK, K) != cudaSuccess) return MSM_ERR_OOM;
-  if (upload((void**)&D.cell_off, offs) != cudaSuccess) return MSM_ERR_OOM;
   if (upload((void**)&D.cell_rows, rowv) != cudaSuccess) return MSM_ERR_OOM;
-  if (P->fp64) {
-    std::vector<R4<double>> sh;
-    for (auto& o : offs) sh.push_back({o.x * P->cw[0], o.y * P->cw[1], o.z * P->cw[2], 0.0});
-    if (upload(&D.cell_shift, sh) != cudaSuccess) return MSM_ERR_OOM;
-  } else {
-    std::vector<R4<float>> sh;
-    for (auto& o : offs)
-      sh.push_back({(float)(o.x * P->cw[0]), (float)(o.y * P->cw[1]), (float)(o.z * P->cw[2]), 0.f});
-    if (upload(&D.cell_shift, sh) != cudaSuccess) return MSM_ERR_OOM;
-  }
   if (P->stencil_fits) {  // the stencil kernel's segment tables (unused, and not built, past its window)
     std::vector<int> start;
     if (P->fp64) {
@@ -627,8 +626,8 @@ int build_plan(const msm_params* pp, const msm_tuning* tune, Plan* P) {
 void free_plan(Plan* P) {
   DeviceBuffers& D = P->d;
   void* ptrs[] = {D.key, D.rank, D.perm, D.count, D.csum, D.cell_start, D.atoms,
-                  D.gfrac, D.gbase, D.phis, D.fs, D.glong, D.topK, D.topq, D.topu, D.seg, D.seg2, D.cell_shift, D.cell_rows,
-                  D.seg_start, D.cell_off, D.partial, D.scalars, D.md_partial, D.md_step, D.status, D.hpos, D.hq,
+                  D.gfrac, D.gbase, D.phis, D.fs, D.glong, D.topK, D.topq, D.topu, D.seg, D.seg2, D.cell_rows,
+                  D.seg_start, D.partial, D.scalars, D.md_partial, D.md_step, D.status, D.hpos, D.hq,
                   D.hphi, D.hforce, D.henergy, D.lparts, D.fft_work};
   for (void* p : ptrs)
     if (p) cudaFree(p);
