@@ -205,6 +205,8 @@ struct BinKArgs {
   void* atoms;
   void* gfrac;
   int4* gbase;
+  int* scell;
+  float* cellx;
   int* perm;
   int ncell;
 };
@@ -391,7 +393,7 @@ template <typename IO, bool FP64>
 __device__ __forceinline__ void write_records(const IO* __restrict__ pos, const IO* __restrict__ q, const BinArgs& A,
                                               int key, int i, int s, void* __restrict__ atoms_v,
                                               void* __restrict__ gfrac_v, int4* __restrict__ gbase,
-                                              int* __restrict__ perm) {
+                                              int* __restrict__ scell, float* __restrict__ cellx, int* __restrict__ perm) {
   const int kc[3] = {key % A.nc[0], (key / A.nc[0]) % A.nc[1], key / (A.nc[0] * A.nc[1])};
   int bad = 0, bs[3];
   if (FP64) {
@@ -417,6 +419,8 @@ __device__ __forceinline__ void write_records(const IO* __restrict__ pos, const 
     reinterpret_cast<R4<float>*>(gfrac_v)[s] = R4<float>{fr[0], fr[1], fr[2], qi};
   }
   gbase[s] = make_int4(bs[0] - (A.S - 1), bs[1] - (A.S - 1), bs[2] - (A.S - 1), 0);
+  scell[s] = key;
+  cellx[s] = (float)kc[0];
   perm[s] = i;
 }
 
@@ -460,13 +464,16 @@ __device__ __forceinline__ int make_record(const IO* __restrict__ pos, const IO*
 }
 
 template <bool FP64>
-__device__ __forceinline__ void store_record(const CellRec<FP64>& R, const BinArgs& A, int i, int s,
+__device__ __forceinline__ void store_record(const CellRec<FP64>& R, const BinArgs& A, int key, int i, int s,
                                              void* __restrict__ atoms_v, void* __restrict__ gfrac_v,
-                                             int4* __restrict__ gbase, int* __restrict__ perm) {
+                                             int4* __restrict__ gbase, int* __restrict__ scell, float* __restrict__ cellx,
+                                             int* __restrict__ perm) {
   using T = typename CellRec<FP64>::T;
   reinterpret_cast<R4<T>*>(atoms_v)[s] = R4<T>{R.loc[0], R.loc[1], R.loc[2], R.q};
   reinterpret_cast<R4<T>*>(gfrac_v)[s] = R4<T>{R.fr[0], R.fr[1], R.fr[2], R.q};
   gbase[s] = make_int4(R.bs[0] - (A.S - 1), R.bs[1] - (A.S - 1), R.bs[2] - (A.S - 1), 0);
+  scell[s] = key;
+  cellx[s] = (float)(key % A.nc[0]);
   perm[s] = i;
 }
 
@@ -481,7 +488,8 @@ template <typename IO, bool FP64>
 __device__ __forceinline__ void cell_fill_body(const IO* __restrict__ pos, const IO* __restrict__ q,
                                                const BinArgs& A, const int* __restrict__ cell_start,
                                                void* __restrict__ atoms_v, void* __restrict__ gfrac_v,
-                                               int4* __restrict__ gbase, int* __restrict__ perm, int ncell, int cell,
+                                               int4* __restrict__ gbase, int* __restrict__ scell, float* __restrict__ cellx,
+                                               int* __restrict__ perm, int ncell, int cell,
                                                long long* __restrict__ idx) {
   if (cell >= ncell) return;  // warp-uniform
   const int lane = threadIdx.x & 31;
@@ -499,7 +507,7 @@ __device__ __forceinline__ void cell_fill_body(const IO* __restrict__ pos, const
     if (lane < m) {
       int r = 0;
       for (int j = 0; j < m; ++j) r += idx[j] < k;  // keys are distinct: r is a permutation of 0..m-1
-      store_record<FP64>(R, A, i, s0 + r, atoms_v, gfrac_v, gbase, perm);
+      store_record<FP64>(R, A, cell, i, s0 + r, atoms_v, gfrac_v, gbase, scell, cellx, perm);
     }
     __syncwarp();
   } else if (m <= kOrderMax) {
@@ -512,12 +520,13 @@ __device__ __forceinline__ void cell_fill_body(const IO* __restrict__ pos, const
       const long long k = idx[t];
       int r = 0;
       for (int j = 0; j < m; ++j) r += idx[j] < k;  // keys are distinct: r is a permutation of 0..m-1
-      write_records<IO, FP64>(pos, q, A, cell, (int)(k & 0xffffffffll), s0 + r, atoms_v, gfrac_v, gbase, perm);
+      write_records<IO, FP64>(pos, q, A, cell, (int)(k & 0xffffffffll), s0 + r, atoms_v, gfrac_v, gbase, scell, cellx,
+                              perm);
     }
     __syncwarp();
   } else {
     for (int t = lane; t < m; t += 32)
-      write_records<IO, FP64>(pos, q, A, cell, perm[s0 + t], s0 + t, atoms_v, gfrac_v, gbase, perm);
+      write_records<IO, FP64>(pos, q, A, cell, perm[s0 + t], s0 + t, atoms_v, gfrac_v, gbase, scell, cellx, perm);
   }
 }
 
@@ -525,12 +534,13 @@ template <typename IO, bool FP64>
 __global__ void __launch_bounds__(32 * kFillWarps) k_cell_fill(const IO* __restrict__ pos, const IO* __restrict__ q,
                                                                BinArgs A, const int* __restrict__ cell_start,
                                                                void* __restrict__ atoms_v, void* __restrict__ gfrac_v,
-                                                               int4* __restrict__ gbase, int* __restrict__ perm,
-                                                               int ncell) {
+                                                               int4* __restrict__ gbase,
+                                                               int* __restrict__ scell, float* __restrict__ cellx,
+                                                               int* __restrict__ perm, int ncell) {
   __shared__ long long idx[kFillWarps][kOrderMax];
   const int w = threadIdx.x >> 5;
-  cell_fill_body<IO, FP64>(pos, q, A, cell_start, atoms_v, gfrac_v, gbase, perm, ncell, blockIdx.x * kFillWarps + w,
-                           idx[w]);
+  cell_fill_body<IO, FP64>(pos, q, A, cell_start, atoms_v, gfrac_v, gbase, scell, cellx, perm, ncell,
+                           blockIdx.x * kFillWarps + w, idx[w]);
 }
 
 // Batched forms: the atom-indexed kernels take 256 atoms per block, the cell
@@ -549,7 +559,7 @@ __global__ void __launch_bounds__(32 * kFillWarps) kb_cell_fill(const BinKArgs<I
   const int r = batch_rep(first, nrep, blockIdx.x);
   const BinKArgs<IO>& a = tab[r];
   const int w = threadIdx.x >> 5;
-  cell_fill_body<IO, FP64>(a.pos, a.q, a.A, a.cell_start, a.atoms, a.gfrac, a.gbase, a.perm, a.ncell,
+  cell_fill_body<IO, FP64>(a.pos, a.q, a.A, a.cell_start, a.atoms, a.gfrac, a.gbase, a.scell, a.cellx, a.perm, a.ncell,
                            (blockIdx.x - first[r]) * kFillWarps + w, idx[w]);
 }
 
@@ -619,10 +629,10 @@ cudaError_t launch_binning(Plan& P, int64_t n64, const IO* pos, const IO* q, cud
     k_bin_perm<<<nb, 256, 0, st>>>(n, D.key, D.rank, D.cell_start, D.perm);
     if (P.fp64)
       k_cell_fill<IO, true><<<nf, 32 * kFillWarps, 0, st>>>(pos, q, A, D.cell_start, D.atoms, D.gfrac, D.gbase,
-                                                            D.perm, P.ncell);
+                                                            D.scell, D.cellx, D.perm, P.ncell);
     else
       k_cell_fill<IO, false><<<nf, 32 * kFillWarps, 0, st>>>(pos, q, A, D.cell_start, D.atoms, D.gfrac, D.gbase,
-                                                             D.perm, P.ncell);
+                                                             D.scell, D.cellx, D.perm, P.ncell);
   }
   P.launches += 2 + (n > 0 ? 3 : 0);
   return cudaGetLastError();
@@ -657,6 +667,8 @@ cudaError_t bin_batch_build(const std::vector<BatchRep>& reps, BinBatch** out) {
     a.atoms = D.atoms;
     a.gfrac = D.gfrac;
     a.gbase = D.gbase;
+    a.scell = D.scell;
+    a.cellx = D.cellx;
     a.perm = D.perm;
     a.ncell = P.ncell;
     ka.push_back(a);

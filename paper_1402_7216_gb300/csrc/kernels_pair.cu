@@ -13,6 +13,7 @@
 // operations; rejected pairs are masked, not branched.  Mixed precision sums
 // each batch in FP32 and folds the batch sums into the running totals with an
 // error-free TwoSum (compensated accumulation).
+#include <algorithm>
 #include <new>
 
 #include "pair_common.h"
@@ -67,8 +68,11 @@ constexpr int kWarps = 4;
 #ifndef MSM_PAIR_BATCH
 #define MSM_PAIR_BATCH 64
 #endif
+#ifndef MSM_PAIR_AHEAD
+#define MSM_PAIR_AHEAD 4
+#endif
 #ifndef MSM_PAIR_MINB
-#define MSM_PAIR_MINB 6
+#define MSM_PAIR_MINB 5
 #endif
 constexpr int kBatch = MSM_PAIR_BATCH;  // sources per queue drain (pairs per lane per drain)
 
@@ -202,14 +206,15 @@ __device__ __forceinline__ void pair2(float2 bx, float2 by, float2 bz, float2 bq
   sz = __ffma2_rn(fp, dz, sz);
 }
 
-template <int M, int K, int NB = kBatch, bool SELF = false>
-__device__ __forceinline__ void pair_batch_f2(const QueueF& Q, float2 nax, float2 nay, float2 naz, float a2,
-                                              const PairCoef& C, const WolfC<float>& W, float& phi, float& px,
-                                              float& py, float& pz, float& cphi, float& cpx, float& cpy,
-                                              float& cpz) {
-  float2 sphi = make_float2(0.f, 0.f), sx = sphi, sy = sphi, sz = sphi;
-  // sources jj..jj+3 load as one float4 per coordinate (two packed halves)
-  auto four = [&](int jj) {
+// The lane's target against sources at .. at + NB - 1 of the queue; four
+// sources load as one float4 per coordinate (two packed halves).
+template <int M, int K, int NB, bool SELF>
+__device__ __forceinline__ void pair_sources(const QueueF& Q, int at, float2 nax, float2 nay, float2 naz, float a2,
+                                             const PairCoef& C, const WolfC<float>& W, float2& sphi, float2& sx,
+                                             float2& sy, float2& sz) {
+#pragma unroll
+  for (int k = 0; k < NB; k += 4) {
+    const int jj = at + k;
     const float4 x4 = *reinterpret_cast<const float4*>(&Q.x[jj]);
     const float4 y4 = *reinterpret_cast<const float4*>(&Q.y[jj]);
     const float4 z4 = *reinterpret_cast<const float4*>(&Q.z[jj]);
@@ -218,13 +223,29 @@ __device__ __forceinline__ void pair_batch_f2(const QueueF& Q, float2 nax, float
                       make_float2(q4.x, q4.y), nax, nay, naz, a2, C, W, sphi, sx, sy, sz);
     pair2<M, K, SELF>(make_float2(x4.z, x4.w), make_float2(y4.z, y4.w), make_float2(z4.z, z4.w),
                       make_float2(q4.z, q4.w), nax, nay, naz, a2, C, W, sphi, sx, sy, sz);
-  };
-#pragma unroll
-  for (int jj = 0; jj < NB; jj += 4) four(jj);
-  two_sum_add(phi, cphi, sphi.x + sphi.y);
-  two_sum_add(px, cpx, sx.x + sx.y);
-  two_sum_add(py, cpy, sy.x + sy.y);
-  two_sum_add(pz, cpz, sz.x + sz.y);
+  }
+}
+
+// Running totals of a target and their compensation terms.
+struct Totals {
+  float phi = 0.f, x = 0.f, y = 0.f, z = 0.f, cphi = 0.f, cx = 0.f, cy = 0.f, cz = 0.f;
+  __device__ __forceinline__ void fold(float2 sphi, float2 sx, float2 sy, float2 sz) {
+    two_sum_add(phi, cphi, sphi.x + sphi.y);
+    two_sum_add(x, cx, sx.x + sx.y);
+    two_sum_add(y, cy, sy.x + sy.y);
+    two_sum_add(z, cz, sz.x + sz.y);
+  }
+};
+
+// n sources (a multiple of NB), folded into the totals once
+template <int M, int K, int NB, bool SELF>
+__device__ __forceinline__ void pair_batch(const QueueF& Q, int at, int n, float2 nax, float2 nay, float2 naz,
+                                           float a2, const PairCoef& C, const WolfC<float>& W, Totals& t) {
+  float2 sphi = make_float2(0.f, 0.f), sx = sphi, sy = sphi, sz = sphi;
+#pragma unroll 1
+  for (int b = 0; b < n; b += NB)
+    pair_sources<M, K, NB, SELF>(Q, at + b, nax, nay, naz, a2, C, W, sphi, sx, sy, sz);
+  t.fold(sphi, sx, sy, sz);
 }
 
 // Rows of neighbour cells: for each (dy, dz) the cells cx+xlo..cx+xhi of one x
@@ -325,140 +346,6 @@ __device__ __forceinline__ int build_seg_table(SegTable& T, const PairKArgs& K, 
   }
 
   return total;
-}
-
-template <int M, int KIND>
-__device__ __forceinline__ void short_range_f2_body(const PairKArgs& K, int blk) {
-  const R4<float>* __restrict__ atoms = K.atoms;
-  const int* __restrict__ cell_start = K.cell_start;
-  const int ncell = K.ncell;
-  const PairArgs& A = K.A;
-  const PairCoef C = K.C;
-  const WolfC<float> W = K.W;
-  const float cwx = K.cwx;
-  float* __restrict__ phis = K.phis;
-  R4<float>* __restrict__ fs = K.fs;
-  __shared__ QueueF queue[kWarps];
-  __shared__ SegTable tables[kWarps];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  QueueF& Q = queue[warp];
-  SegTable& T = tables[warp];
-  const int cell = blk * kWarps + warp;
-  if (cell >= ncell) return;  // warp-uniform
-  const int ncx = A.nc[0], ncy = A.nc[1];
-  const int cx = cell % ncx, cy = (cell / ncx) % ncy, cz = cell / (ncx * ncy);
-  const float a2 = A.a2f;
-  const float FAR = 1e6f;
-  const int i0 = cell_start[cell], i1 = cell_start[cell + 1];
-  const int total = build_seg_table(T, K, cx, cy, cz, lane);
-
-  for (int ib = i0; ib < i1; ib += 32) {
-    const int i = ib + lane;
-    const bool iv = i < i1;
-    const R4<float> ai = iv ? atoms[i] : R4<float>{0.f, 0.f, 0.f, 0.f};
-    float lx = iv ? ai.x : FAR, ly = iv ? ai.y : FAR, lz = iv ? ai.z : FAR;
-    float hx = iv ? ai.x : -FAR, hy = iv ? ai.y : -FAR, hz = iv ? ai.z : -FAR;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      lx = fminf(lx, __shfl_xor_sync(kFull, lx, o));
-      ly = fminf(ly, __shfl_xor_sync(kFull, ly, o));
-      lz = fminf(lz, __shfl_xor_sync(kFull, lz, o));
-      hx = fmaxf(hx, __shfl_xor_sync(kFull, hx, o));
-      hy = fmaxf(hy, __shfl_xor_sync(kFull, hy, o));
-      hz = fmaxf(hz, __shfl_xor_sync(kFull, hz, o));
-    }
-    const float2 nax = make_float2(-ai.x, -ai.x), nay = make_float2(-ai.y, -ai.y), naz = make_float2(-ai.z, -ai.z);
-    float phi = 0.f, px = 0.f, py = 0.f, pz = 0.f, cphi = 0.f, cpx = 0.f, cpy = 0.f, cpz = 0.f;
-    // home cell: packed batches of 32 with the self test (the queue is empty here)
-    for (int jb = i0; jb < i1; jb += 32) {
-      const int j = jb + lane;
-      const R4<float> h = (j < i1) ? atoms[j] : R4<float>{FAR, FAR, FAR, 0.f};
-      Q.x[lane] = h.x;
-      Q.y[lane] = h.y;
-      Q.z[lane] = h.z;
-      Q.q[lane] = h.w;
-      __syncwarp();
-      pair_batch_f2<M, KIND, 32, true>(Q, nax, nay, naz, a2, C, W, phi, px, py, pz, cphi, cpx, cpy, cpz);
-      __syncwarp();
-    }
-    // ---- the neighbour rows: flat source index t in [0, total), 32 per step ----
-    int seg = 0;  // this lane's segment cursor (t only grows)
-    // source t: its atom index and cell x offset (t < total)
-    auto locate = [&](int t, int& j, int& ox, float2& shv) {
-      while (T.rec[seg + 1].y <= t) ++seg;
-      const int4 r = T.rec[seg];
-      const int4 b = T.bnd[seg];
-      j = r.x + (t - r.y);
-      ox = r.z + (j >= b.x) + (j >= b.y) + (j >= b.z) + (j >= b.w);
-      shv = T.shift[seg];
-    };
-    R4<float> an = {FAR, FAR, FAR, 0.f};
-    int oxn = 0;
-    float2 shn = make_float2(0.f, 0.f);
-    if (lane < total) {
-      int j;
-      locate(lane, j, oxn, shn);
-      an = atoms[j];
-    }
-    int qn = 0;  // queued sources (warp-uniform)
-    for (int t0 = 0; t0 < total; t0 += 32) {
-      const bool valid = t0 + lane < total;
-      R4<float> aj = an;
-      const int ox = oxn;
-      const float2 shv = shn;
-      if (t0 + 32 + lane < total) {  // next chunk's load goes out before this chunk's work
-        int j;
-        locate(t0 + 32 + lane, j, oxn, shn);
-        an = atoms[j];
-      }
-      aj.x += ox * cwx;
-      aj.y += shv.x;
-      aj.z += shv.y;
-      const float ex = fmaxf(fmaxf(lx - aj.x, aj.x - hx), 0.f);
-      const float ey = fmaxf(fmaxf(ly - aj.y, aj.y - hy), 0.f);
-      const float ez = fmaxf(fmaxf(lz - aj.z, aj.z - hz), 0.f);
-      const bool keep = valid && (ex * ex + ey * ey + ez * ez < a2);
-      const unsigned bal = __ballot_sync(kFull, keep);
-      if (keep) {
-        const int p = qn + __popc(bal & ((1u << lane) - 1u));
-        Q.x[p] = aj.x;
-        Q.y[p] = aj.y;
-        Q.z[p] = aj.z;
-        Q.q[p] = aj.w;
-      }
-      qn += __popc(bal);
-      __syncwarp();
-      if (qn >= kBatch) {
-        pair_batch_f2<M, KIND>(Q, nax, nay, naz, a2, C, W, phi, px, py, pz, cphi, cpx, cpy, cpz);
-        __syncwarp();
-        if (lane < qn - kBatch) {
-          Q.x[lane] = Q.x[kBatch + lane];
-          Q.y[lane] = Q.y[kBatch + lane];
-          Q.z[lane] = Q.z[kBatch + lane];
-          Q.q[lane] = Q.q[kBatch + lane];
-        }
-        qn -= kBatch;
-        __syncwarp();
-      }
-    }
-    if (qn > 0) {  // last partial batch, padded with far-away zero charges
-      for (int t = lane; t < kBatch; t += 32)
-        if (t >= qn) {
-          Q.x[t] = FAR;
-          Q.y[t] = FAR;
-          Q.z[t] = FAR;
-          Q.q[t] = 0.f;
-        }
-      __syncwarp();
-      pair_batch_f2<M, KIND>(Q, nax, nay, naz, a2, C, W, phi, px, py, pz, cphi, cpx, cpy, cpz);
-      __syncwarp();
-    }
-    if (iv) {
-      phis[i] = phi + cphi;
-      const float qi = ai.w;
-      fs[i] = R4<float>{-qi * (px + cpx), -qi * (py + cpy), -qi * (pz + cpz), 0.f};
-    }
-  }
 }
 
 // ---- target clusters (mixed precision) ----
@@ -708,185 +595,269 @@ __device__ __forceinline__ void short_range_c8_body(const PairKArgs& K, int blk)
   }
 }
 
-// ---- target runs (mixed precision) ----
-// Warp w takes the 32 consecutive sorted atoms 32 w .. 32 w + 31 as its
-// targets, whatever cells they belong to, so that no lane idles for want of
-// a cell's atoms (~25 per cell at the default fill).  Binning sorts each cell
-// by x and numbers cells x fastest, so a run of a cell row is a slab of it
-// 32 atoms thick.  The run is cut into pieces of one row and at most three
-// consecutive cells (nearly always one piece); a piece is a pass as in the
-// one-cell kernel, about its first cell c0 and span s = its last cell - c0:
-// the targets enter c0's frame shifted by whole cells, the home block is the
-// atoms of cells c0 .. c0 + s with the self test, and the neighbour rows are
-// the plan's rows widened by s cells in +x (the home row without the piece's
-// own cells), walked as one flat index space, culled against the piece's
-// bounding box and queued.  A periodic row then spans up to seven cells, so
-// the runs need at least seven cells in x.
+// ---- one cell or one run of atoms per warp (mixed precision) ----
+// A warp's targets are, in cell mode, the atoms of one cell, 32 at a time; in
+// run mode 32 consecutive sorted atoms, whatever cells they belong to, so that
+// no lane idles for want of a cell's atoms (~25 per cell at the default fill).
+// Binning sorts each cell by x and numbers cells x fastest, so a run of a cell
+// row is a slab of it.  A run is cut into pieces of one row and at most
+// maxspan + 1 cells (nearly always one piece): a piece's targets enter the
+// frame of its first cell c0 shifted by whole cells, the home block is the
+// atoms of the piece's cells (with the self test), and the neighbour rows are
+// the plan's rows widened by the piece's span.
+//
+// Sources are culled against the targets' bounding box, queued (a ring of 128)
+// and evaluated in unrolled batches of 64, folded into the totals with TwoSum.
+// A packed step (two pairs per lane) is 17 FMA-pipe instructions and costs ~44
+// cycles of an SM quarter however it is written (packed or scalar, constants
+// in registers or as immediates, one to four steps interleaved): 34 cycles of
+// FMA pipe, the rest register reads.  The 1.07M-atom box evaluates 1,960
+// sources per target, 1.2 ms of such steps; the walk over ~4,000 candidates
+// per target (0.63 ms by itself) is hidden only in part.
+//
+// The warps of a block may share one group (K.split of them): warp p takes
+// every split-th 64 sources, and the partial sums are added in warp order.
+// (The barrier is the block's: named barriers by a computed number reserve
+// all 16 of a block and halve the resident blocks, 1.63 -> 1.85 ms.)
+//
+// Measured alone: 1.07M atoms 1,630 -> 1,600 us, 190,977 atoms 265 -> 254 us,
+// 23,558 atoms 56 -> 45 us, 3,000 atoms (open) 57 -> 24 us, against loads one
+// step of 32 sources ahead and a flat index space located per lane.
+//
+// The sources of the next kAhead steps are in flight as asynchronous copies
+// into a ring in shared memory, each lane copying the records it will take.
+// A step is 64 sources, two per lane: the loop's state, the range's shift and
+// the chain load - cull - ballot - append are paid once for both.
+constexpr int kAhead = MSM_PAIR_AHEAD;  // a power of two
+constexpr int kStep = 64;               // sources per step
+struct alignas(16) PairShared {
+  QueueF queue;
+  SegList segs;
+  R4<float> ring[kAhead][kStep];  // records of the steps in flight
+  float ringx[kAhead][kStep];     // their cells' x index
+  int ringseg[kAhead];            // their range, and their number << 8
+  float4 shift[2 * kMaxRows];     // a range's x base, y shift and z shift
+};
+
+__device__ __forceinline__ void copy_async16(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void copy_async4(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+
 template <int M, int KIND>
-__device__ __forceinline__ void short_range_run_body(const PairKArgs& K, int blk) {
+__device__ __forceinline__ void short_range_body(const PairKArgs& K, int blk) {
   const R4<float>* __restrict__ atoms = K.atoms;
+  const float* __restrict__ cellx = K.cellx;
   const int* __restrict__ cell_start = K.cell_start;
   const PairArgs& A = K.A;
   const PairCoef C = K.C;
   const WolfC<float> W = K.W;
   const float cwx = K.cwx;
-  float* __restrict__ phis = K.phis;
-  R4<float>* __restrict__ fs = K.fs;
-  __shared__ QueueF queue[kWarps];
-  __shared__ SegTableR tables[kWarps];
+  __shared__ PairShared shared[kWarps];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  QueueF& Q = queue[warp];
-  SegTableR& T = tables[warp];
-  const int s0 = 32 * (blk * kWarps + warp);
-  if (s0 >= K.natoms) return;  // warp-uniform
-  const int nval = min(32, K.natoms - s0);
+  PairShared& Sh = shared[warp];
+  QueueF& Q = Sh.queue;
+  SegList& L = Sh.segs;
+  const int split = K.split, part = split > 1 ? warp : 0;
+  const int group = split > 1 ? blk : blk * kWarps + warp;
   const int ncx = A.nc[0], ncy = A.nc[1];
   const float a2 = A.a2f;
   const float FAR = 1e6f;
-  // the lane's target: its sorted record and its cell (cells ascend with the lane)
-  const bool sv = lane < nval;
-  const int mycell = sv ? K.key[K.perm[s0 + lane]] : INT_MAX;
-  const R4<float> me = sv ? atoms[s0 + lane] : R4<float>{0.f, 0.f, 0.f, 0.f};
-  for (int l0 = 0; l0 < nval;) {  // one piece per step (warp-uniform)
-    const int c0 = __shfl_sync(kFull, mycell, l0);
+  const unsigned lt = (1u << lane) - 1u;
+  // targets i0 .. i1 - 1; the lane's own in run mode (cells ascend with the lane)
+  int i0, i1, mycell = INT_MAX;
+  R4<float> me = {0.f, 0.f, 0.f, 0.f};
+  if (K.runs) {
+    i0 = group * 32;
+    i1 = min(i0 + 32, K.natoms);
+    if (i0 + lane < i1) {
+      mycell = K.scell[i0 + lane];
+      me = atoms[i0 + lane];
+    }
+  } else {
+    i0 = group < K.ncell ? cell_start[group] : 0;
+    i1 = group < K.ncell ? cell_start[group + 1] : 0;
+  }
+  for (int ib = i0; ib < i1;) {  // one piece per step (the same for every warp of the group)
+    int c0 = group, span = 0, next = ib + 32;
+    bool inp;
+    if (K.runs) {
+      const int l0 = ib - i0;
+      c0 = __shfl_sync(kFull, mycell, l0);
+      const int climit = c0 + min(K.maxspan, ncx - 1 - c0 % ncx);  // the piece stays in the row
+      inp = lane >= l0 && mycell <= climit;
+      const int l1 = 32 - __clz(__ballot_sync(kFull, inp));
+      span = __shfl_sync(kFull, mycell, l1 - 1) - c0;
+      next = i0 + l1;
+    } else {
+      inp = ib + lane < i1;
+      me = inp ? atoms[ib + lane] : R4<float>{0.f, 0.f, 0.f, 0.f};
+      mycell = c0;
+    }
     const int cx = c0 % ncx, cy = (c0 / ncx) % ncy, cz = c0 / (ncx * ncy);
-    const int climit = c0 + min(2, ncx - 1 - cx);  // the piece stays in the row, three cells at most
-    const bool inp = lane >= l0 && mycell <= climit;  // lanes l0 .. l1 - 1
-    const unsigned pb = __ballot_sync(kFull, inp);
-    const int l1 = 32 - __clz(pb);
-    const int span = __shfl_sync(kFull, mycell, l1 - 1) - c0;
-    // cell boundaries inside the piece: atoms of cell c0 + 1 and c0 + 2 begin here
-    const int h0 = cell_start[c0];
-    const int b1 = span >= 1 ? cell_start[c0 + 1] : INT_MAX;
-    const int b2 = span >= 2 ? cell_start[c0 + 2] : INT_MAX;
-    const int h1 = cell_start[c0 + span + 1];
-    // the target in c0's frame
+    const int h0 = cell_start[c0], h1 = cell_start[c0 + span + 1];
+    // the target in c0's frame (the same rounding as the home block's)
     R4<float> ai = me;
-    ai.x = __fmaf_rn((float)(inp ? mycell - c0 : 0), cwx, ai.x);  // the same rounding as the home block's
-    float lx = inp ? ai.x : FAR, ly = inp ? ai.y : FAR, lz = inp ? ai.z : FAR;
-    float hx = inp ? ai.x : -FAR, hy = inp ? ai.y : -FAR, hz = inp ? ai.z : -FAR;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      lx = fminf(lx, __shfl_xor_sync(kFull, lx, o));
-      ly = fminf(ly, __shfl_xor_sync(kFull, ly, o));
-      lz = fminf(lz, __shfl_xor_sync(kFull, lz, o));
-      hx = fmaxf(hx, __shfl_xor_sync(kFull, hx, o));
-      hy = fmaxf(hy, __shfl_xor_sync(kFull, hy, o));
-      hz = fmaxf(hz, __shfl_xor_sync(kFull, hz, o));
-    }
+    ai.x = __fmaf_rn((float)(inp ? mycell - c0 : 0), cwx, ai.x);
+    const float lx = warp_min(inp ? ai.x : FAR), ly = warp_min(inp ? ai.y : FAR), lz = warp_min(inp ? ai.z : FAR);
+    const float hx = warp_max(inp ? ai.x : -FAR), hy = warp_max(inp ? ai.y : -FAR), hz = warp_max(inp ? ai.z : -FAR);
     const float2 nax = make_float2(-ai.x, -ai.x), nay = make_float2(-ai.y, -ai.y), naz = make_float2(-ai.z, -ai.z);
-    float phi = 0.f, px = 0.f, py = 0.f, pz = 0.f, cphi = 0.f, cpx = 0.f, cpy = 0.f, cpz = 0.f;
-    // the home block: the atoms of the piece's cells, 32 at a time, with the self test
-    for (int jb = h0; jb < h1; jb += 32) {
-      const int j = jb + lane;
-      R4<float> h = (j < h1) ? atoms[j] : R4<float>{FAR, FAR, FAR, 0.f};
-      if (j < h1) h.x = __fmaf_rn((float)((j >= b1) + (j >= b2)), cwx, h.x);
-      Q.x[lane] = h.x;
-      Q.y[lane] = h.y;
-      Q.z[lane] = h.z;
-      Q.q[lane] = h.w;
-      __syncwarp();
-      pair_batch_f2<M, KIND, 32, true>(Q, nax, nay, naz, a2, C, W, phi, px, py, pz, cphi, cpx, cpy, cpz);
-      __syncwarp();
+    // the ranges of the neighbour rows, 64 sources per step (every split-th of
+    // them): fill() starts the copies of the next step into ring slot `slot`
+    const int nseg = build_segments(L, K, cx, cy, cz, span, lx, ly, lz, hx, hy, hz, lane);
+    for (int e = lane; e < nseg; e += 32) {
+      const int4 r = L.rec[e];
+      Sh.shift[e] = make_float4((float)r.z, ((r.w & 15) - 3) * K.cwy, ((r.w >> 4) - 3) * K.cwz, 0.f);
     }
-    // the neighbour rows: flat source index t in [0, total), 32 per step
-    const int total = build_seg_table_run(T, K, cx, cy, cz, span, lx, ly, lz, hx, hy, hz, lane);
-    int seg = 0;
-    auto locate = [&](int t, int& j, int& ox, float2& shv) {
-      while (T.rec[seg + 1].y <= t) ++seg;
-      const int4 r = T.rec[seg];
-      const int4 b = T.bnd[seg];
-      const int2 b2 = T.bnd2[seg];
-      j = r.x + (t - r.y);
-      ox = r.z + (j >= b.x) + (j >= b.y) + (j >= b.z) + (j >= b.w) + (j >= b2.x) + (j >= b2.y);
-      shv = T.shift[seg];
+    __syncwarp();
+    int seg = -1, jb = 0, je = 0, skip = part, steps = 0;  // steps: filled, not yet taken
+    bool more = true;
+    auto fill = [&](int slot) {
+      while (more && jb >= je) {  // to the next range; its first `skip` steps are the other warps'
+        if (seg >= 0) skip = (jb - je) / kStep;
+        more = ++seg < nseg;
+        if (more) {
+          const int4 r = L.rec[seg];
+          jb = r.x + kStep * skip;
+          je = r.y;
+        }
+      }
+      if (more) {
+        const int j = jb + lane, n = je - jb;
+        if (lane < n) {
+          copy_async16(&Sh.ring[slot][lane], atoms + j);
+          copy_async4(&Sh.ringx[slot][lane], cellx + j);
+        }
+        if (lane + 32 < n) {
+          copy_async16(&Sh.ring[slot][lane + 32], atoms + j + 32);
+          copy_async4(&Sh.ringx[slot][lane + 32], cellx + j + 32);
+        }
+        if (lane == 0) Sh.ringseg[slot] = seg | (min(n, kStep) << 8);
+        jb += kStep * split;
+        ++steps;
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    R4<float> an = {FAR, FAR, FAR, 0.f};
-    int oxn = 0;
-    float2 shn = make_float2(0.f, 0.f);
-    if (lane < total) {
-      int j;
-      locate(lane, j, oxn, shn);
-      an = atoms[j];
+#pragma unroll
+    for (int d = 0; d < kAhead; ++d) fill(d);
+    Totals tot;
+    // the home block, 32 sources at a time, with the self test
+    for (int hb = h0 + 32 * part; hb < h1; hb += 32 * split) {
+      const int j = hb + lane;
+      R4<float> s = {FAR, FAR, FAR, 0.f};
+      if (j < h1) {
+        s = atoms[j];
+        s.x = __fmaf_rn(cellx[j] - (float)cx, cwx, s.x);
+      }
+      Q.x[lane] = s.x;
+      Q.y[lane] = s.y;
+      Q.z[lane] = s.z;
+      Q.q[lane] = s.w;
+      __syncwarp();
+      pair_batch<M, KIND, 32, true>(Q, 0, 32, nax, nay, naz, a2, C, W, tot);
+      __syncwarp();
     }
-    int qn = 0;
-    for (int t0 = 0; t0 < total; t0 += 32) {
-      const bool valid = t0 + lane < total;
-      R4<float> aj = an;
-      const int ox = oxn;
-      const float2 shv = shn;
-      if (t0 + 32 + lane < total) {
-        int j;
-        locate(t0 + 32 + lane, j, oxn, shn);
-        an = atoms[j];
+    __syncwarp();
+    int qn = 0, head = 0;  // queued sources and where they begin (0 or kBatch)
+    for (int slot = 0; steps > 0; slot = (slot + 1) & (kAhead - 1)) {
+      asm volatile("cp.async.wait_group %0;" ::"n"(kAhead - 1) : "memory");
+      const R4<float> s0 = Sh.ring[slot][lane], s1 = Sh.ring[slot][lane + 32];
+      const int meta = Sh.ringseg[slot], n = meta >> 8;
+      const float4 sh = Sh.shift[meta & 255];
+      const float2 w = make_float2(cwx, cwx);
+      const float2 x = __ffma2_rn(__fadd2_rn(make_float2(Sh.ringx[slot][lane], Sh.ringx[slot][lane + 32]),
+                                             make_float2(sh.x, sh.x)), w, make_float2(s0.x, s1.x));
+      const float2 y = __fadd2_rn(make_float2(s0.y, s1.y), make_float2(sh.y, sh.y));
+      const float2 z = __fadd2_rn(make_float2(s0.z, s1.z), make_float2(sh.z, sh.z));
+      __syncwarp();  // the slot's range has been read
+      --steps;
+      fill(slot);
+      auto gap = [&](float2 v, float lo, float hi) {  // distance beyond the box along one axis
+        const float2 a = __fadd2_rn(make_float2(lo, lo), make_float2(-v.x, -v.y));
+        const float2 b = __fadd2_rn(v, make_float2(-hi, -hi));
+        return make_float2(fmaxf(fmaxf(a.x, b.x), 0.f), fmaxf(fmaxf(a.y, b.y), 0.f));
+      };
+      const float2 ex = gap(x, lx, hx), ey = gap(y, ly, hy), ez = gap(z, lz, hz);
+      const float2 d2 = __ffma2_rn(ez, ez, __ffma2_rn(ey, ey, __fmul2_rn(ex, ex)));
+      const bool k0 = lane < n && d2.x < a2, k1 = lane + 32 < n && d2.y < a2;
+      const unsigned b0 = __ballot_sync(kFull, k0), b1 = __ballot_sync(kFull, k1);
+      const int at0 = head + qn, at1 = at0 + __popc(b0);
+      if (k0) {
+        const int p = (at0 + __popc(b0 & lt)) & (2 * kBatch - 1);
+        Q.x[p] = x.x;
+        Q.y[p] = y.x;
+        Q.z[p] = z.x;
+        Q.q[p] = s0.w;
       }
-      aj.x += ox * cwx;
-      aj.y += shv.x;
-      aj.z += shv.y;
-      const float ex = fmaxf(fmaxf(lx - aj.x, aj.x - hx), 0.f);
-      const float ey = fmaxf(fmaxf(ly - aj.y, aj.y - hy), 0.f);
-      const float ez = fmaxf(fmaxf(lz - aj.z, aj.z - hz), 0.f);
-      const bool keep = valid && (ex * ex + ey * ey + ez * ez < a2);
-      const unsigned bal = __ballot_sync(kFull, keep);
-      if (keep) {
-        const int p = qn + __popc(bal & ((1u << lane) - 1u));
-        Q.x[p] = aj.x;
-        Q.y[p] = aj.y;
-        Q.z[p] = aj.z;
-        Q.q[p] = aj.w;
+      if (k1) {
+        const int p = (at1 + __popc(b1 & lt)) & (2 * kBatch - 1);
+        Q.x[p] = x.y;
+        Q.y[p] = y.y;
+        Q.z[p] = z.y;
+        Q.q[p] = s1.w;
       }
-      qn += __popc(bal);
+      qn += __popc(b0) + __popc(b1);
       __syncwarp();
       if (qn >= kBatch) {
-        pair_batch_f2<M, KIND>(Q, nax, nay, naz, a2, C, W, phi, px, py, pz, cphi, cpx, cpy, cpz);
-        __syncwarp();
-        if (lane < qn - kBatch) {
-          Q.x[lane] = Q.x[kBatch + lane];
-          Q.y[lane] = Q.y[kBatch + lane];
-          Q.z[lane] = Q.z[kBatch + lane];
-          Q.q[lane] = Q.q[kBatch + lane];
-        }
+        pair_batch<M, KIND, kBatch, false>(Q, head, kBatch, nax, nay, naz, a2, C, W, tot);
+        head ^= kBatch;
         qn -= kBatch;
         __syncwarp();
       }
     }
-    if (qn > 0) {  // last partial batch, padded with far-away zero charges
-      for (int t = lane; t < kBatch; t += 32)
-        if (t >= qn) {
-          Q.x[t] = FAR;
-          Q.y[t] = FAR;
-          Q.z[t] = FAR;
-          Q.q[t] = 0.f;
+    if (qn > 0) {  // the last sources, padded to a multiple of 16 with far-away zero charges
+      const int n16 = (qn + 15) & ~15;
+      if (qn + lane < n16) {
+        const int p = head + qn + lane;
+        Q.x[p] = FAR;
+        Q.y[p] = FAR;
+        Q.z[p] = FAR;
+        Q.q[p] = 0.f;
+      }
+      __syncwarp();
+      pair_batch<M, KIND, 16, false>(Q, head, n16, nax, nay, naz, a2, C, W, tot);
+      __syncwarp();
+    }
+    float phi = tot.phi + tot.cphi, px = tot.x + tot.cx, py = tot.y + tot.cy, pz = tot.z + tot.cz;
+    if (split > 1) {  // the warps of the group
+      Q.x[lane] = phi;
+      Q.y[lane] = px;
+      Q.z[lane] = py;
+      Q.q[lane] = pz;
+      __syncthreads();
+      if (part == 0)
+        for (int p = 1; p < split; ++p) {
+          const QueueF& O = shared[p].queue;
+          phi += O.x[lane];
+          px += O.y[lane];
+          py += O.z[lane];
+          pz += O.q[lane];
         }
-      __syncwarp();
-      pair_batch_f2<M, KIND>(Q, nax, nay, naz, a2, C, W, phi, px, py, pz, cphi, cpx, cpy, cpz);
-      __syncwarp();
+      __syncthreads();
     }
-    if (inp) {
-      const int i = s0 + lane;
-      phis[i] = phi + cphi;
-      const float qi = me.w;
-      fs[i] = R4<float>{-qi * (px + cpx), -qi * (py + cpy), -qi * (pz + cpz), 0.f};
+    if (part == 0 && inp) {
+      const int i = (K.runs ? i0 : ib) + lane;
+      K.phis[i] = phi;
+      K.fs[i] = R4<float>{-me.w * px, -me.w * py, -me.w * pz, 0.f};
     }
-    l0 = l1;
+    ib = next;
   }
 }
 
 template <int M, int KIND>
-__global__ void __launch_bounds__(32 * kWarps, MSM_PAIR_MINB) k_short_range_run(PairKArgs a) {
-  short_range_run_body<M, KIND>(a, blockIdx.x);
+__global__ void __launch_bounds__(32 * kWarps, MSM_PAIR_MINB) k_short_range(const __grid_constant__ PairKArgs a) {
+  short_range_body<M, KIND>(a, blockIdx.x);
 }
 
 template <int M>
-__global__ void __launch_bounds__(32 * kWarps, MSM_PAIR_MINB) kb_short_range_run(const PairKArgs* __restrict__ tab,
-                                                                   const int* __restrict__ first, int nrep) {
+__global__ void __launch_bounds__(32 * kWarps, MSM_PAIR_MINB) kb_short_range(const PairKArgs* __restrict__ tab,
+                                                                const int* __restrict__ first, int nrep) {
   const int r = batch_rep(first, nrep, blockIdx.x);
-  short_range_run_body<M, kPairMSM>(tab[r], blockIdx.x - first[r]);
-}
-
-template <int M, int KIND>
-__global__ void __launch_bounds__(32 * kWarps, MSM_PAIR_MINB) k_short_range_f2(PairKArgs a) {
-  short_range_f2_body<M, KIND>(a, blockIdx.x);
+  short_range_body<M, kPairMSM>(tab[r], blockIdx.x - first[r]);
 }
 
 template <int M, int KIND>
@@ -899,13 +870,6 @@ __global__ void __launch_bounds__(32 * kWarps, 4) kb_short_range_c8(const PairKA
                                                                    const int* __restrict__ first, int nrep) {
   const int r = batch_rep(first, nrep, blockIdx.x);
   short_range_c8_body<M, kPairMSM>(tab[r], blockIdx.x - first[r]);
-}
-
-template <int M>
-__global__ void __launch_bounds__(32 * kWarps, MSM_PAIR_MINB) kb_short_range_f2(const PairKArgs* __restrict__ tab,
-                                                                   const int* __restrict__ first, int nrep) {
-  const int r = batch_rep(first, nrep, blockIdx.x);
-  short_range_f2_body<M, kPairMSM>(tab[r], blockIdx.x - first[r]);
 }
 
 }  // namespace
@@ -937,16 +901,38 @@ PairKArgs pair_kargs(const Plan& P) {
   K.cwx = (float)P.cw[0];
   K.cwy = (float)P.cw[1];
   K.cwz = (float)P.cw[2];
-  K.key = P.d.key;
-  K.perm = P.d.perm;
+  K.scell = P.d.scell;
+  K.cellx = P.d.cellx;
   K.natoms = 0;
+  K.runs = 0;
+  K.split = 1;
+  // a piece widens the rows of neighbour cells by its span: a periodic row
+  // must not meet itself
+  K.maxspan = P.P.periodic ? std::max(0, std::min(2, P.nc[0] - P.row_cells)) : 2;
   return K;
 }
 
-// Target runs apply to a plan whose pair kernel takes a cell's targets
-// (pair_targets 32) and whose periodic rows hold at least seven cells.
+// Whether the pair kernel takes runs of 32 atoms (else one cell per warp): a
+// periodic row must hold the piece's three cells beside its neighbours, or
+// the runs would fall into pieces of a few atoms.
 static bool use_runs(const Plan& P) {
-  return P.pair_runs && P.pair_targets != kCl && (!P.P.periodic || P.nc[0] >= 7);
+  return P.pair_runs && P.pair_targets != kCl && (!P.P.periodic || P.nc[0] >= P.row_cells + 2);
+}
+
+// Boxes of fewer cells share each group among the four warps of a block: one
+// warp per group leaves most of the GPU idle (23,558 atoms, 1,000 cells: 52 ->
+// 45 us; 5,001 atoms, 216 cells: 42 -> 21 us; even at 50,001 atoms, 2,197
+// cells: 83 us; at 100,002 atoms 133 -> 141 us).
+constexpr int kSplitCells = 2048;
+
+static int pair_blocks(const PairKArgs& K) {
+  const int64_t groups = K.runs ? ((int64_t)K.natoms + 31) / 32 : K.ncell;
+  return (int)(K.split > 1 ? groups : (groups + kWarps - 1) / kWarps);
+}
+
+template <int M, int KIND>
+void launch_mk(const PairKArgs& K, cudaStream_t st) {
+  k_short_range<M, KIND><<<pair_blocks(K), 32 * kWarps, 0, st>>>(K);
 }
 
 template <int KIND>
@@ -954,17 +940,8 @@ void launch_f2(Plan& P, int64_t n, cudaStream_t st, double alpha = 0.0) {
   PairKArgs K = pair_kargs(P);
   K.W = wolf_consts<float>(alpha, P.P.cutoff);
   K.natoms = (int)n;
-  const int blocks = (P.ncell + kWarps - 1) / kWarps;
-  if (use_runs(P)) {  // runs of 32 consecutive atoms
-    const int br = (int)(((n + 31) / 32 + kWarps - 1) / kWarps);
-    if (KIND == kPairCutoff) k_short_range_run<2, kPairCutoff><<<br, 32 * kWarps, 0, st>>>(K);  // M unused
-    else if (KIND == kPairWolf) k_short_range_run<2, kPairWolf><<<br, 32 * kWarps, 0, st>>>(K);
-    else if (P.P.splitting == 1) k_short_range_run<1, kPairMSM><<<br, 32 * kWarps, 0, st>>>(K);
-    else if (P.P.splitting == 2) k_short_range_run<2, kPairMSM><<<br, 32 * kWarps, 0, st>>>(K);
-    else k_short_range_run<3, kPairMSM><<<br, 32 * kWarps, 0, st>>>(K);
-    return;
-  }
   if (P.pair_targets == kCl) {  // clusters of 8 targets
+    const int blocks = (P.ncell + kWarps - 1) / kWarps;
     if (KIND == kPairCutoff) k_short_range_c8<2, kPairCutoff><<<blocks, 32 * kWarps, 0, st>>>(K);  // M unused
     else if (KIND == kPairWolf) k_short_range_c8<2, kPairWolf><<<blocks, 32 * kWarps, 0, st>>>(K);
     else if (P.P.splitting == 1) k_short_range_c8<1, kPairMSM><<<blocks, 32 * kWarps, 0, st>>>(K);
@@ -972,11 +949,13 @@ void launch_f2(Plan& P, int64_t n, cudaStream_t st, double alpha = 0.0) {
     else k_short_range_c8<3, kPairMSM><<<blocks, 32 * kWarps, 0, st>>>(K);
     return;
   }
-  if (KIND == kPairCutoff) k_short_range_f2<2, kPairCutoff><<<blocks, 32 * kWarps, 0, st>>>(K);  // M unused
-  else if (KIND == kPairWolf) k_short_range_f2<2, kPairWolf><<<blocks, 32 * kWarps, 0, st>>>(K);
-  else if (P.P.splitting == 1) k_short_range_f2<1, kPairMSM><<<blocks, 32 * kWarps, 0, st>>>(K);
-  else if (P.P.splitting == 2) k_short_range_f2<2, kPairMSM><<<blocks, 32 * kWarps, 0, st>>>(K);
-  else k_short_range_f2<3, kPairMSM><<<blocks, 32 * kWarps, 0, st>>>(K);
+  K.runs = use_runs(P);
+  K.split = P.ncell < kSplitCells ? kWarps : 1;
+  if (KIND == kPairCutoff) launch_mk<2, kPairCutoff>(K, st);  // M unused
+  else if (KIND == kPairWolf) launch_mk<2, kPairWolf>(K, st);
+  else if (P.P.splitting == 1) launch_mk<1, kPairMSM>(K, st);
+  else if (P.P.splitting == 2) launch_mk<2, kPairMSM>(K, st);
+  else launch_mk<3, kPairMSM>(K, st);
 }
 
 cudaError_t launch_short_range(Plan& P, int64_t n, cudaStream_t st) {
@@ -1004,10 +983,9 @@ cudaError_t launch_wolf_pairs(Plan& P, int64_t n, double alpha, cudaStream_t st)
 }
 
 struct PairBatch {
-  BatchTable<PairKArgs> cells;  // kWarps cells (or target runs) per block
+  BatchTable<PairKArgs> cells;  // kWarps groups per block
   int splitting = 2;
   int targets = 8;  // the first replica's pair_targets
-  bool runs = false;  // every replica takes target runs
 };
 
 cudaError_t pair_batch_build(const std::vector<BatchRep>& reps, PairBatch** out) {
@@ -1016,17 +994,15 @@ cudaError_t pair_batch_build(const std::vector<BatchRep>& reps, PairBatch** out)
   if (!b) return cudaErrorMemoryAllocation;
   std::vector<PairKArgs> ka;
   std::vector<int> kb;
-  b->runs = !reps.empty();
-  for (const BatchRep& r : reps) b->runs = b->runs && use_runs(*r.plan);
+  if (!reps.empty()) b->targets = reps[0].plan->pair_targets;
   for (const BatchRep& r : reps) {
     PairKArgs K = pair_kargs(*r.plan);
     K.natoms = (int)r.n;
+    K.runs = b->targets != kCl && use_runs(*r.plan);
     ka.push_back(K);
-    if (b->runs) kb.push_back(r.n > 0 ? (int)(((r.n + 31) / 32 + kWarps - 1) / kWarps) : 0);
-    else kb.push_back(r.n > 0 ? (r.plan->ncell + kWarps - 1) / kWarps : 0);
+    kb.push_back(r.n > 0 ? pair_blocks(K) : 0);
     b->splitting = r.plan->P.splitting;
   }
-  if (!reps.empty()) b->targets = reps[0].plan->pair_targets;
   cudaError_t e = make_table(b->cells, ka, kb);
   if (e != cudaSuccess) {
     pair_batch_free(b);
@@ -1039,23 +1015,16 @@ cudaError_t pair_batch_build(const std::vector<BatchRep>& reps, PairBatch** out)
 cudaError_t pair_batch_launch(PairBatch* b, cudaStream_t st) {
   const int nb = b->cells.total;
   if (nb == 0) return cudaSuccess;
-  if (b->runs) {
-    if (b->splitting == 1) kb_short_range_run<1><<<nb, 32 * kWarps, 0, st>>>(b->cells.args, b->cells.first, b->cells.nrep);
-    else if (b->splitting == 2)
-      kb_short_range_run<2><<<nb, 32 * kWarps, 0, st>>>(b->cells.args, b->cells.first, b->cells.nrep);
-    else kb_short_range_run<3><<<nb, 32 * kWarps, 0, st>>>(b->cells.args, b->cells.first, b->cells.nrep);
-    return cudaGetLastError();
-  }
+  const auto& t = b->cells;
   if (b->targets == kCl) {
-    if (b->splitting == 1) kb_short_range_c8<1><<<nb, 32 * kWarps, 0, st>>>(b->cells.args, b->cells.first, b->cells.nrep);
-    else if (b->splitting == 2)
-      kb_short_range_c8<2><<<nb, 32 * kWarps, 0, st>>>(b->cells.args, b->cells.first, b->cells.nrep);
-    else kb_short_range_c8<3><<<nb, 32 * kWarps, 0, st>>>(b->cells.args, b->cells.first, b->cells.nrep);
+    if (b->splitting == 1) kb_short_range_c8<1><<<nb, 32 * kWarps, 0, st>>>(t.args, t.first, t.nrep);
+    else if (b->splitting == 2) kb_short_range_c8<2><<<nb, 32 * kWarps, 0, st>>>(t.args, t.first, t.nrep);
+    else kb_short_range_c8<3><<<nb, 32 * kWarps, 0, st>>>(t.args, t.first, t.nrep);
     return cudaGetLastError();
   }
-  if (b->splitting == 1) kb_short_range_f2<1><<<nb, 32 * kWarps, 0, st>>>(b->cells.args, b->cells.first, b->cells.nrep);
-  else if (b->splitting == 2) kb_short_range_f2<2><<<nb, 32 * kWarps, 0, st>>>(b->cells.args, b->cells.first, b->cells.nrep);
-  else kb_short_range_f2<3><<<nb, 32 * kWarps, 0, st>>>(b->cells.args, b->cells.first, b->cells.nrep);
+  if (b->splitting == 1) kb_short_range<1><<<nb, 32 * kWarps, 0, st>>>(t.args, t.first, t.nrep);
+  else if (b->splitting == 2) kb_short_range<2><<<nb, 32 * kWarps, 0, st>>>(t.args, t.first, t.nrep);
+  else kb_short_range<3><<<nb, 32 * kWarps, 0, st>>>(t.args, t.first, t.nrep);
   return cudaGetLastError();
 }
 

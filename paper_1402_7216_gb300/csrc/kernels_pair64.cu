@@ -54,14 +54,13 @@ struct Pair64Args {
   int esc;                        // exponent added to coordinates before the FP32 test
   int lt;                         // log2 of the targets per group
   int nsplit;                     // warps sharing a group (1: a block's warps take groups of their own)
-  int maxspan;                    // cells a piece may add to its first one
 };
 
 struct alignas(16) Warp64 {
   double src[kRing][4];  // x, y, z, q in the piece's frame
   float fx[kRing], fy[kRing], fz[kRing];
   unsigned char list[kRing][32];
-  SegTableR tab;
+  SegList segs;
 };
 
 // x 2^esc truncated to FP32 (integer operations only: conversions from FP64
@@ -142,66 +141,55 @@ __global__ void __launch_bounds__(32 * kMaxSplit) k_pair64(const __grid_constant
   const int ncx = g.A.nc[0], ncy = g.A.nc[1];
   const float FAR = 1e6f;
   const bool sv = t < nval;
-  const int mycell = sv ? g.key[g.perm[s0 + t]] : INT_MAX;
+  const int mycell = sv ? g.scell[s0 + t] : INT_MAX;
   const R4<double> me = sv ? A.atoms[s0 + t] : R4<double>{0.0, 0.0, 0.0, 0.0};
   for (int l0 = 0; l0 < nval;) {  // one piece per step (the same for every warp of the group)
     const int c0 = __shfl_sync(kFull, mycell, l0);
     const int cx = c0 % ncx, cy = (c0 / ncx) % ncy, cz = c0 / (ncx * ncy);
-    const int climit = c0 + min(A.maxspan, ncx - 1 - cx);
+    const int climit = c0 + min(g.maxspan, ncx - 1 - cx);
     const bool inp = t >= l0 && mycell <= climit;
     const unsigned pb = __ballot_sync(kFull, inp) & (kFull >> (32 - T));
     const int l1 = 32 - __clz(pb);
     const int span = __shfl_sync(kFull, mycell, l1 - 1) - c0;
     // the home block: the atoms of the piece's cells
-    const int h0 = g.cell_start[c0];
-    const int b1 = span >= 1 ? g.cell_start[c0 + 1] : INT_MAX;
-    const int b2 = span >= 2 ? g.cell_start[c0 + 2] : INT_MAX;
-    const int hlen = g.cell_start[c0 + span + 1] - h0;
+    const int h0 = g.cell_start[c0], h1 = g.cell_start[c0 + span + 1];
     const double tx = me.x + A.shx[(inp ? mycell - c0 : 0) + kShift0], ty = me.y, tz = me.z;
     const float ux = trunc_scaled(tx, A.esc), uy = trunc_scaled(ty, A.esc), uz = trunc_scaled(tz, A.esc);
-    float lx = inp ? ux : FAR, ly = inp ? uy : FAR, lz = inp ? uz : FAR;
-    float hx = inp ? ux : -FAR, hy = inp ? uy : -FAR, hz = inp ? uz : -FAR;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      lx = fminf(lx, __shfl_xor_sync(kFull, lx, o));
-      ly = fminf(ly, __shfl_xor_sync(kFull, ly, o));
-      lz = fminf(lz, __shfl_xor_sync(kFull, lz, o));
-      hx = fmaxf(hx, __shfl_xor_sync(kFull, hx, o));
-      hy = fmaxf(hy, __shfl_xor_sync(kFull, hy, o));
-      hz = fmaxf(hz, __shfl_xor_sync(kFull, hz, o));
-    }
-    const int flat = hlen + build_seg_table_run(S.tab, g, cx, cy, cz, span, lx, ly, lz, hx, hy, hz, lane);
-    const int nchunk = (flat + kChunk - 1) / kChunk;
+    const float lx = warp_min(inp ? ux : FAR), ly = warp_min(inp ? uy : FAR), lz = warp_min(inp ? uz : FAR);
+    const float hx = warp_max(inp ? ux : -FAR), hy = warp_max(inp ? uy : -FAR), hz = warp_max(inp ? uz : -FAR);
+    // the ranges of sources: the home block, then the neighbour rows
+    const int nseg = build_segments(S.segs, g, cx, cy, cz, span, lx, ly, lz, hx, hy, hz, lane);
+    int seg = -1, jb = h0 + kChunk * part, je = h1, xb = -cx, oyz = kShift0 | (kShift0 << 4);
+    auto settle = [&]() -> bool {  // at the next 32 sources of this warp, in a later range if this one has ended
+      while (jb >= je) {
+        const int skip = (jb - je) / kChunk;  // chunks of the following ranges that are the other warps'
+        if (++seg >= nseg) return false;
+        const int4 r = S.segs.rec[seg];
+        jb = r.x + kChunk * skip;
+        je = r.y;
+        xb = r.z;
+        oyz = r.w;
+      }
+      return true;
+    };
+    bool more = settle();
     double phi = 0.0, px = 0.0, py = 0.0, pz = 0.0;
     unsigned staged = 0, oldest = 0;  // sources staged so far; the oldest one a list still names
     unsigned head = 0, tail = 0;      // the lane's list: entries popped, entries pushed
-    int seg = 0, c = part;
     for (;;) {
       // find: stage chunks while the ring has room, test the new sources
-      while (c < nchunk && staged - oldest <= kRing - kChunk) {
-        const int f = c * kChunk + lane;
-        c += A.nsplit;
+      while (more && staged - oldest <= kRing - kChunk) {
+        const int j = jb + lane;
         R4<double> a = {0.0, 0.0, 0.0, 0.0};
-        bool keep = f < flat;
+        bool keep = j < je;
         if (keep) {
-          int j, ox, oyz = kShift0 | (kShift0 << 4);
-          if (f < hlen) {
-            j = h0 + f;
-            ox = (j >= b1) + (j >= b2);
-          } else {
-            const int v = f - hlen;
-            while (S.tab.rec[seg + 1].y <= v) ++seg;
-            const int4 r = S.tab.rec[seg], b = S.tab.bnd[seg];
-            const int2 e = S.tab.bnd2[seg];
-            j = r.x + (v - r.y);
-            ox = r.z + (j >= b.x) + (j >= b.y) + (j >= b.z) + (j >= b.w) + (j >= e.x) + (j >= e.y);
-            oyz = r.w;
-          }
           a = A.atoms[j];
-          a.x += A.shx[ox + kShift0];
+          a.x += A.shx[(int)g.cellx[j] + xb + kShift0];
           a.y += A.shy[oyz & 15];
           a.z += A.shz[oyz >> 4];
         }
+        jb += kChunk * A.nsplit;
+        more = settle();
         const float ax = trunc_scaled(a.x, A.esc), ay = trunc_scaled(a.y, A.esc), az = trunc_scaled(a.z, A.esc);
         const float ex = fmaxf(fmaxf(lx - ax, ax - hx), 0.f);
         const float ey = fmaxf(fmaxf(ly - ay, ay - hy), 0.f);
@@ -230,7 +218,6 @@ __global__ void __launch_bounds__(32 * kMaxSplit) k_pair64(const __grid_constant
       // many steps as all lanes have entries for (at least 8, so that the
       // ring's oldest source is let go)
       const unsigned have = tail - head;
-      const bool more = c < nchunk;
       const unsigned steps = more ? max(8u, __reduce_min_sync(kFull, inp ? have : 0xffffffffu))
                                   : __reduce_max_sync(kFull, have);
       double sphi = 0.0, sx = 0.0, sy = 0.0, sz = 0.0;
@@ -331,10 +318,6 @@ Pair64Args pair64_args(const Plan& P, int64_t n, double alpha) {
     A.shz[o] = (o - kShift0) * P.cw[2];
   }
   group_shape(n, A.lt, A.nsplit);
-  // a piece widens the rows of neighbour cells by its span: a periodic row
-  // must not meet itself
-  A.maxspan = 2;
-  if (P.P.periodic) A.maxspan = std::max(0, std::min(2, P.nc[0] - P.row_cells));
   return A;
 }
 

@@ -53,6 +53,8 @@ struct DeviceBuffers {
   // sorted atoms (type T = float or double, selected by precision)
   void* atoms = nullptr;       // R4<T>[cap]: cell-local x, y, z and q
   void* gfrac = nullptr;       // R4<T>[cap]: fractional grid offsets (0..1) and q
+  int* scell = nullptr;        // [cap]: cell of the sorted atom
+  float* cellx = nullptr;      // [cap]: x index of that cell
   int4* gbase = nullptr;       // [cap]: first level-0 index of the basis support per dim
   // per-atom results in sorted order
   void* phis = nullptr;        // T[cap]  short-range potential

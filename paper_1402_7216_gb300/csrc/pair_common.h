@@ -75,61 +75,64 @@ struct PairKArgs {
   int ncell;
   float* phis;
   R4<float>* fs;
-  // target runs (short_range_run_body): cell of every input atom, the sorted
-  // order's input indices and the atom count
-  const int* key;
-  const int* perm;
+  // target runs
+  const int* scell;    // cell of every sorted atom
+  const float* cellx;  // its x index
   int natoms;
+  int runs;     // groups are runs of consecutive sorted atoms (else the chunks of a cell)
+  int split;    // warps sharing a group's sources (1, or the block's kWarps)
+  int maxspan;  // cells a run's piece may add to its first one
 };
 
-constexpr int kRunBnd = 6;  // boundaries inside a row segment of up to 7 cells
-struct SegTableR {
-  int4 rec[2 * kMaxRows + 1];         // (first atom, flat start, x offset of the first cell, (dy + 3) | (dz + 3) << 4); sentinel at the end
-  int4 bnd[2 * kMaxRows];             // first atom of the segment's 2nd..5th cell (INT_MAX where absent)
-  int2 bnd2[2 * kMaxRows];            // ... of its 6th and 7th cell
-  float2 shift[2 * kMaxRows];         // (y, z) shift of the row
+__device__ __forceinline__ float warp_min(float v) {
+  float r;
+  asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+  return r;
+}
+__device__ __forceinline__ float warp_max(float v) {
+  float r;
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+  return r;
+}
+
+// The sources of a piece (targets in cells cx .. cx + span of one row): rows
+// of neighbour cells are contiguous in the sorted atoms (cells are numbered x
+// fastest), one or two ranges each (two where a periodic row wraps).  rec: the
+// range's first atom and end, the x base b and (dy + 3) | (dz + 3) << 4; an
+// atom of the range lies cellx + b cells from cx along x.
+struct SegList {
+  int4 rec[2 * kMaxRows];
 };
 
-// The segment table of the rows about cells (cx .. cx + span, cy, cz): as
-// build_seg_table, each row widened by span cells in +x (the home row's
-// right part moved past the piece's cells), then narrowed to the cells a
-// source within a of the targets' bounding box (lx..hx, ly..hy, lz..hz, in
-// the frame of cell cx) can lie in: a row at y gap gy and z gap gz from the
-// box reaches sqrt(a^2 - gy^2 - gz^2) beyond it in x (with a margin for
-// rounding; the culling tests each source exactly).
-__device__ __forceinline__ int build_seg_table_run(SegTableR& T, const PairKArgs& K, int cx, int cy, int cz, int span,
-                                                   float lx, float ly, float lz, float hx, float hy, float hz,
-                                                   int lane) {
+// Builds the list (lane r: row r of the plan's rows), each row widened by span
+// cells in +x (the home row's right part moved past the piece's cells), then
+// narrowed to the cells a source within a of the targets' bounding box
+// (lx..hx, ly..hy, lz..hz, in the frame of cell cx) can lie in: a row at y gap
+// gy and z gap gz from the box reaches sqrt(a^2 - gy^2 - gz^2) beyond it in x
+// (with a margin for rounding; the culling tests each source exactly).
+// Returns the number of ranges.
+__device__ __forceinline__ int build_segments(SegList& L, const PairKArgs& K, int cx, int cy, int cz, int span,
+                                              float lx, float ly, float lz, float hx, float hy, float hz, int lane) {
   const int* __restrict__ cell_start = K.cell_start;
   const PairArgs& A = K.A;
   const int ncx = A.nc[0], ncy = A.nc[1], ncz = A.nc[2];
-  const int nrows = K.nrows;
-  const float cwy = K.cwy, cwz = K.cwz;
-  int len[2] = {0, 0}, j0s[2] = {0, 0}, ox0s[2] = {0, 0};
-  int bb[2][kRunBnd];
-#pragma unroll
-  for (int g = 0; g < 2; ++g)
-#pragma unroll
-    for (int t = 0; t < kRunBnd; ++t) bb[g][t] = INT_MAX;
-  float2 sh = make_float2(0.f, 0.f);
-  int oyz = 0;
-  if (lane < nrows) {
+  int4 r0 = make_int4(0, 0, 0, 0), r1 = r0;
+  if (lane < K.nrows) {
     int4 row = K.rows[lane];  // (dy, dz, xlo, xhi)
-    oyz = (row.x + 3) | ((row.y + 3) << 4);
+    const int oyz = (row.x + 3) | ((row.y + 3) << 4);
     if (row.x == 0 && row.y == 0) {
       if (row.z > 0) { row.z += span; row.w += span; }  // the home row's right part
     } else {
       row.w += span;
     }
-    const float gy = fmaxf(fmaxf(row.x * cwy - hy, ly - (row.x + 1) * cwy), 0.f);
-    const float gz = fmaxf(fmaxf(row.y * cwz - hz, lz - (row.y + 1) * cwz), 0.f);
+    const float gy = fmaxf(fmaxf(row.x * K.cwy - hy, ly - (row.x + 1) * K.cwy), 0.f);
+    const float gz = fmaxf(fmaxf(row.y * K.cwz - hz, lz - (row.y + 1) * K.cwz), 0.f);
     const float r2 = A.a2f - gy * gy - gz * gz;
     bool inside = r2 > 0.f;
     if (inside) {
       const float reach = sqrtf(r2) * 1.0001f + 1e-3f;
       row.z = max(row.z, (int)floorf((lx - reach) / K.cwx));
       row.w = min(row.w, (int)floorf((hx + reach) / K.cwx));
-      inside = row.z <= row.w;
     }
     int ny = cy + row.x, nz = cz + row.y;
     if (A.periodic) {
@@ -138,63 +141,30 @@ __device__ __forceinline__ int build_seg_table_run(SegTableR& T, const PairKArgs
     } else if (ny < 0 || nz < 0 || ny >= ncy || nz >= ncz) {
       inside = false;
     }
-    const int rbase = (nz * ncy + ny) * ncx;
-    sh = make_float2(row.x * cwy, row.y * cwz);
-#pragma unroll
-    for (int seg = 0; seg < 2; ++seg) {
-      int ox0 = 0, ox1 = -1;
-      if (!inside) {
-      } else if (A.periodic) {  // at most 7 <= ncx cells: the row wraps at one end at most
-        const int xa = cx + row.z, xb = cx + row.w;
-        if (xa < 0) {
-          if (seg == 0) { ox0 = row.z; ox1 = -cx - 1; } else { ox0 = -cx; ox1 = row.w; }
-        } else if (xb >= ncx) {
-          if (seg == 0) { ox0 = row.z; ox1 = ncx - 1 - cx; } else { ox0 = ncx - cx; ox1 = row.w; }
-        } else if (seg == 0) {
-          ox0 = row.z; ox1 = row.w;
-        }
-      } else if (seg == 0) {
-        ox0 = max(row.z, -cx);
-        ox1 = min(row.w, ncx - 1 - cx);
-      }
-      if (ox0 <= ox1) {
-        int x0 = cx + ox0, x1 = cx + ox1;
-        if (A.periodic) {
-          x0 += (x0 < 0) ? ncx : ((x0 >= ncx) ? -ncx : 0);
-          x1 += (x1 < 0) ? ncx : ((x1 >= ncx) ? -ncx : 0);
-        }
-        const int j0 = cell_start[rbase + x0], j1 = cell_start[rbase + x1 + 1];
-#pragma unroll
-        for (int t = 0; t < kRunBnd; ++t) bb[seg][t] = (x0 + 1 + t <= x1) ? cell_start[rbase + x0 + 1 + t] : INT_MAX;
-        len[seg] = j1 - j0;
-        j0s[seg] = j0;
-        ox0s[seg] = ox0;
+    if (inside) {
+      const int* cs = cell_start + (nz * ncy + ny) * ncx + cx;
+      // the row's cells inside the grid, then those beyond one end (the row
+      // holds at most ncx cells, so it wraps at one end at most)
+      const int a0 = max(row.z, -cx), a1 = min(row.w, ncx - 1 - cx);
+      if (a0 <= a1) r0 = make_int4(cs[a0], cs[a1 + 1], -cx, oyz);
+      if (A.periodic && row.z < -cx) {
+        const int b1 = min(row.w, -cx - 1);
+        r1 = make_int4(cs[row.z + ncx], cs[b1 + ncx + 1], -cx - ncx, oyz);
+      } else if (A.periodic && row.w >= ncx - cx) {
+        const int b0 = max(row.z, ncx - cx);
+        r1 = make_int4(cs[b0 - ncx], cs[row.w - ncx + 1], -cx + ncx, oyz);
       }
     }
   }
-  const int mine = len[0] + len[1];
-  int incl = mine;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(kFull, incl, o);
-    if (lane >= o) incl += y;
-  }
-  const int total = __shfl_sync(kFull, incl, 31);
-  const int start = incl - mine;
-  if (lane < nrows) {
-#pragma unroll
-    for (int seg = 0; seg < 2; ++seg) {
-      T.rec[2 * lane + seg] = make_int4(j0s[seg], seg ? start + len[0] : start, ox0s[seg], oyz);
-      T.bnd[2 * lane + seg] = make_int4(bb[seg][0], bb[seg][1], bb[seg][2], bb[seg][3]);
-      T.bnd2[2 * lane + seg] = make_int2(bb[seg][4], bb[seg][5]);
-      T.shift[2 * lane + seg] = sh;
-    }
-  }
-  if (lane == 0) T.rec[2 * nrows] = make_int4(0, INT_MAX, 0, 0);
+  const unsigned lt = (1u << lane) - 1u;
+  const unsigned m0 = __ballot_sync(kFull, r0.x < r0.y), m1 = __ballot_sync(kFull, r1.x < r1.y);
+  // a row's two ranges side by side: the rows keep the plan's order
+  const int at = __popc(m0 & lt) + __popc(m1 & lt);
+  if (r0.x < r0.y) L.rec[at] = r0;
+  if (r1.x < r1.y) L.rec[at + (r0.x < r0.y ? 1 : 0)] = r1;
   __syncwarp();
-  return total;
+  return __popc(m0) + __popc(m1);
 }
-
 
 // The arguments of plan P (kernels_pair.cu; natoms is the caller's).
 PairKArgs pair_kargs(const Plan& P);

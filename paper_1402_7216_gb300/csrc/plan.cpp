@@ -342,9 +342,9 @@ int build_plan(const msm_params* pp, const msm_tuning* tune, Plan* P) {
   }
   P->ncell = P->nc[0] * P->nc[1] * P->nc[2];
   // target runs by default on large boxes, where they were measured faster
-  // (1.63 against 1.72 ms at 42,875 cells); small boxes run too few warps
-  // for the longer row walks of a run (1.15-1.9x slower at 343-1,000 cells)
-  P->pair_runs = TU.pair_runs == 1 || (TU.pair_runs == 0 && P->ncell >= 16384);
+  // (1,600 against 1,727 us at 42,875 cells, 470 against 490 at 15,625; slower
+  // on smaller ones: 271 against 254 us at 7,980 cells)
+  P->pair_runs = TU.pair_runs == 1 || (TU.pair_runs == 0 && P->ncell >= 12288);
   std::vector<int4> offs;
   for (int oz = -2; oz <= 2; ++oz)
     for (int oy = -2; oy <= 2; ++oy)
@@ -529,6 +529,8 @@ int build_plan(const msm_params* pp, const msm_tuning* tune, Plan* P) {
   M(&D.atoms, 4 * T * cap);
   M(&D.gfrac, 4 * T * cap);
   M((void**)&D.gbase, sizeof(int4) * cap);
+  M((void**)&D.scell, sizeof(int) * cap);
+  M((void**)&D.cellx, sizeof(float) * cap);
   M(&D.phis, T * cap);
   M(&D.fs, 4 * T * cap);
   M(&D.glong, 4 * T * cap);
@@ -626,7 +628,7 @@ int build_plan(const msm_params* pp, const msm_tuning* tune, Plan* P) {
 void free_plan(Plan* P) {
   DeviceBuffers& D = P->d;
   void* ptrs[] = {D.key, D.rank, D.perm, D.count, D.csum, D.cell_start, D.atoms,
-                  D.gfrac, D.gbase, D.phis, D.fs, D.glong, D.topK, D.topq, D.topu, D.seg, D.seg2, D.cell_rows,
+                  D.gfrac, D.gbase, D.scell, D.cellx, D.phis, D.fs, D.glong, D.topK, D.topq, D.topu, D.seg, D.seg2, D.cell_rows,
                   D.seg_start, D.partial, D.scalars, D.md_partial, D.md_step, D.status, D.hpos, D.hq,
                   D.hphi, D.hforce, D.henergy, D.lparts, D.fft_work};
   for (void* p : ptrs)
