@@ -101,12 +101,12 @@ __device__ __forceinline__ int slot(int idx, int n, int lo, int periodic) {
   return idx - lo;  // callers only pass indices inside the open grid
 }
 
-// ---- anterpolation: per-block shared-memory patches ----
+// ---- anterpolation: per-block shared-memory patches (mixed plans) ----
 // A block owns B x B x B short-range cells; the level-0 points their atoms
 // can reach form a patch of at most PD^3 points held in shared memory.  Each
 // atom adds its (2S)^3 weighted charges into the patch (shared-memory
-// atomics); the block then adds the patch into the global FP64 grid, so
-// global atomics only meet where neighbouring patches overlap.
+// reductions); the block then adds the patch into the global grid, so
+// global reductions only meet where neighbouring patches overlap.
 struct AnterpArgs {
   int nc[3];        // short-range cells per dimension
   int B;            // cells per block side
@@ -114,142 +114,94 @@ struct AnterpArgs {
   double cw_h[3];   // cell width in units of h
 };
 
-// One thread per atom, and the lanes of a warp take atoms from different
-// cells of the block: the block's atoms are listed rank-major (the first atom
-// of every cell, then the second of every cell, ...), so consecutive threads
-// work on different cells.  Atoms of one cell share most of their support,
-// so this keeps the shared-memory atomics of one warp instruction on
-// different points, and no lane idles while others finish a fuller cell.
+// A block's atoms: the cells of one x row of the block are contiguous in the
+// sorted order, so they are B * B ranges, found in parallel (thread r: range
+// r) and laid end to end.
 constexpr int kAnterpMaxAtoms = 4096;  // atoms per block listed in shared memory
+constexpr int kBlockRows = 16;         // B <= 4
+constexpr int kPatchThreads = 1024;    // largest block of the anterpolation kernel
 
-__device__ __forceinline__ int block_cells(const AnterpArgs& A, const int* __restrict__ cell_start, const int* c0,
-                                           int* cstart, int* ccount) {
-  int k = 0;
-  for (int bz = 0; bz < A.B; ++bz)
-    for (int by = 0; by < A.B; ++by)
-      for (int bx = 0; bx < A.B; ++bx) {
-        int x = c0[0] + bx, y = c0[1] + by, z = c0[2] + bz;
-        if (x >= A.nc[0] || y >= A.nc[1] || z >= A.nc[2]) continue;
-        int c = (z * A.nc[1] + y) * A.nc[0] + x;
-        cstart[k] = cell_start[c];
-        ccount[k] = cell_start[c + 1] - cell_start[c];
-        ++k;
-      }
-  return k;
-}
+struct BlockAtoms {
+  int start[kBlockRows];    // first atom of a range
+  int pre[kBlockRows + 1];  // atoms in the ranges before it
+};
 
-// Rank-major list of the block's atoms (warp 0 builds it); returns the count,
-// or -1 when the block holds more atoms than the list can take.
-__device__ __forceinline__ int build_rank_list(int nk, const int* cstart, const int* ccount, int* list,
-                                               int* maxc_s) {
-  const int lane = threadIdx.x & 31;
-  int total = 0;
+// Fills R (all threads of the block call this) and returns the atom count.
+__device__ __forceinline__ int block_atoms(const AnterpArgs& A, const int* __restrict__ cell_start, int bx, int by,
+                                           int bz, BlockAtoms& R) {
   if (threadIdx.x < 32) {
-    int mx = 0;
-    for (int c = lane; c < nk; c += 32) mx = max(mx, ccount[c]);
-    for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    for (int r = 0; r < mx; ++r)
-      for (int cb = 0; cb < nk; cb += 32) {
-        const int c = cb + lane;
-        const bool has = c < nk && ccount[c] > r;
-        const unsigned bal = __ballot_sync(0xffffffffu, has);
-        const int p = total + __popc(bal & ((1u << lane) - 1u));
-        if (has && p < kAnterpMaxAtoms) list[p] = cstart[c] + r;
-        total += __popc(bal);
-      }
-    if (lane == 0) *maxc_s = total;
+    const int r = threadIdx.x, x0 = bx * A.B, y = by * A.B + r % A.B, z = bz * A.B + r / A.B;
+    int s = 0, len = 0;
+    if (r < A.B * A.B && y < A.nc[1] && z < A.nc[2]) {
+      const int* row = cell_start + (z * A.nc[1] + y) * A.nc[0];
+      s = row[x0];
+      len = row[min(x0 + A.B, A.nc[0])] - s;
+    }
+    int incl = len;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (r >= o) incl += v;
+    }
+    if (r < kBlockRows) R.start[r] = s;
+    if (r <= kBlockRows) R.pre[r] = incl - len;
   }
   __syncthreads();
-  total = *maxc_s;
-  return total > kAnterpMaxAtoms ? -1 : total;
+  return R.pre[kBlockRows];
 }
 
-template <typename T, typename ACC, int ORDER>
-__global__ void __launch_bounds__(256) k_anterp_patch(const R4<T>* __restrict__ gfrac,
-                                                      const int4* __restrict__ gbase,
-                                                      const int* __restrict__ cell_start, AnterpArgs A,
-                                                      GridDims G, double* __restrict__ grid,
-                                                      const double* __restrict__ dscale, double factor) {
-  constexpr int S = Basis<T, ORDER>::S, W = 2 * S;
-  extern __shared__ unsigned char smem_raw[];
-  ACC* patch = reinterpret_cast<ACC*>(smem_raw);
-  __shared__ int cstart[64], ccount[64], list[kAnterpMaxAtoms], tot_s;
-  const int PD = A.pd, np = PD * PD * PD, tid = threadIdx.x;
-  const int c0[3] = {(int)blockIdx.x * A.B, (int)blockIdx.y * A.B, (int)blockIdx.z * A.B};
-  const int lo0 = (int)floor(c0[0] * A.cw_h[0]) - S - 1;
-  const int lo1 = (int)floor(c0[1] * A.cw_h[1]) - S - 1;
-  const int lo2 = (int)floor(c0[2] * A.cw_h[2]) - S - 1;
-  for (int e = tid; e < np; e += blockDim.x) patch[e] = ACC(0);
-  __shared__ int nk_s;
-  if (tid == 0) nk_s = block_cells(A, cell_start, c0, cstart, ccount);
-  __syncthreads();
-  const int nk = nk_s;
-  int total = build_rank_list(nk, cstart, ccount, list, &tot_s);
-  const T sc_all = T(factor * (dscale ? *dscale : 1.0));
-  const int count = total >= 0 ? total : 0;
-  for (int kk = tid; kk < count; kk += blockDim.x) {
-    const int i = list[kk];
-    const R4<T> f = gfrac[i];
-    const int4 b = gbase[i];
-    const T qi = sc_all * f.w;
-    T wx[W], wy[W], wz[W];
-    weights<T, ORDER>(f.x, wx);
-    weights<T, ORDER>(f.y, wy);
-    weights<T, ORDER>(f.z, wz);
-    const int px = b.x - lo0, py = b.y - lo1, pz = b.z - lo2;
-    if (px >= 0 && py >= 0 && pz >= 0 && px + W <= PD && py + W <= PD && pz + W <= PD) {
+// The block's kk-th atom (0 <= kk < total).
+__device__ __forceinline__ int block_atom(const BlockAtoms& R, int kk) {
+  int r = 0;
 #pragma unroll
-      for (int c = 0; c < W; ++c) {
-        const T qz = qi * wz[c];
+  for (int h = kBlockRows / 2; h > 0; h >>= 1) r += kk >= R.pre[r + h] ? h : 0;
+  return R.start[r] + kk - R.pre[r];
+}
+// The same with neighbours in kk 1/32 of the block apart (kk < 32 ceil(total / 32);
+// -1 past the end): the lanes of a warp then take atoms of different cells.
+__device__ __forceinline__ int spread_atom(const BlockAtoms& R, int kk, int total) {
+  const int k = (kk & 31) * ((total + 31) >> 5) + (kk >> 5);
+  return k < total ? block_atom(R, k) : -1;
+}
+
+// FP64 plans: one thread per atom adds its (2S)^3 weighted charges straight to
+// the grid (FP64 reductions in L2).  Thread t takes atom (t mod 32) stride +
+// t / 32, so the lanes of a warp lie far apart and their reductions fall on
+// different points.  Bound by the FP64 rate and the reductions; patches in
+// shared memory (whose FP64 additions are compare-and-swap loops) took 138 us
+// in the 8 blocks of a 3,000-atom system and 123 us at 23,558 atoms.
+constexpr int kWide = 64;  // threads per block of the FP64 atom kernels: small systems still reach every SM
+
+template <int ORDER>
+__global__ void __launch_bounds__(kWide) k_anterp64(const R4<double>* __restrict__ gfrac,
+                                                   const int4* __restrict__ gbase, int n, int stride, GridDims G,
+                                                   double* __restrict__ grid, const double* __restrict__ dscale,
+                                                   double factor) {
+  constexpr int W = 2 * Basis<double, ORDER>::S;
+  const int t = blockIdx.x * kWide + threadIdx.x, i = (t & 31) * stride + (t >> 5);
+  if ((t >> 5) >= stride || i >= n) return;
+  const R4<double> f = gfrac[i];
+  const int4 b = gbase[i];
+  double wx[W], wy[W], wz[W];
+  weights<double, ORDER>(f.x, wx);
+  weights<double, ORDER>(f.y, wy);
+  weights<double, ORDER>(f.z, wz);
+  const double q = f.w * (factor * (dscale ? *dscale : 1.0));
+  int ix[W];
 #pragma unroll
-        for (int bb = 0; bb < W; ++bb) {
-          const T qyz = qz * wy[bb];
-          ACC* row = patch + ((pz + c) * PD + py + bb) * PD + px;
+  for (int a = 0; a < W; ++a) ix[a] = slot(b.x + a, G.n[0], G.lo[0], G.periodic);
 #pragma unroll
-          for (int a = 0; a < W; ++a) atomicAdd(row + a, ACC(qyz * wx[a]));
-        }
-      }
-    } else {  // outside the patch (cannot happen for atoms inside their cells): straight to the grid
-      for (int c = 0; c < W; ++c)
-        for (int bb = 0; bb < W; ++bb)
-          for (int a = 0; a < W; ++a) {
-            int sx = slot(b.x + a, G.n[0], G.lo[0], G.periodic), sy = slot(b.y + bb, G.n[1], G.lo[1], G.periodic),
-                sz = slot(b.z + c, G.n[2], G.lo[2], G.periodic);
-            atomicAdd(grid + ((size_t)sz * G.n[1] + sy) * G.n[0] + sx, (double)(qi * wz[c] * wy[bb] * wx[a]));
-          }
+  for (int c = 0; c < W; ++c) {
+    const int sz = slot(b.z + c, G.n[2], G.lo[2], G.periodic);
+    const double qz = q * wz[c];
+#pragma unroll
+    for (int bb = 0; bb < W; ++bb) {
+      const int sy = slot(b.y + bb, G.n[1], G.lo[1], G.periodic);
+      const double qyz = qz * wy[bb];
+      double* row = grid + ((size_t)sz * G.n[1] + sy) * G.n[0];
+#pragma unroll
+      for (int a = 0; a < W; ++a) atomicAdd(row + ix[a], qyz * wx[a]);
     }
-  }
-  if (total < 0) {  // more atoms than the list holds: one thread per atom, straight to the grid
-    for (int c = 0; c < nk; ++c)
-      for (int m = tid; m < ccount[c]; m += blockDim.x) {
-        const int i = cstart[c] + m;
-        const R4<T> f = gfrac[i];
-        const int4 b = gbase[i];
-        const T qi = sc_all * f.w;
-        T wx[W], wy[W], wz[W];
-        weights<T, ORDER>(f.x, wx);
-        weights<T, ORDER>(f.y, wy);
-        weights<T, ORDER>(f.z, wz);
-        for (int cc = 0; cc < W; ++cc)
-          for (int bb = 0; bb < W; ++bb)
-            for (int a = 0; a < W; ++a) {
-              int sx = slot(b.x + a, G.n[0], G.lo[0], G.periodic), sy = slot(b.y + bb, G.n[1], G.lo[1], G.periodic),
-                  sz = slot(b.z + cc, G.n[2], G.lo[2], G.periodic);
-              atomicAdd(grid + ((size_t)sz * G.n[1] + sy) * G.n[0] + sx, (double)(qi * wz[cc] * wy[bb] * wx[a]));
-            }
-      }
-  }
-  __syncthreads();
-  for (int e = tid; e < np; e += blockDim.x) {
-    const ACC v = patch[e];
-    if (v == ACC(0)) continue;
-    int ix = lo0 + e % PD, iy = lo1 + (e / PD) % PD, iz = lo2 + e / (PD * PD);
-    if (!G.periodic && (ix < G.lo[0] || iy < G.lo[1] || iz < G.lo[2] || ix >= G.lo[0] + G.n[0] ||
-                        iy >= G.lo[1] + G.n[1] || iz >= G.lo[2] + G.n[2]))
-      continue;
-    int sx = slot(ix, G.n[0], G.lo[0], G.periodic), sy = slot(iy, G.n[1], G.lo[1], G.periodic),
-        sz = slot(iz, G.n[2], G.lo[2], G.periodic);
-    atomicAdd(grid + ((size_t)sz * G.n[1] + sy) * G.n[0] + sx, (double)v);
   }
 }
 
@@ -284,29 +236,42 @@ __device__ __forceinline__ void fx_split(float t, int& hi, int& lo) {
 // their (2S)^3 reductions.  The block therefore buckets its atoms by that
 // bank and lays the list out in rounds of 32 slots, slot L of round r holding
 // the r-th atom of bucket L: the 32 lanes of a warp instruction then touch 32
-// different banks.  Buckets fuller than the round count R = ceil(total/32)
-// spill into the empty slots of the others (those lanes share a bank with one
-// other lane).  Integer sums do not depend on the order, so neither the
+// different banks.  There are as many rounds R as the fullest bucket has atoms
+// (~25 % more than total/32; with R = total/32 the overflow of the fuller
+// buckets shared a bank with another lane in nearly every round, 2.2 passes of
+// shared memory per instruction); where the list is too short for that, the
+// overflow spills into the empty slots of the other buckets.  Integer sums do not depend on the order, so neither the
 // bucket ranks nor the spill order affect the result.  Returns the slot count
-// 32 R (unfilled slots hold -1); scratch (at least total + 32 R ints) is the
-// not yet zeroed patch, else the list stays as it is.
-__device__ __forceinline__ int bank_order(int* list, int total, const int4* __restrict__ gbase, int lo0, int lo1,
-                                          int lo2, int PD, int* scratch, int nscratch) {
-  __shared__ int bcnt[32], bempty[33], ovf;
-  const int R = (total + 31) >> 5, nslot = R << 5;
-  if (total == 0 || nscratch < total + nslot) return total;  // block-uniform
+// 32 R (unfilled slots hold -1); scratch (at least 32 R ints) is the not yet
+// zeroed patch, else the list is in the plain order.
+__device__ __forceinline__ int bank_order(const BlockAtoms& A, int total, int* list,
+                                          const int4* __restrict__ gbase, int lo0, int lo1, int lo2, int PD,
+                                          int* scratch, int nscratch) {
+  __shared__ int bcnt[32], bempty[33], ovf, rounds;
+  const int nspread = ((total + 31) >> 5) << 5;
   const int tid = threadIdx.x;
+  if (total == 0) return 0;  // block-uniform
+  if (nscratch < nspread) {  // a patch smaller than its atoms: the plain order
+    for (int kk = tid; kk < total; kk += blockDim.x) list[kk] = block_atom(A, kk);
+    __syncthreads();
+    return total;
+  }
   if (tid < 32) bcnt[tid] = 0;
   if (tid == 0) ovf = 0;
   __syncthreads();
-  for (int kk = tid; kk < total; kk += blockDim.x) {
-    const int4 b = gbase[list[kk]];
+  for (int kk = tid; kk < nspread; kk += blockDim.x) {
+    const int i = spread_atom(A, kk, total);
+    if (i < 0) continue;
+    const int4 b = gbase[i];
     const int key = (((b.z - lo2) * PD + (b.y - lo1)) * PD + (b.x - lo0)) & 31;
     scratch[kk] = key | (atomicAdd(&bcnt[key], 1) << 5);
   }
   __syncthreads();
-  if (tid < 32) {  // empty slots of bucket L: rounds bcnt[L] .. R-1; exclusive prefix over L
-    const int e = max(0, R - bcnt[tid]);
+  if (tid < 32) {
+    // rounds: the fullest bucket's atoms, as far as the list holds them
+    const int Rm = max(nspread >> 5, min(__reduce_max_sync(0xffffffffu, bcnt[tid]), kAnterpMaxAtoms / 32 + 1));
+    // empty slots of bucket L: rounds bcnt[L] .. R-1; exclusive prefix over L
+    const int e = max(0, Rm - bcnt[tid]);
     int incl = e;
     for (int o = 1; o < 32; o <<= 1) {
       const int y = __shfl_up_sync(0xffffffffu, incl, o);
@@ -314,27 +279,76 @@ __device__ __forceinline__ int bank_order(int* list, int total, const int4* __re
     }
     bempty[tid] = incl - e;
     if (tid == 31) bempty[32] = incl;
+    if (tid == 0) rounds = Rm;
   }
-  int* slots = scratch + total;
-  for (int e = tid; e < nslot; e += blockDim.x) slots[e] = -1;
   __syncthreads();
-  for (int kk = tid; kk < total; kk += blockDim.x) {
-    const int key = scratch[kk] & 31, r = scratch[kk] >> 5;
+  const int R = rounds, nslot = R << 5;
+  for (int e = tid; e < nslot; e += blockDim.x)
+    if ((e >> 5) >= bcnt[e & 31]) list[e] = -1;
+  __syncthreads();
+  for (int kk = tid; kk < nspread; kk += blockDim.x) {
+    const int i = spread_atom(A, kk, total);
+    if (i < 0) continue;
+    const int key = scratch[kk] & 31, rank = scratch[kk] >> 5;
     int slot;
-    if (r < R) {
-      slot = (r << 5) | key;
+    if (rank < R) {
+      slot = (rank << 5) | key;
     } else {
       const int o = atomicAdd(&ovf, 1);  // o < total empty slots, since 32 R >= total
       int L = 0;
       while (bempty[L + 1] <= o) ++L;
       slot = ((bcnt[L] + (o - bempty[L])) << 5) | L;
     }
-    slots[slot] = list[kk];
+    list[slot] = i;
   }
   __syncthreads();
-  for (int e = tid; e < nslot; e += blockDim.x) list[e] = slots[e];
-  __syncthreads();
   return nslot;
+}
+
+// Where the patch's points lie on the level-0 grid: offsets of its rows and
+// planes, wrapped (or -1 outside an open grid) once per block.
+struct PatchMap {
+  int64_t plane[32];
+  int row[32];
+};
+
+__device__ __forceinline__ int wrap_or_out(int i, int n, int lo, int periodic) {
+  if (!periodic) return i - lo < 0 || i - lo >= n ? -1 : i - lo;
+  while (i < 0) i += n;
+  while (i >= n) i -= n;
+  return i;
+}
+
+// Threads 0..63 (PD <= 32); the block synchronises before patch_rows.
+__device__ __forceinline__ void patch_map(int PD, int lo1, int lo2, const GridDims& G, PatchMap& M) {
+  const int t = threadIdx.x & 31;
+  if (t >= PD) return;
+  if (threadIdx.x < 32) {
+    const int y = wrap_or_out(lo1 + t, G.n[1], G.lo[1], G.periodic);
+    M.row[t] = y < 0 ? -1 : y * G.n[0];
+  } else if (threadIdx.x < 64) {
+    const int z = wrap_or_out(lo2 + t, G.n[2], G.lo[2], G.periodic);
+    M.plane[t] = z < 0 ? -1 : (int64_t)z * G.n[1] * G.n[0];
+  }
+}
+
+// Walks the PD x PD rows of a patch, a warp per row, its lanes along x: f(patch
+// index, grid index or -1).
+template <typename F>
+__device__ __forceinline__ void patch_rows(int PD, int lo0, const GridDims& G, const PatchMap& M, F&& f) {
+  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  if (lane >= PD) return;
+  const int x = wrap_or_out(lo0 + lane, G.n[0], G.lo[0], G.periodic);
+  int y = threadIdx.x >> 5, z = 0;
+  for (int e = y * PD + lane; e < PD * PD * PD; e += nw * PD, y += nw) {
+    while (y >= PD) {
+      y -= PD;
+      ++z;
+    }
+    const int r = M.row[y];
+    const int64_t p = M.plane[z];
+    f(e, (x | r) < 0 || p < 0 ? (int64_t)-1 : p + (r + x));
+  }
 }
 
 // One atom's (2S)^3 weighted charges straight into the fixed-point grid
@@ -374,20 +388,20 @@ __device__ __forceinline__ void anterp_fx_body(const R4<float>* __restrict__ gfr
   const int PD = A.pd, np = PD * PD * PD, tid = threadIdx.x;
   int* phi_ = reinterpret_cast<int*>(smem_raw);  // coarse sums
   int* plo = phi_ + np;                          // residual sums
-  __shared__ int cstart[64], ccount[64], list[kAnterpMaxAtoms + 32], tot_s, nk_s;  // + one round of slots
-  const int c0[3] = {bx * A.B, by * A.B, bz * A.B};
-  const int lo0 = (int)floor(c0[0] * A.cw_h[0]) - S - 1;
-  const int lo1 = (int)floor(c0[1] * A.cw_h[1]) - S - 1;
-  const int lo2 = (int)floor(c0[2] * A.cw_h[2]) - S - 1;
-  if (tid == 0) nk_s = block_cells(A, cell_start, c0, cstart, ccount);
-  __syncthreads();
-  const int nk = nk_s;
-  const int total = build_rank_list(nk, cstart, ccount, list, &tot_s);
+  __shared__ int list[kAnterpMaxAtoms + 32];  // + one round of slots
+  __shared__ BlockAtoms R;
+  __shared__ PatchMap M;
+  const int lo0 = (int)floor(bx * A.B * A.cw_h[0]) - S - 1;
+  const int lo1 = (int)floor(by * A.B * A.cw_h[1]) - S - 1;
+  const int lo2 = (int)floor(bz * A.B * A.cw_h[2]) - S - 1;
+  patch_map(PD, lo1, lo2, G, M);
+  const int total = block_atoms(A, cell_start, bx, by, bz, R);
+  if (total == 0) return;
   // |q_j| <= 2^18 / (atoms in the patch) bounds the coarse sums; |q_j| < 2^10
   // keeps |t| < 2^22, where the magic-number rounding of fx_split is exact
-  const float qmax = fminf(262144.0f / (float)max(total, 1), 1023.0f);
-  const int count = total >= 0 ? bank_order(list, total, gbase, lo0, lo1, lo2, PD, phi_, 2 * np) : 0;
-  for (int e = tid; e < 2 * np; e += blockDim.x) phi_[e] = 0;
+  const float qmax = fminf(262144.0f / (float)total, 1023.0f);
+  const int count = total <= kAnterpMaxAtoms ? bank_order(R, total, list, gbase, lo0, lo1, lo2, PD, phi_, 2 * np) : 0;
+  for (int e = tid; e < np; e += blockDim.x) reinterpret_cast<int2*>(phi_)[e] = make_int2(0, 0);
   __syncthreads();
   for (int kk = tid; kk < count; kk += blockDim.x) {
     const int i = list[kk];
@@ -421,32 +435,23 @@ __device__ __forceinline__ void anterp_fx_body(const R4<float>* __restrict__ gfr
       anterp_atom_global<ORDER>(f, b, G, gfx);
     }
   }
-  if (total < 0) {  // more atoms than the list holds: one thread per atom, straight to the grid
-    for (int c = 0; c < nk; ++c)
-      for (int m = tid; m < ccount[c]; m += blockDim.x) {
-        const int i = cstart[c] + m;
-        anterp_atom_global<ORDER>(gfrac[i], gbase[i], G, gfx);
-      }
+  if (total > kAnterpMaxAtoms) {  // more atoms than the list holds: one thread per atom, straight to the grid
+    for (int kk = tid; kk < total; kk += blockDim.x) {
+      const int i = block_atom(R, kk);
+      anterp_atom_global<ORDER>(gfrac[i], gbase[i], G, gfx);
+    }
   }
   __syncthreads();
   // flush: the point's value in 2^-31 units, h 2^19 + l, added to the global
   // fixed-point grid with an integer reduction (no FP64 arithmetic)
-  for (int e = tid; e < np; e += blockDim.x) {
+  patch_rows(PD, lo0, G, M, [&](int e, int64_t g) {
     const int h = phi_[e], l = plo[e];
-    if ((h | l) == 0) continue;
-    int ix = lo0 + e % PD, iy = lo1 + (e / PD) % PD, iz = lo2 + e / (PD * PD);
-    if (!G.periodic && (ix < G.lo[0] || iy < G.lo[1] || iz < G.lo[2] || ix >= G.lo[0] + G.n[0] ||
-                        iy >= G.lo[1] + G.n[1] || iz >= G.lo[2] + G.n[2]))
-      continue;
-    int sx = slot(ix, G.n[0], G.lo[0], G.periodic), sy = slot(iy, G.n[1], G.lo[1], G.periodic),
-        sz = slot(iz, G.n[2], G.lo[2], G.periodic);
-    atomicAdd(gfx + ((size_t)sz * G.n[1] + sy) * G.n[0] + sx,
-              (unsigned long long)((long long)h * 524288LL + (long long)l));
-  }
+    if ((h | l) != 0 && g >= 0) atomicAdd(gfx + g, (unsigned long long)((long long)h * 524288LL + (long long)l));
+  });
 }
 
 template <int ORDER>
-__global__ void __launch_bounds__(256) k_anterp_fx(const R4<float>* __restrict__ gfrac, const int4* __restrict__ gbase,
+__global__ void __launch_bounds__(kPatchThreads) k_anterp_fx(const R4<float>* __restrict__ gfrac, const int4* __restrict__ gbase,
                                                    const int* __restrict__ cell_start, AnterpArgs A, GridDims G,
                                                    unsigned long long* __restrict__ gfx) {
   anterp_fx_body<ORDER>(gfrac, gbase, cell_start, A, G, gfx, blockIdx.x, blockIdx.y, blockIdx.z);
@@ -1246,36 +1251,32 @@ __device__ __forceinline__ void interp_patch_atom(const R4<T>& f, const int4& b,
   }
 }
 
-// Lists the block's atoms (rank-major, then bank-ordered with the patch as
-// scratch: the gathers of one warp instruction then read 32 different banks)
-// and stages the patch of u^0 for the block at cell block c0.  Returns the
-// slot count of the list (unfilled slots hold -1), or -1 when the block holds
-// more atoms than the list takes.
-template <typename T>
+// Lists the block's atoms (bank-ordered with the patch as scratch: the gathers
+// of one warp instruction then read 32 different banks) and stages the patch
+// of u^0.  Returns the slot count of the list (unfilled slots hold -1), or -1
+// when the block holds more atoms than the list takes.
 __device__ __forceinline__ int stage_interp_block(const AnterpArgs& A, const int* __restrict__ cell_start,
-                                                  const int4* __restrict__ gbase, const T* __restrict__ u0,
-                                                  const GridDims& G, T* patch, int lo0, int lo1, int lo2, int* cstart,
-                                                  int* ccount, int* list, int* nk_s, int* tot_s, int bx, int by,
-                                                  int bz) {
-  const int PD = A.pd, np = PD * PD * PD;
-  const int c0[3] = {bx * A.B, by * A.B, bz * A.B};
-  if (threadIdx.x == 0) *nk_s = block_cells(A, cell_start, c0, cstart, ccount);
-  __syncthreads();
-  int total = build_rank_list(*nk_s, cstart, ccount, list, tot_s);
-  if (total >= 0)
-    total = bank_order(list, total, gbase, lo0, lo1, lo2, PD, reinterpret_cast<int*>(patch),
-                       np * (int)(sizeof(T) / sizeof(int)));
-  for (int e = threadIdx.x; e < np; e += blockDim.x) {
-    int ix = lo0 + e % PD, iy = lo1 + (e / PD) % PD, iz = lo2 + e / (PD * PD);
-    T v = T(0);
-    if (G.periodic) {
-      v = u0[((size_t)slot(iz, G.n[2], 0, 1) * G.n[1] + slot(iy, G.n[1], 0, 1)) * G.n[0] + slot(ix, G.n[0], 0, 1)];
-    } else if (ix >= G.lo[0] && iy >= G.lo[1] && iz >= G.lo[2] && ix < G.lo[0] + G.n[0] && iy < G.lo[1] + G.n[1] &&
-               iz < G.lo[2] + G.n[2]) {
-      v = u0[((size_t)(iz - G.lo[2]) * G.n[1] + (iy - G.lo[1])) * G.n[0] + (ix - G.lo[0])];
-    }
-    patch[e] = v;
-  }
+                                                  const int4* __restrict__ gbase, const float* __restrict__ u0,
+                                                  const GridDims& G, float* patch, int lo0, int lo1, int lo2,
+                                                  BlockAtoms& R, int* list, int bx, int by, int bz) {
+  const int PD = A.pd;
+  __shared__ PatchMap M;
+  patch_map(PD, lo1, lo2, G, M);
+  int total = block_atoms(A, cell_start, bx, by, bz, R);
+  if (total == 0) return 0;
+  total = total <= kAnterpMaxAtoms
+              ? bank_order(R, total, list, gbase, lo0, lo1, lo2, PD, reinterpret_cast<int*>(patch), PD * PD * PD)
+              : -1;
+  // asynchronous copies: every row's loads are in flight together
+  patch_rows(PD, lo0, G, M, [&](int e, int64_t g) {
+    if (g >= 0)
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(patch + e)),
+                   "l"(u0 + g)
+                   : "memory");
+    else
+      patch[e] = 0.f;
+  });
+  asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
   return total;
 }
@@ -1308,46 +1309,35 @@ struct InterpKArgs {
 // GATHER: interpolate only (u_long and its gradient into glong; no pair
 // results needed, so this runs while the pair sums are still being computed),
 // else also assemble phi, F and the energy partials.
-template <typename T, int ORDER, typename OUT, bool GATHER = false>
+template <int ORDER, typename OUT, bool GATHER = false>
 __device__ __forceinline__ void interp_fwd_body(
-    const R4<T>* __restrict__ gfrac, const int4* __restrict__ gbase, const int* __restrict__ perm,
-    const int* __restrict__ cell_start, const AnterpArgs& AA, const T* __restrict__ u0, const GridDims& G,
-    const AssembleArgs& A, const T* __restrict__ phis, R4<T>* __restrict__ fs, R4<T>* __restrict__ glong,
+    const R4<float>* __restrict__ gfrac, const int4* __restrict__ gbase, const int* __restrict__ perm,
+    const int* __restrict__ cell_start, const AnterpArgs& AA, const float* __restrict__ u0, const GridDims& G,
+    const AssembleArgs& A, const float* __restrict__ phis, R4<float>* __restrict__ fs, R4<float>* __restrict__ glong,
     OUT* __restrict__ phi_out, OUT* __restrict__ force_out, double* __restrict__ partial, int bx, int by, int bz,
     int lin) {
-  constexpr int S = Basis<T, ORDER>::S;
+  constexpr int S = Basis<float, ORDER>::S;
   extern __shared__ unsigned char smem_raw[];
-  T* patch = reinterpret_cast<T*>(smem_raw);
-  __shared__ int cstart[64], ccount[64], list[kAnterpMaxAtoms + 32], nk_s, tot_s;  // + one round of slots
-  const int c0[3] = {bx * AA.B, by * AA.B, bz * AA.B};
-  const int lo0 = (int)floor(c0[0] * AA.cw_h[0]) - S - 1;
-  const int lo1 = (int)floor(c0[1] * AA.cw_h[1]) - S - 1;
-  const int lo2 = (int)floor(c0[2] * AA.cw_h[2]) - S - 1;
-  const int total = stage_interp_block<T>(AA, cell_start, gbase, u0, G, patch, lo0, lo1, lo2, cstart, ccount, list,
-                                          &nk_s, &tot_s, bx, by, bz);
-  const T ih[3] = {T(A.inv_h[0]), T(A.inv_h[1]), T(A.inv_h[2])};
+  float* patch = reinterpret_cast<float*>(smem_raw);
+  __shared__ int list[kAnterpMaxAtoms + 32];  // + one round of slots
+  __shared__ BlockAtoms R;
+  const int lo0 = (int)floor(bx * AA.B * AA.cw_h[0]) - S - 1;
+  const int lo1 = (int)floor(by * AA.B * AA.cw_h[1]) - S - 1;
+  const int lo2 = (int)floor(bz * AA.B * AA.cw_h[2]) - S - 1;
+  const int total =
+      stage_interp_block(AA, cell_start, gbase, u0, G, patch, lo0, lo1, lo2, R, list, bx, by, bz);
+  const float ih[3] = {(float)A.inv_h[0], (float)A.inv_h[1], (float)A.inv_h[2]};
   double e = 0.0;
-  const int nk = nk_s;
-  // atoms from the list, or (over-full block) walked cell by cell
-  const int nlist = total >= 0 ? total : 0;
-  int walk_c = 0, walk_m = threadIdx.x;
-  for (int kk = threadIdx.x;; kk += blockDim.x) {
-    int i;
-    if (total >= 0) {
-      if (kk >= nlist) break;
-      i = list[kk];
-      if (i < 0) continue;  // unfilled slot of the bank-ordered list
-    } else {
-      while (walk_c < nk && walk_m >= ccount[walk_c]) walk_m -= ccount[walk_c++];
-      if (walk_c >= nk) break;
-      i = cstart[walk_c] + walk_m;
-      walk_m += blockDim.x;
-    }
-    const R4<T> f = gfrac[i];
-    T p, g[3];
-    interp_patch_atom<T, ORDER>(f, gbase[i], patch, AA.pd, lo0, lo1, lo2, u0, G, ih, p, g);
-    if (!GATHER) e += Assemble<T>::forward(A, f.w, phis[i], p, fs[i], g, perm[i], phi_out, force_out);
-    glong[i] = R4<T>{g[0], g[1], g[2], p};
+  // atoms from the list, or (over-full block) in the plain order
+  const int nlist = total >= 0 ? total : R.pre[kBlockRows];
+  for (int kk = threadIdx.x; kk < nlist; kk += blockDim.x) {
+    const int i = total >= 0 ? list[kk] : block_atom(R, kk);
+    if (i < 0) continue;  // unfilled slot of the bank-ordered list
+    const R4<float> f = gfrac[i];
+    float p, g[3];
+    interp_patch_atom<float, ORDER>(f, gbase[i], patch, AA.pd, lo0, lo1, lo2, u0, G, ih, p, g);
+    if (!GATHER) e += Assemble<float>::forward(A, f.w, phis[i], p, fs[i], g, perm[i], phi_out, force_out);
+    glong[i] = R4<float>{g[0], g[1], g[2], p};
   }
   if (!GATHER) {
     double bsum = block_sum<256>(e);
@@ -1355,20 +1345,36 @@ __device__ __forceinline__ void interp_fwd_body(
   }
 }
 
-template <typename T, int ORDER, typename OUT>
-__device__ __forceinline__ void interp_fwd_call(const InterpKArgs<T, OUT>& K, int bx, int by, int bz, int lin) {
-  interp_fwd_body<T, ORDER, OUT>(K.gfrac, K.gbase, K.perm, K.cell_start, K.AA, K.u0, K.G, K.A, K.phis, K.fs, K.glong,
-                                 K.phi_out, K.force_out, K.partial, bx, by, bz, lin);
+template <int ORDER, typename OUT>
+__device__ __forceinline__ void interp_fwd_call(const InterpKArgs<float, OUT>& K, int bx, int by, int bz, int lin) {
+  interp_fwd_body<ORDER, OUT>(K.gfrac, K.gbase, K.perm, K.cell_start, K.AA, K.u0, K.G, K.A, K.phis, K.fs, K.glong,
+                              K.phi_out, K.force_out, K.partial, bx, by, bz, lin);
 }
 
-template <typename T, int ORDER>
-__global__ void __launch_bounds__(256, 3) k_interp_gather(const R4<T>* __restrict__ gfrac,
+template <int ORDER>
+__global__ void __launch_bounds__(256, 3) k_interp_gather(const R4<float>* __restrict__ gfrac,
                                                           const int4* __restrict__ gbase,
                                                           const int* __restrict__ cell_start, AnterpArgs AA,
-                                                          const T* __restrict__ u0, GridDims G, AssembleArgs A,
-                                                          R4<T>* __restrict__ glong) {
-  interp_fwd_body<T, ORDER, double, true>(gfrac, gbase, nullptr, cell_start, AA, u0, G, A, nullptr, nullptr, glong,
-                                          nullptr, nullptr, nullptr, blockIdx.x, blockIdx.y, blockIdx.z, 0);
+                                                          const float* __restrict__ u0, GridDims G, AssembleArgs A,
+                                                          R4<float>* __restrict__ glong) {
+  interp_fwd_body<ORDER, double, true>(gfrac, gbase, nullptr, cell_start, AA, u0, G, A, nullptr, nullptr, glong,
+                                       nullptr, nullptr, nullptr, blockIdx.x, blockIdx.y, blockIdx.z, 0);
+}
+
+// FP64 plans: one thread per atom, taps read through the cache (the FP64
+// instructions, two lanes per SM and clock, are the bound: ~300 per atom for
+// the cubic, ~850 for the quintic basis).  Staged patches ran in 8 to 27
+// blocks on small systems (141 us at 3,000 and 23,558 atoms).
+template <int ORDER>
+__global__ void __launch_bounds__(kWide) k_interp_gather64(const R4<double>* __restrict__ gfrac,
+                                                          const int4* __restrict__ gbase, int n,
+                                                          const double* __restrict__ u0, GridDims G, AssembleArgs A,
+                                                          R4<double>* __restrict__ glong) {
+  const int i = blockIdx.x * kWide + threadIdx.x;
+  if (i >= n) return;
+  double p, g[3];
+  interp_atom<double, ORDER>(gfrac[i], gbase[i], u0, G, A.inv_h, p, g);
+  glong[i] = R4<double>{g[0], g[1], g[2], p};
 }
 
 // Assembly after the pair sums and the gather: phi_i, F_i in the caller's
@@ -1404,60 +1410,65 @@ __global__ void __launch_bounds__(1024) k_energy_final(const double* __restrict_
 }
 
 // adjoint assembly: av0 = M (anterpolated 1/2 gE q) on the grid
-template <typename T, int ORDER, typename OUT>
+template <int ORDER, typename OUT>
 __device__ __forceinline__ void interp_bwd_body(
-    const R4<T>* __restrict__ gfrac, const int4* __restrict__ gbase, const int* __restrict__ perm,
-    const int* __restrict__ cell_start, const AnterpArgs& AA, const T* __restrict__ av0, const GridDims& G,
-    const AssembleArgs& A, const T* __restrict__ phis, const R4<T>* __restrict__ fs,
-    const R4<T>* __restrict__ glong, const double* __restrict__ gE, OUT* __restrict__ grad_pos,
+    const R4<float>* __restrict__ gfrac, const int4* __restrict__ gbase, const int* __restrict__ perm,
+    const int* __restrict__ cell_start, const AnterpArgs& AA, const float* __restrict__ av0, const GridDims& G,
+    const AssembleArgs& A, const float* __restrict__ phis, const R4<float>* __restrict__ fs,
+    const R4<float>* __restrict__ glong, const double* __restrict__ gE, OUT* __restrict__ grad_pos,
     OUT* __restrict__ grad_q, int bx, int by, int bz) {
-  constexpr int S = Basis<T, ORDER>::S;
+  constexpr int S = Basis<float, ORDER>::S;
   extern __shared__ unsigned char smem_raw[];
-  T* patch = reinterpret_cast<T*>(smem_raw);
-  __shared__ int cstart[64], ccount[64], list[kAnterpMaxAtoms + 32], nk_s, tot_s;  // + one round of slots
-  const int c0[3] = {bx * AA.B, by * AA.B, bz * AA.B};
-  const int lo0 = (int)floor(c0[0] * AA.cw_h[0]) - S - 1;
-  const int lo1 = (int)floor(c0[1] * AA.cw_h[1]) - S - 1;
-  const int lo2 = (int)floor(c0[2] * AA.cw_h[2]) - S - 1;
-  const int total = stage_interp_block<T>(AA, cell_start, gbase, av0, G, patch, lo0, lo1, lo2, cstart, ccount,
-                                          list, &nk_s, &tot_s, bx, by, bz);
-  const T ih[3] = {T(A.inv_h[0]), T(A.inv_h[1]), T(A.inv_h[2])};
-  const T gg = (T)*gE;
-  const int nk = nk_s, nlist = total >= 0 ? total : 0;
-  int walk_c = 0, walk_m = threadIdx.x;
-  for (int kk = threadIdx.x;; kk += blockDim.x) {
-    int i;
-    if (total >= 0) {
-      if (kk >= nlist) break;
-      i = list[kk];
-      if (i < 0) continue;  // unfilled slot of the bank-ordered list
-    } else {
-      while (walk_c < nk && walk_m >= ccount[walk_c]) walk_m -= ccount[walk_c++];
-      if (walk_c >= nk) break;
-      i = cstart[walk_c] + walk_m;
-      walk_m += blockDim.x;
-    }
-    const R4<T> f = gfrac[i];
-    T v, gv[3];
-    interp_patch_atom<T, ORDER>(f, gbase[i], patch, AA.pd, lo0, lo1, lo2, av0, G, ih, v, gv);
-    Assemble<T>::backward(A, gg, f.w, phis[i], fs[i], glong[i], v, gv, perm[i], grad_pos, grad_q);
+  float* patch = reinterpret_cast<float*>(smem_raw);
+  __shared__ int list[kAnterpMaxAtoms + 32];  // + one round of slots
+  __shared__ BlockAtoms R;
+  const int lo0 = (int)floor(bx * AA.B * AA.cw_h[0]) - S - 1;
+  const int lo1 = (int)floor(by * AA.B * AA.cw_h[1]) - S - 1;
+  const int lo2 = (int)floor(bz * AA.B * AA.cw_h[2]) - S - 1;
+  const int total =
+      stage_interp_block(AA, cell_start, gbase, av0, G, patch, lo0, lo1, lo2, R, list, bx, by, bz);
+  const float ih[3] = {(float)A.inv_h[0], (float)A.inv_h[1], (float)A.inv_h[2]};
+  const float gg = (float)*gE;
+  const int nlist = total >= 0 ? total : R.pre[kBlockRows];
+  for (int kk = threadIdx.x; kk < nlist; kk += blockDim.x) {
+    const int i = total >= 0 ? list[kk] : block_atom(R, kk);
+    if (i < 0) continue;  // unfilled slot of the bank-ordered list
+    const R4<float> f = gfrac[i];
+    float v, gv[3];
+    interp_patch_atom<float, ORDER>(f, gbase[i], patch, AA.pd, lo0, lo1, lo2, av0, G, ih, v, gv);
+    Assemble<float>::backward(A, gg, f.w, phis[i], fs[i], glong[i], v, gv, perm[i], grad_pos, grad_q);
   }
 }
 
-template <typename T, int ORDER, typename OUT>
-__device__ __forceinline__ void interp_bwd_call(const InterpKArgs<T, OUT>& K, int bx, int by, int bz) {
-  interp_bwd_body<T, ORDER, OUT>(K.gfrac, K.gbase, K.perm, K.cell_start, K.AA, K.u0, K.G, K.A, K.phis, K.fs, K.glong,
-                                 K.gE, K.grad_pos, K.grad_q, bx, by, bz);
+template <int ORDER, typename OUT>
+__device__ __forceinline__ void interp_bwd_call(const InterpKArgs<float, OUT>& K, int bx, int by, int bz) {
+  interp_bwd_body<ORDER, OUT>(K.gfrac, K.gbase, K.perm, K.cell_start, K.AA, K.u0, K.G, K.A, K.phis, K.fs, K.glong,
+                              K.gE, K.grad_pos, K.grad_q, bx, by, bz);
 }
 
-template <typename T, int ORDER, typename OUT>
-__global__ void __launch_bounds__(256) k_interp_bwd(
-    const R4<T>* __restrict__ gfrac, const int4* __restrict__ gbase, const int* __restrict__ perm,
-    const int* __restrict__ cell_start, AnterpArgs AA, const T* __restrict__ av0, GridDims G, AssembleArgs A,
-    const T* __restrict__ phis, const R4<T>* __restrict__ fs, const R4<T>* __restrict__ glong,
+template <int ORDER, typename OUT>
+__global__ void __launch_bounds__(256, 3) k_interp_bwd(
+    const R4<float>* __restrict__ gfrac, const int4* __restrict__ gbase, const int* __restrict__ perm,
+    const int* __restrict__ cell_start, AnterpArgs AA, const float* __restrict__ av0, GridDims G, AssembleArgs A,
+    const float* __restrict__ phis, const R4<float>* __restrict__ fs, const R4<float>* __restrict__ glong,
     const double* __restrict__ gE, OUT* __restrict__ grad_pos, OUT* __restrict__ grad_q) {
-  interp_bwd_body<T, ORDER, OUT>(gfrac, gbase, perm, cell_start, AA, av0, G, A, phis, fs, glong, gE, grad_pos, grad_q,
-                                 blockIdx.x, blockIdx.y, blockIdx.z);
+  interp_bwd_body<ORDER, OUT>(gfrac, gbase, perm, cell_start, AA, av0, G, A, phis, fs, glong, gE, grad_pos, grad_q,
+                              blockIdx.x, blockIdx.y, blockIdx.z);
+}
+
+// FP64 plans: one thread per atom, as k_interp_gather64
+template <int ORDER, typename OUT>
+__global__ void __launch_bounds__(kWide) k_interp_bwd64(
+    const R4<double>* __restrict__ gfrac, const int4* __restrict__ gbase, const int* __restrict__ perm, int n,
+    const double* __restrict__ av0, GridDims G, AssembleArgs A, const double* __restrict__ phis,
+    const R4<double>* __restrict__ fs, const R4<double>* __restrict__ glong, const double* __restrict__ gE,
+    OUT* __restrict__ grad_pos, OUT* __restrict__ grad_q) {
+  const int i = blockIdx.x * kWide + threadIdx.x;
+  if (i >= n) return;
+  const R4<double> f = gfrac[i];
+  double v, gv[3];
+  interp_atom<double, ORDER>(f, gbase[i], av0, G, A.inv_h, v, gv);
+  Assemble<double>::backward(A, *gE, f.w, phis[i], fs[i], glong[i], v, gv, perm[i], grad_pos, grad_q);
 }
 
 template <typename T>
@@ -1503,20 +1514,10 @@ AnterpArgs patch_args(const Plan& P, bool batch = false) {
   return A;
 }
 
-template <typename T, typename ACC, int ORDER>
-void anterp_t(Plan& P, void* grid0, const double* dscale, double factor, cudaStream_t st) {
-  AnterpArgs A;
-  for (int d = 0; d < 3; ++d) {
-    A.nc[d] = P.nc[d];
-    A.cw_h[d] = P.cw[d] / P.h[d];
-  }
-  A.B = P.ablk;
-  A.pd = P.apd;
-  dim3 grid(blocks_for(P.nc[0], A.B), blocks_for(P.nc[1], A.B), blocks_for(P.nc[2], A.B));
-  size_t sm = sizeof(ACC) * (size_t)A.pd * A.pd * A.pd;
-  k_anterp_patch<T, ACC, ORDER><<<grid, 256, sm, st>>>((const R4<T>*)P.d.gfrac, P.d.gbase, P.d.cell_start, A,
-                                                     dims_of(P, 0), (double*)grid0, dscale, factor);
-}
+// Threads per anterpolation block: the patch leaves room for two blocks per SM
+// (512 threads: 1.07M atoms 166 -> 148 us against 256) or, beyond 100 KB, for
+// one (1,024 threads: 4.1M atoms 1,175 -> 907 us).
+static int anterp_threads(size_t patch_bytes) { return patch_bytes > 100 * 1024 ? 1024 : 512; }
 
 // Mixed precision: patch sums into the fixed-point grid (in the restriction
 // temporary tmp[0], free until the first restriction pass), then one
@@ -1531,7 +1532,7 @@ void anterp_fx(Plan& P, int64_t n, void* grid0, const double* dscale, double fac
     AnterpArgs A = patch_args(P);
     dim3 grid(blocks_for(P.nc[0], A.B), blocks_for(P.nc[1], A.B), blocks_for(P.nc[2], A.B));
     size_t sm = 2 * sizeof(int) * (size_t)A.pd * A.pd * A.pd;  // coarse and residual sums
-    k_anterp_fx<ORDER><<<grid, 256, sm, st>>>((const R4<float>*)P.d.gfrac, P.d.gbase, P.d.cell_start, A,
+    k_anterp_fx<ORDER><<<grid, anterp_threads(sm), sm, st>>>((const R4<float>*)P.d.gfrac, P.d.gbase, P.d.cell_start, A,
                                               dims_of(P, 0), gfx);
     P.launches += 1;
   }
@@ -1549,8 +1550,13 @@ cudaError_t launch_anterpolate(Plan& P, int64_t n, void* grid0, const double* ds
   cudaMemsetAsync(grid0, 0, bytes, st);
   P.launches += 1 + (n > 0 ? 1 : 0);
   if (n <= 0) return cudaGetLastError();
-  if (P.P.order == 3) anterp_t<double, double, 3>(P, grid0, dscale, factor, st);
-  else anterp_t<double, double, 5>(P, grid0, dscale, factor, st);
+  const int stride = (int)((n + 31) / 32);
+  const unsigned nb = blocks_for((int64_t)32 * stride, kWide);
+  const R4<double>* f = (const R4<double>*)P.d.gfrac;
+  if (P.P.order == 3)
+    k_anterp64<3><<<nb, kWide, 0, st>>>(f, P.d.gbase, (int)n, stride, dims_of(P, 0), (double*)grid0, dscale, factor);
+  else
+    k_anterp64<5><<<nb, kWide, 0, st>>>(f, P.d.gbase, (int)n, stride, dims_of(P, 0), (double*)grid0, dscale, factor);
   return cudaGetLastError();
 }
 
@@ -1837,9 +1843,6 @@ cudaError_t launch_top(Plan& P, const void* qt, void* ut, cudaStream_t st) {
 }
 
 
-#define INTERP_FWD_ARGS(K)                                                                                   \
-  K.gfrac, K.gbase, K.perm, K.cell_start, K.AA, K.u0, K.G, K.A, K.phis, K.fs, K.glong, K.phi_out, K.force_out, \
-      K.partial
 #define INTERP_BWD_ARGS(K) \
   K.gfrac, K.gbase, K.perm, K.cell_start, K.AA, K.u0, K.G, K.A, K.phis, K.fs, K.glong, K.gE, K.grad_pos, K.grad_q
 
@@ -1872,23 +1875,26 @@ InterpKArgs<T, OUT> interp_kargs(Plan& P, bool backward, OUT* phi, OUT* force, c
 
 cudaError_t launch_interp_gather(Plan& P, int64_t n, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  AnterpArgs AA = patch_args(P);
-  dim3 grid(blocks_for(P.nc[0], AA.B), blocks_for(P.nc[1], AA.B), blocks_for(P.nc[2], AA.B));
-  size_t sm = (P.fp64 ? 8 : 4) * (size_t)AA.pd * AA.pd * AA.pd;
   const GridDims G = dims_of(P, 0);
   const AssembleArgs A = assemble_args(P);
-#define MSM_GATHER(T, O)                                                                                          \
-  k_interp_gather<T, O><<<grid, 256, sm, st>>>((const R4<T>*)P.d.gfrac, P.d.gbase, P.d.cell_start, AA,            \
-                                               (const T*)P.d.gu[0], G, A, (R4<T>*)P.d.glong)
-  if (P.fp64) {
-    if (P.P.order == 3) MSM_GATHER(double, 3);
-    else MSM_GATHER(double, 5);
-  } else {
-    if (P.P.order == 3) MSM_GATHER(float, 3);
-    else MSM_GATHER(float, 5);
-  }
-#undef MSM_GATHER
   P.launches += 1;
+  if (P.fp64) {
+    const unsigned nb = blocks_for(n, kWide);
+    const R4<double>* f = (const R4<double>*)P.d.gfrac;
+    const double* u = (const double*)P.d.gu[0];
+    if (P.P.order == 3) k_interp_gather64<3><<<nb, kWide, 0, st>>>(f, P.d.gbase, (int)n, u, G, A, (R4<double>*)P.d.glong);
+    else k_interp_gather64<5><<<nb, kWide, 0, st>>>(f, P.d.gbase, (int)n, u, G, A, (R4<double>*)P.d.glong);
+    return cudaGetLastError();
+  }
+  AnterpArgs AA = patch_args(P);
+  dim3 grid(blocks_for(P.nc[0], AA.B), blocks_for(P.nc[1], AA.B), blocks_for(P.nc[2], AA.B));
+  size_t sm = sizeof(float) * (size_t)AA.pd * AA.pd * AA.pd;
+  const R4<float>* f = (const R4<float>*)P.d.gfrac;
+  const float* u = (const float*)P.d.gu[0];
+  if (P.P.order == 3)
+    k_interp_gather<3><<<grid, 256, sm, st>>>(f, P.d.gbase, P.d.cell_start, AA, u, G, A, (R4<float>*)P.d.glong);
+  else
+    k_interp_gather<5><<<grid, 256, sm, st>>>(f, P.d.gbase, P.d.cell_start, AA, u, G, A, (R4<float>*)P.d.glong);
   return cudaGetLastError();
 }
 
@@ -1918,19 +1924,23 @@ template <typename OUT>
 cudaError_t launch_interp_backward(Plan& P, int64_t n, const double* gE, OUT* grad_pos, OUT* grad_q,
                                    cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  AnterpArgs AA = patch_args(P);
-  dim3 grid(blocks_for(P.nc[0], AA.B), blocks_for(P.nc[1], AA.B), blocks_for(P.nc[2], AA.B));
-  size_t sm = (P.fp64 ? 8 : 4) * (size_t)AA.pd * AA.pd * AA.pd;
   P.launches += 1;
   if (P.fp64) {
-    auto K = interp_kargs<double, OUT>(P, true, nullptr, nullptr, gE, grad_pos, grad_q, nullptr);
-    if (P.P.order == 3) k_interp_bwd<double, 3, OUT><<<grid, 256, sm, st>>>(INTERP_BWD_ARGS(K));
-    else k_interp_bwd<double, 5, OUT><<<grid, 256, sm, st>>>(INTERP_BWD_ARGS(K));
-  } else {
-    auto K = interp_kargs<float, OUT>(P, true, nullptr, nullptr, gE, grad_pos, grad_q, nullptr);
-    if (P.P.order == 3) k_interp_bwd<float, 3, OUT><<<grid, 256, sm, st>>>(INTERP_BWD_ARGS(K));
-    else k_interp_bwd<float, 5, OUT><<<grid, 256, sm, st>>>(INTERP_BWD_ARGS(K));
+    const unsigned nb = blocks_for(n, kWide);
+    const auto K = interp_kargs<double, OUT>(P, true, nullptr, nullptr, gE, grad_pos, grad_q, nullptr);
+    if (P.P.order == 3)
+      k_interp_bwd64<3, OUT><<<nb, kWide, 0, st>>>(K.gfrac, K.gbase, K.perm, (int)n, K.u0, K.G, K.A, K.phis, K.fs,
+                                                   K.glong, gE, grad_pos, grad_q);
+    else
+      k_interp_bwd64<5, OUT><<<nb, kWide, 0, st>>>(K.gfrac, K.gbase, K.perm, (int)n, K.u0, K.G, K.A, K.phis, K.fs,
+                                                   K.glong, gE, grad_pos, grad_q);
+    return cudaGetLastError();
   }
+  const auto K = interp_kargs<float, OUT>(P, true, nullptr, nullptr, gE, grad_pos, grad_q, nullptr);
+  dim3 grid(K.nbx, K.nby, blocks_for(P.nc[2], K.AA.B));
+  size_t sm = sizeof(float) * (size_t)K.AA.pd * K.AA.pd * K.AA.pd;
+  if (P.P.order == 3) k_interp_bwd<3, OUT><<<grid, 256, sm, st>>>(INTERP_BWD_ARGS(K));
+  else k_interp_bwd<5, OUT><<<grid, 256, sm, st>>>(INTERP_BWD_ARGS(K));
   return cudaGetLastError();
 }
 
@@ -2112,7 +2122,7 @@ __global__ void __launch_bounds__(kEw) kb_f64_to_f32(const ConvKArgs* __restrict
 }
 
 template <int ORDER>
-__global__ void __launch_bounds__(256, 2) kb_anterp_fx(const AntKArgs* __restrict__ tab, const int* __restrict__ first,
+__global__ void __launch_bounds__(512, 2) kb_anterp_fx(const AntKArgs* __restrict__ tab, const int* __restrict__ first,
                                                     int nrep) {
   const int r = batch_rep(first, nrep, blockIdx.x);
   const AntKArgs& a = tab[r];
@@ -2139,21 +2149,21 @@ __global__ void __launch_bounds__(32 * kTopWarps) kb_top(const TopKArgs* __restr
 }
 
 template <int ORDER>
-__global__ void __launch_bounds__(256, 2) kb_interp_fwd(const InterpKArgs<float, double>* __restrict__ tab,
+__global__ void __launch_bounds__(256, 3) kb_interp_fwd(const InterpKArgs<float, double>* __restrict__ tab,
                                                      const int* __restrict__ first, int nrep) {
   const int r = batch_rep(first, nrep, blockIdx.x);
   const InterpKArgs<float, double>& K = tab[r];
   const int b = blockIdx.x - first[r];
-  interp_fwd_call<float, ORDER, double>(K, b % K.nbx, (b / K.nbx) % K.nby, b / (K.nbx * K.nby), b);
+  interp_fwd_call<ORDER, double>(K, b % K.nbx, (b / K.nbx) % K.nby, b / (K.nbx * K.nby), b);
 }
 
 template <int ORDER>
-__global__ void __launch_bounds__(256, 2) kb_interp_bwd(const InterpKArgs<float, double>* __restrict__ tab,
+__global__ void __launch_bounds__(256, 3) kb_interp_bwd(const InterpKArgs<float, double>* __restrict__ tab,
                                                      const int* __restrict__ first, int nrep) {
   const int r = batch_rep(first, nrep, blockIdx.x);
   const InterpKArgs<float, double>& K = tab[r];
   const int b = blockIdx.x - first[r];
-  interp_bwd_call<float, ORDER, double>(K, b % K.nbx, (b / K.nbx) % K.nby, b / (K.nbx * K.nby));
+  interp_bwd_call<ORDER, double>(K, b % K.nbx, (b / K.nbx) % K.nby, b / (K.nbx * K.nby));
 }
 
 __global__ void __launch_bounds__(1024) kb_energy_final(const EnergyKArgs* __restrict__ tab,
@@ -2645,7 +2655,7 @@ cudaError_t grid_batch_front(GridBatch* B, bool backward, cudaStream_t st) {
   if (backward && !B->has_backward) return cudaErrorInvalidValue;
   const bool o3 = B->order == 3;
   launch_table(B->zero_fx, kb_zero, kEw, st);
-  launch_table(B->anterp, o3 ? kb_anterp_fx<3> : kb_anterp_fx<5>, 256, st);
+  launch_table(B->anterp, o3 ? kb_anterp_fx<3> : kb_anterp_fx<5>, 512, st);
   launch_table(B->fx[0], kb_fx_to_f64, kEw, st);
   if (backward) launch_table(B->fx[1], kb_fx_to_f64, kEw, st);
   return cudaGetLastError();
@@ -2705,10 +2715,8 @@ cudaError_t configure_kernels() {
     cudaError_t r = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLatticeSmemMax);
     if (r != cudaSuccess) e = r;
   };
-  set((const void*)k_interp_gather<float, 3>);
-  set((const void*)k_interp_gather<float, 5>);
-  set((const void*)k_interp_gather<double, 3>);
-  set((const void*)k_interp_gather<double, 5>);
+  set((const void*)k_interp_gather<3>);
+  set((const void*)k_interp_gather<5>);
   set((const void*)k_lattice_f2<kLatticeLP, 4, 8>);
   set((const void*)k_lattice_f2<kLatticeLP, 0, 0>);
   set((const void*)kb_lattice_f2);
@@ -2720,16 +2728,10 @@ cudaError_t configure_kernels() {
   set((const void*)kb_interp_bwd<5>);
   set((const void*)k_anterp_fx<3>);
   set((const void*)k_anterp_fx<5>);
-  set((const void*)k_anterp_patch<double, double, 3>);
-  set((const void*)k_anterp_patch<double, double, 5>);
-  set((const void*)k_interp_bwd<float, 3, double>);
-  set((const void*)k_interp_bwd<float, 3, float>);
-  set((const void*)k_interp_bwd<float, 5, double>);
-  set((const void*)k_interp_bwd<float, 5, float>);
-  set((const void*)k_interp_bwd<double, 3, double>);
-  set((const void*)k_interp_bwd<double, 3, float>);
-  set((const void*)k_interp_bwd<double, 5, double>);
-  set((const void*)k_interp_bwd<double, 5, float>);
+  set((const void*)k_interp_bwd<3, double>);
+  set((const void*)k_interp_bwd<3, float>);
+  set((const void*)k_interp_bwd<5, double>);
+  set((const void*)k_interp_bwd<5, float>);
   if (e == cudaSuccess) e = configure_fft_kernels();
   if (e == cudaSuccess) e = configure_pair64_kernels();
   return e;

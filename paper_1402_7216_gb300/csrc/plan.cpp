@@ -410,15 +410,17 @@ int build_plan(const msm_params* pp, const msm_tuning* tune, Plan* P) {
     P->apd_batch = patch_dim(B);
     if (TU.patch_cells == 0 && !P->fp64) {
       // one system alone, mixed precision: by default smaller patches for
-      // small systems, down to 2 cells a side until the patch blocks fill the
-      // 152 SMs once (water23k: 0.40 -> 0.34 ms serialised; the FP64 path
-      // measured 2 % slower with them); a batch fills the GPU with its replicas
+      // small systems, down to 2 cells a side until the patch blocks nearly
+      // fill the 152 SMs once (23,558 atoms, 10 cells a side: anterpolation 24
+      // us with 125 blocks of 2^3 cells, 40 with 64 of 3^3; 190,977 atoms: 54
+      // us with 150 blocks of 4^3 cells, 65 with 343 of 3^3); a batch fills
+      // the GPU with its replicas
       auto blocks = [&](int b) {
         int64_t nb = 1;
         for (int d = 0; d < 3; ++d) nb *= (P->nc[d] + b - 1) / b;
         return nb;
       };
-      while (B > 2 && blocks(B) < 152) --B;
+      while (B > 2 && blocks(B) < 120) --B;
     }
     P->ablk = B;
     P->apd = patch_dim(B);
@@ -513,7 +515,8 @@ int build_plan(const msm_params* pp, const msm_tuning* tune, Plan* P) {
   {  // one energy partial per interpolation block (blocks of ablk^3 cells)
     int64_t nb = 1;
     for (int d = 0; d < 3; ++d) nb *= (P->nc[d] + P->ablk - 1) / P->ablk;
-    P->nblk_partial = (int)std::max<int64_t>(nb, 1);
+    // ... and at least eight blocks per SM of the assembly where the atoms allow
+    P->nblk_partial = (int)std::max<int64_t>(std::max<int64_t>(nb, 1), std::min<int64_t>((cap + 255) / 256, 8 * 152));
   }
   cudaError_t e = cudaSuccess;
   auto M = [&](void** ptr, size_t bytes) {
