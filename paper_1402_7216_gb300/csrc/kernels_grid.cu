@@ -729,130 +729,88 @@ __global__ void k_prolong3(const T* __restrict__ in, T* __restrict__ out, Grid3A
   out[t] = out[t] + acc;  // onto u^{k, cutoff}
 }
 
-// ---- lattice cutoff: z-streaming shared-memory planes, register tiles ----
-// A block of 4 warps owns a brick of outputs 32 (x) x LBY (y) x 4 (z); warp w
+// ---- lattice cutoff by the stencil, FP64 ----
+// One thread per output point, the stencil as rows of taps along x (dy, dz, half
+// length X, coefficients of dx = -X .. X).  Bound by the FP64 rate (2 lanes per
+// SM and clock), so what counts is one FP64 FMA per tap and no other: the rows
+// hold no padding, the coefficients are warp-uniform loads, the charges come
+// through the cache, and all index arithmetic runs beside the FMAs.  Small
+// grids share the rows among gridDim.y blocks, whose parts k_lattice_reduce
+// adds in order (no atomics: reproducible).  Register tiles of 8 outputs with
+// segments of 8 taps spent ~3x the FMAs on padding and idle lanes on a 16^3
+// grid: 251 -> 65 us for both levels of a 3,000-atom open system alone, and
+// 888 -> 146 us beside the pair sums.
+constexpr int kLat64 = 128;  // threads per block
+
+template <bool PERIODIC>
+__global__ void __launch_bounds__(kLat64) k_lattice64(const double* __restrict__ q, double* __restrict__ u,
+                                                     double* __restrict__ up, GridDims G,
+                                                     const int4* __restrict__ rows, const double* __restrict__ coef,
+                                                     int nrows, int per, double scale) {
+  const int n0 = G.n[0], n1 = G.n[1], n2 = G.n[2];
+  const int64_t np = (int64_t)n0 * n1 * n2, p = (int64_t)blockIdx.x * kLat64 + threadIdx.x;
+  if (p >= np) return;
+  const int x = (int)(p % n0), y = (int)((p / n0) % n1), z = (int)(p / ((int64_t)n0 * n1));
+  const int r1 = min(nrows, ((int)blockIdx.y + 1) * per);
+  double acc = 0.0;
+  for (int r = blockIdx.y * per; r < r1; ++r) {
+    const int4 R = rows[r];  // (dy, dz, X, first coefficient)
+    int yy = y + R.x, zz = z + R.y;
+    if (PERIODIC) {
+      while (yy < 0) yy += n1;
+      while (yy >= n1) yy -= n1;
+      while (zz < 0) zz += n2;
+      while (zz >= n2) zz -= n2;
+    } else if (yy < 0 || zz < 0 || yy >= n1 || zz >= n2) {
+      continue;
+    }
+    const double* row = q + ((int64_t)zz * n1 + yy) * n0;
+    const double* g = coef + R.w;
+    double sum = 0.0;
+    if (PERIODIC) {
+      int i = x - R.z;
+      while (i < 0) i += n0;
+#pragma unroll 4
+      for (int k = 0; k <= 2 * R.z; ++k) {
+        sum = fma(g[k], row[i], sum);
+        i = i + 1 == n0 ? 0 : i + 1;
+      }
+    } else {
+#pragma unroll 4
+      for (int k = 0; k <= 2 * R.z; ++k) {
+        const int i = x - R.z + k;
+        const double v = i >= 0 && i < n0 ? row[i] : 0.0;
+        sum = fma(g[k], v, sum);
+      }
+    }
+    acc += sum;
+  }
+  acc *= scale;
+  if (gridDim.y > 1) up[(int64_t)blockIdx.y * np + p] = acc;
+  else u[p] = acc;
+}
+
+// ---- lattice cutoff by the stencil, FP32: z-streaming shared-memory planes, register tiles ----
+// A block of 4 warps owns a brick of outputs 32 (x) x 16 (y) x 4 (z); warp w
 // owns plane z0 + w.  The input planes are staged one at a time in shared
 // memory (a 2-D window with halo Ex, Ey; odd row pitch so the lanes of a warp
 // sit on distinct banks); for staged plane zi, warp w applies the stencil rows
 // of dz = zi - (z0 + w) as segments of 8 taps along x on register tiles of
-// 8 consecutive x outputs per lane.  Coarse levels with few bricks split the
-// input planes over several blocks (nsplit) that add their partial sums into
-// the zeroed output; per-plane partial sums are folded into the totals with
-// TwoSum in mixed precision.
-//   FP64: one row per lane (LBY = 8), scalar FMA.
-//   FP32: two rows per lane (LBY = 16) packed into float2, one FFMA2 per two
-//         outputs, coefficients stored pre-duplicated as float2 pairs.
-constexpr int LBX = 32, LBZ = 4, LPX = 8;
+// 8 consecutive x outputs per lane, two rows packed into float2 (one FFMA2
+// per two outputs).  Coarse levels with few bricks split the input planes over
+// several blocks (nsplit): block part writes its partial sums to
+// up[part][point] and k_lattice_reduce adds the parts in order.
+constexpr int LBX = 32;         // window of the FP64 form's support check (plan geometry)
 constexpr int kLatticeLP = 8;   // x outputs per lane of the FP32 lattice kernel (8 or 16)
 constexpr int kLatticeZ = 4;    // warps (output planes) per block of the FP32 lattice kernel
 constexpr size_t kLatticeSmemMax = 200 * 1024;  // dynamic shared memory the FP32 lattice kernels may use
-
-template <typename T>
-__device__ __forceinline__ void two_sum_add(T& s, T& c, T x) {
-  T t = s + x;
-  T bp = t - s;
-  c += (s - (t - bp)) + (x - bp);
-  s = t;
-}
-
-// Stages plane zi of q into plane[] (rows SY, staged width SXw, pitch SX).
-template <typename T>
-__device__ __forceinline__ void stage_plane(T* plane, const T* __restrict__ q, const GridDims& G, int zi, int x0,
-                                            int y0, int Ex, int Ey, int SXw, int SX, int SY) {
-  int gz;
-  bool zok;
-  if (G.periodic) {
-    gz = zi % G.n[2];
-    if (gz < 0) gz += G.n[2];
-    zok = true;
-  } else {
-    gz = zi;
-    zok = (zi >= 0 && zi < G.n[2]);
-  }
-  for (int e = threadIdx.x; e < SY * SXw; e += blockDim.x) {
-    int xx = e % SXw, yy = e / SXw;
-    int gx = x0 - Ex + xx, gy = y0 - Ey + yy;
-    T v = T(0);
-    if (G.periodic) {
-      gx %= G.n[0];
-      if (gx < 0) gx += G.n[0];
-      gy %= G.n[1];
-      if (gy < 0) gy += G.n[1];
-      v = q[((size_t)gz * G.n[1] + gy) * G.n[0] + gx];
-    } else if (zok && gx >= 0 && gx < G.n[0] && gy >= 0 && gy < G.n[1]) {
-      v = q[((size_t)gz * G.n[1] + gy) * G.n[0] + gx];
-    }
-    plane[yy * SX + xx] = v;
-  }
-}
 
 struct LatticeArgs {
   int Ex, Ey, Ez;
   int nsplit;  // blocks sharing one brick's input planes
   int nbz;     // bricks along z
-  int txn, tyn;  // FP32 kernel: lanes along x (LP outputs each) and along y (two rows each) of a warp's tile
+  int txn, tyn;  // lanes along x (LP outputs each) and along y (two rows each) of a warp's tile
 };
-
-// When several blocks share a brick's input planes (L.nsplit > 1), block
-// part writes its partial sums to up[part][point] and k_lattice_reduce adds
-// the parts in order: no atomics, so the sums are reproducible.
-template <typename T, bool COMP>
-__global__ void __launch_bounds__(128) k_lattice(const T* __restrict__ q, T* __restrict__ u, T* __restrict__ up,
-                                                 GridDims G, const Segment<T>* __restrict__ seg,
-                                                 const int* __restrict__ seg_start, LatticeArgs L, T scale) {
-  constexpr int LBY = 8;
-  extern __shared__ unsigned char smem_raw[];
-  T* plane = reinterpret_cast<T*>(smem_raw);
-  const int Ex = L.Ex, Ey = L.Ey, Ez = L.Ez;
-  const int SXw = LBX + 2 * Ex + kSeg, SX = SXw | 1, SY = LBY + 2 * Ey;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, tx = lane & 3, ty = lane >> 2;
-  const int bz = blockIdx.z % L.nbz, part = blockIdx.z / L.nbz;
-  const int x0 = blockIdx.x * LBX, y0 = blockIdx.y * LBY, z0 = bz * LBZ, zo = z0 + warp;
-  const int nplanes = LBZ + 2 * Ez, per = (nplanes + L.nsplit - 1) / L.nsplit;
-  const int zbeg = z0 - Ez + part * per, zend = min(z0 - Ez + nplanes, zbeg + per);
-  T acc[LPX], cmp[LPX];
-#pragma unroll
-  for (int j = 0; j < LPX; ++j) acc[j] = cmp[j] = T(0);
-  for (int zi = zbeg; zi < zend; ++zi) {
-    __syncthreads();
-    stage_plane(plane, q, G, zi, x0, y0, Ex, Ey, SXw, SX, SY);
-    __syncthreads();
-    const int dz = zi - zo;
-    if (dz < -Ez || dz > Ez || zo >= G.n[2]) continue;  // warp-uniform
-    T part_[LPX];
-#pragma unroll
-    for (int j = 0; j < LPX; ++j) part_[j] = T(0);
-    const int s1 = seg_start[dz + Ez + 1];
-    for (int s = seg_start[dz + Ez]; s < s1; ++s) {
-      const Segment<T> sg = seg[s];
-      const T* row = plane + (ty + Ey + sg.dy) * SX + tx * LPX + Ex + sg.dx0;
-      T win[LPX + kSeg - 1];
-#pragma unroll
-      for (int k = 0; k < LPX + kSeg - 1; ++k) win[k] = row[k];
-#pragma unroll
-      for (int k = 0; k < kSeg; ++k)
-#pragma unroll
-        for (int j = 0; j < LPX; ++j) part_[j] += sg.g[k] * win[j + k];
-    }
-#pragma unroll
-    for (int j = 0; j < LPX; ++j) {
-      if (COMP) two_sum_add(acc[j], cmp[j], part_[j]);
-      else acc[j] += part_[j];
-    }
-  }
-  if (zo >= G.n[2]) return;
-  const int y = y0 + ty;
-  if (y >= G.n[1]) return;
-#pragma unroll
-  for (int j = 0; j < LPX; ++j) {
-    int x = x0 + tx * LPX + j;
-    if (x >= G.n[0]) continue;
-    T v = scale * (acc[j] + cmp[j]);
-    const size_t o = ((size_t)zo * G.n[1] + y) * G.n[0] + x;
-    if (L.nsplit > 1) up[(size_t)part * G.n[0] * G.n[1] * G.n[2] + o] = v;
-    else u[o] = v;
-  }
-}
 
 // Window offsets of a block, computed once (the periodic wrap costs integer
 // divisions): col[xx] = grid x index of window column xx (-1 outside an open
@@ -1722,20 +1680,31 @@ static size_t lattice_smem(int txn, int tyn, const int E[3]) {
   return sizeof(float) * 2 * SX * SY + sizeof(int) * (SXw + SY);
 }
 
-// Lattice cutoff of level k from the FP64 charges qk.  Mixed precision first
-// converts the level's charges to FP32 once (on GB300 the conversion runs on
-// the slow FP64 pipe, so it must not sit in the per-tap loop).
-template <typename T>
-void lattice_t(Plan& P, int k, const double* qk64, T* uk, cudaStream_t st) {
-  GridDims G = dims_of(P, k);
-  const bool f32 = !std::is_same<T, double>::value;
-  const T* qk = (const T*)qk64;
-  if (f32) {
-    float* qf = (float*)P.d.tmp[0];  // free between the restriction and the prolongation passes
-    k_f64_to_f32<<<blocks_for(grid_points(P, k), 256), 256, 0, st>>>(qk64, qf, grid_points(P, k));
+// Lattice cutoff of level k by the stencil from the FP64 charges qk.
+static void lattice_fp64(Plan& P, int k, const double* qk, double* uk, cudaStream_t st) {
+  const GridDims G = dims_of(P, k);
+  const int64_t np = grid_points(P, k);
+  const int ns = lattice_nsplit(P, k), per = (P.nlrows + ns - 1) / ns;
+  double* up = (double*)P.d.lparts;
+  dim3 grid(blocks_for(np, kLat64), ns);
+  const double scale = std::ldexp(1.0, -k);
+  const double* coef = (const double*)P.d.seg;
+  if (G.periodic) k_lattice64<true><<<grid, kLat64, 0, st>>>(qk, uk, up, G, P.d.lrows, coef, P.nlrows, per, scale);
+  else k_lattice64<false><<<grid, kLat64, 0, st>>>(qk, uk, up, G, P.d.lrows, coef, P.nlrows, per, scale);
+  if (ns > 1) {
+    k_lattice_reduce<double><<<blocks_for(np, 256), 256, 0, st>>>(up, uk, np, ns);
     P.launches += 1;
-    qk = (const T*)qf;
   }
+}
+
+// The same on the mixed plan, which first converts the level's charges to
+// FP32 once (the conversion runs on the slow FP64 pipe, so it must not sit in
+// the per-tap loop).
+static void lattice_fp32(Plan& P, int k, const double* qk64, float* uk, cudaStream_t st) {
+  GridDims G = dims_of(P, k);
+  float* qk = (float*)P.d.tmp[0];  // free between the restriction and the prolongation passes
+  k_f64_to_f32<<<blocks_for(grid_points(P, k), 256), 256, 0, st>>>(qk64, qk, grid_points(P, k));
+  P.launches += 1;
   LatticeArgs L;
   L.Ex = P.E[0];
   L.Ey = P.E[1];
@@ -1744,31 +1713,22 @@ void lattice_t(Plan& P, int k, const double* qk64, T* uk, cudaStream_t st) {
   // runtime-tile kernel is slower per tap than the saving on ragged coarse
   // levels), unless the plan's tuning names another tile for level 0
   lattice_tile_of(P, k, L.txn, L.tyn);
-  const int TW = f32 ? kLatticeLP * L.txn : LBX, LBY = f32 ? 2 * L.tyn : 8;
-  const int LBZb = f32 ? kLatticeZ : LBZ;  // output planes (warps) per block
-  L.nbz = (int)blocks_for(G.n[2], LBZb);
+  L.nbz = (int)blocks_for(G.n[2], kLatticeZ);
   L.nsplit = lattice_nsplit(P, k);
-  T* up = (T*)P.d.lparts;
-  dim3 grid(blocks_for(G.n[0], TW), blocks_for(G.n[1], LBY), L.nbz * L.nsplit);
-  int SX = (LBX + 2 * P.E[0] + kSeg) | 1, SY = LBY + 2 * P.E[1];
-  // FP32 double-buffers its planes and keeps the window offsets (SXw + SY ints)
-  size_t sm = f32 ? lattice_smem(L.txn, L.tyn, P.E) : sizeof(T) * SX * SY;
-  T scale = (T)std::ldexp(1.0, -k);
-  if (f32) {
-    if (L.txn == 4 && L.tyn == 8)
-      k_lattice_f2<kLatticeLP, 4, 8><<<grid, 32 * kLatticeZ, sm, st>>>((const float*)qk, (float*)uk, (float*)up, G,
-                                                                      (const Segment2*)P.d.seg2, P.d.seg_start, L,
-                                                                      (float)scale);
-    else
-      k_lattice_f2<kLatticeLP, 0, 0><<<grid, 32 * kLatticeZ, sm, st>>>((const float*)qk, (float*)uk, (float*)up, G,
-                                                                      (const Segment2*)P.d.seg2, P.d.seg_start, L,
-                                                                      (float)scale);
-  } else {
-    k_lattice<T, false><<<grid, 128, sm, st>>>(qk, uk, up, G, (const Segment<T>*)P.d.seg, P.d.seg_start, L, scale);
-  }
+  float* up = (float*)P.d.lparts;
+  dim3 grid(blocks_for(G.n[0], kLatticeLP * L.txn), blocks_for(G.n[1], 2 * L.tyn), L.nbz * L.nsplit);
+  // double-buffered planes and the window offsets (SXw + SY ints)
+  const size_t sm = lattice_smem(L.txn, L.tyn, P.E);
+  const float scale = (float)std::ldexp(1.0, -k);
+  if (L.txn == 4 && L.tyn == 8)
+    k_lattice_f2<kLatticeLP, 4, 8><<<grid, 32 * kLatticeZ, sm, st>>>(qk, uk, up, G, (const Segment2*)P.d.seg2,
+                                                                    P.d.seg_start, L, scale);
+  else
+    k_lattice_f2<kLatticeLP, 0, 0><<<grid, 32 * kLatticeZ, sm, st>>>(qk, uk, up, G, (const Segment2*)P.d.seg2,
+                                                                    P.d.seg_start, L, scale);
   if (L.nsplit > 1) {
     const int64_t np = grid_points(P, k);
-    k_lattice_reduce<T><<<blocks_for(np, 256), 256, 0, st>>>(up, uk, np, L.nsplit);
+    k_lattice_reduce<float><<<blocks_for(np, 256), 256, 0, st>>>(up, uk, np, L.nsplit);
     P.launches += 1;
   }
 }
@@ -1785,17 +1745,21 @@ void lattice_tile_of(const Plan& P, int k, int& txn, int& tyn) {
   }
 }
 
-// Blocks that share one brick's input planes at level k (several on small
-// levels, so that the launch still fills the GPU: lattice_waves blocks per SM).
+// Blocks that share one brick's input planes (FP64: one output's stencil rows)
+// at level k: several on small levels, so that the launch still fills the GPU
+// (lattice_waves blocks per SM; FP64: 16 warps per SM).
 int lattice_nsplit(const Plan& P, int k) {
+  if (P.fp64) {
+    const int64_t warps = blocks_for(grid_points(P, k), 32);
+    return (int)std::min<int64_t>(std::max(P.nlrows, 1), std::max<int64_t>(1, (152 * 16 + warps / 2) / warps));
+  }
   GridDims G = dims_of(P, k);
   int txn, tyn;
   lattice_tile_of(P, k, txn, tyn);
-  const int TW = P.fp64 ? LBX : kLatticeLP * txn, LBY = P.fp64 ? 8 : 2 * tyn;
-  const int LBZb = P.fp64 ? LBZ : kLatticeZ;
-  const int64_t bricks = (int64_t)blocks_for(G.n[0], TW) * blocks_for(G.n[1], LBY) * blocks_for(G.n[2], LBZb);
-  const int64_t target = (int64_t)P.lattice_waves * 152 * 4 / LBZb;
-  return (int)std::min<int64_t>(LBZb + 2 * P.E[2], std::max<int64_t>(1, (target + bricks - 1) / bricks));
+  const int64_t bricks = (int64_t)blocks_for(G.n[0], kLatticeLP * txn) * blocks_for(G.n[1], 2 * tyn) *
+                         blocks_for(G.n[2], kLatticeZ);
+  const int64_t target = (int64_t)P.lattice_waves * 152 * 4 / kLatticeZ;
+  return (int)std::min<int64_t>(kLatticeZ + 2 * P.E[2], std::max<int64_t>(1, (target + bricks - 1) / bricks));
 }
 
 // Elements of the plan's split-partial buffer: the largest nsplit x points of
@@ -1823,8 +1787,8 @@ bool lattice_tile_fits(const Plan& P, int txn, int tyn) {
 
 cudaError_t launch_lattice(Plan& P, int k, const void* qk, void* uk, cudaStream_t st) {
   P.launches += 1;
-  if (P.fp64) lattice_t<double>(P, k, (const double*)qk, (double*)uk, st);
-  else lattice_t<float>(P, k, (const double*)qk, (float*)uk, st);
+  if (P.fp64) lattice_fp64(P, k, (const double*)qk, (double*)uk, st);
+  else lattice_fp32(P, k, (const double*)qk, (float*)uk, st);
   return cudaGetLastError();
 }
 

@@ -25,14 +25,6 @@ struct alignas(4 * sizeof(T)) R4 {
   T x, y, z, w;
 };
 
-// One x-run of the level stencil: taps (dx0 + j, dy, dz), j = 0..kSeg-1,
-// with coefficients g[j] (zero past the end of the run).
-template <typename T>
-struct Segment {
-  int dy, dx0;
-  T g[kSeg];
-};
-
 // A run over two adjacent stencil rows, for packed FP32x2 FMAs: g[j] =
 // (tap (dx0 + j, dy, dz), tap (dx0 + j, dy - 1, dz)), the coefficients that
 // one input row applies to the two output rows y and y + 1 it feeds.
@@ -77,8 +69,9 @@ struct DeviceBuffers {
   double* topq = nullptr;
   double* topu = nullptr;
   // level stencil
-  void* seg = nullptr;         // Segment<T>[nseg]
-  void* seg2 = nullptr;        // Segment2[nseg] (mixed precision only, instead of seg)
+  void* seg = nullptr;         // FP64: double coefficients of the rows in lrows
+  int4* lrows = nullptr;       // FP64: [nlrows] rows (dy, dz, X, first coefficient)
+  void* seg2 = nullptr;        // Segment2[nseg] (mixed precision)
   int* seg_start = nullptr;    // [2*Ez+2]: segments of plane dz live in [start[dz+Ez], start[dz+Ez+1])
   int4* cell_rows = nullptr;   // [nrows]: (dy, dz, xlo, xhi) rows of neighbour cell offsets
   // reductions and status
@@ -146,6 +139,7 @@ struct Plan {
   // level stencil
   int E[3] = {0, 0, 0};        // largest |dx|, |dy|, |dz| of a tap
   int nseg = 0;
+  int nlrows = 0;
   double stencil_taps = 0.0;   // number of taps (for work accounting)
   // top level
   int top_table_dims[3];

@@ -163,35 +163,20 @@ cudaError_t upload(void** dst, const std::vector<T>& v) {
   return cudaMemcpy(*dst, v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice);
 }
 
-template <typename T>
-void build_segments(const Plan& P, const std::vector<double>& G, const int E[3],
-                    std::vector<Segment<T>>& segs, std::vector<int>& start) {
-  int nx = 2 * E[0] + 1, ny = 2 * E[1] + 1;
-  auto at = [&](int dx, int dy, int dz) {
-    return G[((size_t)(dz + E[2]) * ny + (dy + E[1])) * nx + (dx + E[0])];
-  };
-  start.assign(2 * E[2] + 2, 0);
-  for (int dz = -E[2]; dz <= E[2]; ++dz) {
-    start[dz + E[2]] = (int)segs.size();
+// The stencil as rows of taps along x, (dy, dz, X, first coefficient): the
+// coefficients of dx = -X .. X, X the row's largest |dx| with a tap.
+void build_rows64(const std::vector<double>& G, const int E[3], std::vector<int4>& rows, std::vector<double>& coef) {
+  const int nx = 2 * E[0] + 1, ny = 2 * E[1] + 1;
+  for (int dz = -E[2]; dz <= E[2]; ++dz)
     for (int dy = -E[1]; dy <= E[1]; ++dy) {
+      const double* g = &G[((size_t)(dz + E[2]) * ny + (dy + E[1])) * nx + E[0]];
       int X = -1;
       for (int dx = 0; dx <= E[0]; ++dx)
-        if (at(dx, dy, dz) != 0.0) X = dx;
+        if (g[dx] != 0.0) X = dx;
       if (X < 0) continue;
-      for (int dx0 = -X; dx0 <= X; dx0 += kSeg) {
-        Segment<T> s;
-        s.dy = dy;
-        s.dx0 = dx0;
-        for (int j = 0; j < kSeg; ++j) {
-          int dx = dx0 + j;
-          s.g[j] = (dx <= X) ? (T)at(dx, dy, dz) : (T)0;
-        }
-        segs.push_back(s);
-      }
+      rows.push_back(make_int4(dy, dz, X, (int)coef.size()));
+      for (int dx = -X; dx <= X; ++dx) coef.push_back(g[dx]);
     }
-  }
-  start[2 * E[2] + 1] = (int)segs.size();
-  (void)P;
 }
 
 // Row pairs of the stencil for the packed FP32 kernel, whose lanes own two
@@ -457,6 +442,10 @@ int build_plan(const msm_params* pp, const msm_tuning* tune, Plan* P) {
         if (g != 0.0) taps += 1;
       }
   P->stencil_taps = taps;
+  std::vector<int4> rows64;  // the FP64 stencil's rows (their number sizes the split buffer below)
+  std::vector<double> coef64;
+  if (P->fp64 && P->stencil_fits) build_rows64(G, P->E, rows64, coef64);
+  P->nlrows = (int)rows64.size();
 
   // top-level kernel table (FP64)
   int top = P->levels - 1;
@@ -605,19 +594,16 @@ int build_plan(const msm_params* pp, const msm_tuning* tune, Plan* P) {
   if (upload((void**)&D.topK, K) != cudaSuccess) return MSM_ERR_OOM;
   if (upload((void**)&D.cell_rows, rowv) != cudaSuccess) return MSM_ERR_OOM;
   if (P->stencil_fits) {  // the stencil kernel's segment tables (unused, and not built, past its window)
-    std::vector<int> start;
     if (P->fp64) {
-      std::vector<Segment<double>> segs;
-      build_segments<double>(*P, G, P->E, segs, start);
-      P->nseg = (int)segs.size();
-      if (upload(&D.seg, segs) != cudaSuccess) return MSM_ERR_OOM;
+      if (upload(&D.seg, coef64) != cudaSuccess || upload((void**)&D.lrows, rows64) != cudaSuccess) return MSM_ERR_OOM;
     } else {
+      std::vector<int> start;
       std::vector<Segment2> segs2;
       build_row_pairs(G, P->E, segs2, start);
       P->nseg = (int)segs2.size();
       if (upload(&D.seg2, segs2) != cudaSuccess) return MSM_ERR_OOM;
+      if (upload((void**)&D.seg_start, start) != cudaSuccess) return MSM_ERR_OOM;
     }
-    if (upload((void**)&D.seg_start, start) != cudaSuccess) return MSM_ERR_OOM;
   }
   int least = 0, greatest = 0;
   if (cudaDeviceGetStreamPriorityRange(&least, &greatest) != cudaSuccess ||
@@ -632,7 +618,7 @@ void free_plan(Plan* P) {
   DeviceBuffers& D = P->d;
   void* ptrs[] = {D.key, D.rank, D.perm, D.count, D.csum, D.cell_start, D.atoms,
                   D.gfrac, D.gbase, D.scell, D.cellx, D.phis, D.fs, D.glong, D.topK, D.topq, D.topu, D.seg, D.seg2, D.cell_rows,
-                  D.seg_start, D.partial, D.scalars, D.md_partial, D.md_step, D.status, D.hpos, D.hq,
+                  D.seg_start, D.lrows, D.partial, D.scalars, D.md_partial, D.md_step, D.status, D.hpos, D.hq,
                   D.hphi, D.hforce, D.henergy, D.lparts, D.fft_work};
   for (void* p : ptrs)
     if (p) cudaFree(p);
