@@ -583,150 +583,152 @@ __device__ __forceinline__ void prolong_axis_body(const T* __restrict__ in, T* _
   out[t] = accumulate ? out[t] + sum : sum;
 }
 
-template <typename T, int ORDER>
-__global__ void k_prolong_axis(const T* __restrict__ in, T* __restrict__ out, AxisArgs A, int accumulate) {
-  prolong_axis_body<T, ORDER>(in, out, A, accumulate, (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
-}
-
-// ---- restriction and prolongation in one pass (small levels) ----
-// The tensor product of the three axis passes above, each output point
-// gathering its taps directly: the same taps in the same order and the same
-// association (restriction: x innermost, then y, then z; prolongation: z
-// innermost, then y, then x), so the result is bit-identical to the three
-// passes; one launch instead of three and no temporaries.  Used where the
-// gathered taps are few enough (see direct_budget).
+// ---- restriction and prolongation in one launch per level ----
+// A block computes a tile of the output from the input region it reaches,
+// staged in shared memory, as the three axis passes above in turn: the same
+// taps in the same order and association (restriction x, y, z; prolongation z,
+// y, x), so the result is bit-identical to the three passes, in one launch
+// and with no temporaries in global memory.
 struct Grid3Args {
   int nin[3], nout[3];  // array dims (x, y, z) of input and output
   int lo_in[3], lo_out[3];
   int periodic;
 };
 
-// The 1-D taps of a restriction output c in the axis pass's order (offsets
-// -R, .., -1, 0, 1, .., R, odd or 0): input indices and weights in fixed
-// slots; an open grid's taps outside the grid get weight 0 (adding 0 * v
-// leaves a sum unchanged, so the result stays that of the pass, which skips
-// them).
-template <typename T, int ORDER>
-__device__ __forceinline__ void restrict_taps(int c, int lo_out, int lo_in, int n, int periodic, int* s, T* w) {
-  constexpr int R = ORDER;
-  const int nu0 = 2 * (lo_out + c);
-  int k = 0;
+// Array index of absolute index i on an axis, wrapped, or -1 outside an open grid.
+__device__ __forceinline__ int axis_index(int i, int n, int lo, int periodic) {
+  if (!periodic) return i - lo >= 0 && i - lo < n ? i - lo : -1;
+  while (i < 0) i += n;
+  while (i >= n) i -= n;
+  return i;
+}
+
+// Restriction: kTileC^3 coarse points per block of 128 threads.  The FP64
+// arithmetic (2 lanes per SM and clock) of the halo makes the tile cost about
+// twice the axis passes' operations, so large levels keep those (see
+// restrict_by_tiles).
+constexpr int kTileC = 4;
+template <int ORDER>
+struct RestrictTile {
+  static constexpr int R = ORDER, F = 2 * kTileC + 2 * R - 1;  // fine points per side
+  int idx[3][F];
+  double a[F * F * F], b[F * F * kTileC];
+};
+
+template <int ORDER>
+__device__ __forceinline__ void restrict_tile_body(const double* __restrict__ in, double* __restrict__ out,
+                                                   const Grid3Args& A, int tile) {
+  using RT = RestrictTile<ORDER>;
+  constexpr int R = RT::R, F = RT::F, C = kTileC;
+  __shared__ RT S;
+  const int tx = (A.nout[0] + C - 1) / C, ty = (A.nout[1] + C - 1) / C;
+  const int c0[3] = {tile % tx * C, tile / tx % ty * C, tile / (tx * ty) * C};
+  const int tid = threadIdx.x;
+  for (int e = tid; e < 3 * F; e += blockDim.x) {
+    const int d = e / F, f = e - d * F;
+    S.idx[d][f] = axis_index(2 * (A.lo_out[d] + c0[d]) - R + f, A.nin[d], A.lo_in[d], A.periodic);
+  }
+  __syncthreads();
+  for (int e = tid; e < F * F * F; e += blockDim.x) {
+    const int x = S.idx[0][e % F], y = S.idx[1][e / F % F], z = S.idx[2][e / (F * F)];
+    S.a[e] = (x | y | z) < 0 ? 0.0 : in[((size_t)z * A.nin[1] + y) * A.nin[0] + x];
+  }
+  __syncthreads();
+  auto taps = [&](const double* v, int stride) {  // v: the point at offset 0
+    double sum = 0.0;
 #pragma unroll
-  for (int d = -R; d <= R; ++d) {
-    if (d != 0 && (d & 1) == 0) continue;
-    int t = nu0 + d - lo_in;
-    T wt = T(rweight<ORDER>(d < 0 ? -d : d));
-    if (periodic) {
-      t = wrap_periodic(t, n);
-    } else if (t < 0 || t >= n) {
-      t = 0;
-      wt = T(0);
-    }
-    s[k] = t;
-    w[k] = wt;
-    ++k;
+    for (int d = -R; d <= R; ++d)
+      if (d == 0 || (d & 1)) sum += rweight<ORDER>(d < 0 ? -d : d) * v[d * stride];
+    return sum;
+  };
+  for (int e = tid; e < F * F * C; e += blockDim.x) S.b[e] = taps(S.a + e / C * F + 2 * (e % C) + R, 1);
+  __syncthreads();
+  for (int e = tid; e < F * C * C; e += blockDim.x) {
+    const int c = e % C, y = e / C % C, z = e / (C * C);
+    S.a[e] = taps(S.b + (z * F + 2 * y + R) * C + c, C);
+  }
+  __syncthreads();
+  for (int e = tid; e < C * C * C; e += blockDim.x) {
+    const int c = e % C, y = e / C % C, z = e / (C * C);
+    const int x = c0[0] + c, yy = c0[1] + y, zz = c0[2] + z;
+    if (x < A.nout[0] && yy < A.nout[1] && zz < A.nout[2])
+      out[((size_t)zz * A.nout[1] + yy) * A.nout[0] + x] = taps(S.a + ((2 * z + R) * C + y) * C + c, C * C);
   }
 }
 
-// The 1-D taps of a prolongation output f: an even index nu takes the one
-// coarse point nu / 2 (offset 0), an odd one the ORDER + 1 points of the odd
-// offsets -R .. R, in the axis pass's order; fixed slots as above.  Returns
-// the slot count (1 or ORDER + 1).
-template <typename T, int ORDER>
-__device__ __forceinline__ int prolong_taps(int f, int lo_out, int lo_in, int n, int periodic, int* s, T* w) {
-  constexpr int R = ORDER;
-  const int nu = lo_out + f;
-  if ((nu & 1) == 0) {
-    int t = nu / 2 - lo_in;
-    T wt = T(1);
-    if (periodic) {
-      t = wrap_periodic(t, n);
-    } else if (t < 0 || t >= n) {
-      t = 0;
-      wt = T(0);
-    }
-    s[0] = t;
-    w[0] = wt;
-    return 1;
-  }
-  int k = 0;
-#pragma unroll
-  for (int d = -R; d <= R; d += 2) {  // the odd offsets
-    int t = (nu - d) / 2 - lo_in;
-    T wt = T(rweight<ORDER>(d < 0 ? -d : d));
-    if (periodic) {
-      t = wrap_periodic(t, n);
-    } else if (t < 0 || t >= n) {
-      t = 0;
-      wt = T(0);
-    }
-    s[k] = t;
-    w[k] = wt;
-    ++k;
-  }
-  return R + 1;
+template <int ORDER>
+__global__ void __launch_bounds__(128) k_restrict_tile(const double* __restrict__ in, double* __restrict__ out,
+                                                       Grid3Args A) {
+  restrict_tile_body<ORDER>(in, out, A, blockIdx.x);
 }
 
-template <typename T, int ORDER>
-__global__ void k_restrict3(const T* __restrict__ in, T* __restrict__ out, Grid3Args A) {
-  constexpr int NT = ORDER + 2;  // offsets 0 and the odd ones up to ORDER
-  const int np = A.nout[0] * A.nout[1] * A.nout[2];
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= np) return;
-  const int c[3] = {t % A.nout[0], (t / A.nout[0]) % A.nout[1], t / (A.nout[0] * A.nout[1])};
-  int sx[NT], sy[NT], sz[NT];
-  T wx[NT], wy[NT], wz[NT];
-  restrict_taps<T, ORDER>(c[0], A.lo_out[0], A.lo_in[0], A.nin[0], A.periodic, sx, wx);
-  restrict_taps<T, ORDER>(c[1], A.lo_out[1], A.lo_in[1], A.nin[1], A.periodic, sy, wy);
-  restrict_taps<T, ORDER>(c[2], A.lo_out[2], A.lo_in[2], A.nin[2], A.periodic, sz, wz);
-  T acc = 0;
+// Prolongation: 32 x TYZ x TYZ fine points per block of 256 threads, added
+// onto the output.  Bound by memory on large levels (the output read and
+// written once, the coarse grid read once): 240^3 points in 3 axis passes took
+// 352 us.
+constexpr int kTileX = 32;
+template <typename T, int ORDER, int TYZ>
+struct ProlongTile {
+  static constexpr int R = ORDER, CX = kTileX / 2 + R + 1, CY = TYZ / 2 + R + 1;  // coarse points reached
+  int idx[3][CX];
+  T a[CY * CY * CX], b[TYZ * CY * CX];
+};
+
+template <typename T, int ORDER, int TYZ>
+__device__ __forceinline__ void prolong_tile_body(const T* __restrict__ in, T* __restrict__ out, const Grid3Args& A,
+                                                  int tile) {
+  using PT = ProlongTile<T, ORDER, TYZ>;
+  constexpr int R = PT::R, CX = PT::CX, CY = PT::CY;
+  __shared__ PT S;
+  const int tx = (A.nout[0] + kTileX - 1) / kTileX, ty = (A.nout[1] + TYZ - 1) / TYZ;
+  const int f0[3] = {tile % tx * kTileX, tile / tx % ty * TYZ, tile / (tx * ty) * TYZ};
+  const int tid = threadIdx.x;
+  int nu0[3], co[3];  // absolute fine index of the tile's corner, lowest coarse index it reaches
 #pragma unroll
-  for (int iz = 0; iz < NT; ++iz) {
-    T ay = 0;
-#pragma unroll
-    for (int iy = 0; iy < NT; ++iy) {
-      const T* row = in + ((size_t)sz[iz] * A.nin[1] + sy[iy]) * A.nin[0];
-      T ax = 0;
-#pragma unroll
-      for (int ix = 0; ix < NT; ++ix) ax += wx[ix] * row[sx[ix]];
-      ay += wy[iy] * ax;
-    }
-    acc += wz[iz] * ay;
+  for (int d = 0; d < 3; ++d) {
+    nu0[d] = A.lo_out[d] + f0[d];
+    co[d] = (nu0[d] + 1 - R) >> 1;
   }
-  out[t] = acc;
+  for (int e = tid; e < 3 * CX; e += blockDim.x) {
+    const int d = e / CX, c = e - d * CX;
+    S.idx[d][c] = axis_index(co[d] + c, A.nin[d], A.lo_in[d], A.periodic);
+  }
+  __syncthreads();
+  for (int e = tid; e < CY * CY * CX; e += blockDim.x) {
+    const int x = S.idx[0][e % CX], y = S.idx[1][e / CX % CY], z = S.idx[2][e / (CX * CY)];
+    S.a[e] = (x | y | z) < 0 ? T(0) : in[((size_t)z * A.nin[1] + y) * A.nin[0] + x];
+  }
+  __syncthreads();
+  // fine index nu (even: the coarse point nu / 2; odd: those at odd distances up to R); v: coarse point co
+  auto taps = [&](const T* v, int stride, int nu, int c) {
+    if ((nu & 1) == 0) return v[((nu >> 1) - c) * stride];
+    T sum = 0;
+#pragma unroll
+    for (int d = -R; d <= R; d += 2) sum += T(rweight<ORDER>(d < 0 ? -d : d)) * v[(((nu - d) >> 1) - c) * stride];
+    return sum;
+  };
+  for (int e = tid; e < TYZ * CY * CX; e += blockDim.x) {
+    const int z = e / (CY * CX), yx = e - z * CY * CX;
+    S.b[e] = taps(S.a + yx, CY * CX, nu0[2] + z, co[2]);
+  }
+  __syncthreads();
+  for (int e = tid; e < TYZ * TYZ * CX; e += blockDim.x) {
+    const int x = e % CX, y = e / CX % TYZ, z = e / (CX * TYZ);
+    S.a[e] = taps(S.b + z * CY * CX + x, CX, nu0[1] + y, co[1]);
+  }
+  __syncthreads();
+  for (int e = tid; e < TYZ * TYZ * kTileX; e += blockDim.x) {
+    const int x = e % kTileX, y = e / kTileX % TYZ, z = e / (kTileX * TYZ);
+    if (f0[0] + x < A.nout[0] && f0[1] + y < A.nout[1] && f0[2] + z < A.nout[2]) {
+      T* o = out + ((size_t)(f0[2] + z) * A.nout[1] + f0[1] + y) * A.nout[0] + f0[0] + x;
+      *o = *o + taps(S.a + (z * TYZ + y) * CX, 1, nu0[0] + x, co[0]);  // onto u^{k, cutoff}
+    }
+  }
 }
 
-template <typename T, int ORDER>
-__global__ void k_prolong3(const T* __restrict__ in, T* __restrict__ out, Grid3Args A) {
-  constexpr int NO = ORDER + 1;  // the odd offsets
-  const int np = A.nout[0] * A.nout[1] * A.nout[2];
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= np) return;
-  const int f[3] = {t % A.nout[0], (t / A.nout[0]) % A.nout[1], t / (A.nout[0] * A.nout[1])};
-  int sx[NO], sy[NO], sz[NO];
-  T wx[NO], wy[NO], wz[NO];
-  const int kx = prolong_taps<T, ORDER>(f[0], A.lo_out[0], A.lo_in[0], A.nin[0], A.periodic, sx, wx);
-  const int ky = prolong_taps<T, ORDER>(f[1], A.lo_out[1], A.lo_in[1], A.nin[1], A.periodic, sy, wy);
-  const int kz = prolong_taps<T, ORDER>(f[2], A.lo_out[2], A.lo_in[2], A.nin[2], A.periodic, sz, wz);
-  T acc = 0;
-#pragma unroll
-  for (int ix = 0; ix < NO; ++ix) {
-    if (ix < kx) {
-      T ay = 0;
-#pragma unroll
-      for (int iy = 0; iy < NO; ++iy) {
-        if (iy < ky) {
-          T az = 0;
-#pragma unroll
-          for (int iz = 0; iz < NO; ++iz)
-            if (iz < kz) az += wz[iz] * in[((size_t)sz[iz] * A.nin[1] + sy[iy]) * A.nin[0] + sx[ix]];
-          ay += wy[iy] * az;
-        }
-      }
-      acc += wx[ix] * ay;
-    }
-  }
-  out[t] = out[t] + acc;  // onto u^{k, cutoff}
+template <typename T, int ORDER, int TYZ>
+__global__ void __launch_bounds__(256) k_prolong_tile(const T* __restrict__ in, T* __restrict__ out, Grid3Args A) {
+  prolong_tile_body<T, ORDER, TYZ>(in, out, A, blockIdx.x);
 }
 
 // ---- lattice cutoff by the stencil, FP64 ----
@@ -1534,18 +1536,18 @@ cudaError_t launch_scale_grid(Plan& P, const void* src, void* dst, const double*
   return cudaGetLastError();
 }
 
-// Whether a level's restriction or prolongation runs as one gathering pass:
-// on plans whose finest grid has at most 64^3 points, whose evaluations are
-// bound by their chains of small launches (measured 4-7 % faster on 23,558 and
-// 3,000 atoms; on the 1.07 M-atom box, where the grid passes run beside the
-// pair sums, the three-pass form was 1 % faster), and where the gathered taps
-// (points times at most (ORDER + 2)^3) stay few (this GPU's FP64 rate is 1/64
-// of its FP32 rate).
-static bool direct_pass(const Plan& P, int64_t points, bool fp64_values) {
-  if (grid_points(P, 0) > ((int64_t)1 << 18)) return false;
-  const int64_t nt = P.P.order + 2;
-  const int64_t taps = points * nt * nt * nt;
-  return taps <= (fp64_values ? ((int64_t)1 << 17) : ((int64_t)1 << 26));
+// Whether a level's restriction runs by tiles (one launch) or as three axis
+// passes: up to 24^3 coarse points, where the launches are the cost (16^3
+// coarse points, cubic: 14 -> 5 us; 48^3, quintic: 25 us by passes, FP64-bound
+// at about twice that by tiles).
+static bool restrict_by_tiles(int64_t coarse_points) { return coarse_points <= 24 * 24 * 24; }
+// Prolongation tiles: 8 planes a side once the blocks fill the GPU many times over.
+static int prolong_tyz(int64_t fine_points) { return fine_points > ((int64_t)1 << 18) ? 8 : 4; }
+static int64_t restrict_tiles(const int* n) {
+  return (int64_t)((n[0] + kTileC - 1) / kTileC) * ((n[1] + kTileC - 1) / kTileC) * ((n[2] + kTileC - 1) / kTileC);
+}
+static int64_t prolong_tiles(const int* n, int tyz) {
+  return (int64_t)((n[0] + kTileX - 1) / kTileX) * ((n[1] + tyz - 1) / tyz) * ((n[2] + tyz - 1) / tyz);
 }
 
 static Grid3Args grid3_args(const Plan& P, int kin, int kout) {
@@ -1564,11 +1566,12 @@ cudaError_t launch_restrict(Plan& P, int k, const void* fine, void* coarse, cuda
   const int* nf = P.n[k];
   const int* nc = P.n[k + 1];
   const int64_t ncp = (int64_t)nc[0] * nc[1] * nc[2];
-  if (direct_pass(P, ncp, true)) {
+  if (restrict_by_tiles(ncp)) {
     P.launches += 1;
     const Grid3Args A = grid3_args(P, k, k + 1);
-    if (P.P.order == 3) k_restrict3<double, 3><<<blocks_for(ncp, 128), 128, 0, st>>>((const double*)fine, (double*)coarse, A);
-    else k_restrict3<double, 5><<<blocks_for(ncp, 128), 128, 0, st>>>((const double*)fine, (double*)coarse, A);
+    const unsigned nb = (unsigned)restrict_tiles(nc);
+    if (P.P.order == 3) k_restrict_tile<3><<<nb, 128, 0, st>>>((const double*)fine, (double*)coarse, A);
+    else k_restrict_tile<5><<<nb, 128, 0, st>>>((const double*)fine, (double*)coarse, A);
     return cudaGetLastError();
   }
   P.launches += 3;
@@ -1593,50 +1596,24 @@ cudaError_t launch_restrict(Plan& P, int k, const void* fine, void* coarse, cuda
   return cudaGetLastError();
 }
 
-template <typename T>
-void prolong_t(Plan& P, int k, const T* coarse, T* fine, cudaStream_t st) {
-  const int* nf = P.n[k];
-  const int* nc = P.n[k + 1];
-  T* s1 = (T*)P.d.tmp[0];
-  T* s2 = (T*)P.d.tmp[1];
-  const T* src[3] = {coarse, s1, s2};
-  T* dst[3] = {s1, s2, fine};
-  int cur[3] = {nc[0], nc[1], nc[2]};
-  for (int i = 0; i < 3; ++i) {
-    int ax = 2 - i;  // z, then y, then x
-    AxisArgs A;
-    for (int d = 0; d < 3; ++d) A.nin[d] = cur[d];
-    cur[ax] = nf[ax];
-    for (int d = 0; d < 3; ++d) A.nout[d] = cur[d];
-    A.axis = ax;
-    A.lo_in = P.lo[k + 1][ax];
-    A.lo_out = P.lo[k][ax];
-    A.periodic = P.P.periodic;
-    unsigned nb = blocks_for((int64_t)cur[0] * cur[1] * cur[2], 256);
-    int acc = (i == 2) ? 1 : 0;  // the last pass adds onto u^{k,cutoff}
-    if (P.P.order == 3) k_prolong_axis<T, 3><<<nb, 256, 0, st>>>(src[i], dst[i], A, acc);
-    else k_prolong_axis<T, 5><<<nb, 256, 0, st>>>(src[i], dst[i], A, acc);
-  }
+template <typename T, int TYZ>
+static void prolong_t(Plan& P, int k, const T* coarse, T* fine, cudaStream_t st) {
+  const Grid3Args A = grid3_args(P, k + 1, k);
+  const unsigned nb = (unsigned)prolong_tiles(P.n[k], TYZ);
+  if (P.P.order == 3) k_prolong_tile<T, 3, TYZ><<<nb, 256, 0, st>>>(coarse, fine, A);
+  else k_prolong_tile<T, 5, TYZ><<<nb, 256, 0, st>>>(coarse, fine, A);
 }
 
 cudaError_t launch_prolong(Plan& P, int k, const void* coarse, void* fine, cudaStream_t st) {
-  const int64_t nfp = grid_points(P, k);
-  if (direct_pass(P, nfp, P.fp64)) {
-    P.launches += 1;
-    const Grid3Args A = grid3_args(P, k + 1, k);
-    const unsigned nb = blocks_for(nfp, 256);
-    if (P.fp64) {
-      if (P.P.order == 3) k_prolong3<double, 3><<<nb, 256, 0, st>>>((const double*)coarse, (double*)fine, A);
-      else k_prolong3<double, 5><<<nb, 256, 0, st>>>((const double*)coarse, (double*)fine, A);
-    } else {
-      if (P.P.order == 3) k_prolong3<float, 3><<<nb, 256, 0, st>>>((const float*)coarse, (float*)fine, A);
-      else k_prolong3<float, 5><<<nb, 256, 0, st>>>((const float*)coarse, (float*)fine, A);
-    }
-    return cudaGetLastError();
+  P.launches += 1;
+  const bool big = prolong_tyz(grid_points(P, k)) == 8;
+  if (P.fp64) {
+    if (big) prolong_t<double, 8>(P, k, (const double*)coarse, (double*)fine, st);
+    else prolong_t<double, 4>(P, k, (const double*)coarse, (double*)fine, st);
+  } else {
+    if (big) prolong_t<float, 8>(P, k, (const float*)coarse, (float*)fine, st);
+    else prolong_t<float, 4>(P, k, (const float*)coarse, (float*)fine, st);
   }
-  P.launches += 3;
-  if (P.fp64) prolong_t<double>(P, k, (const double*)coarse, (double*)fine, st);
-  else prolong_t<float>(P, k, (const float*)coarse, (float*)fine, st);
   return cudaGetLastError();
 }
 
@@ -1993,6 +1970,12 @@ struct AxisKArgs {
   AxisArgs A;
   int acc;
 };
+template <typename T>
+struct TileKArgs {
+  const T* in;
+  T* out;
+  Grid3Args A;
+};
 struct ConvKArgs {
   const double* src;
   float* dst;
@@ -2065,11 +2048,17 @@ __global__ void __launch_bounds__(kEw) kb_restrict_axis(const AxisKArgs<double>*
 }
 
 template <int ORDER>
-__global__ void __launch_bounds__(kEw) kb_prolong_axis(const AxisKArgs<float>* __restrict__ tab,
+__global__ void __launch_bounds__(128) kb_restrict_tile(const TileKArgs<double>* __restrict__ tab,
+                                                        const int* __restrict__ first, int nrep) {
+  const int r = batch_rep(first, nrep, blockIdx.x);
+  restrict_tile_body<ORDER>(tab[r].in, tab[r].out, tab[r].A, blockIdx.x - first[r]);
+}
+
+template <int ORDER>
+__global__ void __launch_bounds__(256) kb_prolong_tile(const TileKArgs<float>* __restrict__ tab,
                                                        const int* __restrict__ first, int nrep) {
   const int r = batch_rep(first, nrep, blockIdx.x);
-  const AxisKArgs<float>& a = tab[r];
-  prolong_axis_body<float, ORDER>(a.in, a.out, a.A, a.acc, ew_index(first, r));
+  prolong_tile_body<float, ORDER, 8>(tab[r].in, tab[r].out, tab[r].A, blockIdx.x - first[r]);
 }
 
 __global__ void __launch_bounds__(kEw) kb_lattice_reduce(const ReduceKArgs* __restrict__ tab,
@@ -2230,7 +2219,11 @@ struct GridBatch {
   BatchTable<LatKArgs> lattice[2];
   FftBatch* fft[2] = {nullptr, nullptr};  // the FFT form, when every replica's plan took it
   BatchTable<TopKArgs> top[2];
-  std::vector<BatchTable<AxisKArgs<float>>> prol[2];  // [dir][3 k + pass]
+  std::vector<BatchTable<AxisKArgs<float>>> prol[2];  // [dir][3 k + pass] (persistent chains)
+  // one launch per level: restriction where every replica's level is small
+  // enough (else the axis passes), prolongation
+  std::vector<BatchTable<TileKArgs<double>>> restr_tile[2];
+  std::vector<BatchTable<TileKArgs<float>>> prol_tile[2];
   BatchTable<InterpKArgs<float, double>> interp[2];
   BatchTable<EnergyKArgs> energy;
   // persistent chains: pass descriptors of the restriction and prolongation
@@ -2260,6 +2253,8 @@ void grid_batch_free(GridBatch* b) {
     fft_batch_free(b->fft[d]);
     b->top[d].release();
     for (auto& t : b->prol[d]) t.release();
+    for (auto& t : b->restr_tile[d]) t.release();
+    for (auto& t : b->prol_tile[d]) t.release();
     b->interp[d].release();
   }
   b->energy.release();
@@ -2383,6 +2378,35 @@ cudaError_t grid_batch_build(const std::vector<BatchRep>& reps, bool backward, G
         }
         chk(make_table(B->restr[dir][3 * k + ax], ra, rb));
       }
+    B->restr_tile[dir].resize(std::max(B->maxlev - 1, 0));
+    B->prol_tile[dir].resize(std::max(B->maxlev - 1, 0));
+    for (int k = 0; k + 1 < B->maxlev; ++k) {
+      std::vector<TileKArgs<double>> ra;
+      std::vector<TileKArgs<float>> pa;
+      std::vector<int> rb, pb;
+      bool small = true;
+      for (const BatchRep& r : reps) {
+        Plan& P = *r.plan;
+        TileKArgs<double> a{};
+        TileKArgs<float> p{};
+        int na = 0, np = 0;
+        if (k + 1 < P.levels) {
+          void* const* q = dir ? P.d.aq : P.d.gq;
+          void* const* u = dir ? P.d.au : P.d.gu;
+          small = small && restrict_by_tiles(grid_points(P, k + 1));
+          a = TileKArgs<double>{(const double*)q[k], (double*)q[k + 1], grid3_args(P, k, k + 1)};
+          na = (int)restrict_tiles(P.n[k + 1]);
+          p = TileKArgs<float>{(const float*)u[k + 1], (float*)u[k], grid3_args(P, k + 1, k)};
+          np = (int)prolong_tiles(P.n[k], 8);
+        }
+        ra.push_back(a);
+        rb.push_back(na);
+        pa.push_back(p);
+        pb.push_back(np);
+      }
+      if (small) chk(make_table(B->restr_tile[dir][k], ra, rb));
+      chk(make_table(B->prol_tile[dir][k], pa, pb));
+    }
     // lattice cutoff of every level below the top.  FFT form (every plan
     // periodic and built with it): five launches over all levels of all
     // replicas, level k of a replica working at offset sum_{j<k} N_j of its
@@ -2634,9 +2658,14 @@ cudaError_t grid_batch_levels(GridBatch* B, int d, cudaStream_t st) {
     cudaError_t e = launch_chain(B, o3 ? kb_restrict_chain<3> : kb_restrict_chain<5>, B->chain_restr[d], B->n_restr, st);
     if (e != cudaSuccess) return e;
   } else {
-    for (int k = 0; k + 1 < B->maxlev; ++k)
+    for (int k = 0; k + 1 < B->maxlev; ++k) {
+      if (B->restr_tile[d][k].total > 0) {
+        launch_table(B->restr_tile[d][k], o3 ? kb_restrict_tile<3> : kb_restrict_tile<5>, 128, st);
+        continue;
+      }
       for (int ax = 0; ax < 3; ++ax)
         launch_table(B->restr[d][3 * k + ax], o3 ? kb_restrict_axis<3> : kb_restrict_axis<5>, kEw, st);
+    }
   }
   if (B->fft[d]) {
     cudaError_t e = fft_batch_launch(B->fft[d], st);
@@ -2652,8 +2681,7 @@ cudaError_t grid_batch_levels(GridBatch* B, int d, cudaStream_t st) {
     if (e != cudaSuccess) return e;
   } else {
     for (int k = B->maxlev - 2; k >= 0; --k)
-      for (int i = 0; i < 3; ++i)
-        launch_table(B->prol[d][3 * k + i], o3 ? kb_prolong_axis<3> : kb_prolong_axis<5>, kEw, st);
+      launch_table(B->prol_tile[d][k], o3 ? kb_prolong_tile<3> : kb_prolong_tile<5>, 256, st);
   }
   return cudaGetLastError();
 }
