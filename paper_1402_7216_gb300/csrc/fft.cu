@@ -12,7 +12,12 @@
 // the level's grid instead of (taps) multiply-adds per point:
 //   x forward (reading the FP64 charges), y forward, z forward with the
 //   product by K^ and z inverse fused (the z line stays in shared memory),
-//   y inverse, x inverse (writing the real part as the potential).
+//   y inverse, x inverse (writing the potential).
+// Charges and potentials are real, so of the transform along x only the
+// n0 / 2 + 1 columns of non-negative frequency are kept: the x passes take two
+// real rows as one complex line (the transforms separate by symmetry), and the
+// y and z passes have half the lines (the 4.1M-atom box's sweep, 240^3 ..
+// 30^3, took 770 us with full complex grids and takes 385 us).
 // Each pass is one launch over every lattice level of a plan (or of every
 // replica of a batch), a table of per-level arguments mapping blocks to
 // levels.  The 1-D transforms are mixed-radix Stockham FFTs (radices 4, 2,
@@ -251,12 +256,13 @@ __device__ __forceinline__ Cx<T>* fft_lines(Cx<T>* X, Cx<T>* Y, int sL, int P, i
 template <typename T>
 struct FftPassArgs {
   int n[3];
-  int axis;              // 0 (x), 1 (y), 2 (z)
+  int h;                 // columns kept along x, n[0] / 2 + 1
+  int axis;              // 0 (x, two rows per line), 1 (y), 2 (z)
   int sL;                // lines per block L = 2^sL
-  int groups_per_row;    // axis 1, 2: x-groups of L lines per row of the other dimension
+  int groups_per_row;    // axis 1, 2: groups of L columns per row of the other dimension
   FftAxisDesc D;
   const Cx<T>* tw;       // this axis's stage tables and roots (n - 1 + kRoots entries)
-  Cx<T>* buf;            // the level's complex grid
+  Cx<T>* buf;            // the level's complex grid, h x n[1] x n[2]
   const double* qin;     // x forward: the FP64 charges (real input)
   T* uout;               // x inverse: the potential (real output)
   const T* khat;         // z pass: the kernel's transform (real), scaled
@@ -267,14 +273,14 @@ struct FftPassArgs {
 // banks.
 __host__ __device__ __forceinline__ int line_pitch(int n) { return (pad(n - 1) + 1) | 1; }
 
-// MODE: 0 x forward from real FP64 input, 1 forward (any axis), 2 z forward
-// x K^ x z inverse, 3 inverse (y), 4 x inverse to real output.  The block's
+// MODE: 0 x forward from real FP64 input, 1 forward (y or z), 2 z forward x K^
+// x z inverse, 3 inverse (y), 4 x inverse to real output.  The block's
 // descriptor fields are read once into registers.
 template <typename T, int MODE>
 __device__ __forceinline__ void fft_pass_body(const FftPassArgs<T>* __restrict__ Ap, int blk) {
   extern __shared__ __align__(16) unsigned char fft_smem[];
   const int ax = Ap->axis, sL = Ap->sL, gpr = Ap->groups_per_row;
-  const int n0 = Ap->n[0], n1 = Ap->n[1], n2 = Ap->n[2];
+  const int n0 = Ap->n[0], n1 = Ap->n[1], n2 = Ap->n[2], h = Ap->h;
   const int n = Ap->D.n, c = Ap->D.c, sn = Ap->D.s, nst = Ap->D.nst;
   const unsigned long long radix_code = Ap->D.radix_code;
   const Cx<T>* tw = Ap->tw;
@@ -284,59 +290,101 @@ __device__ __forceinline__ void fft_pass_body(const FftPassArgs<T>* __restrict__
   Cx<T>* Y = X + L * P;
   Cx<T>* w = Y + L * P;
   for (int i = threadIdx.x; i < n - 1 + kRoots; i += blockDim.x) w[i] = tw[i];
-  // the block's lines: element e of line l at global offset base + l * ls + e * es
-  long long base, ls, es;
-  int nl;  // valid lines
-  if (ax == 0) {
-    base = (long long)blk * L * n0;
-    ls = n0;
-    es = 1;
-    nl = min(L, n1 * n2 - blk * L);
+  const int total = n << sL;
+  // y and z: the block's lines are columns x0 .. x0 + nl - 1; element e of line l
+  // at base + l + e * es
+  long long base = 0, es = 0;
+  int nl = 0;
+  // x: line l is the rows r0 + 2 l and r0 + 2 l + 1
+  const int rows = n1 * n2, r0 = blk << (sL + 1);
+  if (MODE == 0) {
+    // load (consecutive threads on consecutive addresses); kFftBatch elements
+    // per thread are issued before their shared-memory stores, so that they are
+    // in flight together
+    for (int t0 = threadIdx.x; t0 < total; t0 += kFftBatch * blockDim.x) {
+      double v[kFftBatch][2];
+      int at[kFftBatch];
+#pragma unroll
+      for (int u = 0; u < kFftBatch; ++u) {
+        const int t = t0 + u * (int)blockDim.x;
+        v[u][0] = v[u][1] = 0.0;
+        at[u] = -1;
+        if (t < total) {
+          const int l = div_c(t >> sn, c), e = t - l * n, r = r0 + 2 * l;
+          at[u] = l * P + pad(e);
+          if (r < rows) v[u][0] = Ap->qin[(long long)r * n0 + e];
+          if (r + 1 < rows) v[u][1] = Ap->qin[(long long)(r + 1) * n0 + e];
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kFftBatch; ++u)
+        if (at[u] >= 0) X[at[u]] = Cx<T>{(T)v[u][0], (T)v[u][1]};
+    }
+  } else if (MODE == 4) {
+    // the two rows' half spectra A, B as one line: A + i B, and by symmetry
+    // conj(A) + i conj(B) at the negative frequency
+    int l = 0, k = threadIdx.x;
+    auto settle = [&] {
+      while (k >= h) {
+        k -= h;
+        ++l;
+      }
+    };
+    settle();
+    while (l < L) {
+      Cx<T> a[2], b[2];
+      int ll[2], kk[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int r = r0 + 2 * l;
+        a[u] = b[u] = Cx<T>{T(0), T(0)};
+        ll[u] = l;
+        kk[u] = k;
+        if (l < L) {
+          if (r < rows) a[u] = buf[(long long)r * h + k];
+          if (r + 1 < rows) b[u] = buf[(long long)(r + 1) * h + k];
+          k += blockDim.x;
+          settle();
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+        if (ll[u] < L) {
+          Cx<T>* x = X + ll[u] * P;
+          const int q = kk[u];
+          x[pad(q)] = Cx<T>{a[u].x - b[u].y, a[u].y + b[u].x};
+          if (q > 0 && 2 * q != n) x[pad(n - q)] = Cx<T>{a[u].x + b[u].y, b[u].x - a[u].y};
+        }
+    }
   } else {
     const int g = blk % gpr, other = blk / gpr;  // other: z (axis 1) or y (axis 2)
     const int x0 = g * L;
-    nl = min(L, n0 - x0);
-    ls = 1;
+    nl = min(L, h - x0);
     if (ax == 1) {
-      base = (long long)other * n1 * n0 + x0;
-      es = n0;
+      base = (long long)other * n1 * h + x0;
+      es = h;
     } else {
-      base = (long long)other * n0 + x0;
-      es = (long long)n0 * n1;
+      base = (long long)other * h + x0;
+      es = (long long)h * n1;
     }
-  }
-  // load (consecutive threads on consecutive global addresses): axis 0 takes
-  // t = l n + e, the others t = e L + l; kFftBatch loads per thread are issued
-  // before their shared-memory stores, so that they are in flight together
-  const int total = n << sL;
-  for (int t0 = threadIdx.x; t0 < total; t0 += kFftBatch * blockDim.x) {
-    Cx<T> v[kFftBatch];
-    int at[kFftBatch];
+    for (int t0 = threadIdx.x; t0 < total; t0 += kFftBatch * blockDim.x) {
+      Cx<T> v[kFftBatch];
+      int at[kFftBatch];
 #pragma unroll
-    for (int u = 0; u < kFftBatch; ++u) {
-      const int t = t0 + u * (int)blockDim.x;
-      v[u] = Cx<T>{T(0), T(0)};
-      at[u] = -1;
-      if (t < total) {
-        int l, e;
-        if (ax == 0) {
-          l = div_c(t >> sn, c);
-          e = t - l * n;
-        } else {
-          e = t >> sL;
-          l = t & (L - 1);
-        }
-        at[u] = l * P + pad(e);
-        if (l < nl) {
-          const long long o = base + l * ls + e * es;
-          if (MODE == 0) v[u].x = (T)Ap->qin[o];
-          else v[u] = buf[o];
+      for (int u = 0; u < kFftBatch; ++u) {
+        const int t = t0 + u * (int)blockDim.x;
+        v[u] = Cx<T>{T(0), T(0)};
+        at[u] = -1;
+        if (t < total) {
+          const int e = t >> sL, l = t & (L - 1);
+          at[u] = l * P + pad(e);
+          if (l < nl) v[u] = buf[base + l + e * es];
         }
       }
-    }
 #pragma unroll
-    for (int u = 0; u < kFftBatch; ++u)
-      if (at[u] >= 0) X[at[u]] = v[u];
+      for (int u = 0; u < kFftBatch; ++u)
+        if (at[u] >= 0) X[at[u]] = v[u];
+    }
   }
   __syncthreads();
   const T s = (MODE == 3 || MODE == 4) ? T(1) : T(-1);
@@ -348,7 +396,7 @@ __device__ __forceinline__ void fft_pass_body(const FftPassArgs<T>* __restrict__
 #pragma unroll
       for (int u = 0; u < kFftBatch; ++u) {
         const int t = t0 + u * (int)blockDim.x, e = t >> sL, l = t & (L - 1);
-        kh[u] = (t < total && l < nl) ? khat[base + l * ls + e * es] : T(0);
+        kh[u] = (t < total && l < nl) ? khat[base + l + e * es] : T(0);
       }
 #pragma unroll
       for (int u = 0; u < kFftBatch; ++u) {
@@ -362,20 +410,33 @@ __device__ __forceinline__ void fft_pass_body(const FftPassArgs<T>* __restrict__
     __syncthreads();
     R = fft_lines(R, R == X ? Y : X, sL, P, n, c, sn, nst, radix_code, w, T(1));
   }
-  T* uout = Ap->uout;
-  for (int t = threadIdx.x; t < total; t += blockDim.x) {
-    int l, e;
-    if (ax == 0) {
-      l = div_c(t >> sn, c);
-      e = t - l * n;
-    } else {
-      e = t >> sL;
-      l = t & (L - 1);
+  if (MODE == 4) {
+    T* uout = Ap->uout;
+    for (int t = threadIdx.x; t < total; t += blockDim.x) {
+      const int l = div_c(t >> sn, c), e = t - l * n, r = r0 + 2 * l;
+      const Cx<T> v = R[l * P + pad(e)];
+      if (r < rows) uout[(long long)r * n0 + e] = v.x;
+      if (r + 1 < rows) uout[(long long)(r + 1) * n0 + e] = v.y;
     }
-    if (l < nl) {
-      const long long o = base + l * ls + e * es;
-      if (MODE == 4) uout[o] = R[l * P + pad(e)].x;
-      else buf[o] = R[l * P + pad(e)];
+  } else if (MODE == 0) {
+    // Z = A + i B with A and B Hermitian: A = (Z[k] + conj Z[n-k]) / 2,
+    // B = -i (Z[k] - conj Z[n-k]) / 2
+    const T half = (T)0.5;
+    for (int l = 0, k = threadIdx.x; l < L; k += blockDim.x) {
+      while (k >= h) {
+        k -= h;
+        ++l;
+      }
+      if (l >= L) break;
+      const int r = r0 + 2 * l;
+      const Cx<T> z = R[l * P + pad(k)], y = R[l * P + pad(k > 0 ? n - k : 0)];
+      if (r < rows) buf[(long long)r * h + k] = Cx<T>{half * (z.x + y.x), half * (z.y - y.y)};
+      if (r + 1 < rows) buf[(long long)(r + 1) * h + k] = Cx<T>{half * (z.y + y.y), half * (y.x - z.x)};
+    }
+  } else {
+    for (int t = threadIdx.x; t < total; t += blockDim.x) {
+      const int e = t >> sL, l = t & (L - 1);
+      if (l < nl) buf[base + l + e * es] = R[l * P + pad(e)];
     }
   }
 }
@@ -440,9 +501,10 @@ FftPassArgs<T> pass_args(const int dims[3], int axis, const void* tw, void* buf,
   FftPassArgs<T> A;
   for (int d = 0; d < 3; ++d) A.n[d] = dims[d];
   const int n = dims[axis];
+  A.h = dims[0] / 2 + 1;
   A.axis = axis;
   A.sL = lines_per_block_log2<T>(n);
-  A.groups_per_row = (dims[0] + (1 << A.sL) - 1) >> A.sL;
+  A.groups_per_row = (A.h + (1 << A.sL) - 1) >> A.sL;
   factorize(n, A.D, sizeof(T) == sizeof(float));
   A.tw = reinterpret_cast<const Cx<T>*>(tw);
   A.buf = reinterpret_cast<Cx<T>*>(buf);
@@ -454,7 +516,7 @@ FftPassArgs<T> pass_args(const int dims[3], int axis, const void* tw, void* buf,
 
 template <typename T>
 int pass_blocks(const FftPassArgs<T>& A) {
-  if (A.axis == 0) return (A.n[1] * A.n[2] + (1 << A.sL) - 1) >> A.sL;
+  if (A.axis == 0) return ((A.n[1] * A.n[2] + 1) / 2 + (1 << A.sL) - 1) >> A.sL;
   const int other = A.axis == 1 ? A.n[2] : A.n[1];
   return A.groups_per_row * other;
 }
@@ -543,6 +605,7 @@ cudaError_t fft_build_level(Plan& P, int k, const std::vector<double>& K, void* 
   FftLevel& F = P.fftl[k];
   for (int d = 0; d < 3; ++d) F.n[d] = P.n[k][d];
   const int64_t N = (int64_t)F.n[0] * F.n[1] * F.n[2];
+  const int64_t H = (int64_t)(F.n[0] / 2 + 1) * F.n[1] * F.n[2];  // kept columns
   cudaError_t e = cudaSuccess;
   void* tw64[3] = {nullptr, nullptr, nullptr};
   for (int d = 0; d < 3 && e == cudaSuccess; ++d) {
@@ -562,7 +625,7 @@ cudaError_t fft_build_level(Plan& P, int k, const std::vector<double>& K, void* 
       if (e == cudaSuccess) e = cudaMemcpy(F.tw[d], twf.data(), sizeof(float) * twf.size(), cudaMemcpyHostToDevice);
     }
   }
-  if (e == cudaSuccess) e = cudaMalloc(&F.khat, (P.fp64 ? sizeof(double) : sizeof(float)) * (size_t)N);
+  if (e == cudaSuccess) e = cudaMalloc(&F.khat, (P.fp64 ? sizeof(double) : sizeof(float)) * (size_t)H);
   double* kd = nullptr;
   if (e == cudaSuccess) e = cudaMalloc((void**)&kd, sizeof(double) * (size_t)N);
   if (e == cudaSuccess) e = cudaMemcpy(kd, K.data(), sizeof(double) * (size_t)N, cudaMemcpyHostToDevice);
@@ -578,9 +641,9 @@ cudaError_t fft_build_level(Plan& P, int k, const std::vector<double>& K, void* 
     run_pass<double, 1>(t[1], 0);
     run_pass<double, 1>(t[2], 0);
     const double scale = std::ldexp(1.0, -k) / (double)N;
-    k_take_real<<<(unsigned)((N + 255) / 256), 256>>>((const Cx<double>*)work, scale,
+    k_take_real<<<(unsigned)((H + 255) / 256), 256>>>((const Cx<double>*)work, scale,
                                                       P.fp64 ? nullptr : (float*)F.khat,
-                                                      P.fp64 ? (double*)F.khat : nullptr, N);
+                                                      P.fp64 ? (double*)F.khat : nullptr, H);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
