@@ -67,7 +67,7 @@ cudaError_t grid_sweep(Plan& P, int dir, cudaStream_t st) {
   if (e == cudaSuccess && P.lattice_fft)
     e = stage(P, MSM_STAGE_LATTICE, st, [&] {
       P.launches += 5;
-      return fft_batch_launch(P.fftb[dir], st);
+      return fft_batch_launch(P.fftb[dir], st, P.pdl);
     });
   if (e == cudaSuccess) e = stage(P, MSM_STAGE_TOP, st, [&] { return launch_top(P, q[l - 1], u[l - 1], st); });
   for (int k = l - 2; k >= 0 && e == cudaSuccess; --k)
@@ -85,7 +85,10 @@ cudaError_t grid_sweep(Plan& P, int dir, cudaStream_t st) {
 // st takes the side stream in and the graph gets two parallel branches.
 template <typename IO>
 int forward(Plan& P, int64_t n, const IO* pos, const IO* q, double* energy, IO* phi, IO* force, cudaStream_t st) {
-  cudaError_t e = stage(P, MSM_STAGE_BINNING, st, [&] { return launch_binning(P, n, pos, q, st); });
+  // the grid the anterpolation adds into: fixed point in tmp[0], or the FP64 grid itself
+  auto* charge = (unsigned long long*)(P.fp64 ? P.d.gq[0] : P.d.tmp[0]);
+  cudaError_t e = stage(P, MSM_STAGE_BINNING, st,
+                        [&] { return launch_binning(P, n, pos, q, st, charge, grid_points(P, 0)); });
   cudaStream_t gs = st;
   if (e == cudaSuccess && P.overlap) {
     gs = P.side;

@@ -446,6 +446,7 @@ __device__ __forceinline__ void fft_pass_body(const FftPassArgs<T>* __restrict__
 template <typename T, int MODE>
 __global__ void __launch_bounds__(kFftThreads, sizeof(T) == 4 ? 4 : 2) k_fft_pass(const FftPassArgs<T>* __restrict__ tab,
                                                           const int* __restrict__ first, int nitems) {
+  pdl_sync();
   const int r = batch_rep(first, nitems, blockIdx.x);
   fft_pass_body<T, MODE>(tab + r, (int)blockIdx.x - __ldg(first + r));
 }
@@ -522,8 +523,8 @@ int pass_blocks(const FftPassArgs<T>& A) {
 }
 
 template <typename T, int MODE>
-void run_pass(const BatchTable<FftPassArgs<T>>& t, cudaStream_t st) {
-  if (t.total > 0) k_fft_pass<T, MODE><<<t.total, kFftThreads, t.smem, st>>>(t.args, t.first, t.nrep);
+void run_pass(const BatchTable<FftPassArgs<T>>& t, cudaStream_t st, bool pdl = false) {
+  if (t.total > 0) klaunch(pdl, k_fft_pass<T, MODE>, t.total, kFftThreads, t.smem, st, t.args, t.first, t.nrep);
 }
 
 // The twiddle table of one axis of length n, FP64: the stage tables
@@ -698,17 +699,17 @@ cudaError_t fft_batch_build(const std::vector<FftBatchItem>& items, bool fp64, F
 }
 
 template <typename T>
-static void launch_tables(const BatchTable<FftPassArgs<T>>* t, cudaStream_t st) {
-  run_pass<T, 0>(t[0], st);
-  run_pass<T, 1>(t[1], st);
-  run_pass<T, 2>(t[2], st);
-  run_pass<T, 3>(t[3], st);
-  run_pass<T, 4>(t[4], st);
+static void launch_tables(const BatchTable<FftPassArgs<T>>* t, cudaStream_t st, bool pdl) {
+  run_pass<T, 0>(t[0], st, pdl);
+  run_pass<T, 1>(t[1], st, pdl);
+  run_pass<T, 2>(t[2], st, pdl);
+  run_pass<T, 3>(t[3], st, pdl);
+  run_pass<T, 4>(t[4], st, pdl);
 }
 
-cudaError_t fft_batch_launch(const FftBatch* b, cudaStream_t st) {
-  if (b->fp64) launch_tables<double>(b->d, st);
-  else launch_tables<float>(b->f, st);
+cudaError_t fft_batch_launch(const FftBatch* b, cudaStream_t st, bool pdl) {
+  if (b->fp64) launch_tables<double>(b->d, st, pdl);
+  else launch_tables<float>(b->f, st, pdl);
   return cudaGetLastError();
 }
 

@@ -36,6 +36,7 @@
 // if they had been computed in FP64 and rounded.  FP32 inputs (hi = x, lo = 0)
 // take the same path.  Positions outside [0, L) of a periodic box are folded
 // in FP64 first (rare).
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -250,7 +251,10 @@ __device__ __forceinline__ void bin_count_body(const IO* __restrict__ pos, const
 template <typename IO, bool FP64>
 __global__ void __launch_bounds__(256) k_bin_count(const IO* __restrict__ pos, const IO* __restrict__ q, int n,
                                                    BinArgs A, int* __restrict__ count, int* __restrict__ key_out,
-                                                   int* __restrict__ rank_out, int* __restrict__ status) {
+                                                   int* __restrict__ rank_out, int* __restrict__ status,
+                                                   unsigned long long* __restrict__ zero, int64_t nzero) {
+  pdl_sync();
+  for (int64_t k = (int64_t)blockIdx.x * 256 + threadIdx.x; k < nzero; k += (int64_t)gridDim.x * 256) zero[k] = 0ull;
   bin_count_body<IO, FP64>(pos, q, n, A, count, key_out, rank_out, status, blockIdx.x);
 }
 
@@ -292,6 +296,7 @@ __device__ __forceinline__ void cell_sums_body(const int* __restrict__ count, in
 }
 
 __global__ void __launch_bounds__(1024) k_cell_sums(const int* __restrict__ count, int ncell, int* __restrict__ sums) {
+  pdl_sync();
   cell_sums_body(count, ncell, sums, blockIdx.x);
 }
 
@@ -346,6 +351,7 @@ __device__ __forceinline__ void cell_scan_body(int* __restrict__ count, int ncel
 
 __global__ void __launch_bounds__(1024) k_cell_scan(int* __restrict__ count, int ncell,
                                                     const int* __restrict__ sums, int* __restrict__ cell_start) {
+  pdl_sync();
   cell_scan_body(count, ncell, sums, cell_start, blockIdx.x);
 }
 
@@ -366,6 +372,7 @@ __device__ __forceinline__ void bin_perm_body(int n, const int* __restrict__ key
 __global__ void __launch_bounds__(256) k_bin_perm(int n, const int* __restrict__ key_in,
                                                   const int* __restrict__ rank_in, const int* __restrict__ cell_start,
                                                   int* __restrict__ perm) {
+  pdl_sync();
   bin_perm_body(n, key_in, rank_in, cell_start, perm, blockIdx.x);
 }
 
@@ -537,6 +544,7 @@ __global__ void __launch_bounds__(32 * kFillWarps) k_cell_fill(const IO* __restr
                                                                int4* __restrict__ gbase,
                                                                int* __restrict__ scell, float* __restrict__ cellx,
                                                                int* __restrict__ perm, int ncell) {
+  pdl_sync();
   __shared__ long long idx[kFillWarps][kOrderMax];
   const int w = threadIdx.x >> 5;
   cell_fill_body<IO, FP64>(pos, q, A, cell_start, atoms_v, gfrac_v, gbase, scell, cellx, perm, ncell,
@@ -610,31 +618,36 @@ BinArgs bin_args(const Plan& P) {
 }  // namespace
 
 template <typename IO>
-cudaError_t launch_binning(Plan& P, int64_t n64, const IO* pos, const IO* q, cudaStream_t st) {
+cudaError_t launch_binning(Plan& P, int64_t n64, const IO* pos, const IO* q, cudaStream_t st,
+                           unsigned long long* zero, int64_t nzero) {
   const int n = (int)n64;
   DeviceBuffers& D = P.d;
   const BinArgs A = bin_args(P);
   const unsigned nb = (unsigned)((n + 255) / 256);
   const unsigned nsc = (unsigned)((P.ncell + kScanChunk - 1) / kScanChunk);
   if (n > 0) {
+    // enough blocks for the zeroed words too, at eight per thread
+    const unsigned nz = std::max(nb, (unsigned)std::min<int64_t>((nzero + 2047) / 2048, 8 * 152));
     if (P.fp64)
-      k_bin_count<IO, true><<<nb, 256, 0, st>>>(pos, q, n, A, D.count, D.key, D.rank, D.status);
+      klaunch(false, k_bin_count<IO, true>, nz, 256, 0, st, pos, q, n, A, D.count, D.key, D.rank, D.status, zero, nzero);
     else
-      k_bin_count<IO, false><<<nb, 256, 0, st>>>(pos, q, n, A, D.count, D.key, D.rank, D.status);
+      klaunch(false, k_bin_count<IO, false>, nz, 256, 0, st, pos, q, n, A, D.count, D.key, D.rank, D.status, zero, nzero);
+  } else if (nzero > 0) {
+    cudaMemsetAsync(zero, 0, sizeof(unsigned long long) * (size_t)nzero, st);
   }
-  k_cell_sums<<<nsc, 1024, 0, st>>>(D.count, P.ncell, D.csum);
-  k_cell_scan<<<nsc, 1024, 0, st>>>(D.count, P.ncell, D.csum, D.cell_start);
+  if (nsc > 1) klaunch(P.pdl, k_cell_sums, nsc, 1024, 0, st, D.count, P.ncell, D.csum);  // one chunk has no offset
+  klaunch(P.pdl, k_cell_scan, nsc, 1024, 0, st, D.count, P.ncell, D.csum, D.cell_start);
   if (n > 0) {
     const unsigned nf = (unsigned)((P.ncell + kFillWarps - 1) / kFillWarps);
-    k_bin_perm<<<nb, 256, 0, st>>>(n, D.key, D.rank, D.cell_start, D.perm);
+    klaunch(P.pdl, k_bin_perm, nb, 256, 0, st, n, D.key, D.rank, D.cell_start, D.perm);
     if (P.fp64)
-      k_cell_fill<IO, true><<<nf, 32 * kFillWarps, 0, st>>>(pos, q, A, D.cell_start, D.atoms, D.gfrac, D.gbase,
-                                                            D.scell, D.cellx, D.perm, P.ncell);
+      klaunch(P.pdl, k_cell_fill<IO, true>, nf, 32 * kFillWarps, 0, st, pos, q, A, D.cell_start, D.atoms, D.gfrac,
+              D.gbase, D.scell, D.cellx, D.perm, P.ncell);
     else
-      k_cell_fill<IO, false><<<nf, 32 * kFillWarps, 0, st>>>(pos, q, A, D.cell_start, D.atoms, D.gfrac, D.gbase,
-                                                             D.scell, D.cellx, D.perm, P.ncell);
+      klaunch(P.pdl, k_cell_fill<IO, false>, nf, 32 * kFillWarps, 0, st, pos, q, A, D.cell_start, D.atoms, D.gfrac,
+              D.gbase, D.scell, D.cellx, D.perm, P.ncell);
   }
-  P.launches += 2 + (n > 0 ? 3 : 0);
+  P.launches += 1 + (nsc > 1 ? 1 : 0) + (n > 0 ? 3 : 0);
   return cudaGetLastError();
 }
 
@@ -709,7 +722,9 @@ void bin_batch_free(BinBatch* b) {
   delete b;
 }
 
-template cudaError_t launch_binning<double>(Plan&, int64_t, const double*, const double*, cudaStream_t);
-template cudaError_t launch_binning<float>(Plan&, int64_t, const float*, const float*, cudaStream_t);
+template cudaError_t launch_binning<double>(Plan&, int64_t, const double*, const double*, cudaStream_t,
+                                            unsigned long long*, int64_t);
+template cudaError_t launch_binning<float>(Plan&, int64_t, const float*, const float*, cudaStream_t,
+                                           unsigned long long*, int64_t);
 
 }  // namespace msm

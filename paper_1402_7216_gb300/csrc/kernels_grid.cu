@@ -177,6 +177,7 @@ __global__ void __launch_bounds__(kWide) k_anterp64(const R4<double>* __restrict
                                                    const int4* __restrict__ gbase, int n, int stride, GridDims G,
                                                    double* __restrict__ grid, const double* __restrict__ dscale,
                                                    double factor) {
+  pdl_sync();
   constexpr int W = 2 * Basis<double, ORDER>::S;
   const int t = blockIdx.x * kWide + threadIdx.x, i = (t & 31) * stride + (t >> 5);
   if ((t >> 5) >= stride || i >= n) return;
@@ -454,6 +455,7 @@ template <int ORDER>
 __global__ void __launch_bounds__(kPatchThreads) k_anterp_fx(const R4<float>* __restrict__ gfrac, const int4* __restrict__ gbase,
                                                    const int* __restrict__ cell_start, AnterpArgs A, GridDims G,
                                                    unsigned long long* __restrict__ gfx) {
+  pdl_sync();
   anterp_fx_body<ORDER>(gfrac, gbase, cell_start, A, G, gfx, blockIdx.x, blockIdx.y, blockIdx.z);
 }
 
@@ -469,6 +471,7 @@ __device__ __forceinline__ void fx_to_f64_body(const unsigned long long* __restr
 
 __global__ void k_fx_to_f64(const unsigned long long* __restrict__ gfx, double* __restrict__ q0, int64_t count,
                             const double* __restrict__ dscale, double factor) {
+  pdl_sync();
   fx_to_f64_body(gfx, q0, count, dscale, factor, (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
@@ -549,6 +552,7 @@ __device__ __forceinline__ void restrict_axis_body(const T* __restrict__ in, T* 
 
 template <typename T, int ORDER>
 __global__ void k_restrict_axis(const T* __restrict__ in, T* __restrict__ out, AxisArgs A) {
+  pdl_sync();
   restrict_axis_body<T, ORDER>(in, out, A, (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
@@ -659,6 +663,7 @@ __device__ __forceinline__ void restrict_tile_body(const double* __restrict__ in
 template <int ORDER>
 __global__ void __launch_bounds__(128) k_restrict_tile(const double* __restrict__ in, double* __restrict__ out,
                                                        Grid3Args A) {
+  pdl_sync();
   restrict_tile_body<ORDER>(in, out, A, blockIdx.x);
 }
 
@@ -728,6 +733,7 @@ __device__ __forceinline__ void prolong_tile_body(const T* __restrict__ in, T* _
 
 template <typename T, int ORDER, int TYZ>
 __global__ void __launch_bounds__(256) k_prolong_tile(const T* __restrict__ in, T* __restrict__ out, Grid3Args A) {
+  pdl_sync();
   prolong_tile_body<T, ORDER, TYZ>(in, out, A, blockIdx.x);
 }
 
@@ -749,6 +755,7 @@ __global__ void __launch_bounds__(kLat64) k_lattice64(const double* __restrict__
                                                      double* __restrict__ up, GridDims G,
                                                      const int4* __restrict__ rows, const double* __restrict__ coef,
                                                      int nrows, int per, double scale) {
+  pdl_sync();
   const int n0 = G.n[0], n1 = G.n[1], n2 = G.n[2];
   const int64_t np = (int64_t)n0 * n1 * n2, p = (int64_t)blockIdx.x * kLat64 + threadIdx.x;
   if (p >= np) return;
@@ -968,6 +975,7 @@ __global__ void __launch_bounds__(32 * kLatticeZ, 6) k_lattice_f2(const float* _
                                                                const Segment2* __restrict__ seg,
                                                                const int* __restrict__ seg_start, LatticeArgs L,
                                                                float scale) {
+  pdl_sync();
   lattice_f2_body<LP, TXC, TYC>(q, u, up, G, seg, seg_start, L, scale, blockIdx.x, blockIdx.y, blockIdx.z);
 }
 
@@ -984,6 +992,7 @@ __device__ __forceinline__ void lattice_reduce_body(const T* __restrict__ up, T*
 template <typename T>
 __global__ void __launch_bounds__(256) k_lattice_reduce(const T* __restrict__ up, T* __restrict__ u, int64_t np,
                                                         int nsplit) {
+  pdl_sync();
   lattice_reduce_body<T>(up, u, np, nsplit, (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
@@ -1028,6 +1037,7 @@ template <typename T>
 __global__ void __launch_bounds__(32 * kTopWarps) k_top(const double* __restrict__ qt, T* __restrict__ ut,
                                                         double* __restrict__ ut64, GridDims G,
                                                         const double* __restrict__ K, int tx, int ty, int tz) {
+  pdl_sync();
   top_body<T>(qt, ut, ut64, G, K, tx, ty, (int64_t)blockIdx.x * kTopWarps + (threadIdx.x >> 5));
   (void)tz;
 }
@@ -1317,6 +1327,7 @@ __global__ void __launch_bounds__(256, 3) k_interp_gather(const R4<float>* __res
                                                           const int* __restrict__ cell_start, AnterpArgs AA,
                                                           const float* __restrict__ u0, GridDims G, AssembleArgs A,
                                                           R4<float>* __restrict__ glong) {
+  pdl_sync();
   interp_fwd_body<ORDER, double, true>(gfrac, gbase, nullptr, cell_start, AA, u0, G, A, nullptr, nullptr, glong,
                                        nullptr, nullptr, nullptr, blockIdx.x, blockIdx.y, blockIdx.z, 0);
 }
@@ -1330,11 +1341,35 @@ __global__ void __launch_bounds__(kWide) k_interp_gather64(const R4<double>* __r
                                                           const int4* __restrict__ gbase, int n,
                                                           const double* __restrict__ u0, GridDims G, AssembleArgs A,
                                                           R4<double>* __restrict__ glong) {
+  pdl_sync();
   const int i = blockIdx.x * kWide + threadIdx.x;
   if (i >= n) return;
   double p, g[3];
   interp_atom<double, ORDER>(gfrac[i], gbase[i], u0, G, A.inv_h, p, g);
   glong[i] = R4<double>{g[0], g[1], g[2], p};
+}
+
+// The energy from the blocks' partials, by the block that finishes last (ticket:
+// one counter, back to 0 afterwards), in a fixed order: thread t takes partials
+// t, t + 256, ...
+__device__ __forceinline__ void energy_by_last_block(double bsum, double* __restrict__ partial, int* ticket,
+                                                     double* __restrict__ energy) {
+  __shared__ bool last;
+  if (threadIdx.x == 0) {
+    partial[blockIdx.x] = bsum;
+    __threadfence();
+    last = atomicAdd(ticket, 1) == (int)gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double v = 0.0;
+  for (int i = threadIdx.x; i < (int)gridDim.x; i += 256) v += __ldcg(partial + i);
+  const double s = block_sum<256>(v);
+  if (threadIdx.x == 0) {
+    *energy = 0.5 * s;
+    *ticket = 0;
+  }
 }
 
 // Assembly after the pair sums and the gather: phi_i, F_i in the caller's
@@ -1345,7 +1380,9 @@ __global__ void __launch_bounds__(256) k_interp_assemble(int64_t n, const int* _
                                                          const R4<T>* __restrict__ fs,
                                                          const R4<T>* __restrict__ glong, AssembleArgs A,
                                                          OUT* __restrict__ phi_out, OUT* __restrict__ force_out,
-                                                         double* __restrict__ partial) {
+                                                         double* __restrict__ partial, int* ticket,
+                                                         double* __restrict__ energy) {
+  pdl_sync();
   double e = 0.0;
   for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
     const R4<T> gl = glong[i];
@@ -1353,7 +1390,8 @@ __global__ void __launch_bounds__(256) k_interp_assemble(int64_t n, const int* _
     e += Assemble<T>::forward(A, gfrac[i].w, phis[i], gl.w, fs[i], g, perm[i], phi_out, force_out);
   }
   const double bsum = block_sum<256>(e);
-  if (threadIdx.x == 0) partial[blockIdx.x] = bsum;
+  __syncthreads();  // block_sum's buffer is used again by the last block
+  energy_by_last_block(bsum, partial, ticket, energy);
 }
 
 __device__ __forceinline__ void energy_final_body(const double* __restrict__ partial, int nb,
@@ -1366,6 +1404,7 @@ __device__ __forceinline__ void energy_final_body(const double* __restrict__ par
 
 __global__ void __launch_bounds__(1024) k_energy_final(const double* __restrict__ partial, int nb,
                                                        double* __restrict__ energy) {
+  pdl_sync();
   energy_final_body(partial, nb, energy);
 }
 
@@ -1412,6 +1451,7 @@ __global__ void __launch_bounds__(256, 3) k_interp_bwd(
     const int* __restrict__ cell_start, AnterpArgs AA, const float* __restrict__ av0, GridDims G, AssembleArgs A,
     const float* __restrict__ phis, const R4<float>* __restrict__ fs, const R4<float>* __restrict__ glong,
     const double* __restrict__ gE, OUT* __restrict__ grad_pos, OUT* __restrict__ grad_q) {
+  pdl_sync();
   interp_bwd_body<ORDER, OUT>(gfrac, gbase, perm, cell_start, AA, av0, G, A, phis, fs, glong, gE, grad_pos, grad_q,
                               blockIdx.x, blockIdx.y, blockIdx.z);
 }
@@ -1423,6 +1463,7 @@ __global__ void __launch_bounds__(kWide) k_interp_bwd64(
     const double* __restrict__ av0, GridDims G, AssembleArgs A, const double* __restrict__ phis,
     const R4<double>* __restrict__ fs, const R4<double>* __restrict__ glong, const double* __restrict__ gE,
     OUT* __restrict__ grad_pos, OUT* __restrict__ grad_q) {
+  pdl_sync();
   const int i = blockIdx.x * kWide + threadIdx.x;
   if (i >= n) return;
   const R4<double> f = gfrac[i];
@@ -1480,23 +1521,22 @@ AnterpArgs patch_args(const Plan& P, bool batch = false) {
 static int anterp_threads(size_t patch_bytes) { return patch_bytes > 100 * 1024 ? 1024 : 512; }
 
 // Mixed precision: patch sums into the fixed-point grid (in the restriction
-// temporary tmp[0], free until the first restriction pass), then one
+// temporary tmp[0], free until the first restriction pass, zeroed by the binning), then one
 // conversion to the FP64 level-0 grid that applies the scale.
 template <int ORDER>
 void anterp_fx(Plan& P, int64_t n, void* grid0, const double* dscale, double factor, cudaStream_t st) {
   const int64_t np = grid_points(P, 0);
   auto* gfx = (unsigned long long*)P.d.tmp[0];
-  cudaMemsetAsync(gfx, 0, sizeof(unsigned long long) * (size_t)np, st);
-  P.launches += 2;
+  P.launches += 1;
   if (n > 0) {
     AnterpArgs A = patch_args(P);
     dim3 grid(blocks_for(P.nc[0], A.B), blocks_for(P.nc[1], A.B), blocks_for(P.nc[2], A.B));
     size_t sm = 2 * sizeof(int) * (size_t)A.pd * A.pd * A.pd;  // coarse and residual sums
-    k_anterp_fx<ORDER><<<grid, anterp_threads(sm), sm, st>>>((const R4<float>*)P.d.gfrac, P.d.gbase, P.d.cell_start, A,
+    klaunch(false, k_anterp_fx<ORDER>, grid, anterp_threads(sm), sm, st, (const R4<float>*)P.d.gfrac, P.d.gbase, P.d.cell_start, A,
                                               dims_of(P, 0), gfx);
     P.launches += 1;
   }
-  k_fx_to_f64<<<blocks_for(np, 256), 256, 0, st>>>(gfx, (double*)grid0, np, dscale, factor);
+  klaunch(P.pdl, k_fx_to_f64, blocks_for(np, 256), 256, 0, st, gfx, (double*)grid0, np, dscale, factor);
 }
 
 cudaError_t launch_anterpolate(Plan& P, int64_t n, void* grid0, const double* dscale, double factor,
@@ -1506,23 +1546,22 @@ cudaError_t launch_anterpolate(Plan& P, int64_t n, void* grid0, const double* ds
     else anterp_fx<5>(P, n, grid0, dscale, factor, st);
     return cudaGetLastError();
   }
-  size_t bytes = sizeof(double) * (size_t)grid_points(P, 0);
-  cudaMemsetAsync(grid0, 0, bytes, st);
-  P.launches += 1 + (n > 0 ? 1 : 0);
   if (n <= 0) return cudaGetLastError();
+  P.launches += 1;
   const int stride = (int)((n + 31) / 32);
   const unsigned nb = blocks_for((int64_t)32 * stride, kWide);
   const R4<double>* f = (const R4<double>*)P.d.gfrac;
   if (P.P.order == 3)
-    k_anterp64<3><<<nb, kWide, 0, st>>>(f, P.d.gbase, (int)n, stride, dims_of(P, 0), (double*)grid0, dscale, factor);
+    klaunch(false, k_anterp64<3>, nb, kWide, 0, st, f, P.d.gbase, (int)n, stride, dims_of(P, 0), (double*)grid0, dscale, factor);
   else
-    k_anterp64<5><<<nb, kWide, 0, st>>>(f, P.d.gbase, (int)n, stride, dims_of(P, 0), (double*)grid0, dscale, factor);
+    klaunch(false, k_anterp64<5>, nb, kWide, 0, st, f, P.d.gbase, (int)n, stride, dims_of(P, 0), (double*)grid0, dscale, factor);
   return cudaGetLastError();
 }
 
 // dst = factor * dscale[0] * src over the level-0 grid (FP64)
 __global__ void k_scale_grid(const double* __restrict__ src, double* __restrict__ dst, int64_t count,
                              const double* __restrict__ dscale, double factor) {
+  pdl_sync();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   dst[i] = src[i] * (factor * *dscale);
@@ -1532,7 +1571,7 @@ cudaError_t launch_scale_grid(Plan& P, const void* src, void* dst, const double*
                               cudaStream_t st) {
   P.launches += 1;
   const int64_t np = grid_points(P, 0);
-  k_scale_grid<<<blocks_for(np, 256), 256, 0, st>>>((const double*)src, (double*)dst, np, dscale, factor);
+  klaunch(false, k_scale_grid, blocks_for(np, 256), 256, 0, st, (const double*)src, (double*)dst, np, dscale, factor);
   return cudaGetLastError();
 }
 
@@ -1570,8 +1609,8 @@ cudaError_t launch_restrict(Plan& P, int k, const void* fine, void* coarse, cuda
     P.launches += 1;
     const Grid3Args A = grid3_args(P, k, k + 1);
     const unsigned nb = (unsigned)restrict_tiles(nc);
-    if (P.P.order == 3) k_restrict_tile<3><<<nb, 128, 0, st>>>((const double*)fine, (double*)coarse, A);
-    else k_restrict_tile<5><<<nb, 128, 0, st>>>((const double*)fine, (double*)coarse, A);
+    if (P.P.order == 3) klaunch(P.pdl, k_restrict_tile<3>, nb, 128, 0, st, (const double*)fine, (double*)coarse, A);
+    else klaunch(P.pdl, k_restrict_tile<5>, nb, 128, 0, st, (const double*)fine, (double*)coarse, A);
     return cudaGetLastError();
   }
   P.launches += 3;
@@ -1590,8 +1629,8 @@ cudaError_t launch_restrict(Plan& P, int k, const void* fine, void* coarse, cuda
     A.lo_out = P.lo[k + 1][ax];
     A.periodic = P.P.periodic;
     unsigned nb = blocks_for((int64_t)cur[0] * cur[1] * cur[2], 256);
-    if (P.P.order == 3) k_restrict_axis<double, 3><<<nb, 256, 0, st>>>(src[ax], dst[ax], A);
-    else k_restrict_axis<double, 5><<<nb, 256, 0, st>>>(src[ax], dst[ax], A);
+    if (P.P.order == 3) klaunch(P.pdl, k_restrict_axis<double, 3>, nb, 256, 0, st, src[ax], dst[ax], A);
+    else klaunch(P.pdl, k_restrict_axis<double, 5>, nb, 256, 0, st, src[ax], dst[ax], A);
   }
   return cudaGetLastError();
 }
@@ -1600,8 +1639,8 @@ template <typename T, int TYZ>
 static void prolong_t(Plan& P, int k, const T* coarse, T* fine, cudaStream_t st) {
   const Grid3Args A = grid3_args(P, k + 1, k);
   const unsigned nb = (unsigned)prolong_tiles(P.n[k], TYZ);
-  if (P.P.order == 3) k_prolong_tile<T, 3, TYZ><<<nb, 256, 0, st>>>(coarse, fine, A);
-  else k_prolong_tile<T, 5, TYZ><<<nb, 256, 0, st>>>(coarse, fine, A);
+  if (P.P.order == 3) klaunch(P.pdl, k_prolong_tile<T, 3, TYZ>, nb, 256, 0, st, coarse, fine, A);
+  else klaunch(P.pdl, k_prolong_tile<T, 5, TYZ>, nb, 256, 0, st, coarse, fine, A);
 }
 
 cudaError_t launch_prolong(Plan& P, int k, const void* coarse, void* fine, cudaStream_t st) {
@@ -1623,6 +1662,7 @@ __device__ __forceinline__ void f64_to_f32_body(const double* __restrict__ src, 
 }
 
 __global__ void k_f64_to_f32(const double* __restrict__ src, float* __restrict__ dst, int64_t count) {
+  pdl_sync();
   f64_to_f32_body(src, dst, count, (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
@@ -1666,10 +1706,10 @@ static void lattice_fp64(Plan& P, int k, const double* qk, double* uk, cudaStrea
   dim3 grid(blocks_for(np, kLat64), ns);
   const double scale = std::ldexp(1.0, -k);
   const double* coef = (const double*)P.d.seg;
-  if (G.periodic) k_lattice64<true><<<grid, kLat64, 0, st>>>(qk, uk, up, G, P.d.lrows, coef, P.nlrows, per, scale);
-  else k_lattice64<false><<<grid, kLat64, 0, st>>>(qk, uk, up, G, P.d.lrows, coef, P.nlrows, per, scale);
+  if (G.periodic) klaunch(P.pdl, k_lattice64<true>, grid, kLat64, 0, st, qk, uk, up, G, P.d.lrows, coef, P.nlrows, per, scale);
+  else klaunch(P.pdl, k_lattice64<false>, grid, kLat64, 0, st, qk, uk, up, G, P.d.lrows, coef, P.nlrows, per, scale);
   if (ns > 1) {
-    k_lattice_reduce<double><<<blocks_for(np, 256), 256, 0, st>>>(up, uk, np, ns);
+    klaunch(P.pdl, k_lattice_reduce<double>, blocks_for(np, 256), 256, 0, st, up, uk, np, ns);
     P.launches += 1;
   }
 }
@@ -1680,7 +1720,7 @@ static void lattice_fp64(Plan& P, int k, const double* qk, double* uk, cudaStrea
 static void lattice_fp32(Plan& P, int k, const double* qk64, float* uk, cudaStream_t st) {
   GridDims G = dims_of(P, k);
   float* qk = (float*)P.d.tmp[0];  // free between the restriction and the prolongation passes
-  k_f64_to_f32<<<blocks_for(grid_points(P, k), 256), 256, 0, st>>>(qk64, qk, grid_points(P, k));
+  klaunch(P.pdl, k_f64_to_f32, blocks_for(grid_points(P, k), 256), 256, 0, st, qk64, qk, grid_points(P, k));
   P.launches += 1;
   LatticeArgs L;
   L.Ex = P.E[0];
@@ -1698,14 +1738,14 @@ static void lattice_fp32(Plan& P, int k, const double* qk64, float* uk, cudaStre
   const size_t sm = lattice_smem(L.txn, L.tyn, P.E);
   const float scale = (float)std::ldexp(1.0, -k);
   if (L.txn == 4 && L.tyn == 8)
-    k_lattice_f2<kLatticeLP, 4, 8><<<grid, 32 * kLatticeZ, sm, st>>>(qk, uk, up, G, (const Segment2*)P.d.seg2,
+    klaunch(P.pdl, k_lattice_f2<kLatticeLP, 4, 8>, grid, 32 * kLatticeZ, sm, st, qk, uk, up, G, (const Segment2*)P.d.seg2,
                                                                     P.d.seg_start, L, scale);
   else
-    k_lattice_f2<kLatticeLP, 0, 0><<<grid, 32 * kLatticeZ, sm, st>>>(qk, uk, up, G, (const Segment2*)P.d.seg2,
+    klaunch(P.pdl, k_lattice_f2<kLatticeLP, 0, 0>, grid, 32 * kLatticeZ, sm, st, qk, uk, up, G, (const Segment2*)P.d.seg2,
                                                                     P.d.seg_start, L, scale);
   if (L.nsplit > 1) {
     const int64_t np = grid_points(P, k);
-    k_lattice_reduce<float><<<blocks_for(np, 256), 256, 0, st>>>(up, uk, np, L.nsplit);
+    klaunch(P.pdl, k_lattice_reduce<float>, blocks_for(np, 256), 256, 0, st, up, uk, np, L.nsplit);
     P.launches += 1;
   }
 }
@@ -1775,10 +1815,10 @@ cudaError_t launch_top(Plan& P, const void* qt, void* ut, cudaStream_t st) {
   GridDims G = dims_of(P, top);
   unsigned nb = blocks_for(grid_points(P, top), kTopWarps);
   if (P.fp64)
-    k_top<double><<<nb, 32 * kTopWarps, 0, st>>>((const double*)qt, (double*)ut, P.d.topu, G, P.d.topK,
+    klaunch(P.pdl, k_top<double>, nb, 32 * kTopWarps, 0, st, (const double*)qt, (double*)ut, P.d.topu, G, P.d.topK,
                                      P.top_table_dims[0], P.top_table_dims[1], P.top_table_dims[2]);
   else
-    k_top<float><<<nb, 32 * kTopWarps, 0, st>>>((const double*)qt, (float*)ut, P.d.topu, G, P.d.topK,
+    klaunch(P.pdl, k_top<float>, nb, 32 * kTopWarps, 0, st, (const double*)qt, (float*)ut, P.d.topu, G, P.d.topK,
                                     P.top_table_dims[0], P.top_table_dims[1], P.top_table_dims[2]);
   return cudaGetLastError();
 }
@@ -1823,8 +1863,8 @@ cudaError_t launch_interp_gather(Plan& P, int64_t n, cudaStream_t st) {
     const unsigned nb = blocks_for(n, kWide);
     const R4<double>* f = (const R4<double>*)P.d.gfrac;
     const double* u = (const double*)P.d.gu[0];
-    if (P.P.order == 3) k_interp_gather64<3><<<nb, kWide, 0, st>>>(f, P.d.gbase, (int)n, u, G, A, (R4<double>*)P.d.glong);
-    else k_interp_gather64<5><<<nb, kWide, 0, st>>>(f, P.d.gbase, (int)n, u, G, A, (R4<double>*)P.d.glong);
+    if (P.P.order == 3) klaunch(P.pdl, k_interp_gather64<3>, nb, kWide, 0, st, f, P.d.gbase, (int)n, u, G, A, (R4<double>*)P.d.glong);
+    else klaunch(P.pdl, k_interp_gather64<5>, nb, kWide, 0, st, f, P.d.gbase, (int)n, u, G, A, (R4<double>*)P.d.glong);
     return cudaGetLastError();
   }
   AnterpArgs AA = patch_args(P);
@@ -1833,9 +1873,9 @@ cudaError_t launch_interp_gather(Plan& P, int64_t n, cudaStream_t st) {
   const R4<float>* f = (const R4<float>*)P.d.gfrac;
   const float* u = (const float*)P.d.gu[0];
   if (P.P.order == 3)
-    k_interp_gather<3><<<grid, 256, sm, st>>>(f, P.d.gbase, P.d.cell_start, AA, u, G, A, (R4<float>*)P.d.glong);
+    klaunch(P.pdl, k_interp_gather<3>, grid, 256, sm, st, f, P.d.gbase, P.d.cell_start, AA, u, G, A, (R4<float>*)P.d.glong);
   else
-    k_interp_gather<5><<<grid, 256, sm, st>>>(f, P.d.gbase, P.d.cell_start, AA, u, G, A, (R4<float>*)P.d.glong);
+    klaunch(P.pdl, k_interp_gather<5>, grid, 256, sm, st, f, P.d.gbase, P.d.cell_start, AA, u, G, A, (R4<float>*)P.d.glong);
   return cudaGetLastError();
 }
 
@@ -1845,16 +1885,18 @@ cudaError_t launch_interp_assemble(Plan& P, int64_t n, double* energy, OUT* phi,
   const AssembleArgs A = assemble_args(P);
   if (nb > 0) {
     if (P.fp64)
-      k_interp_assemble<double, OUT><<<nb, 256, 0, st>>>(n, P.d.perm, (const R4<double>*)P.d.gfrac,
+      klaunch(false, k_interp_assemble<double, OUT>, nb, 256, 0, st, n, P.d.perm, (const R4<double>*)P.d.gfrac,
                                                         (const double*)P.d.phis, (const R4<double>*)P.d.fs,
-                                                        (const R4<double>*)P.d.glong, A, phi, force, P.d.partial);
+                                                        (const R4<double>*)P.d.glong, A, phi, force, P.d.partial,
+                                                        P.d.ticket, energy);
     else
-      k_interp_assemble<float, OUT><<<nb, 256, 0, st>>>(n, P.d.perm, (const R4<float>*)P.d.gfrac,
+      klaunch(false, k_interp_assemble<float, OUT>, nb, 256, 0, st, n, P.d.perm, (const R4<float>*)P.d.gfrac,
                                                        (const float*)P.d.phis, (const R4<float>*)P.d.fs,
-                                                       (const R4<float>*)P.d.glong, A, phi, force, P.d.partial);
+                                                       (const R4<float>*)P.d.glong, A, phi, force, P.d.partial,
+                                                        P.d.ticket, energy);
   }
-  k_energy_final<<<1, 1024, 0, st>>>(P.d.partial, nb, energy);
-  P.launches += 1 + (nb > 0 ? 1 : 0);
+  if (nb == 0) klaunch(false, k_energy_final, 1, 1024, 0, st, P.d.partial, nb, energy);
+  P.launches += 1;
   return cudaGetLastError();
 }
 
@@ -1870,18 +1912,18 @@ cudaError_t launch_interp_backward(Plan& P, int64_t n, const double* gE, OUT* gr
     const unsigned nb = blocks_for(n, kWide);
     const auto K = interp_kargs<double, OUT>(P, true, nullptr, nullptr, gE, grad_pos, grad_q, nullptr);
     if (P.P.order == 3)
-      k_interp_bwd64<3, OUT><<<nb, kWide, 0, st>>>(K.gfrac, K.gbase, K.perm, (int)n, K.u0, K.G, K.A, K.phis, K.fs,
+      klaunch(P.pdl, k_interp_bwd64<3, OUT>, nb, kWide, 0, st, K.gfrac, K.gbase, K.perm, (int)n, K.u0, K.G, K.A, K.phis, K.fs,
                                                    K.glong, gE, grad_pos, grad_q);
     else
-      k_interp_bwd64<5, OUT><<<nb, kWide, 0, st>>>(K.gfrac, K.gbase, K.perm, (int)n, K.u0, K.G, K.A, K.phis, K.fs,
+      klaunch(P.pdl, k_interp_bwd64<5, OUT>, nb, kWide, 0, st, K.gfrac, K.gbase, K.perm, (int)n, K.u0, K.G, K.A, K.phis, K.fs,
                                                    K.glong, gE, grad_pos, grad_q);
     return cudaGetLastError();
   }
   const auto K = interp_kargs<float, OUT>(P, true, nullptr, nullptr, gE, grad_pos, grad_q, nullptr);
   dim3 grid(K.nbx, K.nby, blocks_for(P.nc[2], K.AA.B));
   size_t sm = sizeof(float) * (size_t)K.AA.pd * K.AA.pd * K.AA.pd;
-  if (P.P.order == 3) k_interp_bwd<3, OUT><<<grid, 256, sm, st>>>(INTERP_BWD_ARGS(K));
-  else k_interp_bwd<5, OUT><<<grid, 256, sm, st>>>(INTERP_BWD_ARGS(K));
+  if (P.P.order == 3) klaunch(P.pdl, k_interp_bwd<3, OUT>, grid, 256, sm, st, INTERP_BWD_ARGS(K));
+  else klaunch(P.pdl, k_interp_bwd<5, OUT>, grid, 256, sm, st, INTERP_BWD_ARGS(K));
   return cudaGetLastError();
 }
 
@@ -1893,8 +1935,8 @@ cudaError_t launch_grid_to_double(Plan& P, const void* src, double* dst, int64_t
                                   cudaStream_t st) {
   unsigned nb = blocks_for(count, 256);
   if (count <= 0) return cudaSuccess;
-  if (P.fp64 || is_double) k_to_double<double><<<nb, 256, 0, st>>>((const double*)src, dst, count);
-  else k_to_double<float><<<nb, 256, 0, st>>>((const float*)src, dst, count);
+  if (P.fp64 || is_double) klaunch(false, k_to_double<double>, nb, 256, 0, st, (const double*)src, dst, count);
+  else klaunch(false, k_to_double<float>, nb, 256, 0, st, (const float*)src, dst, count);
   return cudaGetLastError();
 }
 
@@ -1906,7 +1948,9 @@ template <typename T, typename OUT>
 __global__ void __launch_bounds__(256) k_cutoff_assemble(int64_t n, const int* __restrict__ perm,
                                                          const R4<T>* __restrict__ atoms, const T* __restrict__ phis,
                                                          const R4<T>* __restrict__ fs, T kc, T selfc, OUT* __restrict__ phi_out,
-                                                         OUT* __restrict__ force_out, double* __restrict__ partial) {
+                                                         OUT* __restrict__ force_out, double* __restrict__ partial,
+                                                         int* ticket, double* __restrict__ energy) {
+  pdl_sync();
   double e = 0.0;
   for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
     const T p = phis[i] - selfc * atoms[i].w;  // selfc: the method's self term (0 for the cutoff method)
@@ -1921,7 +1965,8 @@ __global__ void __launch_bounds__(256) k_cutoff_assemble(int64_t n, const int* _
     e += (double)(atoms[i].w * (kc * p));
   }
   const double bsum = block_sum<256>(e);
-  if (threadIdx.x == 0) partial[blockIdx.x] = bsum;
+  __syncthreads();  // block_sum's buffer is used again by the last block
+  energy_by_last_block(bsum, partial, ticket, energy);
 }
 
 template <typename OUT>
@@ -1930,17 +1975,17 @@ cudaError_t launch_cutoff_assemble(Plan& P, int64_t n, double* energy, OUT* phi,
   const int nb = (int)std::max<int64_t>(0, std::min<int64_t>(P.nblk_partial, (n + 255) / 256));
   if (nb > 0) {
     if (P.fp64)
-      k_cutoff_assemble<double, OUT><<<nb, 256, 0, st>>>(n, P.d.perm, (const R4<double>*)P.d.atoms,
+      klaunch(false, k_cutoff_assemble<double, OUT>, nb, 256, 0, st, n, P.d.perm, (const R4<double>*)P.d.atoms,
                                                         (const double*)P.d.phis, (const R4<double>*)P.d.fs,
-                                                        P.P.coulomb_k, self_c, phi, force, P.d.partial);
+                                                        P.P.coulomb_k, self_c, phi, force, P.d.partial, P.d.ticket, energy);
     else
-      k_cutoff_assemble<float, OUT><<<nb, 256, 0, st>>>(n, P.d.perm, (const R4<float>*)P.d.atoms,
+      klaunch(false, k_cutoff_assemble<float, OUT>, nb, 256, 0, st, n, P.d.perm, (const R4<float>*)P.d.atoms,
                                                        (const float*)P.d.phis, (const R4<float>*)P.d.fs,
                                                        (float)P.P.coulomb_k, (float)self_c, phi, force,
-                                                       P.d.partial);
+                                                       P.d.partial, P.d.ticket, energy);
   }
-  k_energy_final<<<1, 1024, 0, st>>>(P.d.partial, nb, energy);
-  P.launches += 1 + (nb > 0 ? 1 : 0);
+  if (nb == 0) klaunch(false, k_energy_final, 1, 1024, 0, st, P.d.partial, nb, energy);
+  P.launches += 1;
   return cudaGetLastError();
 }
 

@@ -850,6 +850,7 @@ __device__ __forceinline__ void short_range_body(const PairKArgs& K, int blk) {
 
 template <int M, int KIND>
 __global__ void __launch_bounds__(32 * kWarps, MSM_PAIR_MINB) k_short_range(const __grid_constant__ PairKArgs a) {
+  pdl_sync();
   short_range_body<M, KIND>(a, blockIdx.x);
 }
 
@@ -931,8 +932,8 @@ static int pair_blocks(const PairKArgs& K) {
 }
 
 template <int M, int KIND>
-void launch_mk(const PairKArgs& K, cudaStream_t st) {
-  k_short_range<M, KIND><<<pair_blocks(K), 32 * kWarps, 0, st>>>(K);
+void launch_mk(const Plan& P, const PairKArgs& K, cudaStream_t st) {
+  klaunch(P.pdl, k_short_range<M, KIND>, pair_blocks(K), 32 * kWarps, 0, st, K);
 }
 
 template <int KIND>
@@ -951,11 +952,11 @@ void launch_f2(Plan& P, int64_t n, cudaStream_t st, double alpha = 0.0) {
   }
   K.runs = use_runs(P);
   K.split = P.ncell < kSplitCells ? kWarps : 1;
-  if (KIND == kPairCutoff) launch_mk<2, kPairCutoff>(K, st);  // M unused
-  else if (KIND == kPairWolf) launch_mk<2, kPairWolf>(K, st);
-  else if (P.P.splitting == 1) launch_mk<1, kPairMSM>(K, st);
-  else if (P.P.splitting == 2) launch_mk<2, kPairMSM>(K, st);
-  else launch_mk<3, kPairMSM>(K, st);
+  if (KIND == kPairCutoff) launch_mk<2, kPairCutoff>(P, K, st);  // M unused
+  else if (KIND == kPairWolf) launch_mk<2, kPairWolf>(P, K, st);
+  else if (P.P.splitting == 1) launch_mk<1, kPairMSM>(P, K, st);
+  else if (P.P.splitting == 2) launch_mk<2, kPairMSM>(P, K, st);
+  else launch_mk<3, kPairMSM>(P, K, st);
 }
 
 cudaError_t launch_short_range(Plan& P, int64_t n, cudaStream_t st) {

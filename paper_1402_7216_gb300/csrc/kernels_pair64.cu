@@ -128,6 +128,7 @@ __device__ __forceinline__ void pair64(const Pair64Args& A, double tx, double ty
 
 template <int M, int K>
 __global__ void __launch_bounds__(32 * kMaxSplit) k_pair64(const __grid_constant__ Pair64Args A) {
+  pdl_sync();
   extern __shared__ __align__(16) unsigned char smem64[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   Warp64& S = reinterpret_cast<Warp64*>(smem64)[warp];
@@ -322,12 +323,11 @@ Pair64Args pair64_args(const Plan& P, int64_t n, double alpha) {
 }
 
 template <int M, int K>
-cudaError_t launch_k(const Pair64Args& A, cudaStream_t st) {
+cudaError_t launch_k(const Plan& P, const Pair64Args& A, cudaStream_t st) {
   const int64_t groups = ((int64_t)A.g.natoms + (1 << A.lt) - 1) >> A.lt;
   const int warps = A.nsplit > 1 ? A.nsplit : 2;
   const unsigned blocks = (unsigned)(A.nsplit > 1 ? groups : (groups + warps - 1) / warps);
-  k_pair64<M, K><<<blocks, 32 * warps, warps * sizeof(Warp64), st>>>(A);
-  return cudaGetLastError();
+  return klaunch(P.pdl, k_pair64<M, K>, blocks, 32 * warps, warps * sizeof(Warp64), st, A);
 }
 
 template <int M, int K>
@@ -349,11 +349,11 @@ cudaError_t configure_pair64_kernels() {
 
 cudaError_t launch_pair64(Plan& P, int kind, int64_t n, double alpha, cudaStream_t st) {
   const Pair64Args A = pair64_args(P, n, alpha);
-  if (kind == kPairCutoff) return launch_k<2, kPairCutoff>(A, st);  // M unused
-  if (kind == kPairWolf) return launch_k<2, kPairWolf>(A, st);
-  if (P.P.splitting == 1) return launch_k<1, kPairMSM>(A, st);
-  if (P.P.splitting == 2) return launch_k<2, kPairMSM>(A, st);
-  return launch_k<3, kPairMSM>(A, st);
+  if (kind == kPairCutoff) return launch_k<2, kPairCutoff>(P, A, st);  // M unused
+  if (kind == kPairWolf) return launch_k<2, kPairWolf>(P, A, st);
+  if (P.P.splitting == 1) return launch_k<1, kPairMSM>(P, A, st);
+  if (P.P.splitting == 2) return launch_k<2, kPairMSM>(P, A, st);
+  return launch_k<3, kPairMSM>(P, A, st);
 }
 
 }  // namespace msm

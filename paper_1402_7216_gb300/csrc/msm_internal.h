@@ -77,6 +77,7 @@ struct DeviceBuffers {
   // reductions and status
   double* partial = nullptr;   // per-block energy partials
   double* scalars = nullptr;   // [8] scratch scalars (0: backward scale; 1, 2..7: MD energy and record when none is kept)
+  int* ticket = nullptr;       // [1] blocks of the assembly that are done (zero between evaluations)
   double* md_partial = nullptr;  // [4 * kMdBlocks] per-block kinetic energy and momentum of the MD loop
   int* md_step = nullptr;        // [1] record counter of MD steps replayed from a graph
   int* status = nullptr;
@@ -147,6 +148,7 @@ struct Plan {
   int64_t cap = 0;
   int nblk_partial = 0;
   DeviceBuffers d;
+  bool pdl = false;  // small plan: dependent launches scheduled early (klaunch)
   // concurrency: the grid passes of a forward evaluation run on `side` (a
   // plan-owned stream of the highest priority) while the pair sums run on the
   // caller's stream; fork and join are event waits
@@ -174,6 +176,35 @@ struct Plan {
   int64_t launches = 0;
   int64_t evals = 0;
 };
+
+#ifdef __CUDACC__
+// Launches of a plan's chains of small kernels.  With pdl (small plans) the
+// kernel may be scheduled while its predecessor in the stream drains and then
+// waits in pdl_sync() for the predecessor's results: that hides the launch gap
+// between dependent kernels, which is most of a small system's time.  On large
+// plans blocks waiting early would take the SMs from the concurrent pair sums.
+template <typename... P, typename... A>
+inline cudaError_t klaunch(bool pdl, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                           A&&... args) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  cudaLaunchAttribute at[1] = {};
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = at;
+  c.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+// First statement of every kernel launched so: waits until the kernels before
+// it have completed, then lets the next one be scheduled.
+__device__ __forceinline__ void pdl_sync() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+#endif
 
 // ---- batches of independent systems (one launch per stage over all replicas) ----
 // A batched launch numbers the blocks of all replicas consecutively; first[r]
@@ -278,8 +309,11 @@ int64_t grid_points(const Plan& P, int k);
 
 // ---- launchers (.cu files); all asynchronous on stream ----
 // binning: keys, stable radix sort by cell, cell_start, gather of sorted atoms
+// and, on the way, nzero 8-byte words at zero set to 0 (the charge grid the
+// anterpolation adds into)
 template <typename IO>  // IO = double or float (caller's position and charge type)
-cudaError_t launch_binning(Plan& P, int64_t n, const IO* pos, const IO* q, cudaStream_t s);
+cudaError_t launch_binning(Plan& P, int64_t n, const IO* pos, const IO* q, cudaStream_t s,
+                           unsigned long long* zero = nullptr, int64_t nzero = 0);
 // short-range pair sums (phis, fs.xyz)
 cudaError_t launch_short_range(Plan& P, int64_t n, cudaStream_t s);
 // the cutoff method: Coulomb pair sums within the cutoff (phis, fs.xyz); Wolf
@@ -340,7 +374,7 @@ struct FftBatchItem {
   void* work;
 };
 cudaError_t fft_batch_build(const std::vector<FftBatchItem>& items, bool fp64, FftBatch** out);
-cudaError_t fft_batch_launch(const FftBatch* b, cudaStream_t s);
+cudaError_t fft_batch_launch(const FftBatch* b, cudaStream_t s, bool pdl = false);
 void fft_batch_free(FftBatch* b);
 cudaError_t launch_top(Plan& P, const void* qt, void* ut, cudaStream_t s);
 cudaError_t launch_prolong(Plan& P, int k, const void* coarse, void* fine, cudaStream_t s);

@@ -551,13 +551,16 @@ int build_plan(const msm_params* pp, const msm_tuning* tune, Plan* P) {
   M((void**)&D.md_partial, sizeof(double) * 4 * kMdBlocks);
   M((void**)&D.md_step, sizeof(int));
   M((void**)&D.status, sizeof(int));
+  M((void**)&D.ticket, sizeof(int));
   if (want_fft) {  // complex FP64 per point of every lattice level (the kernel's transforms use level 0's share)
     size_t pts = 0;
     for (int k = 0; k + 1 < P->levels; ++k) pts += (size_t)grid_points(*P, k);
     M(&D.fft_work, 16 * pts);
   }
   if (e != cudaSuccess) return MSM_ERR_OOM;
-  if (cudaMemset(D.status, 0, sizeof(int)) != cudaSuccess) return MSM_ERR_CUDA;
+  if (cudaMemset(D.status, 0, sizeof(int)) != cudaSuccess || cudaMemset(D.ticket, 0, sizeof(int)) != cudaSuccess)
+    return MSM_ERR_CUDA;
+  P->pdl = cap <= 262144 && grid_points(*P, 0) <= 80 * 80 * 80;
   if (want_fft) {
     // the folded kernel of level k on its own grid: taps n wrapped modulo the
     // level's dimensions (the images of the sphere where it is wider than the
@@ -618,7 +621,7 @@ void free_plan(Plan* P) {
   DeviceBuffers& D = P->d;
   void* ptrs[] = {D.key, D.rank, D.perm, D.count, D.csum, D.cell_start, D.atoms,
                   D.gfrac, D.gbase, D.scell, D.cellx, D.phis, D.fs, D.glong, D.topK, D.topq, D.topu, D.seg, D.seg2, D.cell_rows,
-                  D.seg_start, D.lrows, D.partial, D.scalars, D.md_partial, D.md_step, D.status, D.hpos, D.hq,
+                  D.seg_start, D.lrows, D.partial, D.scalars, D.md_partial, D.md_step, D.status, D.ticket, D.hpos, D.hq,
                   D.hphi, D.hforce, D.henergy, D.lparts, D.fft_work};
   for (void* p : ptrs)
     if (p) cudaFree(p);
