@@ -32,8 +32,19 @@ def _ptr(t):
 
 
 def _stream(stream):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return C.c_void_p(s.cuda_stream)
+    return C.c_void_p(_raw_stream(stream))
+
+
+def _raw_stream(stream):
+    """The stream's handle as an integer (the current stream's without making
+    a Stream object, which costs several microseconds)."""
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+
+
+def _addr(t):
+    return t.data_ptr() if t is not None else None
 
 
 class MSM:
@@ -111,6 +122,8 @@ class MSM:
         """Forward pass: returns (E [0-d] float64, phi [N] or None, F [N,3] or
         None).  float64 inputs go through msm_eval, float32 inputs through
         msm_eval_f32io (phi and F then come back as float32)."""
+        # integers and bound functions straight to ctypes: on small systems the
+        # marshalling of a call costs as much host time as its launches
         pos, q = self._check_inputs(pos, q)
         n = pos.shape[0]
         io = pos.dtype
@@ -120,9 +133,11 @@ class MSM:
             F = torch.empty((n, 3), dtype=io, device=pos.device) if want_force else None
         else:
             E, phi, F = out
-        fn = lib().msm_eval if io == torch.float64 else lib().msm_eval_f32io
-        rc = fn(self._h, n, _ptr(pos), _ptr(q), _ptr(E), _ptr(phi), _ptr(F), _stream(stream))
-        _capi.check(rc, "msm_eval" if io == torch.float64 else "msm_eval_f32io")
+        L = lib()
+        fn = L.msm_eval if io is torch.float64 else L.msm_eval_f32io
+        rc = fn(self._h, n, pos.data_ptr(), q.data_ptr(), _addr(E), _addr(phi), _addr(F), _raw_stream(stream))
+        if rc:
+            _capi.check(rc, "msm_eval" if io is torch.float64 else "msm_eval_f32io")
         self._last_n = n
         self._last_io = io
         return E, phi, F
@@ -223,7 +238,9 @@ class MSM:
     def forward_id(self):
         """msm_forward_id: the id of this plan's latest forward pass (0: none)."""
         fid = C.c_int64()
-        _capi.check(lib().msm_forward_id(self._h, C.byref(fid)), "msm_forward_id")
+        rc = lib().msm_forward_id(self._h, C.byref(fid))
+        if rc:
+            _capi.check(rc, "msm_forward_id")
         return fid.value
 
     def backward(self, grad_E, want_pos=True, want_q=True, stream=None, dtype=None, forward_id=None):
@@ -243,10 +260,14 @@ class MSM:
         dev = grad_E.device
         gp = torch.empty((n, 3), dtype=io, device=dev) if want_pos else None
         gq = torch.empty(n, dtype=io, device=dev) if want_q else None
-        g = grad_E.to(torch.float64).reshape(()).contiguous()
-        fn = lib().msm_eval_backward if io == torch.float64 else lib().msm_eval_backward_f32io
-        rc = fn(self._h, fid, _ptr(g), _ptr(gp), _ptr(gq), _stream(stream))
-        _capi.check(rc, "msm_eval_backward" if io == torch.float64 else "msm_eval_backward_f32io")
+        g = grad_E
+        if g.dtype is not torch.float64 or g.numel() != 1:
+            g = g.to(torch.float64).reshape(())
+        L = lib()
+        fn = L.msm_eval_backward if io is torch.float64 else L.msm_eval_backward_f32io
+        rc = fn(self._h, fid, g.data_ptr(), _addr(gp), _addr(gq), _raw_stream(stream))
+        if rc:
+            _capi.check(rc, "msm_eval_backward" if io is torch.float64 else "msm_eval_backward_f32io")
         return gp, gq
 
     def eval_host(self, pos, q, want_phi=False, want_force=False, stream=None, out=None):
