@@ -607,7 +607,22 @@ __device__ __forceinline__ int axis_index(int i, int n, int lo, int periodic) {
   return i;
 }
 
-// Restriction: kTileC^3 coarse points per block of 128 threads.  The FP64
+// One value from global to shared memory without waiting (0 where g < 0);
+// tile_wait() completes the thread's copies.
+template <typename T>
+__device__ __forceinline__ void tile_copy(T* dst, const T* __restrict__ src, int64_t g) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  const T* p = g >= 0 ? src + g : src;
+  const int bytes = g >= 0 ? (int)sizeof(T) : 0;
+  if (sizeof(T) == 8) asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(p), "r"(bytes) : "memory");
+  else asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(p), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void tile_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// Restriction: kTileC^3 coarse points per block of 256 threads; small levels
+// are bound by latency, so the tile's loads are all in flight at once (against
+// a loop of loads and 128 threads, all levels: 80^3 fine points 80 -> 57 us,
+// 32^3 27 -> 19 us, 16^3 23 -> 17 us).  The FP64
 // arithmetic (2 lanes per SM and clock) of the halo makes the tile cost about
 // twice the axis passes' operations, so large levels keep those (see
 // restrict_by_tiles).
@@ -635,8 +650,9 @@ __device__ __forceinline__ void restrict_tile_body(const double* __restrict__ in
   __syncthreads();
   for (int e = tid; e < F * F * F; e += blockDim.x) {
     const int x = S.idx[0][e % F], y = S.idx[1][e / F % F], z = S.idx[2][e / (F * F)];
-    S.a[e] = (x | y | z) < 0 ? 0.0 : in[((size_t)z * A.nin[1] + y) * A.nin[0] + x];
+    tile_copy(S.a + e, in, (x | y | z) < 0 ? (int64_t)-1 : ((int64_t)z * A.nin[1] + y) * A.nin[0] + x);
   }
+  tile_wait();
   __syncthreads();
   auto taps = [&](const double* v, int stride) {  // v: the point at offset 0
     double sum = 0.0;
@@ -661,7 +677,7 @@ __device__ __forceinline__ void restrict_tile_body(const double* __restrict__ in
 }
 
 template <int ORDER>
-__global__ void __launch_bounds__(128) k_restrict_tile(const double* __restrict__ in, double* __restrict__ out,
+__global__ void __launch_bounds__(256) k_restrict_tile(const double* __restrict__ in, double* __restrict__ out,
                                                        Grid3Args A) {
   pdl_sync();
   restrict_tile_body<ORDER>(in, out, A, blockIdx.x);
@@ -701,8 +717,9 @@ __device__ __forceinline__ void prolong_tile_body(const T* __restrict__ in, T* _
   __syncthreads();
   for (int e = tid; e < CY * CY * CX; e += blockDim.x) {
     const int x = S.idx[0][e % CX], y = S.idx[1][e / CX % CY], z = S.idx[2][e / (CX * CY)];
-    S.a[e] = (x | y | z) < 0 ? T(0) : in[((size_t)z * A.nin[1] + y) * A.nin[0] + x];
+    tile_copy(S.a + e, in, (x | y | z) < 0 ? (int64_t)-1 : ((int64_t)z * A.nin[1] + y) * A.nin[0] + x);
   }
+  tile_wait();
   __syncthreads();
   // fine index nu (even: the coarse point nu / 2; odd: those at odd distances up to R); v: coarse point co
   auto taps = [&](const T* v, int stride, int nu, int c) {
@@ -1609,8 +1626,8 @@ cudaError_t launch_restrict(Plan& P, int k, const void* fine, void* coarse, cuda
     P.launches += 1;
     const Grid3Args A = grid3_args(P, k, k + 1);
     const unsigned nb = (unsigned)restrict_tiles(nc);
-    if (P.P.order == 3) klaunch(P.pdl, k_restrict_tile<3>, nb, 128, 0, st, (const double*)fine, (double*)coarse, A);
-    else klaunch(P.pdl, k_restrict_tile<5>, nb, 128, 0, st, (const double*)fine, (double*)coarse, A);
+    if (P.P.order == 3) klaunch(P.pdl, k_restrict_tile<3>, nb, 256, 0, st, (const double*)fine, (double*)coarse, A);
+    else klaunch(P.pdl, k_restrict_tile<5>, nb, 256, 0, st, (const double*)fine, (double*)coarse, A);
     return cudaGetLastError();
   }
   P.launches += 3;
@@ -2093,7 +2110,7 @@ __global__ void __launch_bounds__(kEw) kb_restrict_axis(const AxisKArgs<double>*
 }
 
 template <int ORDER>
-__global__ void __launch_bounds__(128) kb_restrict_tile(const TileKArgs<double>* __restrict__ tab,
+__global__ void __launch_bounds__(256) kb_restrict_tile(const TileKArgs<double>* __restrict__ tab,
                                                         const int* __restrict__ first, int nrep) {
   const int r = batch_rep(first, nrep, blockIdx.x);
   restrict_tile_body<ORDER>(tab[r].in, tab[r].out, tab[r].A, blockIdx.x - first[r]);
@@ -2705,7 +2722,7 @@ cudaError_t grid_batch_levels(GridBatch* B, int d, cudaStream_t st) {
   } else {
     for (int k = 0; k + 1 < B->maxlev; ++k) {
       if (B->restr_tile[d][k].total > 0) {
-        launch_table(B->restr_tile[d][k], o3 ? kb_restrict_tile<3> : kb_restrict_tile<5>, 128, st);
+        launch_table(B->restr_tile[d][k], o3 ? kb_restrict_tile<3> : kb_restrict_tile<5>, 256, st);
         continue;
       }
       for (int ax = 0; ax < 3; ++ax)
