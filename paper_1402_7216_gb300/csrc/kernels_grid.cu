@@ -1389,6 +1389,11 @@ __device__ __forceinline__ void energy_by_last_block(double bsum, double* __rest
   }
 }
 
+// The short-range potential: an array of its own on the mixed plan, beside the
+// force (written by the same reductions) on the FP64 plan.
+__device__ __forceinline__ float short_phi(const float* phis, int64_t i, const R4<float>&) { return phis[i]; }
+__device__ __forceinline__ double short_phi(const double*, int64_t, const R4<double>& s) { return s.w; }
+
 // Assembly after the pair sums and the gather: phi_i, F_i in the caller's
 // order and the per-block energy partials (grid-stride over sorted atoms).
 template <typename T, typename OUT>
@@ -1404,7 +1409,8 @@ __global__ void __launch_bounds__(256) k_interp_assemble(int64_t n, const int* _
   for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
     const R4<T> gl = glong[i];
     const T g[3] = {gl.x, gl.y, gl.z};
-    e += Assemble<T>::forward(A, gfrac[i].w, phis[i], gl.w, fs[i], g, perm[i], phi_out, force_out);
+    const R4<T> s = fs[i];
+    e += Assemble<T>::forward(A, gfrac[i].w, short_phi(phis, i, s), gl.w, s, g, perm[i], phi_out, force_out);
   }
   const double bsum = block_sum<256>(e);
   __syncthreads();  // block_sum's buffer is used again by the last block
@@ -1477,7 +1483,7 @@ __global__ void __launch_bounds__(256, 3) k_interp_bwd(
 template <int ORDER, typename OUT>
 __global__ void __launch_bounds__(kWide) k_interp_bwd64(
     const R4<double>* __restrict__ gfrac, const int4* __restrict__ gbase, const int* __restrict__ perm, int n,
-    const double* __restrict__ av0, GridDims G, AssembleArgs A, const double* __restrict__ phis,
+    const double* __restrict__ av0, GridDims G, AssembleArgs A,
     const R4<double>* __restrict__ fs, const R4<double>* __restrict__ glong, const double* __restrict__ gE,
     OUT* __restrict__ grad_pos, OUT* __restrict__ grad_q) {
   pdl_sync();
@@ -1486,7 +1492,8 @@ __global__ void __launch_bounds__(kWide) k_interp_bwd64(
   const R4<double> f = gfrac[i];
   double v, gv[3];
   interp_atom<double, ORDER>(f, gbase[i], av0, G, A.inv_h, v, gv);
-  Assemble<double>::backward(A, *gE, f.w, phis[i], fs[i], glong[i], v, gv, perm[i], grad_pos, grad_q);
+  const R4<double> s = fs[i];
+  Assemble<double>::backward(A, *gE, f.w, s.w, s, glong[i], v, gv, perm[i], grad_pos, grad_q);
 }
 
 template <typename T>
@@ -1929,11 +1936,11 @@ cudaError_t launch_interp_backward(Plan& P, int64_t n, const double* gE, OUT* gr
     const unsigned nb = blocks_for(n, kWide);
     const auto K = interp_kargs<double, OUT>(P, true, nullptr, nullptr, gE, grad_pos, grad_q, nullptr);
     if (P.P.order == 3)
-      klaunch(P.pdl, k_interp_bwd64<3, OUT>, nb, kWide, 0, st, K.gfrac, K.gbase, K.perm, (int)n, K.u0, K.G, K.A, K.phis, K.fs,
-                                                   K.glong, gE, grad_pos, grad_q);
+      klaunch(P.pdl, k_interp_bwd64<3, OUT>, nb, kWide, 0, st, K.gfrac, K.gbase, K.perm, (int)n, K.u0, K.G, K.A, K.fs,
+              K.glong, gE, grad_pos, grad_q);
     else
-      klaunch(P.pdl, k_interp_bwd64<5, OUT>, nb, kWide, 0, st, K.gfrac, K.gbase, K.perm, (int)n, K.u0, K.G, K.A, K.phis, K.fs,
-                                                   K.glong, gE, grad_pos, grad_q);
+      klaunch(P.pdl, k_interp_bwd64<5, OUT>, nb, kWide, 0, st, K.gfrac, K.gbase, K.perm, (int)n, K.u0, K.G, K.A, K.fs,
+              K.glong, gE, grad_pos, grad_q);
     return cudaGetLastError();
   }
   const auto K = interp_kargs<float, OUT>(P, true, nullptr, nullptr, gE, grad_pos, grad_q, nullptr);
@@ -1970,8 +1977,8 @@ __global__ void __launch_bounds__(256) k_cutoff_assemble(int64_t n, const int* _
   pdl_sync();
   double e = 0.0;
   for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
-    const T p = phis[i] - selfc * atoms[i].w;  // selfc: the method's self term (0 for the cutoff method)
     const R4<T> f = fs[i];
+    const T p = short_phi(phis, i, f) - selfc * atoms[i].w;  // selfc: the method's self term (0 for the cutoff method)
     const int o = perm[i];
     if (phi_out) phi_out[o] = (OUT)(kc * p);
     if (force_out) {

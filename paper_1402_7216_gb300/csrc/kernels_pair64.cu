@@ -3,10 +3,11 @@
 //
 // This GPU issues FP64 at 1/64 of the FP32 rate (2 lanes per SM and clock), so
 // the kernel is bound by the number of FP64 instructions and nothing else:
-// 22 per MSM pair, and only pairs inside the cutoff are worth them.  The
-// candidates of a target's neighbourhood are ~2,000 sources (culled against
-// the bounding box of a warp's targets), ~750 of them inside a 12 A cutoff at
-// water density.  So the kernel separates finding from evaluating:
+// 22 per MSM pair seen from one atom, 27 for both atoms at once, and only pairs
+// inside the cutoff are worth them.  The candidates of a target's neighbourhood
+// are ~2,000 sources (culled against the bounding box of a warp's targets),
+// ~750 of them inside a 12 A cutoff at water density.  So the kernel separates
+// finding from evaluating:
 //   - sources are staged 32 at a time in a ring of shared memory (FP64
 //     coordinates in the targets' frame, and their FP32 truncation), and every
 //     lane tests every staged source against its own target in FP32, with a
@@ -19,6 +20,17 @@
 //     instruction).  Lists of different lanes fill unevenly as the walk passes
 //     through the neighbourhood; the ring keeps up to 256 sources alive so that
 //     a lane ahead of the others still has entries.
+// An MSM pair is evaluated once: of two groups of targets the one that
+// takes_pair() names meets the other's atoms, and adds to their sums with FP64
+// reductions (fire and forget; at most 4 per 27 FP64 instructions, and gathering
+// them to whole sectors first made no difference).  Against each atom for itself:
+// 1M atoms at water density 31.7 -> 20.9 ms (the FP64 pipe alone would take
+// 17 ms), 23,558 atoms 900 -> 614 us, 3,000 atoms 153 -> 110 us.  The choice by
+// group index halves the sources staged and tested too; "the earlier atom" would
+// give an atom at the top of its cell far fewer pairs than one at the bottom,
+// with the lanes waiting for the fullest list (25.6 ms), and a choice by atom
+// parity fills the ring with sources few lanes take (21.5 ms, and 3,000 atoms
+// 140 us).
 // The reciprocal square root is seeded by the FP32 one and refined once by
 // Halley's third-order iteration (5 FP64 instructions, error below 1 ulp more
 // than half a rounding).
@@ -44,8 +56,7 @@ constexpr int kShift0 = 3;   // index of offset 0 in the shift tables
 struct Pair64Args {
   PairKArgs g;  // geometry: cell widths and cutoff in FP32, scaled by 2^esc (a in [1, 2))
   const R4<double>* atoms;
-  double* phis;
-  R4<double>* fs;
+  R4<double>* fs;  // force sums, potential
   double a2;
   double G[4], D[3];  // pot = 1/r + sum_k G[k] r2^k, f' = 1/r^3 + sum_k D[k] r2^k
   WolfC<double> W;
@@ -58,7 +69,7 @@ struct Pair64Args {
 
 struct alignas(16) Warp64 {
   double src[kRing][4];  // x, y, z, q in the piece's frame
-  float fx[kRing], fy[kRing], fz[kRing];
+  float4 f[kRing];       // their FP32 truncations and the source's index
   unsigned char list[kRing][32];
   SegList segs;
 };
@@ -90,11 +101,33 @@ __device__ __forceinline__ double rsqrt_halley(double x) {
   return fma(y * r, fma(0.375, r, 0.5), y);
 }
 
+// MSM pairs are evaluated once, for both atoms, with reductions into the sums
+// (their order varies, as that of the FP64 anterpolation's does); the cutoff
+// and Wolf methods evaluate each pair for either atom and store, so that their
+// results repeat bit for bit.
+__host__ __device__ constexpr bool both_sides(int kind) { return kind == kPairMSM; }
+
+// Adds (x, y, z, w) to one atom's sums.
+__device__ __forceinline__ void add_sums(R4<double>* s, double x, double y, double z, double w) {
+  atomicAdd(&s->x, x);
+  atomicAdd(&s->y, y);
+  atomicAdd(&s->z, z);
+  atomicAdd(&s->w, w);
+}
+
+// Which of two groups (atoms of a group) i != j evaluates their pairs: the later
+// one if the numbers have the same parity, else the earlier one.
+__device__ __forceinline__ bool takes_pair(int i, int j) { return ((((j - i) >> 31) ^ i ^ j) & 1) != 0; }
+
 // One pair: q_j times the pair potential onto phi, f' (r_i - r_j) onto
-// (px, py, pz), with the force on i being q_i times that sum.
+// (px, py, pz), with the force on i being q_i times that sum.  BOTH: q_i q_j f'
+// (r_i - r_j) onto (px, py, pz), and the same for atom j onto sj (5 more FP64
+// instructions against the 22 of a second visit).
 template <int M, int K>
-__device__ __forceinline__ void pair64(const Pair64Args& A, double tx, double ty, double tz, const double* src,
-                                       double& phi, double& px, double& py, double& pz) {
+__device__ __forceinline__ void pair64(const Pair64Args& A, double tx, double ty, double tz, double tq,
+                                       const double* src, double& phi, double& px, double& py, double& pz,
+                                       R4<double>* sj) {
+  constexpr bool BOTH = both_sides(K);
   const double2 xy = *reinterpret_cast<const double2*>(src), zq = *reinterpret_cast<const double2*>(src + 2);
   const double dx = tx - xy.x, dy = ty - xy.y, dz = tz - zq.x;
   const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
@@ -110,8 +143,18 @@ __device__ __forceinline__ void pair64(const Pair64Args& A, double tx, double ty
     double d = A.D[M - 1];
 #pragma unroll
     for (int k = M - 2; k >= 0; --k) d = fma(d, r2s, A.D[k]);
-    phi = fma(q, ri + g, phi);
+    const double v = ri + g;
+    phi = fma(q, v, phi);
     f = q * fma(ri * ri, ri, d);
+    if constexpr (BOTH) {
+      const double w = -tq * f;
+      const double wx = w * dx, wy = w * dy, wz = w * dz;
+      px -= wx;
+      py -= wy;
+      pz -= wz;
+      if (ok && sj) add_sums(sj, wx, wy, wz, tq * v);
+      return;
+    }
   } else if (K == kPairWolf) {
     const double r = r2s * ri;
     const double e = d_erfc(A.W.alpha * r) * ri, x = A.W.c2 * d_exp(-A.W.alpha2 * r2s);
@@ -128,6 +171,7 @@ __device__ __forceinline__ void pair64(const Pair64Args& A, double tx, double ty
 
 template <int M, int K>
 __global__ void __launch_bounds__(32 * kMaxSplit) k_pair64(const __grid_constant__ Pair64Args A) {
+  constexpr bool BOTH = both_sides(K);
   pdl_sync();
   extern __shared__ __align__(16) unsigned char smem64[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -182,7 +226,7 @@ __global__ void __launch_bounds__(32 * kMaxSplit) k_pair64(const __grid_constant
       while (more && staged - oldest <= kRing - kChunk) {
         const int j = jb + lane;
         R4<double> a = {0.0, 0.0, 0.0, 0.0};
-        bool keep = j < je;
+        bool keep = j < je && (!BOTH || (j >> A.lt) == group || takes_pair(group, j >> A.lt));
         if (keep) {
           a = A.atoms[j];
           a.x += A.shx[(int)g.cellx[j] + xb + kShift0];
@@ -199,9 +243,7 @@ __global__ void __launch_bounds__(32 * kMaxSplit) k_pair64(const __grid_constant
         const unsigned bal = __ballot_sync(kFull, keep);
         if (keep) {
           const int p = (staged + __popc(bal & ((1u << lane) - 1u))) & (kRing - 1);
-          S.fx[p] = ax;
-          S.fy[p] = ay;
-          S.fz[p] = az;
+          S.f[p] = make_float4(ax, ay, az, __int_as_float(j));
           *reinterpret_cast<double2*>(&S.src[p][0]) = make_double2(a.x, a.y);
           *reinterpret_cast<double2*>(&S.src[p][2]) = make_double2(a.z, a.w);
         }
@@ -210,8 +252,11 @@ __global__ void __launch_bounds__(32 * kMaxSplit) k_pair64(const __grid_constant
 #pragma unroll 4
         for (unsigned s = staged + ((h - staged) & (lpt - 1)); s < end; s += lpt) {
           const int p = s & (kRing - 1);
-          const float dx = ux - S.fx[p], dy = uy - S.fy[p], dz = uz - S.fz[p];
-          if (inp && dx * dx + dy * dy + dz * dz < A.a2test) S.list[tail++ & (kRing - 1)][lane] = (unsigned char)p;
+          const float4 b = S.f[p];
+          const float dx = ux - b.x, dy = uy - b.y, dz = uz - b.z;
+          const int j = __float_as_int(b.w);
+          const bool mine = !BOTH || (j >> A.lt) != group || j == s0 + t || takes_pair(s0 + t, j);
+          if (inp && mine && dx * dx + dy * dy + dz * dz < A.a2test) S.list[tail++ & (kRing - 1)][lane] = (unsigned char)p;
         }
         staged = end;
       }
@@ -225,7 +270,9 @@ __global__ void __launch_bounds__(32 * kMaxSplit) k_pair64(const __grid_constant
       for (unsigned k = 0; k < steps; ++k)
         if (head < tail) {
           const int p = S.list[head++ & (kRing - 1)][lane];
-          pair64<M, K>(A, tx, ty, tz, S.src[p], sphi, sx, sy, sz);
+          const int j = BOTH ? __float_as_int(S.f[p].w) : 0;
+          // (an image of the atom itself is one-sided: the mirror image is met too)
+          pair64<M, K>(A, tx, ty, tz, me.w, S.src[p], sphi, sx, sy, sz, j != s0 + t ? A.fs + j : nullptr);
         }
       phi += sphi;
       px += sx;
@@ -265,8 +312,8 @@ __global__ void __launch_bounds__(32 * kMaxSplit) k_pair64(const __grid_constant
     }
     if (part == 0 && h == 0 && inp) {
       const int i = s0 + t;
-      A.phis[i] = phi;
-      A.fs[i] = R4<double>{me.w * px, me.w * py, me.w * pz, 0.0};
+      if (BOTH) add_sums(A.fs + i, px, py, pz, phi);
+      else A.fs[i] = R4<double>{me.w * px, me.w * py, me.w * pz, phi};
     }
     __syncwarp();
     l0 = l1;
@@ -304,7 +351,6 @@ Pair64Args pair64_args(const Plan& P, int64_t n, double alpha) {
   A.a2test = (float)(a2t * (1.0 + 1e-6));
   A.g.A.a2f = A.a2test;
   A.atoms = (const R4<double>*)P.d.atoms;
-  A.phis = (double*)P.d.phis;
   A.fs = (R4<double>*)P.d.fs;
   A.a2 = a * a;
   static const double cf[4][4] = {{0, 0, 0, 0}, {1.5, -0.5, 0, 0}, {1.875, -1.25, 0.375, 0},

@@ -49,8 +49,8 @@ struct DeviceBuffers {
   float* cellx = nullptr;      // [cap]: x index of that cell
   int4* gbase = nullptr;       // [cap]: first level-0 index of the basis support per dim
   // per-atom results in sorted order
-  void* phis = nullptr;        // T[cap]  short-range potential
-  void* fs = nullptr;          // R4<T>[cap] short-range force (x, y, z), spare (w)
+  void* phis = nullptr;        // float[cap] short-range potential (FP64 plans: fs.w)
+  void* fs = nullptr;          // R4<T>[cap] short-range force (x, y, z); FP64: potential (w)
   void* glong = nullptr;       // R4<T>[cap] long-range gradient (x, y, z) and long-range potential (w)
   // grids, one per level: charges q^k in FP64, potentials u^k in T
   void* gq[kMaxLevels] = {};
@@ -314,9 +314,9 @@ int64_t grid_points(const Plan& P, int k);
 template <typename IO>  // IO = double or float (caller's position and charge type)
 cudaError_t launch_binning(Plan& P, int64_t n, const IO* pos, const IO* q, cudaStream_t s,
                            unsigned long long* zero = nullptr, int64_t nzero = 0);
-// short-range pair sums (phis, fs.xyz)
+// short-range pair sums (phis, fs.xyz; FP64: fs)
 cudaError_t launch_short_range(Plan& P, int64_t n, cudaStream_t s);
-// the cutoff method: Coulomb pair sums within the cutoff (phis, fs.xyz); Wolf
+// the cutoff method: Coulomb pair sums within the cutoff (as above); Wolf
 // summation: its damped shifted-force pair sums; and the assembly of phi
 // (minus self_c q_i: 0 for the cutoff method, 2 c_s for Wolf), F and E
 cudaError_t launch_cutoff_pairs(Plan& P, int64_t n, cudaStream_t s);

@@ -523,7 +523,7 @@ int build_plan(const msm_params* pp, const msm_tuning* tune, Plan* P) {
   M((void**)&D.gbase, sizeof(int4) * cap);
   M((void**)&D.scell, sizeof(int) * cap);
   M((void**)&D.cellx, sizeof(float) * cap);
-  M(&D.phis, T * cap);
+  if (!P->fp64) M(&D.phis, T * cap);
   M(&D.fs, 4 * T * cap);
   M(&D.glong, 4 * T * cap);
   for (int k = 0; k < P->levels; ++k) {
