@@ -35,7 +35,7 @@
 // Halley's third-order iteration (5 FP64 instructions, error below 1 ulp more
 // than half a rounding).
 //
-// A group of T = 8, 16 or 32 consecutive sorted atoms is a warp's targets,
+// A group of T = 8 or 16 consecutive sorted atoms is a warp's targets,
 // 32 / T lanes sharing one (each tests every (32 / T)-th source); small systems
 // also split a group's sources over 2 to 8 warps of a block, combined in a
 // fixed order.  Groups are cut into pieces of one cell row as the target runs
@@ -320,14 +320,19 @@ __global__ void __launch_bounds__(32 * kMaxSplit) k_pair64(const __grid_constant
   }
 }
 
-// Targets per group and warps per group: full warps of targets once their
-// number fills the GPU (152 SMs x 8 warps), else smaller groups, then several
-// warps per group.
+// Targets per group and warps per group: groups of 16 once they make 152 SMs x
+// 8 warps, else groups of 8, then several warps per group.  Groups of 32 are
+// the same at 1M atoms (20.9 against 20.8 ms) and leave the chip waiting for
+// its last warps below (200,000 atoms 4.46 against 4.24 ms, 100,000 2,419
+// against 2,185 us, 50,000 1,429 against 1,178); groups of 8 stage each source
+// for fewer targets (1M 22.1 ms; at 23,558 566 against 611 us alone, but 663
+// against 653 us an evaluation with gradients).  Warps per group at 3,000
+// atoms: 214, 126, 108 and 114 us with 1, 2, 4 and 8; at 6,000 241, 180, 190
+// and 219.
 void group_shape(int64_t n, int& lt, int& nsplit) {
   constexpr int64_t kFill = 152 * 8;
-  lt = 5;
+  lt = (n + 15) >> 4 >= kFill ? 4 : 3;
   nsplit = 1;
-  while (lt > 3 && ((n + (1 << lt) - 1) >> lt) < kFill) --lt;
   while (nsplit < kMaxSplit && ((n + (1 << lt) - 1) >> lt) * nsplit < kFill * 3 / 4) nsplit *= 2;
 }
 

@@ -39,3 +39,22 @@ def test_pairs_once_for_both_atoms(n, periodic):
         assert abs(E.item() - ref["E"]) <= TOL * 0.5 * np.abs(q[:m] * ref["phi"]).sum() + 1e-300
         assert_atoms(F.cpu().numpy(), ref["F"], TOL)
         assert_atoms(phi.cpu().numpy(), ref["phi"], TOL)
+
+
+@pytest.mark.parametrize("n", [19440, 19441, 65536])
+def test_groups_of_8_and_16(n):
+    """Both sides of the change of targets per group, and a size well above."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1402_7216_gb300 import MSM
+    dev = torch.device("cuda:0")
+    box = np.array([88.0, 86.0, 90.0]) * (n / 65536) ** (1 / 3)
+    rng = np.random.default_rng(n)
+    pos, q = rng.uniform(0.0, 1.0, (n, 3)) * box, rng.uniform(-1.0, 1.0, n)
+    par = dict(box=tuple(box), periodic=True, cutoff=8.0, spacing=3.0, order=3)
+    E, phi, F = MSM(splitting=2, precision="fp64", max_atoms=n, **par).eval(torch.tensor(pos, device=dev),
+                                                                            torch.tensor(q, device=dev))
+    ref = O.msm(O.Params(split=2, **par), pos, q)
+    assert abs(E.item() - ref["E"]) <= TOL * 0.5 * np.abs(q * ref["phi"]).sum()
+    assert_atoms(F.cpu().numpy(), ref["F"], TOL)
+    assert_atoms(phi.cpu().numpy(), ref["phi"], TOL)
