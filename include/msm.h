@@ -83,7 +83,7 @@ typedef struct {
  *   patch_cells   short-range cells per side of the shared-memory patch blocks
  *                 of anterpolation and interpolation (default: 4, lowered to
  *                 3 or 2 on a mixed-precision plan evaluated alone while fewer
- *                 than 152 patch blocks cover its box, and lower still where
+ *                 than 120 patch blocks cover its box, and lower still where
  *                 the patch would not fit shared memory; batched launches
  *                 keep the largest patch that fits)
  *   lattice_waves blocks per SM the lattice cutoff aims for when it splits the
@@ -97,7 +97,7 @@ typedef struct {
  *                 warp takes 32 consecutive atoms of the sorted order as its
  *                 targets (runs across the cells of a row, which binning
  *                 sorts by x), 2 a warp takes one cell's atoms; 0 the
- *                 default, 1 on plans of at least 16,384 cells and 2 below.
+ *                 default, 1 on plans of at least 12,288 cells and 2 below.
  *                 Runs need at least seven cells along x on a periodic plan
  *                 and fall back to cells otherwise
  *   lattice_txn, lattice_tyn  warp tile of the mixed-precision lattice

@@ -1,5 +1,6 @@
 // kernels_pair.cu -- short-range part of MSM on mixed plans (FP64 plans:
-// kernels_pair64.cu) (Sec. "Multilevel Summation Method"): u_i^short = sum_{j != i, r_ij < a} q_j g*(r_ij) with
+// kernels_pair64.cu; Sec. "Multilevel Summation Method"):
+// u_i^short = sum_{j != i, r_ij < a} q_j g*(r_ij) with
 // g*(r) = 1/r - gamma(r/a)/a (Eq. msmgrid), and the force
 // F_i = -q_i grad_i u_i^short.
 //
