@@ -236,6 +236,18 @@ struct Totals {
     two_sum_add(y, cy, sy.x + sy.y);
     two_sum_add(z, cz, sz.x + sz.y);
   }
+  // another warp's totals, laid down in its queue: x, y, z and q hold phi and
+  // the force sums at [lane] and their compensation terms at [32 + lane]
+  __device__ __forceinline__ void join(const QueueF& O, int lane) {
+    two_sum_add(phi, cphi, O.x[lane]);
+    two_sum_add(x, cx, O.y[lane]);
+    two_sum_add(y, cy, O.z[lane]);
+    two_sum_add(z, cz, O.q[lane]);
+    cphi += O.x[32 + lane];
+    cx += O.y[32 + lane];
+    cy += O.z[32 + lane];
+    cz += O.q[32 + lane];
+  }
 };
 
 // n sources (a multiple of NB), folded into the totals once
@@ -617,7 +629,9 @@ __device__ __forceinline__ void short_range_c8_body(const PairKArgs& K, int blk)
 // per target (0.63 ms by itself) is hidden only in part.
 //
 // The warps of a block may share one group (K.split of them): warp p takes
-// every split-th 64 sources, and the partial sums are added in warp order.
+// every split-th 64 sources, and the warps' totals are joined in warp order
+// with their compensation terms (one FP32 number per warp would round off what
+// the warps' totals cancel to).
 // (The barrier is the block's: named barriers by a computed number reserve
 // all 16 of a block and halve the resident blocks, 1.63 -> 1.85 ms.)
 //
@@ -823,23 +837,20 @@ __device__ __forceinline__ void short_range_body(const PairKArgs& K, int blk) {
       pair_batch<M, KIND, 16, false>(Q, head, n16, nax, nay, naz, a2, C, W, tot);
       __syncwarp();
     }
-    float phi = tot.phi + tot.cphi, px = tot.x + tot.cx, py = tot.y + tot.cy, pz = tot.z + tot.cz;
-    if (split > 1) {  // the warps of the group
-      Q.x[lane] = phi;
-      Q.y[lane] = px;
-      Q.z[lane] = py;
-      Q.q[lane] = pz;
+    if (split > 1) {  // the warps' totals, each with its compensation term, joined in warp order
+      float* mine[4] = {Q.x, Q.y, Q.z, Q.q};
+      const float total[4] = {tot.phi, tot.x, tot.y, tot.z}, comp[4] = {tot.cphi, tot.cx, tot.cy, tot.cz};
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        mine[c][lane] = total[c];
+        mine[c][32 + lane] = comp[c];
+      }
       __syncthreads();
       if (part == 0)
-        for (int p = 1; p < split; ++p) {
-          const QueueF& O = shared[p].queue;
-          phi += O.x[lane];
-          px += O.y[lane];
-          py += O.z[lane];
-          pz += O.q[lane];
-        }
+        for (int p = 1; p < split; ++p) tot.join(shared[p].queue, lane);
       __syncthreads();
     }
+    const float phi = tot.phi + tot.cphi, px = tot.x + tot.cx, py = tot.y + tot.cy, pz = tot.z + tot.cz;
     if (part == 0 && inp) {
       const int i = (K.runs ? i0 : ib) + lane;
       K.phis[i] = phi;
