@@ -72,7 +72,7 @@ struct BinArgs {
   int fmax[3];  // open grids: largest floor(x/h) the level-0 grid covers
   int periodic;
   int S;
-  R4<double>* sums;  // FP64 plan: the atoms' pair sums, set to 0 with their records
+  R4<double>* react;  // FP64 plan, MSM force: the atoms' reaction sums (two each), set to 0 with their records
 };
 
 // Splits a finite y >= 0 into hi + lo with integer operations only: hi keeps
@@ -414,7 +414,7 @@ __device__ __forceinline__ void write_records(const IO* __restrict__ pos, const 
     const double qi = finite_bits(q[i]) ? (double)q[i] : 0.0;
     reinterpret_cast<R4<double>*>(atoms_v)[s] = R4<double>{loc[0], loc[1], loc[2], qi};
     reinterpret_cast<R4<double>*>(gfrac_v)[s] = R4<double>{fr[0], fr[1], fr[2], qi};
-    A.sums[s] = R4<double>{0.0, 0.0, 0.0, 0.0};
+    if (A.react) A.react[2 * (int64_t)s] = A.react[2 * (int64_t)s + 1] = R4<double>{0.0, 0.0, 0.0, 0.0};
   } else {
     float loc[3], fr[3];
     for (int d = 0; d < 3; ++d) {
@@ -480,7 +480,8 @@ __device__ __forceinline__ void store_record(const CellRec<FP64>& R, const BinAr
   using T = typename CellRec<FP64>::T;
   reinterpret_cast<R4<T>*>(atoms_v)[s] = R4<T>{R.loc[0], R.loc[1], R.loc[2], R.q};
   reinterpret_cast<R4<T>*>(gfrac_v)[s] = R4<T>{R.fr[0], R.fr[1], R.fr[2], R.q};
-  if constexpr (FP64) A.sums[s] = R4<double>{0.0, 0.0, 0.0, 0.0};
+  if constexpr (FP64)
+    if (A.react) A.react[2 * (int64_t)s] = A.react[2 * (int64_t)s + 1] = R4<double>{0.0, 0.0, 0.0, 0.0};
   gbase[s] = make_int4(R.bs[0] - (A.S - 1), R.bs[1] - (A.S - 1), R.bs[2] - (A.S - 1), 0);
   scell[s] = key;
   cellx[s] = (float)(key % A.nc[0]);
@@ -615,7 +616,7 @@ BinArgs bin_args(const Plan& P) {
   }
   A.periodic = P.P.periodic;
   A.S = P.S;
-  A.sums = P.fp64 ? (R4<double>*)P.d.fs : nullptr;
+  A.react = nullptr;
   return A;
 }
 
@@ -626,7 +627,8 @@ cudaError_t launch_binning(Plan& P, int64_t n64, const IO* pos, const IO* q, cud
                            unsigned long long* zero, int64_t nzero) {
   const int n = (int)n64;
   DeviceBuffers& D = P.d;
-  const BinArgs A = bin_args(P);
+  BinArgs A = bin_args(P);
+  if (P.fp64 && zero) A.react = (R4<double>*)D.react;
   const unsigned nb = (unsigned)((n + 255) / 256);
   const unsigned nsc = (unsigned)((P.ncell + kScanChunk - 1) / kScanChunk);
   if (n > 0) {

@@ -1389,8 +1389,16 @@ __device__ __forceinline__ void energy_by_last_block(double bsum, double* __rest
   }
 }
 
+// An atom's short-range sums: on the FP64 plan its own and the two of the pairs
+// that other atoms evaluated.
+__device__ __forceinline__ R4<float> short_sums(const R4<float>* fs, const R4<double>*, int64_t i) { return fs[i]; }
+__device__ __forceinline__ R4<double> short_sums(const R4<double>* fs, const R4<double>* react, int64_t i) {
+  const R4<double> a = fs[i], n = react[2 * i], f = react[2 * i + 1];
+  return R4<double>{a.x + (n.x + f.x), a.y + (n.y + f.y), a.z + (n.z + f.z), a.w + (n.w + f.w)};
+}
+
 // The short-range potential: an array of its own on the mixed plan, beside the
-// force (written by the same reductions) on the FP64 plan.
+// force on the FP64 plan.
 __device__ __forceinline__ float short_phi(const float* phis, int64_t i, const R4<float>&) { return phis[i]; }
 __device__ __forceinline__ double short_phi(const double*, int64_t, const R4<double>& s) { return s.w; }
 
@@ -1400,6 +1408,7 @@ template <typename T, typename OUT>
 __global__ void __launch_bounds__(256) k_interp_assemble(int64_t n, const int* __restrict__ perm,
                                                          const R4<T>* __restrict__ gfrac, const T* __restrict__ phis,
                                                          const R4<T>* __restrict__ fs,
+                                                         const R4<double>* __restrict__ react,
                                                          const R4<T>* __restrict__ glong, AssembleArgs A,
                                                          OUT* __restrict__ phi_out, OUT* __restrict__ force_out,
                                                          double* __restrict__ partial, int* ticket,
@@ -1409,7 +1418,7 @@ __global__ void __launch_bounds__(256) k_interp_assemble(int64_t n, const int* _
   for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256) {
     const R4<T> gl = glong[i];
     const T g[3] = {gl.x, gl.y, gl.z};
-    const R4<T> s = fs[i];
+    const R4<T> s = short_sums(fs, react, i);
     e += Assemble<T>::forward(A, gfrac[i].w, short_phi(phis, i, s), gl.w, s, g, perm[i], phi_out, force_out);
   }
   const double bsum = block_sum<256>(e);
@@ -1484,15 +1493,15 @@ template <int ORDER, typename OUT>
 __global__ void __launch_bounds__(kWide) k_interp_bwd64(
     const R4<double>* __restrict__ gfrac, const int4* __restrict__ gbase, const int* __restrict__ perm, int n,
     const double* __restrict__ av0, GridDims G, AssembleArgs A,
-    const R4<double>* __restrict__ fs, const R4<double>* __restrict__ glong, const double* __restrict__ gE,
-    OUT* __restrict__ grad_pos, OUT* __restrict__ grad_q) {
+    const R4<double>* __restrict__ fs, const R4<double>* __restrict__ react, const R4<double>* __restrict__ glong,
+    const double* __restrict__ gE, OUT* __restrict__ grad_pos, OUT* __restrict__ grad_q) {
   pdl_sync();
   const int i = blockIdx.x * kWide + threadIdx.x;
   if (i >= n) return;
   const R4<double> f = gfrac[i];
   double v, gv[3];
   interp_atom<double, ORDER>(f, gbase[i], av0, G, A.inv_h, v, gv);
-  const R4<double> s = fs[i];
+  const R4<double> s = short_sums(fs, react, i);
   Assemble<double>::backward(A, *gE, f.w, s.w, s, glong[i], v, gv, perm[i], grad_pos, grad_q);
 }
 
@@ -1911,11 +1920,12 @@ cudaError_t launch_interp_assemble(Plan& P, int64_t n, double* energy, OUT* phi,
     if (P.fp64)
       klaunch(false, k_interp_assemble<double, OUT>, nb, 256, 0, st, n, P.d.perm, (const R4<double>*)P.d.gfrac,
                                                         (const double*)P.d.phis, (const R4<double>*)P.d.fs,
+                                                        (const R4<double>*)P.d.react,
                                                         (const R4<double>*)P.d.glong, A, phi, force, P.d.partial,
                                                         P.d.ticket, energy);
     else
       klaunch(false, k_interp_assemble<float, OUT>, nb, 256, 0, st, n, P.d.perm, (const R4<float>*)P.d.gfrac,
-                                                       (const float*)P.d.phis, (const R4<float>*)P.d.fs,
+                                                       (const float*)P.d.phis, (const R4<float>*)P.d.fs, nullptr,
                                                        (const R4<float>*)P.d.glong, A, phi, force, P.d.partial,
                                                         P.d.ticket, energy);
   }
@@ -1937,10 +1947,10 @@ cudaError_t launch_interp_backward(Plan& P, int64_t n, const double* gE, OUT* gr
     const auto K = interp_kargs<double, OUT>(P, true, nullptr, nullptr, gE, grad_pos, grad_q, nullptr);
     if (P.P.order == 3)
       klaunch(P.pdl, k_interp_bwd64<3, OUT>, nb, kWide, 0, st, K.gfrac, K.gbase, K.perm, (int)n, K.u0, K.G, K.A, K.fs,
-              K.glong, gE, grad_pos, grad_q);
+              (const R4<double>*)P.d.react, K.glong, gE, grad_pos, grad_q);
     else
       klaunch(P.pdl, k_interp_bwd64<5, OUT>, nb, kWide, 0, st, K.gfrac, K.gbase, K.perm, (int)n, K.u0, K.G, K.A, K.fs,
-              K.glong, gE, grad_pos, grad_q);
+              (const R4<double>*)P.d.react, K.glong, gE, grad_pos, grad_q);
     return cudaGetLastError();
   }
   const auto K = interp_kargs<float, OUT>(P, true, nullptr, nullptr, gE, grad_pos, grad_q, nullptr);

@@ -21,9 +21,13 @@
 //     through the neighbourhood; the ring keeps up to 256 sources alive so that
 //     a lane ahead of the others still has entries.
 // An MSM pair is evaluated once: of two groups of targets the one that
-// takes_pair() names meets the other's atoms, and adds to their sums with FP64
-// reductions (fire and forget; at most 4 per 27 FP64 instructions, and gathering
-// them to whole sectors first made no difference).  Against each atom for itself:
+// takes_pair() names meets the other's atoms, and adds to their reaction sums
+// with FP64 reductions (fire and forget; at most 4 per 27 FP64 instructions, and
+// gathering them to whole sectors first made no difference).  An atom has two
+// reaction sums, for pairs nearer and farther than kNear a: the many small terms
+// of the far pairs would else round onto the few large ones (force error of
+// 3,000 atoms 4.3e-16 with every pair from both atoms, 6.8e-16 with one sum that
+// also took the atom's own total, 4.4e-16 with the two, at the same speed).  Against each atom for itself:
 // 1M atoms at water density 31.7 -> 20.9 ms (the FP64 pipe alone would take
 // 17 ms), 23,558 atoms 900 -> 614 us, 3,000 atoms 153 -> 110 us.  The choice by
 // group index halves the sources staged and tested too; "the earlier atom" would
@@ -41,6 +45,7 @@
 // fixed order.  Groups are cut into pieces of one cell row as the target runs
 // of kernels_pair.cu are.
 #include <algorithm>
+#include <cstring>
 
 #include "pair_common.h"
 
@@ -52,15 +57,22 @@ constexpr int kRing = 256;   // staged sources (a list entry is one byte)
 constexpr int kChunk = 32;   // sources staged together
 constexpr int kMaxSplit = 8; // warps sharing a group
 constexpr int kShift0 = 3;   // index of offset 0 in the shift tables
+// Near pairs: r^2 <= kNear2 a^2.  In a CPU model of the sums' order (water, a
+// gas and like charges, 420 to 750 pairs an atom) the rounding error of force
+// and potential is 0.4 to 1.0 of that of every pair from both atoms for 0.14 to
+// 0.22, up to 1.6 below 0.05 and 1.2 at 0.36; one reaction sum has 1.5 to 2.0.
+constexpr double kNear2 = 0.1875;
 
 struct Pair64Args {
   PairKArgs g;  // geometry: cell widths and cutoff in FP32, scaled by 2^esc (a in [1, 2))
   const R4<double>* atoms;
-  R4<double>* fs;  // force sums, potential
+  R4<double>* fs;     // force sums, potential of the pairs an atom's own group evaluates
+  R4<double>* react;  // [2 i], [2 i + 1]: the same from the other pairs, near and far (both_sides)
   double a2;
   double G[4], D[3];  // pot = 1/r + sum_k G[k] r2^k, f' = 1/r^3 + sum_k D[k] r2^k
   WolfC<double> W;
   double shx[8], shy[8], shz[8];  // offset (index - kShift0) times the cell width
+  int near_hi;                    // high word of the near pairs' largest r^2
   float a2test;                   // scaled cutoff^2 with the margin of the FP32 test
   int esc;                        // exponent added to coordinates before the FP32 test
   int lt;                         // log2 of the targets per group
@@ -121,8 +133,8 @@ __device__ __forceinline__ bool takes_pair(int i, int j) { return ((((j - i) >> 
 
 // One pair: q_j times the pair potential onto phi, f' (r_i - r_j) onto
 // (px, py, pz), with the force on i being q_i times that sum.  BOTH: q_i q_j f'
-// (r_i - r_j) onto (px, py, pz), and the same for atom j onto sj (5 more FP64
-// instructions against the 22 of a second visit).
+// (r_i - r_j) onto (px, py, pz), and the same for atom j onto its reaction sums
+// sj (5 more FP64 instructions against the 22 of a second visit).
 template <int M, int K>
 __device__ __forceinline__ void pair64(const Pair64Args& A, double tx, double ty, double tz, double tq,
                                        const double* src, double& phi, double& px, double& py, double& pz,
@@ -152,7 +164,7 @@ __device__ __forceinline__ void pair64(const Pair64Args& A, double tx, double ty
       px -= wx;
       py -= wy;
       pz -= wz;
-      if (ok && sj) add_sums(sj, wx, wy, wz, tq * v);
+      if (ok && sj) add_sums(sj + (__double2hiint(r2) > A.near_hi), wx, wy, wz, tq * v);
       return;
     }
   } else if (K == kPairWolf) {
@@ -272,7 +284,7 @@ __global__ void __launch_bounds__(32 * kMaxSplit) k_pair64(const __grid_constant
           const int p = S.list[head++ & (kRing - 1)][lane];
           const int j = BOTH ? __float_as_int(S.f[p].w) : 0;
           // (an image of the atom itself is one-sided: the mirror image is met too)
-          pair64<M, K>(A, tx, ty, tz, me.w, S.src[p], sphi, sx, sy, sz, j != s0 + t ? A.fs + j : nullptr);
+          pair64<M, K>(A, tx, ty, tz, me.w, S.src[p], sphi, sx, sy, sz, j != s0 + t ? A.react + 2 * (int64_t)j : nullptr);
         }
       phi += sphi;
       px += sx;
@@ -312,8 +324,7 @@ __global__ void __launch_bounds__(32 * kMaxSplit) k_pair64(const __grid_constant
     }
     if (part == 0 && h == 0 && inp) {
       const int i = s0 + t;
-      if (BOTH) add_sums(A.fs + i, px, py, pz, phi);
-      else A.fs[i] = R4<double>{me.w * px, me.w * py, me.w * pz, phi};
+      A.fs[i] = BOTH ? R4<double>{px, py, pz, phi} : R4<double>{me.w * px, me.w * py, me.w * pz, phi};
     }
     __syncwarp();
     l0 = l1;
@@ -357,7 +368,12 @@ Pair64Args pair64_args(const Plan& P, int64_t n, double alpha) {
   A.g.A.a2f = A.a2test;
   A.atoms = (const R4<double>*)P.d.atoms;
   A.fs = (R4<double>*)P.d.fs;
+  A.react = (R4<double>*)P.d.react;
   A.a2 = a * a;
+  const double near2 = kNear2 * A.a2;
+  uint64_t near_bits;
+  std::memcpy(&near_bits, &near2, sizeof near_bits);
+  A.near_hi = (int)(near_bits >> 32);
   static const double cf[4][4] = {{0, 0, 0, 0}, {1.5, -0.5, 0, 0}, {1.875, -1.25, 0.375, 0},
                                   {2.1875, -2.1875, 1.3125, -0.3125}};
   const int m = P.P.splitting;

@@ -49,8 +49,9 @@ struct DeviceBuffers {
   float* cellx = nullptr;      // [cap]: x index of that cell
   int4* gbase = nullptr;       // [cap]: first level-0 index of the basis support per dim
   // per-atom results in sorted order
-  void* phis = nullptr;        // float[cap] short-range potential (FP64 plans: fs.w)
+  void* phis = nullptr;        // float[cap] short-range potential (FP64 plans: fs.w, react.w)
   void* fs = nullptr;          // R4<T>[cap] short-range force (x, y, z); FP64: potential (w)
+  void* react = nullptr;       // FP64: R4<double>[2 cap] MSM pair sums from the other atom of a pair, near and far
   void* glong = nullptr;       // R4<T>[cap] long-range gradient (x, y, z) and long-range potential (w)
   // grids, one per level: charges q^k in FP64, potentials u^k in T
   void* gq[kMaxLevels] = {};
@@ -309,12 +310,12 @@ int64_t grid_points(const Plan& P, int k);
 
 // ---- launchers (.cu files); all asynchronous on stream ----
 // binning: keys, stable radix sort by cell, cell_start, gather of sorted atoms
-// and, on the way, nzero 8-byte words at zero set to 0 (the charge grid the
-// anterpolation adds into)
+// and, for the MSM force, nzero 8-byte words at zero set to 0 (the charge grid
+// the anterpolation adds into) and the FP64 plan's reaction sums (react)
 template <typename IO>  // IO = double or float (caller's position and charge type)
 cudaError_t launch_binning(Plan& P, int64_t n, const IO* pos, const IO* q, cudaStream_t s,
                            unsigned long long* zero = nullptr, int64_t nzero = 0);
-// short-range pair sums (phis, fs.xyz; FP64: fs)
+// short-range pair sums (phis, fs.xyz; FP64: fs, and react with MSM)
 cudaError_t launch_short_range(Plan& P, int64_t n, cudaStream_t s);
 // the cutoff method: Coulomb pair sums within the cutoff (as above); Wolf
 // summation: its damped shifted-force pair sums; and the assembly of phi

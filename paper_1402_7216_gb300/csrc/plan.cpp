@@ -525,6 +525,7 @@ int build_plan(const msm_params* pp, const msm_tuning* tune, Plan* P) {
   M((void**)&D.cellx, sizeof(float) * cap);
   if (!P->fp64) M(&D.phis, T * cap);
   M(&D.fs, 4 * T * cap);
+  if (P->fp64) M(&D.react, 8 * T * cap);
   M(&D.glong, 4 * T * cap);
   for (int k = 0; k < P->levels; ++k) {
     size_t np = (size_t)grid_points(*P, k);
@@ -620,7 +621,7 @@ int build_plan(const msm_params* pp, const msm_tuning* tune, Plan* P) {
 void free_plan(Plan* P) {
   DeviceBuffers& D = P->d;
   void* ptrs[] = {D.key, D.rank, D.perm, D.count, D.csum, D.cell_start, D.atoms,
-                  D.gfrac, D.gbase, D.scell, D.cellx, D.phis, D.fs, D.glong, D.topK, D.topq, D.topu, D.seg, D.seg2, D.cell_rows,
+                  D.gfrac, D.gbase, D.scell, D.cellx, D.phis, D.fs, D.react, D.glong, D.topK, D.topq, D.topu, D.seg, D.seg2, D.cell_rows,
                   D.seg_start, D.lrows, D.partial, D.scalars, D.md_partial, D.md_step, D.status, D.ticket, D.hpos, D.hq,
                   D.hphi, D.hforce, D.henergy, D.lparts, D.fft_work};
   for (void* p : ptrs)

@@ -43,3 +43,35 @@ def test_warps_join_their_totals_without_rounding(step, x, runs, dev):
     plan.check_status()
     assert abs(phi[n].item() * 2.0 / (2 * small) - 1) <= 1e-6
     assert abs(F[n, 0].item() * 4.0 / (2 * small) - 1) <= 2e-6
+
+
+# FP64 plans evaluate an MSM pair once, and add to the other atom's sums in
+# memory.  A target between strong close charges (+2^47 at 0.5, -2^47 at 1.0: a
+# potential of about 2^47, whose last bit is 2^-5) and 2,000 unit charges 5.5 to
+# 7.8 away, each worth at most 0.011 there, under half that bit: added one by
+# one onto the strong pairs' sum they vanish (their potential is about 8, some
+# half of it by reactions).  The potential is linear in the charges, so the three
+# evaluations may differ by a few last bits only (16 allowed: the sums a lane
+# makes of 8 pairs and more before it adds them, the joins, the grid).  Which
+# atom's group evaluates the strong pairs depends on the sorted order, hence
+# several directions.
+def test_far_pairs_survive_beside_close_ones(dev):
+    from paper_1402_7216_gb300 import MSM
+    n, big = 2000, 2.0 ** 47
+    rng = np.random.default_rng(3)
+    plan = MSM(box=24.0, periodic=False, cutoff=8.0, spacing=2.0, order=3, splitting=2, precision="fp64",
+               max_atoms=n + 3)
+    strong, weak = np.zeros(n + 3), np.ones(n + 3)
+    strong[1:3] = big, -big
+    weak[1:3] = 0.0
+    Q = [torch.tensor(q, device=dev) for q in (strong + weak, strong, weak)]
+    for _ in range(24):
+        d = rng.normal(size=(n + 1, 3))
+        d /= np.linalg.norm(d, axis=1)[:, None]
+        near = np.outer([0.0, 0.5, -1.0], d[n])
+        far = d[:n] * (rng.uniform(5.5 ** 3, 7.8 ** 3, n) ** (1 / 3))[:, None]
+        P = torch.tensor(np.concatenate([near, far]) + 12.0, device=dev)
+        both, s, w = (plan.eval(P, q)[1][0].item() for q in Q)
+        assert 0.5 * big < s < 2 * big
+        assert abs((both - s) - w) <= 16 * 2.0 ** -5
+    plan.check_status()
