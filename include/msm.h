@@ -97,7 +97,8 @@ typedef struct {
  *                 warp takes 32 consecutive atoms of the sorted order as its
  *                 targets (runs across the cells of a row, which binning
  *                 sorts by x), 2 a warp takes one cell's atoms; 0 the
- *                 default, 1 on plans of at least 12,288 cells and 2 below.
+ *                 default, 1 for calls of at least 57,344 atoms on plans of at
+ *                 least 11,264 cells and 2 otherwise.
  *                 Runs need at least seven cells along x on a periodic plan
  *                 and fall back to cells otherwise
  *   lattice_txn, lattice_tyn  warp tile of the mixed-precision lattice

@@ -925,11 +925,22 @@ PairKArgs pair_kargs(const Plan& P) {
   return K;
 }
 
-// Whether the pair kernel takes runs of 32 atoms (else one cell per warp): a
-// periodic row must hold the piece's three cells beside its neighbours, or
-// the runs would fall into pieces of a few atoms.
-static bool use_runs(const Plan& P) {
-  return P.pair_runs && P.pair_targets != kCl && (!P.P.periodic || P.nc[0] >= P.row_cells + 2);
+// How the pair kernel shares its work, by the plan's cells and the call's atoms.
+// A plan of the default capacity has cells of half a cutoff, which may hold far
+// fewer atoms than the 24 that a plan of its system's own size gives them, so the
+// lines below lie on both (pair sums alone, us; cells of a/2, 0.3 to 32 atoms each).
+//
+// Runs of 32 atoms (else one cell per warp): a periodic row must hold the piece's
+// three cells beside its neighbours, or the runs would fall into pieces of a few
+// atoms.  By default from 11,264 cells and 57,344 atoms: at 24 atoms a cell runs
+// against cells take 271 and 254 at 7,980 cells, 552 and 621 at 12,167; with fewer
+// atoms than 152 SMs x 12 warps of 32 the chip waits for a run's pieces one after
+// another: 15,625 cells with 4,687 atoms 107 and 29, 31,250 113 and 94, 62,500 134
+// and 150, 12,167 cells with 48,668 atoms 122 and 115, 97,336 172 and 203.
+constexpr int64_t kRunCells = 11264, kRunAtoms = 57344;
+static bool use_runs(const Plan& P, int64_t n) {
+  const bool wanted = P.pair_runs == 1 || (P.pair_runs == 0 && P.ncell >= kRunCells && n >= kRunAtoms);
+  return wanted && P.pair_targets != kCl && (!P.P.periodic || P.nc[0] >= P.row_cells + 2);
 }
 
 // Boxes of fewer cells share each group among the four warps of a block: one
@@ -962,7 +973,7 @@ void launch_f2(Plan& P, int64_t n, cudaStream_t st, double alpha = 0.0) {
     else k_short_range_c8<3, kPairMSM><<<blocks, 32 * kWarps, 0, st>>>(K);
     return;
   }
-  K.runs = use_runs(P);
+  K.runs = use_runs(P, n);
   K.split = P.ncell < kSplitCells ? kWarps : 1;
   if (KIND == kPairCutoff) launch_mk<2, kPairCutoff>(P, K, st);  // M unused
   else if (KIND == kPairWolf) launch_mk<2, kPairWolf>(P, K, st);
@@ -1011,7 +1022,7 @@ cudaError_t pair_batch_build(const std::vector<BatchRep>& reps, PairBatch** out)
   for (const BatchRep& r : reps) {
     PairKArgs K = pair_kargs(*r.plan);
     K.natoms = (int)r.n;
-    K.runs = b->targets != kCl && use_runs(*r.plan);
+    K.runs = b->targets != kCl && use_runs(*r.plan, r.n);
     ka.push_back(K);
     kb.push_back(r.n > 0 ? pair_blocks(K) : 0);
     b->splitting = r.plan->P.splitting;

@@ -326,10 +326,7 @@ int build_plan(const msm_params* pp, const msm_tuning* tune, Plan* P) {
     P->cw[d] = p.box[d] / c;
   }
   P->ncell = P->nc[0] * P->nc[1] * P->nc[2];
-  // target runs by default on large boxes, where they were measured faster
-  // (1,600 against 1,727 us at 42,875 cells, 470 against 490 at 15,625; slower
-  // on smaller ones: 271 against 254 us at 7,980 cells)
-  P->pair_runs = TU.pair_runs == 1 || (TU.pair_runs == 0 && P->ncell >= 12288);
+  P->pair_runs = TU.pair_runs;
   std::vector<int4> offs;
   for (int oz = -2; oz <= 2; ++oz)
     for (int oy = -2; oy <= 2; ++oy)
