@@ -66,16 +66,7 @@ __device__ __forceinline__ void two_sum_add(T& s, T& c, T x) {
 }
 
 constexpr int kWarps = 4;
-#ifndef MSM_PAIR_BATCH
-#define MSM_PAIR_BATCH 64
-#endif
-#ifndef MSM_PAIR_AHEAD
-#define MSM_PAIR_AHEAD 4
-#endif
-#ifndef MSM_PAIR_MINB
-#define MSM_PAIR_MINB 5
-#endif
-constexpr int kBatch = MSM_PAIR_BATCH;  // sources per queue drain (pairs per lane per drain)
+constexpr int kBatch = 64;  // sources per queue drain (pairs per lane per drain)
 
 __device__ __forceinline__ float fast_rsqrt(float x) {  // one MUFU.RSQ; inputs are >= a^2/... never denormal
   float y;
@@ -643,8 +634,19 @@ __device__ __forceinline__ void short_range_c8_body(const PairKArgs& K, int blk)
 // into a ring in shared memory, each lane copying the records it will take.
 // A step is 64 sources, two per lane: the loop's state, the range's shift and
 // the chain load - cull - ballot - append are paid once for both.
-constexpr int kAhead = MSM_PAIR_AHEAD;  // a power of two
-constexpr int kStep = 64;               // sources per step
+constexpr int kStep = 64;  // sources per step
+// Where cells hold few atoms (flat_walk) most steps within one range would be
+// nearly empty, and a FLAT walk takes its sources across the ranges, each lane
+// keeping the ranges of its two sources.  Such walks are a few steps long: two in
+// flight are enough, and the smaller ring and 80 registers (six blocks an SM)
+// leave more cache and warps (27,000 cells of 4 atoms in runs: 229 us by ranges,
+// 217 across them with four steps in flight and five blocks, 181 so).
+template <bool FLAT>
+struct Walk {
+  static constexpr int kAhead = FLAT ? 2 : 4;      // steps in flight, a power of two
+  static constexpr int kMinBlocks = FLAT ? 6 : 5;  // resident blocks per SM
+};
+template <int kAhead>
 struct alignas(16) PairShared {
   QueueF queue;
   SegList segs;
@@ -663,7 +665,31 @@ __device__ __forceinline__ void copy_async4(void* dst, const void* src) {
                : "memory");
 }
 
-template <int M, int KIND>
+// The ranges laid end to end: rec becomes (first atom minus flat start, flat
+// end, .., ..); returns the number of sources.
+__device__ __forceinline__ int flatten_segments(SegList& L, int nseg, int lane) {
+  int total = 0;
+  for (int b = 0; b < nseg; b += 32) {
+    const int e = b + lane;
+    const int first = e < nseg ? L.rec[e].x : 0, len = e < nseg ? L.rec[e].y - first : 0;
+    int incl = len;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(kFull, incl, o);
+      if (lane >= o) incl += v;
+    }
+    if (e < nseg) {
+      L.rec[e].x = first - (total + incl - len);
+      L.rec[e].y = total + incl;
+    }
+    total += __shfl_sync(kFull, incl, 31);
+  }
+  __syncwarp();
+  return total;
+}
+
+// SHARE: the block's warps share a group (K.split of them).
+template <int M, int KIND, bool FLAT, bool SHARE>
 __device__ __forceinline__ void short_range_body(const PairKArgs& K, int blk) {
   const R4<float>* __restrict__ atoms = K.atoms;
   const float* __restrict__ cellx = K.cellx;
@@ -672,12 +698,13 @@ __device__ __forceinline__ void short_range_body(const PairKArgs& K, int blk) {
   const PairCoef C = K.C;
   const WolfC<float> W = K.W;
   const float cwx = K.cwx;
-  __shared__ PairShared shared[kWarps];
+  constexpr int kAhead = Walk<FLAT>::kAhead;
+  __shared__ PairShared<kAhead> shared[kWarps];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  PairShared& Sh = shared[warp];
+  PairShared<kAhead>& Sh = shared[warp];
   QueueF& Q = Sh.queue;
   SegList& L = Sh.segs;
-  const int split = K.split, part = split > 1 ? warp : 0;
+  const int split = SHARE ? K.split : 1, part = split > 1 ? warp : 0;
   const int group = split > 1 ? blk : blk * kWarps + warp;
   const int ncx = A.nc[0], ncy = A.nc[1];
   const float a2 = A.a2f;
@@ -722,7 +749,8 @@ __device__ __forceinline__ void short_range_body(const PairKArgs& K, int blk) {
     const float hx = warp_max(inp ? ai.x : -FAR), hy = warp_max(inp ? ai.y : -FAR), hz = warp_max(inp ? ai.z : -FAR);
     const float2 nax = make_float2(-ai.x, -ai.x), nay = make_float2(-ai.y, -ai.y), naz = make_float2(-ai.z, -ai.z);
     // the ranges of the neighbour rows, 64 sources per step (every split-th of
-    // them): fill() starts the copies of the next step into ring slot `slot`
+    // them), a step within one range or, FLAT, across ranges laid end to end:
+    // fill() starts the copies of the next step into ring slot `slot`
     const int nseg = build_segments(L, K, cx, cy, cz, span, lx, ly, lz, hx, hy, hz, lane);
     for (int e = lane; e < nseg; e += 32) {
       const int4 r = L.rec[e];
@@ -731,7 +759,36 @@ __device__ __forceinline__ void short_range_body(const PairKArgs& K, int blk) {
     __syncwarp();
     int seg = -1, jb = 0, je = 0, skip = part, steps = 0;  // steps: filled, not yet taken
     bool more = true;
+    // FLAT: sources in all ranges, the first source of the next step to fill and
+    // to take, and the ranges the lane's two sources lie in (it fills and takes
+    // the same ones); rec then holds atom minus flat index, and the flat end
+    int total = 0, tf = kStep * part, tt = tf, sf0 = 0, sf1 = 0, st0 = 0, st1 = 0;
+    if (FLAT) total = flatten_segments(L, nseg, lane);
+    auto range_of = [&](int t, int& e) {  // e: a range not after t's
+      while (L.rec[e].y <= t) ++e;
+    };
     auto fill = [&](int slot) {
+      if (FLAT) {
+        if (tf < total) {
+          const int t0 = tf + lane, t1 = t0 + 32;
+          if (t0 < total) {
+            range_of(t0, sf0);
+            const int j = L.rec[sf0].x + t0;
+            copy_async16(&Sh.ring[slot][lane], atoms + j);
+            copy_async4(&Sh.ringx[slot][lane], cellx + j);
+          }
+          if (t1 < total) {
+            range_of(t1, sf1);
+            const int j = L.rec[sf1].x + t1;
+            copy_async16(&Sh.ring[slot][lane + 32], atoms + j);
+            copy_async4(&Sh.ringx[slot][lane + 32], cellx + j);
+          }
+          tf += kStep * split;
+          ++steps;
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        return;
+      }
       while (more && jb >= je) {  // to the next range; its first `skip` steps are the other warps'
         if (seg >= 0) skip = (jb - je) / kStep;
         more = ++seg < nseg;
@@ -781,13 +838,25 @@ __device__ __forceinline__ void short_range_body(const PairKArgs& K, int blk) {
     for (int slot = 0; steps > 0; slot = (slot + 1) & (kAhead - 1)) {
       asm volatile("cp.async.wait_group %0;" ::"n"(kAhead - 1) : "memory");
       const R4<float> s0 = Sh.ring[slot][lane], s1 = Sh.ring[slot][lane + 32];
-      const int meta = Sh.ringseg[slot], n = meta >> 8;
-      const float4 sh = Sh.shift[meta & 255];
+      int n;
+      float4 sh, sh1;  // the ranges' shifts
+      if (FLAT) {
+        n = total - tt;
+        if (tt + lane < total) range_of(tt + lane, st0);
+        if (tt + lane + 32 < total) range_of(tt + lane + 32, st1);
+        tt += kStep * split;
+        sh = Sh.shift[st0];
+        sh1 = Sh.shift[st1];
+      } else {
+        const int meta = Sh.ringseg[slot];
+        n = meta >> 8;
+        sh = sh1 = Sh.shift[meta & 255];
+      }
       const float2 w = make_float2(cwx, cwx);
       const float2 x = __ffma2_rn(__fadd2_rn(make_float2(Sh.ringx[slot][lane], Sh.ringx[slot][lane + 32]),
-                                             make_float2(sh.x, sh.x)), w, make_float2(s0.x, s1.x));
-      const float2 y = __fadd2_rn(make_float2(s0.y, s1.y), make_float2(sh.y, sh.y));
-      const float2 z = __fadd2_rn(make_float2(s0.z, s1.z), make_float2(sh.z, sh.z));
+                                             make_float2(sh.x, sh1.x)), w, make_float2(s0.x, s1.x));
+      const float2 y = __fadd2_rn(make_float2(s0.y, s1.y), make_float2(sh.y, sh1.y));
+      const float2 z = __fadd2_rn(make_float2(s0.z, s1.z), make_float2(sh.z, sh1.z));
       __syncwarp();  // the slot's range has been read
       --steps;
       fill(slot);
@@ -860,17 +929,17 @@ __device__ __forceinline__ void short_range_body(const PairKArgs& K, int blk) {
   }
 }
 
-template <int M, int KIND>
-__global__ void __launch_bounds__(32 * kWarps, MSM_PAIR_MINB) k_short_range(const __grid_constant__ PairKArgs a) {
+template <int M, int KIND, bool FLAT, bool SHARE>
+__global__ void __launch_bounds__(32 * kWarps, Walk<FLAT>::kMinBlocks) k_short_range(const __grid_constant__ PairKArgs a) {
   pdl_sync();
-  short_range_body<M, KIND>(a, blockIdx.x);
+  short_range_body<M, KIND, FLAT, SHARE>(a, blockIdx.x);
 }
 
-template <int M>
-__global__ void __launch_bounds__(32 * kWarps, MSM_PAIR_MINB) kb_short_range(const PairKArgs* __restrict__ tab,
+template <int M, bool FLAT>
+__global__ void __launch_bounds__(32 * kWarps, Walk<FLAT>::kMinBlocks) kb_short_range(const PairKArgs* __restrict__ tab,
                                                                 const int* __restrict__ first, int nrep) {
   const int r = batch_rep(first, nrep, blockIdx.x);
-  short_range_body<M, kPairMSM>(tab[r], blockIdx.x - first[r]);
+  short_range_body<M, kPairMSM, FLAT, false>(tab[r], blockIdx.x - first[r]);
 }
 
 template <int M, int KIND>
@@ -943,11 +1012,22 @@ static bool use_runs(const Plan& P, int64_t n) {
   return wanted && P.pair_targets != kCl && (!P.P.periodic || P.nc[0] >= P.row_cells + 2);
 }
 
-// Boxes of fewer cells share each group among the four warps of a block: one
-// warp per group leaves most of the GPU idle (23,558 atoms, 1,000 cells: 52 ->
-// 45 us; 5,001 atoms, 216 cells: 42 -> 21 us; even at 50,001 atoms, 2,197
-// cells: 83 us; at 100,002 atoms 133 -> 141 us).
-constexpr int kSplitCells = 2048;
+// Sources across ranges (FLAT) below 8 atoms a cell, where a range (a row of 5
+// cells) rarely fills a step of 64: 12,167 cells of 1, 4, 8 and 12 atoms 75 -> 45,
+// 139 -> 115, 210 -> 203 and 291 -> 294; runs on 27,000 cells of 4 and 8 atoms
+// 229 -> 181 and 333 -> 339.
+static bool flat_walk(int64_t n, int64_t ncell) { return n < 8 * ncell; }
+
+// Small boxes share each group among the four warps of a block: one warp per group
+// leaves most of the GPU idle (23,558 atoms, 1,000 cells: 52 -> 45; 5,001 atoms,
+// 216 cells: 42 -> 21; at 50,001 atoms, 2,197 cells: 83; at 100,002 atoms 133 ->
+// 141).  With cells of few atoms the sharing ends earlier: 1,728 cells of 8 and 16
+// atoms 46 alone and 49 shared, 78 and 82 (Wolf 103 and 117, 164 and 208), of 24
+// atoms 147 and 113; 1,000 cells of 8 atoms 41 and 37.
+static int split_of(bool runs, int64_t n, int64_t ncell) {
+  const bool share = ncell < 1408 || (ncell < 2048 && (runs || n >= 18 * ncell));
+  return share ? kWarps : 1;
+}
 
 static int pair_blocks(const PairKArgs& K) {
   const int64_t groups = K.runs ? ((int64_t)K.natoms + 31) / 32 : K.ncell;
@@ -956,7 +1036,9 @@ static int pair_blocks(const PairKArgs& K) {
 
 template <int M, int KIND>
 void launch_mk(const Plan& P, const PairKArgs& K, cudaStream_t st) {
-  klaunch(P.pdl, k_short_range<M, KIND>, pair_blocks(K), 32 * kWarps, 0, st, K);
+  auto run = [&](auto kernel) { klaunch(P.pdl, kernel, pair_blocks(K), 32 * kWarps, 0, st, K); };
+  if (flat_walk(K.natoms, K.ncell)) run(K.split > 1 ? k_short_range<M, KIND, true, true> : k_short_range<M, KIND, true, false>);
+  else run(K.split > 1 ? k_short_range<M, KIND, false, true> : k_short_range<M, KIND, false, false>);
 }
 
 template <int KIND>
@@ -974,7 +1056,7 @@ void launch_f2(Plan& P, int64_t n, cudaStream_t st, double alpha = 0.0) {
     return;
   }
   K.runs = use_runs(P, n);
-  K.split = P.ncell < kSplitCells ? kWarps : 1;
+  K.split = split_of(K.runs, n, P.ncell);
   if (KIND == kPairCutoff) launch_mk<2, kPairCutoff>(P, K, st);  // M unused
   else if (KIND == kPairWolf) launch_mk<2, kPairWolf>(P, K, st);
   else if (P.P.splitting == 1) launch_mk<1, kPairMSM>(P, K, st);
@@ -1010,6 +1092,7 @@ struct PairBatch {
   BatchTable<PairKArgs> cells;  // kWarps groups per block
   int splitting = 2;
   int targets = 8;  // the first replica's pair_targets
+  bool flat = false;
 };
 
 cudaError_t pair_batch_build(const std::vector<BatchRep>& reps, PairBatch** out) {
@@ -1018,6 +1101,7 @@ cudaError_t pair_batch_build(const std::vector<BatchRep>& reps, PairBatch** out)
   if (!b) return cudaErrorMemoryAllocation;
   std::vector<PairKArgs> ka;
   std::vector<int> kb;
+  int64_t natoms = 0, ncell = 0;
   if (!reps.empty()) b->targets = reps[0].plan->pair_targets;
   for (const BatchRep& r : reps) {
     PairKArgs K = pair_kargs(*r.plan);
@@ -1026,7 +1110,10 @@ cudaError_t pair_batch_build(const std::vector<BatchRep>& reps, PairBatch** out)
     ka.push_back(K);
     kb.push_back(r.n > 0 ? pair_blocks(K) : 0);
     b->splitting = r.plan->P.splitting;
+    natoms += r.n;
+    ncell += K.ncell;
   }
+  b->flat = flat_walk(natoms, ncell);
   cudaError_t e = make_table(b->cells, ka, kb);
   if (e != cudaSuccess) {
     pair_batch_free(b);
@@ -1046,9 +1133,10 @@ cudaError_t pair_batch_launch(PairBatch* b, cudaStream_t st) {
     else kb_short_range_c8<3><<<nb, 32 * kWarps, 0, st>>>(t.args, t.first, t.nrep);
     return cudaGetLastError();
   }
-  if (b->splitting == 1) kb_short_range<1><<<nb, 32 * kWarps, 0, st>>>(t.args, t.first, t.nrep);
-  else if (b->splitting == 2) kb_short_range<2><<<nb, 32 * kWarps, 0, st>>>(t.args, t.first, t.nrep);
-  else kb_short_range<3><<<nb, 32 * kWarps, 0, st>>>(t.args, t.first, t.nrep);
+  auto run = [&](auto kernel) { kernel<<<nb, 32 * kWarps, 0, st>>>(t.args, t.first, t.nrep); };
+  if (b->splitting == 1) run(b->flat ? kb_short_range<1, true> : kb_short_range<1, false>);
+  else if (b->splitting == 2) run(b->flat ? kb_short_range<2, true> : kb_short_range<2, false>);
+  else run(b->flat ? kb_short_range<3, true> : kb_short_range<3, false>);
   return cudaGetLastError();
 }
 
