@@ -2299,8 +2299,8 @@ struct GridBatch {
   FftBatch* fft[2] = {nullptr, nullptr};  // the FFT form, when every replica's plan took it
   BatchTable<TopKArgs> top[2];
   std::vector<BatchTable<AxisKArgs<float>>> prol[2];  // [dir][3 k + pass] (persistent chains)
-  // one launch per level: restriction where every replica's level is small
-  // enough (else the axis passes), prolongation
+  // one launch per level (without persistent chains): restriction where every
+  // replica's level is small enough (else the axis passes), prolongation
   std::vector<BatchTable<TileKArgs<double>>> restr_tile[2];
   std::vector<BatchTable<TileKArgs<float>>> prol_tile[2];
   BatchTable<InterpKArgs<float, double>> interp[2];
@@ -2353,6 +2353,7 @@ cudaError_t grid_batch_build(const std::vector<BatchRep>& reps, bool backward, G
   const int R = (int)reps.size();
   B->order = reps.empty() ? 3 : reps[0].plan->P.order;
   B->has_backward = backward;
+  const bool chains = !reps.empty() && reps[0].plan->batch_persistent;  // restriction and prolongation
   for (const BatchRep& r : reps) B->maxlev = std::max(B->maxlev, r.plan->levels);
   cudaError_t e = cudaSuccess;
   auto chk = [&](cudaError_t x) {
@@ -2424,10 +2425,17 @@ cudaError_t grid_batch_build(const std::vector<BatchRep>& reps, bool backward, G
       fb.push_back(ew_blocks(np));
     }
     chk(make_table(B->fx[dir], fa, fb));
-    // restriction k -> k+1: three axis passes (fine -> tmp[0] -> tmp[1] -> coarse), FP64
+    // restriction k -> k+1, FP64: tiles (one launch) where every replica's level
+    // is small enough, else three axis passes (fine -> tmp[0] -> tmp[1] -> coarse),
+    // which the persistent chains take on every level
     B->restr[dir].resize(3 * std::max(B->maxlev - 1, 0));
-    for (int k = 0; k + 1 < B->maxlev; ++k)
-      for (int ax = 0; ax < 3; ++ax) {
+    B->restr_tile[dir].resize(std::max(B->maxlev - 1, 0));
+    B->prol_tile[dir].resize(std::max(B->maxlev - 1, 0));
+    for (int k = 0; k + 1 < B->maxlev; ++k) {
+      bool small = !chains;
+      for (const BatchRep& r : reps)
+        if (k + 1 < r.plan->levels) small = small && restrict_by_tiles(grid_points(*r.plan, k + 1));
+      for (int ax = 0; ax < 3 && !small; ++ax) {
         std::vector<AxisKArgs<double>> ra;
         std::vector<int> rb;
         for (const BatchRep& r : reps) {
@@ -2457,13 +2465,10 @@ cudaError_t grid_batch_build(const std::vector<BatchRep>& reps, bool backward, G
         }
         chk(make_table(B->restr[dir][3 * k + ax], ra, rb));
       }
-    B->restr_tile[dir].resize(std::max(B->maxlev - 1, 0));
-    B->prol_tile[dir].resize(std::max(B->maxlev - 1, 0));
-    for (int k = 0; k + 1 < B->maxlev; ++k) {
+      if (chains) continue;  // restriction and prolongation run as persistent chains
       std::vector<TileKArgs<double>> ra;
       std::vector<TileKArgs<float>> pa;
       std::vector<int> rb, pb;
-      bool small = true;
       for (const BatchRep& r : reps) {
         Plan& P = *r.plan;
         TileKArgs<double> a{};
@@ -2472,7 +2477,6 @@ cudaError_t grid_batch_build(const std::vector<BatchRep>& reps, bool backward, G
         if (k + 1 < P.levels) {
           void* const* q = dir ? P.d.aq : P.d.gq;
           void* const* u = dir ? P.d.au : P.d.gu;
-          small = small && restrict_by_tiles(grid_points(P, k + 1));
           a = TileKArgs<double>{(const double*)q[k], (double*)q[k + 1], grid3_args(P, k, k + 1)};
           na = (int)restrict_tiles(P.n[k + 1]);
           p = TileKArgs<float>{(const float*)u[k + 1], (float*)u[k], grid3_args(P, k + 1, k)};
@@ -2601,9 +2605,10 @@ cudaError_t grid_batch_build(const std::vector<BatchRep>& reps, bool backward, G
       }
       chk(make_table(B->top[dir], ta, tb));
     }
-    // prolongation k+1 -> k: three passes (coarse -> tmp[0] -> tmp[1] -> fine, the last one adding), FP32
+    // prolongation k+1 -> k in the persistent chains: three passes (coarse ->
+    // tmp[0] -> tmp[1] -> fine, the last one adding), FP32
     B->prol[dir].resize(3 * std::max(B->maxlev - 1, 0));
-    for (int k = B->maxlev - 2; k >= 0; --k)
+    for (int k = B->maxlev - 2; k >= 0 && chains; --k)
       for (int i = 0; i < 3; ++i) {
         std::vector<AxisKArgs<float>> pa;
         std::vector<int> pb;
@@ -2661,7 +2666,7 @@ cudaError_t grid_batch_build(const std::vector<BatchRep>& reps, bool backward, G
   (void)R;
   // persistent chains (replica 0's plan asks for them): one cooperative launch
   // per chain, as many blocks as are co-resident
-  if (e == cudaSuccess && !reps.empty() && reps[0].plan->batch_persistent) {
+  if (e == cudaSuccess && chains) {
     const bool o3 = B->order == 3;
     int dev = 0, nsm = 0, per_r = 0, per_p = 0;
     chk(cudaGetDevice(&dev));
