@@ -36,8 +36,7 @@
 // parity fills the ring with sources few lanes take (21.5 ms, and 3,000 atoms
 // 140 us).
 // The reciprocal square root is seeded by the FP32 one and refined once by
-// Halley's third-order iteration (5 FP64 instructions, error below 1 ulp more
-// than half a rounding).
+// Halley's third-order iteration (5 FP64 instructions, error below 1 ulp).
 //
 // A group of T = 8 or 16 consecutive sorted atoms is a warp's targets,
 // 32 / T lanes sharing one (each tests every (32 / T)-th source); small systems
@@ -99,7 +98,7 @@ __device__ __forceinline__ float trunc_scaled(double x, int esc) {
 // 1 / sqrt(x), x > 0 and normal: the FP32 approximation of the mantissa, its
 // exponent halved with integers, then y (1 + r/2 + 3 r^2/8), r = 1 - x y^2
 // (Halley's iteration; the next term, 5 r^3/16 with |r| < 2^-21, is below
-// 2^-64).
+// 2^-64).  The rounding of x y and the last one are half an ulp each at most.
 __device__ __forceinline__ double rsqrt_halley(double x) {
   const int hi = __double2hiint(x);
   const int e = (hi >> 20) - 1023, odd = e & 1;
