@@ -37,10 +37,14 @@ def _stream(stream):
 
 def _raw_stream(stream):
     """The stream's handle as an integer (the current stream's without making
-    a Stream object, which costs several microseconds)."""
+    a Stream object, which costs several microseconds, where this torch has the
+    call for it; its name is not public)."""
     if stream is not None:
         return stream.cuda_stream
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    current = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if current is None:
+        return torch.cuda.current_stream().cuda_stream
+    return current(torch.cuda.current_device())
 
 
 def _addr(t):
