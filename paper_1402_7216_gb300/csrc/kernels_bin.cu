@@ -1,7 +1,8 @@
 // kernels_bin.cu -- atom binning (link cells, Sec. "Short-range interactions":
 // atoms are binned into cells so that each atom only examines nearby cells).
 //
-// A counting sort over cells in five launches:
+// A counting sort over cells in five launches (four on plans of up to 4,096
+// cells, whose scan is one chunk):
 //   k_bin_count    cell key of every atom; a provisional rank inside the cell
 //                  from one warp-aggregated atomic per (warp, cell)
 //   k_cell_sums    per-chunk sums of the cell counts

@@ -826,7 +826,7 @@ __global__ void __launch_bounds__(kLat64) k_lattice64(const double* __restrict__
 // per two outputs).  Coarse levels with few bricks split the input planes over
 // several blocks (nsplit): block part writes its partial sums to
 // up[part][point] and k_lattice_reduce adds the parts in order.
-constexpr int LBX = 32;         // window of the FP64 form's support check (plan geometry)
+constexpr int LBX = 32;         // see lattice_fits
 constexpr int kLatticeLP = 8;   // x outputs per lane of the FP32 lattice kernel (8 or 16)
 constexpr int kLatticeZ = 4;    // warps (output planes) per block of the FP32 lattice kernel
 constexpr size_t kLatticeSmemMax = 200 * 1024;  // dynamic shared memory the FP32 lattice kernels may use
@@ -1823,6 +1823,8 @@ int64_t lattice_parts_elems(const Plan& P) {
   return m;
 }
 
+// The FP64 kernel needs no shared memory; the line is that of the stencils its
+// plans accept (2a/h up to about 27 spacings), as its 48 KB window once set it.
 bool lattice_fits(const Plan& P) {
   if (P.fp64) {
     const int SX = (LBX + 2 * P.E[0] + kSeg) | 1, SY = 8 + 2 * P.E[1];

@@ -1022,8 +1022,8 @@ static bool flat_walk(int64_t n, int64_t ncell) { return n < 8 * ncell; }
 // leaves most of the GPU idle (23,558 atoms, 1,000 cells: 52 -> 45; 5,001 atoms,
 // 216 cells: 42 -> 21; at 50,001 atoms, 2,197 cells: 83; at 100,002 atoms 133 ->
 // 141).  With cells of few atoms the sharing ends earlier: 1,728 cells of 8 and 16
-// atoms 46 alone and 49 shared, 78 and 82 (Wolf 103 and 117, 164 and 208), of 24
-// atoms 147 and 113; 1,000 cells of 8 atoms 41 and 37.
+// atoms 46 alone and 49 shared, 74 and 82 (Wolf 102 and 117, 157 and 208), of 24
+// atoms 147 (by the kernel without sharing) and 113; 1,000 cells of 8 atoms 41 and 37.
 static int split_of(bool runs, int64_t n, int64_t ncell) {
   const bool share = ncell < 1408 || (ncell < 2048 && (runs || n >= 18 * ncell));
   return share ? kWarps : 1;

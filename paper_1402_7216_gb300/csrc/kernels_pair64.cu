@@ -24,17 +24,18 @@
 // takes_pair() names meets the other's atoms, and adds to their reaction sums
 // with FP64 reductions (fire and forget; at most 4 per 27 FP64 instructions, and
 // gathering them to whole sectors first made no difference).  An atom has two
-// reaction sums, for pairs nearer and farther than kNear a: the many small terms
-// of the far pairs would else round onto the few large ones (force error of
-// 3,000 atoms 4.3e-16 with every pair from both atoms, 6.8e-16 with one sum that
-// also took the atom's own total, 4.4e-16 with the two, at the same speed).  Against each atom for itself:
-// 1M atoms at water density 31.7 -> 20.9 ms (the FP64 pipe alone would take
-// 17 ms), 23,558 atoms 900 -> 614 us, 3,000 atoms 153 -> 110 us.  The choice by
-// group index halves the sources staged and tested too; "the earlier atom" would
-// give an atom at the top of its cell far fewer pairs than one at the bottom,
-// with the lanes waiting for the fullest list (25.6 ms), and a choice by atom
-// parity fills the ring with sources few lanes take (21.5 ms, and 3,000 atoms
-// 140 us).
+// reaction sums, for near and far pairs (kNear2), beside its own total: the many
+// small terms of the far pairs would else round onto the few large ones (force
+// error of 3,000 atoms 4.3e-16 with every pair from both atoms, 6.8e-16 with one
+// sum that also took the atom's own total, 4.4e-16 with the three, at the same
+// speed).  Against each atom for itself: 1,066,628 atoms (a = 12) 36.4 -> 24.0 ms
+// (the FP64 pipe alone would take 18.4), 100,000 (a = 10) 2.63 -> 1.63 ms, 23,558
+// 735 -> 533 us, 3,000 open 154 -> 114 us.  The choice by group index halves the
+// sources staged and tested too.  At a million atoms where it takes 20.9 ms, "the
+// earlier atom" takes 25.6 (an atom at the top of its cell has far fewer later
+// neighbours than one at the bottom, and the lanes wait for the fullest list), and
+// a choice by atom parity 21.5 (the ring fills with sources few lanes take; 3,000
+// atoms 140 against 110 us).
 // The reciprocal square root is seeded by the FP32 one and refined once by
 // Halley's third-order iteration (5 FP64 instructions, error below 1 ulp).
 //
@@ -331,14 +332,14 @@ __global__ void __launch_bounds__(32 * kMaxSplit) k_pair64(const __grid_constant
 }
 
 // Targets per group and warps per group: groups of 16 once they make 152 SMs x
-// 8 warps, else groups of 8, then several warps per group.  Groups of 32 are
-// the same at 1M atoms (20.9 against 20.8 ms) and leave the chip waiting for
-// its last warps below (200,000 atoms 4.46 against 4.24 ms, 100,000 2,419
-// against 2,185 us, 50,000 1,429 against 1,178); groups of 8 stage each source
-// for fewer targets (1M 22.1 ms; at 23,558 566 against 611 us alone, but 663
-// against 653 us an evaluation with gradients).  Warps per group at 3,000
-// atoms: 214, 126, 108 and 114 us with 1, 2, 4 and 8; at 6,000 241, 180, 190
-// and 219.
+// 8 warps, else groups of 8, then several warps per group.  Pair sums alone with
+// groups of 8, 16 and 32: 12,000 atoms 320, 439 and 716 us, 23,558 502, 533 and 798
+// (groups of 8 stage each source for fewer targets, and beside the grid passes an
+// evaluation with gradients takes 663 against 653 us), 50,000 942, 1,004 and 1,233,
+// 100,000 1.65, 1.63 and 1.87 ms, 200,000 3.12, 2.92 and 3.12, 1,066,628 25.5, 24.0
+// and 24.1 (groups of 32 leave the chip waiting for its last warps).  Warps per
+// group of 8, 1, 2, 4 and 8: 3,000 atoms 231, 135, 113 and 117 us; 6,000 262, 191,
+// 206 and 214.
 void group_shape(int64_t n, int& lt, int& nsplit) {
   constexpr int64_t kFill = 152 * 8;
   lt = (n + 15) >> 4 >= kFill ? 4 : 3;
