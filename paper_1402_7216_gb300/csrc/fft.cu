@@ -17,7 +17,8 @@
 // n0 / 2 + 1 columns of non-negative frequency are kept: the x passes take two
 // real rows as one complex line (the transforms separate by symmetry), and the
 // y and z passes have half the lines (the 4.1M-atom box's sweep, 240^3 ..
-// 30^3, took 770 us with full complex grids and takes 385 us).
+// 30^3, took 770 us with full complex grids and 385 us so; 410 us with the
+// smoothing of kEdge).
 // Each pass is one launch over every lattice level of a plan (or of every
 // replica of a batch), a table of per-level arguments mapping blocks to
 // levels.  The 1-D transforms are mixed-radix Stockham FFTs (radices 4, 2,
