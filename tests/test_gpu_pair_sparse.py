@@ -2,8 +2,7 @@
 default capacity leaves cells of half a cutoff), on both sides of each line of
 its dispatch: sources taken across ranges below 8 atoms a cell, a group shared by
 four warps or not at 1,728 cells, runs of atoms from 57,344 atoms on.  Against
-the oracle at the mixed path's tolerances (force rel-RMS 1e-5, potential 1e-6;
-the cutoff method outside the shell of pairs within rounding of the cutoff)."""
+the oracle at the mixed path's tolerances (force rel-RMS 1e-5, potential 1e-6)."""
 import numpy as np
 import pytest
 
