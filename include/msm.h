@@ -98,7 +98,8 @@ typedef struct {
  *                 targets (runs across the cells of a row, which binning
  *                 sorts by x), 2 a warp takes one cell's atoms; 0 the
  *                 default, 1 for calls of at least 57,344 atoms on plans of at
- *                 least 11,264 cells and 2 otherwise.
+ *                 least 11,264 cells, 1 on plans of at least 16,384 cells, and
+ *                 2 otherwise.
  *                 Runs need at least seven cells along x on a periodic plan
  *                 and fall back to cells otherwise
  *   lattice_txn, lattice_tyn  warp tile of the mixed-precision lattice

@@ -5,7 +5,8 @@ The tunables change speed, never results beyond summation order:
                  or 8 (clusters of 8 consecutive atoms)
   pair_runs      with 32: a warp's targets are one cell's atoms (2) or 32
                  consecutive atoms of an x-sorted cell row (1); the default
-                 takes runs from 57,344 atoms on plans of at least 11,264 cells
+                 takes runs from 57,344 atoms on plans of at least 11,264 cells,
+                 and on plans of at least 16,384
   cell_fill      target atoms per short-range cell (pair-kernel lane use vs
                  candidate volume)
   patch_cells    cells per side of the anterpolation/interpolation patch blocks

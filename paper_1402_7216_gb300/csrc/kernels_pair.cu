@@ -1005,10 +1005,15 @@ PairKArgs pair_kargs(const Plan& P) {
 // against cells take 271 and 254 at 7,980 cells, 552 and 621 at 12,167; with fewer
 // atoms than 152 SMs x 12 warps of 32 the chip waits for a run's pieces one after
 // another: 15,625 cells with 4,687 atoms 107 and 29, 31,250 113 and 94, 62,500 134
-// and 150, 12,167 cells with 48,668 atoms 122 and 115, 97,336 172 and 203.
-constexpr int64_t kRunCells = 11264, kRunAtoms = 57344;
+// and 150, 12,167 cells with 48,668 atoms 122 and 115, 97,336 172 and 203.  From
+// 16,384 cells on always: there a system may well be a cluster in a great box, in
+// few cells of many atoms (a droplet of 5,000 atoms in 42,875 cells of 11.4, a = 8:
+// calls of the cutoff method 100 with runs, 304 with a warp per cell; 5,000 spread
+// evenly 115 and 63).
+constexpr int64_t kRunCells = 11264, kRunAtoms = 57344, kRunCellsAlways = 16384;
 static bool use_runs(const Plan& P, int64_t n) {
-  const bool wanted = P.pair_runs == 1 || (P.pair_runs == 0 && P.ncell >= kRunCells && n >= kRunAtoms);
+  const bool many = P.ncell >= kRunCellsAlways || (P.ncell >= kRunCells && n >= kRunAtoms);
+  const bool wanted = P.pair_runs == 1 || (P.pair_runs == 0 && many);
   return wanted && P.pair_targets != kCl && (!P.P.periodic || P.nc[0] >= P.row_cells + 2);
 }
 

@@ -60,11 +60,12 @@ def test_sparse_cells_match_oracle(cells, n, periodic, runs, dev):
 
 
 # Cells and runs sum in different orders, so the bits tell which of the two the
-# default took: runs leave most of the chip waiting below 57,344 atoms.
-@pytest.mark.parametrize("cells,n,same", [(25, 5000, 2), (23, 57343, 2), (23, 57344, 1)], ids=str)
+# default took: below 16,384 cells runs leave most of the chip waiting unless there
+# are 57,344 atoms.
+@pytest.mark.parametrize("cells,n,same", [(25, 5000, 2), (23, 57343, 2), (23, 57344, 1), (26, 5000, 1)], ids=str)
 def test_default_takes_runs_by_atoms(cells, n, same, dev):
     box = 4.001 * cells
-    pos, q = gas(n, box, seed=n)
+    pos, q = gas(n, min(box, 92.0), seed=n)  # dense enough for sums whose order shows
     P = torch.tensor(pos, device=dev), torch.tensor(q, device=dev)
     F = {r: plan_of(box, True, pair_runs=r).cutoff_eval(*P)[2] for r in (0, 1, 2)}
     assert torch.equal(F[0], F[same]) and not torch.equal(F[0], F[3 - same])
