@@ -915,8 +915,9 @@ __device__ __forceinline__ void short_range_body(const PairKArgs& K, int blk) {
         mine[c][32 + lane] = comp[c];
       }
       __syncthreads();
+      tot = Totals();
       if (part == 0)
-        for (int p = 1; p < split; ++p) tot.join(shared[p].queue, lane);
+        for (int p = 0; p < split; ++p) tot.join(shared[p].queue, lane);
       __syncthreads();
     }
     const float phi = tot.phi + tot.cphi, px = tot.x + tot.cx, py = tot.y + tot.cy, pz = tot.z + tot.cz;
@@ -929,8 +930,14 @@ __device__ __forceinline__ void short_range_body(const PairKArgs& K, int blk) {
   }
 }
 
+// Wolf's pair function is short of registers where the warps also join their
+// totals: four blocks with 128 of them instead of five with 96 (calls at 3,000 atoms
+// open 55 -> 47 us, 23,558 with a = 20 515 -> 453, with a = 10 123 -> 125).
+template <int KIND, bool FLAT, bool SHARE>
+constexpr int kPairBlocks = KIND == kPairWolf && SHARE && !FLAT ? 4 : Walk<FLAT>::kMinBlocks;
+
 template <int M, int KIND, bool FLAT, bool SHARE>
-__global__ void __launch_bounds__(32 * kWarps, Walk<FLAT>::kMinBlocks) k_short_range(const __grid_constant__ PairKArgs a) {
+__global__ void __launch_bounds__(32 * kWarps, kPairBlocks<KIND, FLAT, SHARE>) k_short_range(const __grid_constant__ PairKArgs a) {
   pdl_sync();
   short_range_body<M, KIND, FLAT, SHARE>(a, blockIdx.x);
 }
