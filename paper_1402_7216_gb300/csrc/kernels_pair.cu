@@ -839,24 +839,29 @@ __device__ __forceinline__ void short_range_body(const PairKArgs& K, int blk) {
       asm volatile("cp.async.wait_group %0;" ::"n"(kAhead - 1) : "memory");
       const R4<float> s0 = Sh.ring[slot][lane], s1 = Sh.ring[slot][lane + 32];
       int n;
-      float4 sh, sh1;  // the ranges' shifts
-      if (FLAT) {
+      float2 shx, shy, shz;  // the shifts of the two sources' ranges
+      if constexpr (FLAT) {
         n = total - tt;
         if (tt + lane < total) range_of(tt + lane, st0);
         if (tt + lane + 32 < total) range_of(tt + lane + 32, st1);
         tt += kStep * split;
-        sh = Sh.shift[st0];
-        sh1 = Sh.shift[st1];
+        const float4 a = Sh.shift[st0], b = Sh.shift[st1];
+        shx = make_float2(a.x, b.x);
+        shy = make_float2(a.y, b.y);
+        shz = make_float2(a.z, b.z);
       } else {
         const int meta = Sh.ringseg[slot];
         n = meta >> 8;
-        sh = sh1 = Sh.shift[meta & 255];
+        const float4 a = Sh.shift[meta & 255];
+        shx = make_float2(a.x, a.x);
+        shy = make_float2(a.y, a.y);
+        shz = make_float2(a.z, a.z);
       }
       const float2 w = make_float2(cwx, cwx);
-      const float2 x = __ffma2_rn(__fadd2_rn(make_float2(Sh.ringx[slot][lane], Sh.ringx[slot][lane + 32]),
-                                             make_float2(sh.x, sh1.x)), w, make_float2(s0.x, s1.x));
-      const float2 y = __fadd2_rn(make_float2(s0.y, s1.y), make_float2(sh.y, sh1.y));
-      const float2 z = __fadd2_rn(make_float2(s0.z, s1.z), make_float2(sh.z, sh1.z));
+      const float2 x = __ffma2_rn(__fadd2_rn(make_float2(Sh.ringx[slot][lane], Sh.ringx[slot][lane + 32]), shx), w,
+                                  make_float2(s0.x, s1.x));
+      const float2 y = __fadd2_rn(make_float2(s0.y, s1.y), shy);
+      const float2 z = __fadd2_rn(make_float2(s0.z, s1.z), shz);
       __syncwarp();  // the slot's range has been read
       --steps;
       fill(slot);
@@ -1027,8 +1032,16 @@ static bool use_runs(const Plan& P, int64_t n) {
 // Sources across ranges (FLAT) below 8 atoms a cell, where a range (a row of 5
 // cells) rarely fills a step of 64: 12,167 cells of 1, 4, 8 and 12 atoms 75 -> 45,
 // 139 -> 115, 210 -> 203 and 291 -> 294; runs on 27,000 cells of 4 and 8 atoms
-// 229 -> 181 and 333 -> 339.
-static bool flat_walk(int64_t n, int64_t ncell) { return n < 8 * ncell; }
+// 229 -> 181 and 333 -> 339.  Not for runs on smaller boxes (4,096 cells of 4 and 8
+// atoms 102 and 105, 107 and 119: too few warps for a ring of two), nor where the
+// capacity and not the cutoff set the cells' width: so few atoms there are a cluster
+// in a great box, in full cells (20,000 atoms in 42,875 cells of 8.6, a = 10, calls of
+// the cutoff method 98 and 120).
+static bool flat_walk(const Plan& P, int64_t n, bool runs) {
+  const double a = P.P.cutoff;
+  const bool narrow = P.cw[0] * P.cw[1] * P.cw[2] < 0.216 * a * a * a;  // cells of up to 0.6 a
+  return n < 8 * (int64_t)P.ncell && narrow && (!runs || P.ncell >= kRunCellsAlways);
+}
 
 // Small boxes share each group among the four warps of a block: one warp per group
 // leaves most of the GPU idle (23,558 atoms, 1,000 cells: 52 -> 45; 5,001 atoms,
@@ -1049,7 +1062,7 @@ static int pair_blocks(const PairKArgs& K) {
 template <int M, int KIND>
 void launch_mk(const Plan& P, const PairKArgs& K, cudaStream_t st) {
   auto run = [&](auto kernel) { klaunch(P.pdl, kernel, pair_blocks(K), 32 * kWarps, 0, st, K); };
-  if (flat_walk(K.natoms, K.ncell)) run(K.split > 1 ? k_short_range<M, KIND, true, true> : k_short_range<M, KIND, true, false>);
+  if (flat_walk(P, K.natoms, K.runs)) run(K.split > 1 ? k_short_range<M, KIND, true, true> : k_short_range<M, KIND, true, false>);
   else run(K.split > 1 ? k_short_range<M, KIND, false, true> : k_short_range<M, KIND, false, false>);
 }
 
@@ -1113,7 +1126,7 @@ cudaError_t pair_batch_build(const std::vector<BatchRep>& reps, PairBatch** out)
   if (!b) return cudaErrorMemoryAllocation;
   std::vector<PairKArgs> ka;
   std::vector<int> kb;
-  int64_t natoms = 0, ncell = 0;
+  int64_t sparse = 0, dense = 0;
   if (!reps.empty()) b->targets = reps[0].plan->pair_targets;
   for (const BatchRep& r : reps) {
     PairKArgs K = pair_kargs(*r.plan);
@@ -1122,10 +1135,10 @@ cudaError_t pair_batch_build(const std::vector<BatchRep>& reps, PairBatch** out)
     ka.push_back(K);
     kb.push_back(r.n > 0 ? pair_blocks(K) : 0);
     b->splitting = r.plan->P.splitting;
-    natoms += r.n;
-    ncell += K.ncell;
+    // one kernel for all replicas: the walk that suits most of their atoms
+    (flat_walk(*r.plan, r.n, K.runs) ? sparse : dense) += r.n;
   }
-  b->flat = flat_walk(natoms, ncell);
+  b->flat = sparse > dense;
   cudaError_t e = make_table(b->cells, ka, kb);
   if (e != cudaSuccess) {
     pair_batch_free(b);
