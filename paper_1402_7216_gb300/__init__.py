@@ -41,10 +41,10 @@ def _raw_stream(stream):
     call for it; its name is not public)."""
     if stream is not None:
         return stream.cuda_stream
-    current = getattr(torch._C, "_cuda_getCurrentRawStream", None)
-    if current is None:
+    try:
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    except AttributeError:
         return torch.cuda.current_stream().cuda_stream
-    return current(torch.cuda.current_device())
 
 
 def _addr(t):
